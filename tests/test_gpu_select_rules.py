@@ -243,3 +243,30 @@ def test_rownorm_threshold_matches_oracle(w):
         vb.vmoba_select_rule_apply(L.shape, L.scores, vb.SELECT_THRESHOLD_GLOBAL_ROWNORM, 0.25, 1, L.mask_bits, L.kb_ptr,
                                    L.q_idx, L.q_ptr, L.q_pairs, L.capacity, L.k_per_head, L.cutoff, L.dev_status,
                                    L.ws[:vb.workspace_bytes(L.shape, vb.STAGE_SELECT, 0)])
+
+
+@pytest.mark.parametrize("n_blocks", [1, 8, 9, 16, 24, 25, 32, 33, 64, 65, 140, 280, 320, 513, 1024])
+def test_topk_local_row_lengths_ties_and_infinite_scores(n_blocks):
+    """Every instantiation of the top-k kernels (rows of up to 32 blocks by thread, longer ones by warp) at the edges of
+    its range, with k from one block to all; scores of three kinds in one head: continuous, quantised to a few values
+    (ties at the cutoff) and with infinities (blocks a caller has ruled out)."""
+    S, heads = 192, 2
+    grid = (n_blocks, 1, S // n_blocks) if S % n_blocks == 0 else (n_blocks, 1, 1)
+    shape = vb.make_shape(1, heads, 128, grid, (1, 1, grid[2]), "bf16")
+    S = shape.S
+    rng = np.random.default_rng(n_blocks)
+    sc = (3.0 * rng.standard_normal((heads, S, n_blocks))).astype(np.float32)
+    sc[:, 1::3] = np.round(sc[:, 1::3])
+    sc[:, 2::6][rng.random(sc[:, 2::6].shape) < 0.4] = -np.inf
+    sc[:, 5::6][rng.random(sc[:, 5::6].shape) < 0.1] = np.inf
+    L = VmobaLayer(shape, capacity=heads * S * n_blocks)
+    L.scores.copy_(torch.from_numpy(sc.reshape(1, heads, S, n_blocks)))
+    for k in sorted({1, 2, max(1, n_blocks // 3), max(1, n_blocks - 1), n_blocks}):
+        L.dev_status.zero_()
+        L.select_rule(vb.SELECT_TOPK_LOCAL, topk=k)
+        L.check_status()
+        got = U.unpack_mask(L.mask_bits, heads, S, n_blocks)
+        for h in range(heads):
+            ref = orc.select_topk_per_query(sc[h], k)
+            assert np.array_equal(got[h], ref), (k, h)
+            assert float(L.cutoff[h]) == float(sc[h][ref].min())
