@@ -19,12 +19,12 @@ int tc_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, co
 int tc_dense_fwd(const Dims& D, const void* q, const void* k, const void* v, void* o, void* o_resid, float* lse,
                  int32_t* status, cudaStream_t st);
 
-// attn_tc_bwd.cu: tensor-core backward kernels (bf16, head_dim 128)
+// attn_tc_bwd.cu: tensor-core backward kernel (bf16, head_dim 128)
 int tc_sparse_bwd(const Dims& D, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
                   const float* Dv, const int* kb_ptr, const int* q_idx, long long cap, float* dq_acc, void* dk, void* dv,
                   int32_t* status, cudaStream_t st, const RowMap& out_map, const RowMap& do_map);
 int tc_dense_bwd(const Dims& D, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
-                 const float* Dv, void* dq, void* dk, void* dv, int32_t* status, cudaStream_t st);
+                 const float* Dv, float* dq_acc, void* dk, void* dv, int32_t* status, cudaStream_t st);
 
 static bool use_tensor_cores(const Dims& D) { return D.dtype == VMOBA_BF16 && D.d == 128; }
 
@@ -52,7 +52,7 @@ static BwdWs carve_bwd(const Dims& D, bool dense, void* ws, long long cap = 0) {
   w.item_ptr = c.take<int>((size_t)D.BH * D.Nb + 1);
   w.item_tab = dense ? nullptr : c.take<int>((size_t)max_items_128(D, cap));
   w.Dv = c.take<float>((size_t)D.BH * D.S);
-  w.dq_acc = dense ? nullptr : c.take<float>((size_t)D.BH * D.S * D.d);
+  w.dq_acc = dense && !use_tensor_cores(D) ? nullptr : c.take<float>((size_t)D.BH * D.S * D.d);
   w.o_resid = (dense && D.dtype == VMOBA_BF16) ? c.take<__nv_bfloat16>((size_t)D.BH * D.S * D.d) : nullptr;
   w.bytes = c.total();
   w.guards = c.guards;
@@ -143,11 +143,16 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
     count_launches(1);
   }
   if (d_o) {
+    // (the tensor-core backward adds dQ into the fp32 accumulator, cleared in the same pass; null on the other path)
     simt::rowdot_kernel<T, DH><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>((const T*)o, (const T*)w.o_resid,
-                                                                          (const T*)d_o, nq, w.Dv);
+                                                                          (const T*)d_o, nq, w.Dv, RowMap(), RowMap(), w.dq_acc);
     if (use_tensor_cores(D)) {
       VMOBA_LAUNCH_OK(1);
-      return tc_dense_bwd(D, q, k, v, d_o, lse, w.Dv, dq, dk, dv, status, st);
+      int rc = tc_dense_bwd(D, q, k, v, d_o, lse, w.Dv, w.dq_acc, dk, dv, status, st);
+      if (rc) return rc;
+      simt::cast_kernel<T><<<grid_for((nq * DH / 4 + 255) / 256, 16), 256, 0, st>>>(w.dq_acc, (T*)dq, nq * DH / 4);
+      VMOBA_LAUNCH_OK(1);
+      return VMOBA_OK;
     }
     simt::attn_bwd_dkdv_kernel<T, DH, true><<<grid_for(D.BH * tiles, 4), simt::kThreads, 0, st>>>(
         (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, D.S, 1, D.S, D.BH,

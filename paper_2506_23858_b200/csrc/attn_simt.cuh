@@ -426,7 +426,8 @@ merge_batched_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pa
 // ------------------------------------------------------------------------------ backward
 // D = rowsum(dO * O), one warp per query; o and dO block-major or in raster order through their maps, the
 // rounding residual of o always block-major.  If zero_acc is given, the fp32 dQ accumulator rows of the queries
-// with at least one selected block are cleared in the same pass (the only rows the backward kernel adds into).
+// with at least one selected block (of every query without q_ptr) are cleared in the same pass: the only rows the
+// backward kernel adds into.
 template <typename T, int DH>
 __global__ void __launch_bounds__(256)
 rowdot_kernel(const T* __restrict__ o, const T* __restrict__ o_resid, const T* __restrict__ d_o, long long n_queries,
@@ -448,7 +449,7 @@ rowdot_kernel(const T* __restrict__ o, const T* __restrict__ o_resid, const T* _
       for (int r = 0; r < R; ++r) {
         const long long g = min(g0 + r, n_queries - 1);
         used[r] = !q_ptr || __ldg(q_ptr + g + 1) - __ldg(q_ptr + g) >= 1;
-        zero[r] = zero_acc && q_ptr && g0 + r < n_queries && used[r];
+        zero[r] = zero_acc && g0 + r < n_queries && used[r];
       }
 #pragma unroll
       for (int r = 0; r < R; ++r) {
@@ -487,7 +488,7 @@ rowdot_kernel(const T* __restrict__ o, const T* __restrict__ o_resid, const T* _
     float a = 0.f;
     const T* do_row = d_o + do_map.off(g, DH);
     const T* o_row = o + o_map.off(g, DH);
-    if (zero_acc && __ldg(q_ptr + g + 1) - __ldg(q_ptr + g) >= 1) {
+    if (zero_acc && (!q_ptr || __ldg(q_ptr + g + 1) - __ldg(q_ptr + g) >= 1)) {
       float4* row = reinterpret_cast<float4*>(zero_acc + g * DH);
       for (int c = lane; c < DH / 4; c += 32) row[c] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
