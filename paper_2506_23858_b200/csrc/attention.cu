@@ -98,13 +98,12 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
   if (use_tensor_cores(D)) {
     // the backward kernel adds every dQ contribution into the fp32 accumulator: the row-dot pass also clears the
     // rows of all selecting queries; they are converted afterwards (rows of queries without a block become zero)
-    const int min_nb = 1;
     simt::rowdot_kernel<T, DH><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>(
         (const T*)o, (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, o_map, w.dq_acc, q_ptr);
     count_launches(1);
     int rc = tc_sparse_bwd(D, q, k, v, d_o, lse, w.Dv, kb_ptr, q_idx, cap, w.dq_acc, dk, dv, status, st, out_map, do_map);
     if (rc) return rc;
-    simt::cast_rows_kernel<T, DH><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>(w.dq_acc, (T*)dq, q_ptr, nq, 1, min_nb, out_map);
+    simt::cast_rows_kernel<T><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>(w.dq_acc, (T*)dq, q_ptr, nq, out_map);
     VMOBA_LAUNCH_OK(1);
     VMOBA_GUARDS_CHECK(w.guards, status, st);
     return VMOBA_OK;
@@ -150,7 +149,7 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
       VMOBA_LAUNCH_OK(1);
       int rc = tc_dense_bwd(D, q, k, v, d_o, lse, w.Dv, w.dq_acc, dk, dv, status, st);
       if (rc) return rc;
-      simt::cast_kernel<T><<<grid_for((nq * DH / 4 + 255) / 256, 16), 256, 0, st>>>(w.dq_acc, (T*)dq, nq * DH / 4);
+      simt::cast_rows_kernel<T><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>(w.dq_acc, (T*)dq, nullptr, nq, RowMap());
       VMOBA_LAUNCH_OK(1);
       return VMOBA_OK;
     }

@@ -688,48 +688,44 @@ attn_bwd_dq_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
   }
 }
 
-// fp32 accumulator rows -> output dtype, one warp per query.  With `sparse_rows` set only queries with
-// two or more selected blocks own an accumulator row: queries with exactly one block were written
-// directly by the attention kernel (skipped here) and queries with none get zeros without a read.
-template <typename T, int DH>
+// Rows of the tensor-core backward's fp32 dQ accumulator -> output dtype.  The accumulator keeps its 128 columns in the
+// order that kernel reduces them in: position 32 w + 4 r + a holds column 32 w + r + 8 a.  Queries without a selected
+// block (q_ptr given) get zeros without a read.
+template <typename T>
 __global__ void __launch_bounds__(256)
 cast_rows_kernel(const float* __restrict__ src, T* __restrict__ dst, const int* __restrict__ q_ptr, long long n_queries,
-                 int sparse_rows, int min_nb, const RowMap map = RowMap()) {
-  constexpr int C = DH / 32;
+                 const RowMap map) {
+  constexpr int DH = 128;
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-  if constexpr (C == 4) {
-    // Four rows per warp and trip, in phases (list bounds, row offsets, loads, stores), so that the
-    // loads of the four rows are in flight together.
-    constexpr int R = 4;
-    for (long long g0 = warp * R; g0 < n_queries; g0 += nwarps * R) {
-      int nb[R];
-      long long off[R];
-      float4 v[R];
+  // this lane's output columns 4 lane .. 4 lane + 3 sit at positions at, at + 4, at + 8, at + 12: one line of the row
+  const int at = (lane & ~7) * 4 + 16 * (lane & 1) + ((lane & 7) >> 1);
+  // Four rows per warp and trip, in phases (list bounds, row offsets, loads, stores), so that the
+  // loads of the four rows are in flight together.
+  constexpr int R = 4;
+  for (long long g0 = warp * R; g0 < n_queries; g0 += nwarps * R) {
+    bool used[R];
+    long long off[R];
+    float4 v[R];
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const long long g = g0 + r;
-        nb[r] = g >= n_queries ? 1 : (sparse_rows ? __ldg(q_ptr + g + 1) - __ldg(q_ptr + g) : 2);
-        if (g >= n_queries || (nb[r] > 0 && nb[r] < min_nb)) nb[r] = -1;   // no row, or written by the attention kernel
+    for (int r = 0; r < R; ++r) {
+      const long long g = min(g0 + r, n_queries - 1);
+      used[r] = !q_ptr || __ldg(q_ptr + g + 1) > __ldg(q_ptr + g);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) off[r] = map.off(min(g0 + r, n_queries - 1), DH);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      v[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (used[r]) {
+        const float* row = src + min(g0 + r, n_queries - 1) * DH + at;
+        v[r] = make_float4(__ldg(row), __ldg(row + 4), __ldg(row + 8), __ldg(row + 12));
       }
-#pragma unroll
-      for (int r = 0; r < R; ++r) off[r] = nb[r] >= 0 ? map.off(g0 + r, DH) : 0;
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        v[r] = nb[r] > 0 ? *reinterpret_cast<const float4*>(src + (g0 + r) * DH + lane * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int r = 0; r < R; ++r)
-        if (nb[r] >= 0) store4(dst + off[r] + lane * 4, v[r]);
     }
-  } else {
-    for (long long g = warp; g < n_queries; g += nwarps) {
-      const int nb = sparse_rows ? q_ptr[g + 1] - q_ptr[g] : 2;
-      if (nb > 0 && nb < min_nb) continue;   // written directly by the attention kernel
-      T* out = dst + map.off(g, DH);
 #pragma unroll
-      for (int c = 0; c < C; ++c) out[lane * C + c] = from_f32<T>(nb == 0 ? 0.f : src[g * DH + lane * C + c]);
-    }
+    for (int r = 0; r < R; ++r)
+      if (g0 + r < n_queries) store4(dst + off[r] + lane * 4, v[r]);
   }
 }
 

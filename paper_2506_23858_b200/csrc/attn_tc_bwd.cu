@@ -12,18 +12,18 @@
 //     dQ^T = K^T dS^T                                    (SS: K tile read MN-major as A, dS^T as the [keys][queries] tile;
 //                                                         lands in the dP^T columns)
 //   Every key belongs to exactly one item: dK and dV are written once, no atomics.  dQ^T is read out of TMEM by eight
-//   writer warps (lane = head-dim index), transposed four queries at a time among groups of four lanes with shuffles,
-//   and added into an fp32 accumulator with red.global.add.v4.f32 (per warp instruction: complete 128-byte lines of
-//   four query rows).
+//   writer warps and added into an fp32 accumulator with red.global.add.v4.f32 (per warp instruction: complete 128-byte
+//   lines of four query rows).
 //
 // What bounds it is the shared-memory port (128 bytes per cycle).  A shared-memory MMA with N = 128 fetches 8 KB of
 // operands in its 64 cycles, a TS one 4 KB; per 128 x 128 unit that is 2048 cycles of operands against 2560 cycles of
-// tensor math, beside 512 cycles for the landing Q / dO rows, 256 for the dS^T tile and 512 for the dQ shuffles.  Hence
+// tensor math, beside 512 cycles for the landing Q / dO rows and 256 for the dS^T tile.  Hence
 //   * units of 128 queries: with 64 (N = 64) an SS MMA fetches 6 KB for half the math;
 //   * P^T and dS^T as TMEM operands; dQ^T in the columns that dP^T and dS^T no longer need (S^T | dP^T | dV | dK fill the
 //     512 columns, so nothing is double-buffered and the order of the MMAs carries the overlap, see the MMA warp);
 //   * scores read and results written in the 16-row fragment shapes (16x256b in, 16x128b out, stmatrix): a thread then
-//     holds 16 different queries instead of 64, and lse and D are 16 eight-byte shared-memory reads instead of 128 shuffles.
+//     holds 16 different queries instead of 64, and lse and D are 16 eight-byte shared-memory reads instead of 128 shuffles;
+//     dQ^T read in the same shape needs no transposition before the reductions.
 //
 // D = rowsum(dO * O) and lse come in per query; exp runs in the exp2 domain (c = scale * log2 e).
 #include <algorithm>
@@ -42,6 +42,7 @@ constexpr int PANEL = 128 * 128;             // bytes of one 64-column panel of 
 constexpr int TILE = 2 * PANEL;              // [128 x 128] bf16 (32 KB)
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t ST_COL = 0, DPT_COL = 128, DV_COL = 256, DK_COL = 384;
+constexpr uint32_t ROW16 = 16u << 16;        // TMEM lanes 16 .. 31 of a warp's quarter
 constexpr float LOG2E = 1.4426950408889634f;
 // Diagnostics: when a device buffer of 16 counters is registered, the kernel adds the cycles its roles spend in each
 // wait (one representative thread per role and CTA).
@@ -65,7 +66,7 @@ constexpr size_t SMEM_BYTES = 7 * TILE + sizeof(KvSmem) + 32;
 static_assert(SMEM_BYTES <= 232448, "backward: shared memory");
 // Warp groups: {TMA, MMA, 2 dO loaders}, 4 Q loaders, 2 x 4 compute, 2 x 4 dQ writers.  768 threads start with 80
 // registers each; the compute groups, which keep a unit's 64 weights per thread from the first to the second step, take
-// 128, the writers keep 64, the first two groups 48: 2 x 128 + 2 x 64 + 2 x 48 = 6 x 80.
+// 120, the writers (64 values of dQ) keep 80, the first two groups 40: 2 x 120 + 2 x 80 + 2 x 40 = 6 x 80.
 constexpr int THREADS = 768;
 constexpr uint32_t IDESC_TN = make_idesc_bf16(128, 128, false, true);    // dV, dK: A from TMEM, B MN-major
 
@@ -80,7 +81,8 @@ struct KvParams {
   int dkv_32;                  // dk and dv are 32-byte aligned: rows go out with 32-byte stores
   RowMap out_map;              // where the dK / dV rows go (block-major, or raster order through perm)
   RowMap do_map;               // where the dO rows come from (likewise)
-  float* dq_acc;               // fp32 [queries][head_dim], zeroed rows of all selecting queries
+  float* dq_acc;               // fp32 [queries][head_dim], zeroed rows of all selecting queries; columns in the order of the
+                               // dQ writers: position 32 w + 4 r + a holds column 32 w + r + 8 a (r < 8, a < 4)
   int32_t* status;
   unsigned long long* prof;    // optional wait-time counters (diagnostics), or null
 };
@@ -267,7 +269,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   const int n_items = p.BH * (DENSE ? 1 : p.Nb) * tiles;
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     if (warp == 0) {
       // ---------------------------------------------------------------- TMA: K and V tiles, one pair per item
       if (lane == 0) {
@@ -309,9 +311,9 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       //
       // The compute warps alternate between the two element-wise steps, the tensor pipe must have work during both.
       // Order per unit i, with what overlaps it:
-      //   dK(i), dQ^T(i)            | P^T(i+1) from S^T(i+1), which was issued one unit early
-      //   dV(i+1)                   | dQ^T(i) read out by the writers
-      //   dP^T(i+1), S^T(i+2)       | dS^T(i+1) as soon as dP^T(i+1) is complete
+      //   dK(i), dQ^T(i)            | P^T(i+1) from S^T(i+1), which was issued one unit early; dQ^T(i) read out
+      //   dP^T(i+1)                 | rest of P^T(i+1)
+      //   dV(i+1), S^T(i+2)         | dS^T(i+1)
       const bool leader = elect_one();
       auto wwait = [&](int site, uint64_t* bar, uint32_t parity) { twait(site, bar, parity); __syncwarp(); };
       uint32_t n = 0, g = 0;      // items and units done so far
@@ -339,7 +341,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         };
         auto issue_dp = [&](int i) {
           const uint32_t u = g + i, st = u & 1;
-          if (i == 0) wwait(1, &sm->do_full[st], (u >> 1) & 1);     // (later units: waited for by their dV)
+          wwait(1, &sm->do_full[st], (u >> 1) & 1);
           if (u >= 1) wwait(3, &sm->dq_free, (u - 1) & 1);          // the columns held dQ^T of the unit before
           tc_fence_after();
           const uint32_t idesc = make_idesc_bf16(128, 16 * rows16(i), false, false);
@@ -352,7 +354,6 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         };
         auto issue_dv = [&](int i) {
           const uint32_t u = g + i, st = u & 1;
-          if (i > 0) wwait(1, &sm->do_full[st], (u >> 1) & 1);
           wwait(2, &sm->p_ready, u & 1);
           // dV / dK still hold the previous item until its epilogue has read them
           if (i == 0 && n > 0) wwait(3, &sm->acc_free, (n - 1) & 1);
@@ -391,8 +392,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
             if (leader) mma_commit(&sm->dq_full);
           }
           if (i + 1 < n_units) {
-            issue_dv(i + 1);
             issue_dp(i + 1);
+            issue_dv(i + 1);
             if (leader) mma_commit(&sm->do_empty[(u + 1) & 1]);
             if (i + 2 < n_units) issue_s(i + 2);
           }
@@ -449,7 +450,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       if (g >= 1) mbar_arrive(&sm->do_full[(g - 1) & 1]);
     }
   } else if (warp < 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     // ------------------------------------------------------------------ Q loaders (4 warps): gather the Q rows of a unit and
     // its lse and D (run ahead).  The rows go from global to shared memory as asynchronous 16-byte copies; a unit is
     // published in the next iteration, once its copies have landed.  A lane fetches the list entry of one row of each
@@ -496,34 +497,21 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     if (g >= 1) mbar_arrive(&sm->q_full[(g - 1) & 1]);
     if (lt == 0) tflush(7, 1);     // [7] q_empty, [8] total
   } else if (warp >= 16) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
-    // ------------------------------------------------------------------ dQ writers: thread = head-dim index
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+    // ------------------------------------------------------------------ dQ writers
     // Read dQ^T of a unit out of TMEM (lane = head-dim index, 128 query columns; two warps per TMEM lane quarter, each
-    // taking 64 of them in two rounds) and add it into the fp32 accumulator.  The four lanes 4i .. 4i+3 transpose each
-    // group of four queries among themselves with two exchange steps (one shuffle per value), after which lane 4i + j
-    // holds head-dim columns 4i .. 4i+3 of query j of the group: one red.global.add.v4.f32 warp instruction then adds
-    // four complete 128-byte lines, one in each of four accumulator rows.  (Measured per SM with all SMs busy: reductions
-    // that cover whole 128-byte lines reach 23 B/cycle however the lines are spread over rows; 16 bytes per lane in 32
-    // different rows reach 12.5; scalar line-wide reductions reach 23 alone but made the kernel 1.5x slower.)
+    // taking 64 columns) and add it into the fp32 accumulator.  In the 16x256b shape a thread's registers hold the head-dim
+    // indices r, r + 8, r + 16, r + 24 (r = lane / 4) of its quarter for the same query, so that four of them are one
+    // red.global.add.v4.f32 without any exchange between lanes: the accumulator keeps a quarter's 32 columns in the order
+    // 4 r + a <-> r + 8 a, and cast_rows undoes it.  A warp instruction covers four complete 128-byte lines, one in each of
+    // four accumulator rows.  (Measured per SM with all SMs busy: reductions that cover whole 128-byte lines reach 23
+    // B/cycle however the lines are spread over rows; 16 bytes per lane in 32 different rows reach 12.5.  With the rows
+    // lane = head-dim index and shuffles between four lanes instead, the writers' own instructions were the slowest
+    // part of a unit.)
     const int quad = warp & 3;
     const int qhalf = (warp - 16) >> 2;
     const uint32_t dq_tmem = tmem + ((uint32_t)(quad * 32) << 16) + DPT_COL + 64 * qhalf;
-    const int j4 = lane & 3;
-    const bool odd1 = (lane & 1) != 0, odd2 = (lane & 2) != 0;
     float* acc_col = p.dq_acc + quad * 32 + (lane & ~3);
-    // x[0..3]: this lane's head-dim column for four queries -> head-dim columns 4i .. 4i+3 of query j4
-    auto transpose4 = [&](float x0, float x1, float x2, float x3, float4& y) {
-      // step 1, partner lane ^ 1: even lanes keep queries 0, 2, odd lanes keep queries 1, 3
-      const float r0 = __shfl_xor_sync(0xffffffffu, odd1 ? x0 : x1, 1);
-      const float r1 = __shfl_xor_sync(0xffffffffu, odd1 ? x2 : x3, 1);
-      // (query 0 or 1: columns c, c ^ 1), (query 2 or 3: likewise), in column order
-      const float a0 = odd1 ? r0 : x0, a1 = odd1 ? x1 : r0;
-      const float b0 = odd1 ? r1 : x2, b1 = odd1 ? x3 : r1;
-      // step 2, partner lane ^ 2: lanes 0, 1 keep the first query of their pair, lanes 2, 3 the second
-      const float s0 = __shfl_xor_sync(0xffffffffu, odd2 ? a0 : b0, 2);
-      const float s1 = __shfl_xor_sync(0xffffffffu, odd2 ? a1 : b1, 2);
-      y = odd2 ? make_float4(s0, s1, b0, b1) : make_float4(a0, a1, s0, s1);
-    };
     uint32_t g = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
       const KvItem it = kv_decode<DENSE>(p, item, tiles);
@@ -539,47 +527,33 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         }
         twait(0, &sm->dq_full, g & 1);
         tc_fence_after();
+        // everything out of TMEM first: the next dP^T waits for these columns
+        uint32_t x[2][32];
+        tmem_ld_16x256_x8(dq_tmem, x[0]);
+        tmem_ld_16x256_x8(dq_tmem + ROW16, x[1]);
+        tmem_ld_wait();
+        tc_fence_before();
+        mbar_arrive(&sm->dq_free);
+        // A reduction holds its source registers until the load/store unit has taken them, so each has its own four.
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t x[32];
-          tmem_ld32(dq_tmem + 32 * h, x);
-          tmem_ld_wait();
-          if (h == 1) {
-            tc_fence_before();
-            mbar_arrive(&sm->dq_free);
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {        // query 8 j + 2 (lane % 4) + e of this half
+            const int rw = __shfl_sync(0xffffffffu, row_lane[j >> 2], (8 * j + 2 * (lane & 3) + e) & 31);
+            if (rw >= 0)
+              red_add_v4(acc_head + (long long)rw * DH, __uint_as_float(x[0][4 * j + e]) * p.scale, __uint_as_float(x[0][4 * j + 2 + e]) * p.scale,
+                         __uint_as_float(x[1][4 * j + e]) * p.scale, __uint_as_float(x[1][4 * j + 2 + e]) * p.scale);
           }
-          if (first + 32 * h >= it.n_list) continue;      // (uniform) nobody here
-          // The transpositions first, in place, then the eight reductions back to back from eight different
-          // register quadruples: a reduction holds its source registers until the load/store unit has taken them
-          // (about 200 cycles under this kernel's memory traffic), so a loop that reuses one quadruple sends one
-          // reduction per 200 cycles.
-          int rw[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            float4 y;
-            transpose4(__uint_as_float(x[4 * q]), __uint_as_float(x[4 * q + 1]), __uint_as_float(x[4 * q + 2]),
-                       __uint_as_float(x[4 * q + 3]), y);
-            x[4 * q] = __float_as_uint(y.x * p.scale); x[4 * q + 1] = __float_as_uint(y.y * p.scale);
-            x[4 * q + 2] = __float_as_uint(y.z * p.scale); x[4 * q + 3] = __float_as_uint(y.w * p.scale);
-            rw[q] = __shfl_sync(0xffffffffu, row_lane[h], 4 * q + j4);
-          }
-#pragma unroll
-          for (int q = 0; q < 8; ++q)
-            if (rw[q] >= 0)
-              red_add_v4(acc_head + (long long)rw[q] * DH, __uint_as_float(x[4 * q]), __uint_as_float(x[4 * q + 1]),
-                         __uint_as_float(x[4 * q + 2]), __uint_as_float(x[4 * q + 3]));
-        }
       }
     }
     if (warp == 16 && lane == 0) tflush(14, 1);     // [14] dq_full, [15] total
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
     // ------------------------------------------------------------------ compute: warp = 32 keys x half of the unit's queries
     const int quad = warp & 3;
     const int half = (warp - 8) >> 2;
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
     const uint32_t st_t = tmem + lane_addr + ST_COL + 64 * half, dp_t = tmem + lane_addr + DPT_COL + 64 * half;
-    constexpr uint32_t ROW16 = 16u << 16;            // TMEM lanes 16 .. 31 of the warp's quarter
     // this lane's row address for stmatrix: matrices (keys 0-7, queries 8j), (keys 8-15, same), (keys 0-7, 8j + 8), ...
     const int mrow = quad * 32 + 8 * ((lane >> 3) & 1) + (lane & 7), mj = lane >> 4;
     const uint32_t ds_row = smem_u32(sDS) + half * PANEL + mrow * 128;
@@ -744,7 +718,8 @@ static int launch(const Dims& D, const void* k, const void* v, KvParams& kp, cud
 }  // namespace tcb
 
 // Backward over the work lists (bf16, head_dim 128).  Dv holds rowsum(dO * O) per query; dq_acc is
-// an fp32 accumulator whose rows of selecting queries are zero; the caller converts it to bf16.
+// an fp32 accumulator whose rows of selecting queries are zero; the caller converts it to bf16 (simt::cast_rows_kernel
+// knows the order of its columns).
 int tc_sparse_bwd(const Dims& D, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
                   const float* Dv, const int* kb_ptr, const int* q_idx, long long cap, float* dq_acc, void* dk, void* dv,
                   int32_t* status, cudaStream_t st, const RowMap& out_map, const RowMap& do_map) {
