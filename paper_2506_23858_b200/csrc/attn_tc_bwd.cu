@@ -48,26 +48,31 @@ constexpr float LOG2E = 1.4426950408889634f;
 // wait (one representative thread per role and CTA).
 static unsigned long long* g_wait_profile = nullptr;
 
+// A unit's Q tile is held from S^T, issued one unit early, to dK at its end; its dO tile only from dP^T to dV, in the
+// middle.  So three Q tiles and one dO tile keep both gathers ahead (with two of each the MMA warp waited 1250 of a unit's
+// 5000 cycles for Q rows).
+constexpr int NQ = 3;
+
 struct KvSmem {
   uint64_t k_full, k_empty, v_full, v_empty;                       // K / V tile of an item (TMA / commit)
-  uint64_t q_full[2], q_empty[2], do_full[2], do_empty[2];         // gathered Q / dO rows of a unit (loader arrivals / commit)
+  uint64_t q_full[NQ], q_empty[NQ], do_full, do_empty;             // gathered Q / dO rows of a unit (loader arrivals / commit)
   uint64_t s_full, p_ready;                                        // S^T complete (commit) / P^T written (256 arrivals)
   uint64_t dp_full, ds_ready;                                      // dP^T complete (commit) / dS^T written (256 arrivals)
   uint64_t dq_full, dq_free;                                       // dQ^T complete (commit) / read out of TMEM (256 arrivals)
   uint64_t acc_done, acc_free;                                     // dV / dK of an item complete (commit) / read (256 arrivals)
   uint32_t tmem_base;
   int abort_flag;
-  alignas(16) float lse2[2][QU];             // per unit slot: lse * log2 e
-  alignas(16) float negD[2][QU];             // and -rowsum(dO * O)
+  alignas(16) float lse2[NQ][QU];            // lse * log2 e, with the Q rows of a unit
+  alignas(16) float negD[2][QU];             // -rowsum(dO * O), with its dO rows
 };
-// K, V, two Q and two dO tiles, the dS^T tile ([128 keys][128 queries] bf16)
+// K, V, three Q tiles and a dO tile, the dS^T tile ([128 keys][128 queries] bf16)
 // no alignment slack: the kernel checks that its dynamic shared memory starts on a 1024-byte boundary
 constexpr size_t SMEM_BYTES = 7 * TILE + sizeof(KvSmem) + 32;
 static_assert(SMEM_BYTES <= 232448, "backward: shared memory");
-// Warp groups: {TMA, MMA, 2 dO loaders}, 4 Q loaders, 2 x 4 compute, 2 x 4 dQ writers.  768 threads start with 80
+// Warp groups: {TMA, MMA, -, -}, 4 Q loaders, 4 dO loaders, 2 x 4 compute, 2 x 4 dQ writers.  896 threads start with 72
 // registers each; the compute groups, which keep a unit's 64 weights per thread from the first to the second step, take
-// 120, the writers (64 values of dQ) keep 80, the first two groups 40: 2 x 120 + 2 x 80 + 2 x 40 = 6 x 80.
-constexpr int THREADS = 768;
+// 112, the writers (64 values of dQ) 80, the first three groups keep 40: 2 x 112 + 2 x 80 + 3 x 40 = 7 x 72.
+constexpr int THREADS = 896;
 constexpr uint32_t IDESC_TN = make_idesc_bf16(128, 128, false, true);    // dV, dK: A from TMEM, B MN-major
 
 struct KvParams {
@@ -89,7 +94,7 @@ struct KvParams {
 
 struct KvItem {
   int bh, key0, valid, n_list, n_units, first_unit;
-  long long list_lo, head_off;
+  int list_lo, head_off;       // positions and rows fit 31 bits (capacity, B * heads * S <= 2^30)
 };
 
 template <bool DENSE>
@@ -101,7 +106,7 @@ __device__ __forceinline__ KvItem kv_decode(const KvParams& p, int item, int til
   const int j = kbi - it.bh * (DENSE ? 1 : p.Nb);
   it.key0 = (DENSE ? 0 : j * p.sb) + tile * BN;
   it.valid = min(BN, (DENSE ? p.S : p.sb) - tile * BN);
-  it.head_off = (long long)it.bh * p.S;
+  it.head_off = it.bh * p.S;
   if constexpr (DENSE) {
     it.list_lo = 0;
     it.n_list = p.S;
@@ -113,7 +118,7 @@ __device__ __forceinline__ KvItem kv_decode(const KvParams& p, int item, int til
       lo = hi = 0;
     }
 #endif
-    it.list_lo = lo;
+    it.list_lo = (int)lo;
     it.n_list = (int)(hi - lo);
   }
   it.n_units = (it.n_list + QU - 1) / QU;
@@ -129,6 +134,32 @@ __device__ __forceinline__ int unit_of(const KvItem& it, int i) {
   const int u = it.first_unit + i;
   return u >= it.n_units ? u - it.n_units : u;
 }
+
+// Walks the units of all items of this CTA, one per next().
+template <bool DENSE>
+struct UnitWalk {
+  KvItem it;
+  int item, i, n_items, tiles, first, rows;
+  __device__ __forceinline__ UnitWalk(const KvParams& p, int n_items_, int tiles_)
+      : item((int)blockIdx.x - (int)gridDim.x), i(0), n_items(n_items_), tiles(tiles_), first(0), rows(0) { it.n_units = 0; }
+  __device__ __forceinline__ bool next(const KvParams& p) {
+    while (i >= it.n_units) {
+      item += gridDim.x;
+      if (item >= n_items) return false;
+      it = kv_decode<DENSE>(p, item, tiles);
+      i = 0;
+    }
+    first = unit_of<DENSE>(it, i) * QU;
+    rows = min(QU, it.n_list - first);
+    ++i;
+    return true;
+  }
+  // in-head position of the query in row `row` of the unit, -1 for a padding row
+  __device__ __forceinline__ int entry(const KvParams& p, int row) const {
+    if (row >= rows) return -1;
+    return DENSE ? first + row : checked_index(__ldg(p.q_idx + it.list_lo + first + row), p.S, p.status);
+  }
+};
 
 // Asynchronous 16-byte copy global -> shared (bypassing L1); `bytes` = 16, or 0 to write zeros.
 __device__ __forceinline__ void cp_async16(uint32_t smem_dst, const void* gsrc, uint32_t bytes) {
@@ -206,7 +237,8 @@ __device__ __forceinline__ void stmatrix_x4(uint32_t addr, uint32_t a, uint32_t 
 
 template <bool DENSE, bool PROF>
 __global__ void __launch_bounds__(THREADS, 1)
-attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const KvParams p) {
+attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
+                      const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmO, const KvParams p) {
   extern __shared__ uint8_t smem_raw[];
   // the swizzled tiles need 1024-byte alignment and there is no room for alignment slack
   if ((smem_u32(smem_raw) & 1023u) != 0) {
@@ -215,8 +247,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   }
   uint8_t* sK = smem_raw;
   uint8_t* sV = smem_raw + TILE;
-  uint8_t* sQ = smem_raw + 2 * TILE;           // [2]
-  uint8_t* sO = smem_raw + 4 * TILE;           // [2] dO
+  uint8_t* sQ = smem_raw + 2 * TILE;           // [NQ]
+  uint8_t* sO = smem_raw + (2 + NQ) * TILE;    // dO
   uint8_t* sDS = smem_raw + 6 * TILE;
   KvSmem* sm = reinterpret_cast<KvSmem*>(smem_raw + 7 * TILE);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -243,10 +275,8 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   if (threadIdx.x == 0) {
     mbar_init(&sm->k_full, 1); mbar_init(&sm->k_empty, 1);
     mbar_init(&sm->v_full, 1); mbar_init(&sm->v_empty, 1);
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&sm->q_full[b], 128); mbar_init(&sm->q_empty[b], 1);
-      mbar_init(&sm->do_full[b], 64); mbar_init(&sm->do_empty[b], 1);
-    }
+    for (int b = 0; b < NQ; ++b) { mbar_init(&sm->q_full[b], 128); mbar_init(&sm->q_empty[b], 1); }
+    mbar_init(&sm->do_full, 128); mbar_init(&sm->do_empty, 1);
     mbar_init(&sm->s_full, 1); mbar_init(&sm->p_ready, 256);
     mbar_init(&sm->dp_full, 1); mbar_init(&sm->ds_ready, 256);
     mbar_init(&sm->dq_full, 1); mbar_init(&sm->dq_free, 256);
@@ -277,7 +307,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
           const KvItem it = kv_decode<DENSE>(p, item, tiles);
           if (it.n_units == 0) continue;
-          const int y = (int)it.head_off + it.key0;
+          const int y = it.head_off + it.key0;
           // V is free after the item's last dP^T, K only after its last dQ^T
           if (n >= 1) twait(0, &sm->v_empty, (n - 1) & 1);
           mbar_expect_tx(&sm->v_full, TILE);
@@ -291,7 +321,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           // the one K / V pair is reloaded when the item is over: ask the L2 for the next item's tiles now
           if (item + (int)gridDim.x < n_items) {
             const KvItem nx = kv_decode<DENSE>(p, item + gridDim.x, tiles);
-            const int yn = (int)nx.head_off + nx.key0;
+            const int yn = nx.head_off + nx.key0;
             if (nx.n_units > 0) {
               tma_prefetch_2d(&tmK, 0, yn); tma_prefetch_2d(&tmK, 64, yn);
               tma_prefetch_2d(&tmV, 0, yn); tma_prefetch_2d(&tmV, 64, yn);
@@ -317,6 +347,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       const bool leader = elect_one();
       auto wwait = [&](int site, uint64_t* bar, uint32_t parity) { twait(site, bar, parity); __syncwarp(); };
       uint32_t n = 0, g = 0;      // items and units done so far
+      uint32_t s_slot = 0, s_par = 0, k_slot = 0;      // Q ring: next unit's slot and parity for S^T, slot of the current dK
       const uint32_t kK = lo_k(smem_u32(sK)), kV = lo_k(smem_u32(sV)), mK = lo_mn(smem_u32(sK)), mS = lo_mn(smem_u32(sDS));
       const uint32_t kQ = lo_k(smem_u32(sQ)), kO = lo_k(smem_u32(sO)), mQ = lo_mn(smem_u32(sQ)), mO = lo_mn(smem_u32(sO));
       constexpr uint32_t STAGE = TILE >> 4;
@@ -329,61 +360,60 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         const int key_steps = (it.valid + 15) >> 4;
         auto rows16 = [&](int i) { return (min(QU, n_list - unit_of<DENSE>(it, i) * QU) + 15) >> 4; };   // 16-query steps of a unit
         auto issue_s = [&](int i) {
-          const uint32_t u = g + i, st = u & 1;
-          wwait(1, &sm->q_full[st], (u >> 1) & 1);
+          wwait(1, &sm->q_full[s_slot], s_par);
           tc_fence_after();
           const uint32_t idesc = make_idesc_bf16(128, 16 * rows16(i), false, false);
-          const uint32_t b = kQ + st * STAGE;
+          const uint32_t b = kQ + s_slot * STAGE;
+          if (++s_slot == NQ) { s_slot = 0; s_par ^= 1; }
 #pragma unroll
           for (int ks = 0; ks < DH / 16; ++ks)
             if (leader) mma_ss_lo(tmem + ST_COL, kK + koff(ks), b + koff(ks), idesc, ks > 0 ? 1u : 0u);
           if (leader) mma_commit(&sm->s_full);
         };
         auto issue_dp = [&](int i) {
-          const uint32_t u = g + i, st = u & 1;
-          wwait(1, &sm->do_full[st], (u >> 1) & 1);
+          const uint32_t u = g + i;
+          wwait(1, &sm->do_full, u & 1);
           if (u >= 1) wwait(3, &sm->dq_free, (u - 1) & 1);          // the columns held dQ^T of the unit before
           tc_fence_after();
           const uint32_t idesc = make_idesc_bf16(128, 16 * rows16(i), false, false);
-          const uint32_t b = kO + st * STAGE;
 #pragma unroll
           for (int ks = 0; ks < DH / 16; ++ks)
-            if (leader) mma_ss_lo(tmem + DPT_COL, kV + koff(ks), b + koff(ks), idesc, ks > 0 ? 1u : 0u);
+            if (leader) mma_ss_lo(tmem + DPT_COL, kV + koff(ks), kO + koff(ks), idesc, ks > 0 ? 1u : 0u);
           if (leader) mma_commit(&sm->dp_full);
           if (leader && i == n_units - 1) mma_commit(&sm->v_empty);
         };
         auto issue_dv = [&](int i) {
-          const uint32_t u = g + i, st = u & 1;
+          const uint32_t u = g + i;
           wwait(2, &sm->p_ready, u & 1);
           // dV / dK still hold the previous item until its epilogue has read them
           if (i == 0 && n > 0) wwait(3, &sm->acc_free, (n - 1) & 1);
           tc_fence_after();
           const int ksteps = rows16(i);
-          const uint32_t b = mO + st * STAGE;
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)       // P^T of queries 64 h .. sits in columns 64 h .. 64 h + 31
             if (leader && ks < ksteps)
-              mma_ts_lo(tmem + DV_COL, tmem + ST_COL + (ks >> 2) * 64 + (ks & 3) * 8, b + mnoff(ks), IDESC_TN, (ks > 0 || i > 0) ? 1u : 0u);
+              mma_ts_lo(tmem + DV_COL, tmem + ST_COL + (ks >> 2) * 64 + (ks & 3) * 8, mO + mnoff(ks), IDESC_TN, (ks > 0 || i > 0) ? 1u : 0u);
+          if (leader) mma_commit(&sm->do_empty);
         };
         wwait(0, &sm->k_full, n & 1);
         issue_s(0);
         wwait(0, &sm->v_full, n & 1);
         issue_dp(0);
         issue_dv(0);
-        if (leader) mma_commit(&sm->do_empty[g & 1]);
         if (n_units > 1) issue_s(1);
         for (int i = 0; i < n_units; ++i) {
-          const uint32_t u = g + i, st = u & 1;
+          const uint32_t u = g + i;
           wwait(2, &sm->ds_ready, u & 1);
           tc_fence_after();
           {
             const int ksteps = rows16(i);
-            const uint32_t b = mQ + st * STAGE;
+            const uint32_t b = mQ + k_slot * STAGE;
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks)
               if (leader && ks < ksteps)
                 mma_ts_lo(tmem + DK_COL, tmem + DPT_COL + (ks >> 2) * 64 + (ks & 3) * 8, b + mnoff(ks), IDESC_TN, (ks > 0 || i > 0) ? 1u : 0u);
-            if (leader) mma_commit(&sm->q_empty[st]);
+            if (leader) mma_commit(&sm->q_empty[k_slot]);
+            if (++k_slot == NQ) k_slot = 0;
             // dQ^T over dP^T and dS^T: in order behind the dK MMAs that read dS^T there
             const uint32_t idesc = make_idesc_bf16(128, 16 * ksteps, true, true);
 #pragma unroll
@@ -394,7 +424,6 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           if (i + 1 < n_units) {
             issue_dp(i + 1);
             issue_dv(i + 1);
-            if (leader) mma_commit(&sm->do_empty[(u + 1) & 1]);
             if (i + 2 < n_units) issue_s(i + 2);
           }
         }
@@ -404,100 +433,87 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         ++n;
       }
       if (leader) tflush(2, 4);      // [2] k_full + v_full, [3] q_full + do_full, [4] p_ready + ds_ready, [5] dq_free + acc_free, [6] total
-    } else {
-      // ---------------------------------------------------------------- dO loaders (2 warps): see the Q loaders
-      const int w = warp - 2, chunk = lane & 15;
-      const uint32_t dst0 = smem_u32(sO) + (chunk >> 3) * PANEL;
-      const bool raster = p.do_map.perm != nullptr;
-      const long long stride = raster ? p.do_map.st : (long long)DH;
-      uint32_t g = 0;
-      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const KvItem it = kv_decode<DENSE>(p, item, tiles);
-        const int b_ = it.bh / p.do_map.heads, hd_ = it.bh - b_ * p.do_map.heads;
-        const __nv_bfloat16* src = p.d_o + (raster ? b_ * p.do_map.sb + hd_ * p.do_map.sh : it.head_off * DH) + chunk * 8;
-        for (int i = 0; i < it.n_units; ++i, ++g) {
-          const int st = g & 1;
-          const int first = unit_of<DENSE>(it, i) * QU, rows = min(QU, it.n_list - first);
-          int idx[2];        // rows 2 w + (lane >> 4) + 4 k of k = lane % 16 and 16 + lane % 16
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int row = 2 * w + (lane >> 4) + 4 * ((lane & 15) + 16 * h);
-            idx[h] = -1;
-            if (row < rows) {
-              idx[h] = DENSE ? first + row : checked_index(__ldg(p.q_idx + it.list_lo + first + row), p.S, p.status);
-              if (raster) idx[h] = __ldg(p.do_map.perm + idx[h]);
-            }
-          }
-          if (g >= 1) {
-            cp_async_wait<0>();
-            fence_async_proxy();
-            mbar_arrive(&sm->do_full[(g - 1) & 1]);
-          }
-          if (g >= 2) mbar_wait(&sm->do_empty[st], ((g >> 1) - 1) & 1, abort_flag, p.status);
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-#pragma unroll 8
-            for (int k = 0; k < 16; ++k) {
-              const int row = 2 * w + (lane >> 4) + 4 * (k + 16 * h);
-              const int ik = __shfl_sync(0xffffffffu, idx[h], (lane & 16) + k);
-              cp_async16(dst0 + st * TILE + row * 128 + (((chunk & 7) ^ (row & 7)) << 4), src + (long long)max(ik, 0) * stride, ik < 0 ? 0u : 16u);
-            }
-          cp_async_commit();
-        }
-      }
-      cp_async_wait<0>();
-      fence_async_proxy();
-      if (g >= 1) mbar_arrive(&sm->do_full[(g - 1) & 1]);
     }
-  } else if (warp < 8) {
+  } else if (warp < 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-    // ------------------------------------------------------------------ Q loaders (4 warps): gather the Q rows of a unit and
-    // its lse and D (run ahead).  The rows go from global to shared memory as asynchronous 16-byte copies; a unit is
-    // published in the next iteration, once its copies have landed.  A lane fetches the list entry of one row of each
-    // 16 that its half-warp copies and hands it round.
-    const int w = warp - 4, lt = threadIdx.x - 128, chunk = lane & 15;
-    const uint32_t dst0 = smem_u32(sQ) + (chunk >> 3) * PANEL;
-    uint32_t g = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-      const KvItem it = kv_decode<DENSE>(p, item, tiles);
-      const __nv_bfloat16* src = p.q + it.head_off * DH + chunk * 8;
-      for (int i = 0; i < it.n_units; ++i, ++g) {
-        const int st = g & 1;
-        const int first = unit_of<DENSE>(it, i) * QU, rows = min(QU, it.n_list - first);
-        auto entry = [&](int row) {
-          if (row >= rows) return -1;          // padding row, zero-filled
-          return DENSE ? first + row : checked_index(__ldg(p.q_idx + it.list_lo + first + row), p.S, p.status);
-        };
-        const int idx = entry(2 * w + (lane >> 4) + 8 * (lane & 15));
-        const int mine = entry(lt);
-        float l2 = INFINITY, nd = 0.f;         // padded queries: P = exp2(-inf) = 0
-        if (mine >= 0) {
-          l2 = p.lse[it.head_off + mine] * LOG2E;
-          nd = -p.Dv[it.head_off + mine];
+    // ------------------------------------------------------------------ loaders: the Q rows of the units with their lse (warps
+    // 4-7), the dO rows with -rowsum(dO * O) (warps 8-11); they run ahead.
+    // Sparse: the rows go from global to shared memory as asynchronous 16-byte copies, eight threads per 128-byte half
+    // row; a thread keeps the list entries of its eight rows and fetches those of the next unit while the copies are in
+    // flight.  Next to a busy tensor pipe a warp gets shared-memory and load instructions through at about one in 100
+    // cycles, hence four warps for each tensor (six for both: the kernel waited for rows) and no shuffles.
+    // Dense: consecutive rows, TMA tiles requested by one of the threads that bring the scalars.
+    const bool is_q = warp < 8;
+    const int lt = threadIdx.x & 127, r0 = 4 * (warp & 3) + (lane >> 3), chunk = lane & 7;      // rows r0 + 16 k
+    UnitWalk<DENSE> walk(p, n_items, tiles);
+    const bool raster = !is_q && p.do_map.perm != nullptr;
+    const long long stride = raster ? p.do_map.st : (long long)DH;
+    const uint32_t tile0 = smem_u32(is_q ? sQ : sO);
+    const __nv_bfloat16* src = nullptr;
+    int idx[8];
+    float sc = 0.f;
+    auto fetch = [&]() {
+      if constexpr (!DENSE) {
+        const int b_ = walk.it.bh / p.do_map.heads, hd_ = walk.it.bh - b_ * p.do_map.heads;
+        src = (is_q ? p.q : p.d_o) + (raster ? b_ * p.do_map.sb + hd_ * p.do_map.sh : (long long)walk.it.head_off * DH) + chunk * 8;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) idx[k] = walk.entry(p, r0 + 16 * k);
+        if (raster) {
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (idx[k] >= 0) idx[k] = __ldg(p.do_map.perm + idx[k]);
         }
-        if (g >= 1) {
-          cp_async_wait<0>();
-          fence_async_proxy();
-          mbar_arrive(&sm->q_full[(g - 1) & 1]);
-        }
-        if (g >= 2) twait(0, &sm->q_empty[st], ((g >> 1) - 1) & 1);
-#pragma unroll 8
-        for (int k = 0; k < 16; ++k) {
-          const int row = 2 * w + (lane >> 4) + 8 * k;
-          const int ik = __shfl_sync(0xffffffffu, idx, (lane & 16) + k);
-          cp_async16(dst0 + st * TILE + row * 128 + (((chunk & 7) ^ (row & 7)) << 4), src + (long long)max(ik, 0) * DH, ik < 0 ? 0u : 16u);
-        }
-        sm->lse2[st][lt] = l2;
-        sm->negD[st][lt] = nd;
-        cp_async_commit();
       }
+      const int mine = walk.entry(p, lt);
+      sc = is_q ? INFINITY : 0.f;                          // padded queries: P = exp2(-inf) = 0
+      if (mine >= 0) sc = is_q ? __ldg(p.lse + walk.it.head_off + mine) * LOG2E : -__ldg(p.Dv + walk.it.head_off + mine);
+    };
+    bool more = walk.next(p);
+    if (more) fetch();
+    uint32_t slot = 0, par = 1;
+    for (uint32_t g = 0; more; ++g) {
+      uint64_t* full = is_q ? &sm->q_full[slot] : &sm->do_full;
+      // (the first waits pass at once: the parity of the phase before the first)
+      twait(0, is_q ? &sm->q_empty[slot] : &sm->do_empty, par);
+      // -rowsum(dO * O) of unit g goes to slot g % 2, which dS^T of unit g - 2 has left behind when dV of unit g - 1, which
+      // follows P^T of unit g - 1, has freed the dO tile
+      (is_q ? sm->lse2[slot] : sm->negD[g & 1])[lt] = sc;
+      if constexpr (DENSE) {
+        if (lt == 0) {
+          const CUtensorMap* map = is_q ? &tmQ : &tmO;
+          uint8_t* tile = is_q ? sQ + slot * TILE : sO;
+          mbar_expect_tx(full, TILE);
+          tma_load_3d(tile, map, full, 0, walk.first, walk.it.bh);
+          tma_load_3d(tile + PANEL, map, full, 64, walk.first, walk.it.bh);
+        } else {
+          mbar_arrive(full);
+        }
+        more = walk.next(p);
+        if (more) fetch();
+        // drain: every issued load must have landed before the CTA may exit (only matters after a timeout)
+        if (lt == 0 && *abort_flag) mbar_wait(full, par ^ 1, abort_flag, p.status);
+      } else {
+        const uint32_t dst = tile0 + slot * TILE + r0 * 128 + ((chunk ^ (r0 & 7)) << 4);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const __nv_bfloat16* row = src + (long long)max(idx[k], 0) * stride;
+          const uint32_t bytes = idx[k] < 0 ? 0u : 16u;
+          cp_async16(dst + k * 2048, row, bytes);
+          cp_async16(dst + k * 2048 + PANEL, row + 64, bytes);
+        }
+        cp_async_commit();
+        more = walk.next(p);
+        if (more) fetch();
+        cp_async_wait<0>();
+        fence_async_proxy();
+        mbar_arrive(full);
+      }
+      if (!is_q) par ^= 1;
+      else if (++slot == NQ) { slot = 0; par ^= 1; }
     }
-    cp_async_wait<0>();
-    fence_async_proxy();
-    if (g >= 1) mbar_arrive(&sm->q_full[(g - 1) & 1]);
-    if (lt == 0) tflush(7, 1);     // [7] q_empty, [8] total
-  } else if (warp >= 16) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+    if (lt == 0 && is_q) tflush(7, 1);     // [7] q_empty, [8] total
+  } else if (warp >= 20) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 80;");
     // ------------------------------------------------------------------ dQ writers
     // Read dQ^T of a unit out of TMEM (lane = head-dim index, 128 query columns; two warps per TMEM lane quarter, each
     // taking 64 columns) and add it into the fp32 accumulator.  In the 16x256b shape a thread's registers hold the head-dim
@@ -509,13 +525,13 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     // lane = head-dim index and shuffles between four lanes instead, the writers' own instructions were the slowest
     // part of a unit.)
     const int quad = warp & 3;
-    const int qhalf = (warp - 16) >> 2;
+    const int qhalf = (warp - 20) >> 2;
     const uint32_t dq_tmem = tmem + ((uint32_t)(quad * 32) << 16) + DPT_COL + 64 * qhalf;
     float* acc_col = p.dq_acc + quad * 32 + (lane & ~3);
     uint32_t g = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
       const KvItem it = kv_decode<DENSE>(p, item, tiles);
-      float* acc_head = acc_col + it.head_off * DH;
+      float* acc_head = acc_col + (long long)it.head_off * DH;
       for (int i = 0; i < it.n_units; ++i, ++g) {
         const int first = unit_of<DENSE>(it, i) * QU + 64 * qhalf;
         // accumulator rows of queries lane and 32 + lane of this half of the unit (-1 beyond the list)
@@ -546,25 +562,25 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           }
       }
     }
-    if (warp == 16 && lane == 0) tflush(14, 1);     // [14] dq_full, [15] total
+    if (warp == 20 && lane == 0) tflush(14, 1);     // [14] dq_full, [15] total
   } else {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
     // ------------------------------------------------------------------ compute: warp = 32 keys x half of the unit's queries
     const int quad = warp & 3;
-    const int half = (warp - 8) >> 2;
+    const int half = (warp - 12) >> 2;
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
     const uint32_t st_t = tmem + lane_addr + ST_COL + 64 * half, dp_t = tmem + lane_addr + DPT_COL + 64 * half;
     // this lane's row address for stmatrix: matrices (keys 0-7, queries 8j), (keys 8-15, same), (keys 0-7, 8j + 8), ...
     const int mrow = quad * 32 + 8 * ((lane >> 3) & 1) + (lane & 7), mj = lane >> 4;
     const uint32_t ds_row = smem_u32(sDS) + half * PANEL + mrow * 128;
-    uint32_t n = 0, g = 0;
+    uint32_t n = 0, g = 0, slot = 0, par = 0;        // items and units done; slot and parity of the Q ring
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
       const KvItem it = kv_decode<DENSE>(p, item, tiles);
       if (it.n_units == 0) {
         // no query selected this block: its keys get zero gradients
         const int r = quad * 32 + lane;
         if (r < it.valid) {
-          const long long row_off = p.out_map.off(it.head_off + it.key0 + r, DH);
+          const long long row_off = p.out_map.off((long long)it.head_off + it.key0 + r, DH);
           const uint4 z = make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
@@ -577,10 +593,13 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       // rows beyond the key range hold other blocks' keys and must not contribute to dQ
       const int key = quad * 32 + (lane >> 2);
       for (int i = 0; i < it.n_units; ++i, ++g) {
-        const int slot = g & 1;
         const float2* lse2 = reinterpret_cast<const float2*>(sm->lse2[slot] + 64 * half) + (lane & 3);
-        const float2* negD = reinterpret_cast<const float2*>(sm->negD[slot] + 64 * half) + (lane & 3);
-        twait(0, &sm->q_full[slot], (g >> 1) & 1);     // publishes lse2 / negD of this unit
+        const float2* negD = reinterpret_cast<const float2*>(sm->negD[g & 1] + 64 * half) + (lane & 3);
+        twait(0, &sm->q_full[slot], par);              // publishes lse2 of this unit
+        if (++slot == NQ) { slot = 0; par ^= 1; }
+        float2 l[8];                                   // (fetched before the wait: next to a busy tensor pipe a load takes its time)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) l[j] = lse2[4 * j];
         twait(1, &sm->s_full, g & 1);
         tc_fence_after();
         // ---- P^T: thread holds keys key + 8 r (r = 0 .. 3) x queries 8 j + 2 (lane % 4) + {0, 1} of the half
@@ -594,14 +613,13 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
             const int j = 4 * c + jj;
-            const float2 l = lse2[4 * j];
 #pragma unroll
             for (int rh = 0; rh < 2; ++rh)
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 float x0, x1;
                 fma2(x0, x1, __uint_as_float(pv[rh][4 * j + 2 * e]), __uint_as_float(pv[rh][4 * j + 2 * e + 1]), p.scale_log2,
-                     p.scale_log2, -l.x, -l.y);
+                     p.scale_log2, -l[j].x, -l[j].y);
                 x0 = ex2(x0);
                 x1 = ex2(x1);
                 pv[rh][4 * j + 2 * e] = __float_as_uint(x0);
@@ -612,10 +630,15 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
           tmem_st_16x128_x4(st_t + 16 * c, pk[0]);
           tmem_st_16x128_x4(st_t + ROW16 + 16 * c, pk[1]);
         }
+        // negD of this unit (dV needs the dO rows anyway; asked before dV can run, so that the barrier cannot be a phase ahead)
+        twait(0, &sm->do_full, g & 1);
         tmem_st_wait();
         tc_fence_before();
         mbar_arrive(&sm->p_ready);
         // ---- dS^T = P^T (dP^T - D).  The dS^T tile in shared memory is free: dP^T was issued behind the dQ^T that read it.
+        float2 d[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) d[j] = negD[4 * j];
         twait(2, &sm->dp_full, g & 1);
         tc_fence_after();
 #pragma unroll
@@ -630,11 +653,10 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 #pragma unroll
             for (int jj = 0; jj < 4; ++jj) {
               const int j = 4 * c + jj;
-              const float2 d = negD[4 * j];
 #pragma unroll
               for (int e = 0; e < 2; ++e) {
                 float x0, x1;
-                add2(x0, x1, __uint_as_float(dp[rh][4 * jj + 2 * e]), __uint_as_float(dp[rh][4 * jj + 2 * e + 1]), d.x, d.y);
+                add2(x0, x1, __uint_as_float(dp[rh][4 * jj + 2 * e]), __uint_as_float(dp[rh][4 * jj + 2 * e + 1]), d[j].x, d[j].y);
                 mul2(x0, x1, x0, x1, __uint_as_float(pv[rh][4 * j + 2 * e]), __uint_as_float(pv[rh][4 * j + 2 * e + 1]));
                 dk_[2 * jj + e] = key + 16 * rh + 8 * e < it.valid ? pack_bf16(x0, x1) : 0u;
               }
@@ -655,7 +677,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       twait(3, &sm->acc_done, n & 1);
       tc_fence_after();
       const int r = quad * 32 + lane;
-      const long long row_off = r < it.valid ? p.out_map.off(it.head_off + it.key0 + r, DH) : 0;
+      const long long row_off = r < it.valid ? p.out_map.off((long long)it.head_off + it.key0 + r, DH) : 0;
 #pragma unroll 1
       for (int pass = 0; pass < 4; ++pass) {      // dV columns, then dK columns, 32 at a time
         const int cgrp = half * 2 + (pass & 1);
@@ -687,7 +709,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       }
       ++n;
     }
-    if (threadIdx.x == 256) tflush(9, 4);   // [9] q_full, [10] s_full, [11] dp_full, [12] acc_done, [13] total
+    if (threadIdx.x == 384) tflush(9, 4);   // [9] q_full, [10] s_full, [11] dp_full, [12] acc_done, [13] total
   }
   tc_fence_before();
   __syncthreads();
@@ -696,9 +718,12 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 
 template <bool DENSE>
 static int launch(const Dims& D, const void* k, const void* v, KvParams& kp, cudaStream_t st) {
-  CUtensorMap tmK, tmV;
+  CUtensorMap tmK, tmV, tmQ, tmO;
   const uint64_t rows = (uint64_t)D.BH * D.S;
   if (!sm100::make_tmap_bf16_rows(&tmK, k, rows, DH, BN) || !sm100::make_tmap_bf16_rows(&tmV, v, rows, DH, BN))
+    return VMOBA_ERR_CUDA;
+  // dense: units of consecutive rows (rows beyond a head's S read as zeros); sparse: not used
+  if (!sm100::make_tmap_bf16_heads(&tmQ, kp.q, D.BH, D.S, DH, QU) || !sm100::make_tmap_bf16_heads(&tmO, kp.d_o, D.BH, D.S, DH, QU))
     return VMOBA_ERR_CUDA;
   kp.S = D.S; kp.Nb = DENSE ? 1 : D.Nb; kp.sb = DENSE ? D.S : D.sb; kp.BH = D.BH;
   kp.scale = D.scale; kp.scale_log2 = D.scale * LOG2E;
@@ -710,7 +735,7 @@ static int launch(const Dims& D, const void* k, const void* v, KvParams& kp, cud
   const int grid = (int)std::max<long long>(1, std::min<long long>(items, sm_count()));
   auto kernel = kp.prof ? attn_bwd_fused_kernel<DENSE, true> : attn_bwd_fused_kernel<DENSE, false>;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-  kernel<<<grid, THREADS, SMEM_BYTES, st>>>(tmK, tmV, kp);
+  kernel<<<grid, THREADS, SMEM_BYTES, st>>>(tmK, tmV, tmQ, tmO, kp);
   VMOBA_LAUNCH_OK(1);
   return VMOBA_OK;
 }
