@@ -34,12 +34,20 @@ item_ptr_kernel(const int* __restrict__ kb_ptr, long long n_kb, int rows, long l
       item_ptr, n_kb, &total);
 }
 
-// item_tab[item] = index of the (batch, head, key block) list the item belongs to.
+// item_desc[item] = {index of the (batch, head, key block) list, first list position, rows (<= rows_per_item), 0}; a warp
+// per list (a thread per list took 13 us for 240 lists of 77 items, bound by the latency of its loop).
 static __global__ void __launch_bounds__(256)
-item_tab_kernel(const int* __restrict__ item_ptr, long long n_kb, long long max_items, int* __restrict__ item_tab) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_kb; i += (long long)gridDim.x * blockDim.x) {
-    const long long lo = item_ptr[i], hi = min((long long)item_ptr[i + 1], max_items);
-    for (long long t = lo; t < hi; ++t) item_tab[t] = (int)i;
+item_desc_kernel(const int* __restrict__ item_ptr, const int* __restrict__ kb_ptr, long long n_kb, long long max_items,
+                 long long capacity, int rows_per_item, int4* __restrict__ desc) {
+  const int lane = threadIdx.x & 31;
+  const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n_kb; i += n_warps) {
+    const long long t0 = item_ptr[i], t1 = min((long long)item_ptr[i + 1], max_items);
+    const long long lo = min((long long)kb_ptr[i], capacity), hi = min((long long)kb_ptr[i + 1], capacity);
+    for (long long t = t0 + lane; t < t1; t += 32) {
+      const long long l = lo + (t - t0) * rows_per_item;
+      desc[t] = make_int4((int)i, (int)l, (int)min((long long)rows_per_item, hi - l), 0);
+    }
   }
 }
 

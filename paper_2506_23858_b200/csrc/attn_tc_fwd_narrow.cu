@@ -101,20 +101,6 @@ __device__ __forceinline__ Item item_from_desc(const Params& p, const int4 d) {
   return it;
 }
 
-// item_desc[item] = {index of the (batch, head, key block) list, first list position, rows (<= rows_per_item), 0}
-static __global__ void __launch_bounds__(256)
-item_desc_kernel(const int* __restrict__ item_ptr, const int* __restrict__ kb_ptr, long long n_kb, long long max_items,
-                 long long capacity, int rows_per_item, int4* __restrict__ desc) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_kb; i += (long long)gridDim.x * blockDim.x) {
-    const long long t0 = item_ptr[i], t1 = min((long long)item_ptr[i + 1], max_items);
-    const long long lo = min((long long)kb_ptr[i], capacity), hi = min((long long)kb_ptr[i + 1], capacity);
-    for (long long t = t0; t < t1; ++t) {
-      const long long l = lo + (t - t0) * rows_per_item;
-      desc[t] = make_int4((int)i, (int)l, (int)min((long long)rows_per_item, hi - l), 0);
-    }
-  }
-}
-
 __device__ __forceinline__ constexpr uint32_t koff(int ks) { return (uint32_t)(((ks >> 2) * PANEL + (ks & 3) * 32) >> 4); }
 __device__ __forceinline__ constexpr uint32_t mnoff(int ks) { return (uint32_t)((ks * 2048) >> 4); }
 
@@ -696,7 +682,7 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
     return VMOBA_ERR_CUDA;
   const long long n_kb = (long long)D.BH * D.Nb;
   simt::item_ptr_kernel<<<1, 1024, 0, st>>>(kb_ptr, n_kb, BM, cap, item_ptr);
-  item_desc_kernel<<<(int)std::min<long long>((n_kb + 255) / 256, sm_count() * 4), 256, 0, st>>>(
+  simt::item_desc_kernel<<<(int)std::min<long long>((n_kb + 7) / 8, sm_count() * 8), 256, 0, st>>>(
       item_ptr, kb_ptr, n_kb, max_items, cap, BM, reinterpret_cast<int4*>(item_tab));
   Params p;
   p.q = (const __nv_bfloat16*)q; p.q_idx = q_idx; p.q_ptr = q_ptr; p.item_ptr = item_ptr;
