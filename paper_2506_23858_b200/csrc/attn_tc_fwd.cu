@@ -11,7 +11,7 @@
 //   warp 1        MMA issuer (the whole warp walks the loop, one elected lane issues)
 //   warps 4-7     softmax of tile A: thread = one query row, all 128 keys of the tile
 //   warps 8-11    softmax of tile B
-//   warps 12-15   loaders: gather the 256 Q rows (and per-row output bookkeeping) of the NEXT item
+//   warps 12-15   loaders: gather the 256 Q rows of the NEXT item
 //
 // TMEM: ONE score buffer S (128 columns) that A and B use in turn, P_A and P_B (64 columns each, bf16), the accumulators
 // O_A and O_B (128 columns each).  A softmax thread (200 registers) takes its whole row of 128 scores out of S at once and
@@ -36,7 +36,9 @@ constexpr int BM = 128;              // rows per query tile
 constexpr int IM = 2 * BM;           // query rows per item
 constexpr int BN = 128;              // keys per tile
 constexpr int DH = 128;              // head dim
-constexpr int STAGES = 2;            // K ring depth = V ring depth
+// K and V ring depths.  A V tile is needed by A and, half a period later, by B, and is reloaded after that: with two
+// stages the MMA warp waited for V tiles (700 of 4550 cycles per pair of tiles).
+constexpr int KST = 2, VST = 3;
 constexpr int PANEL = BM * 128;      // bytes of one 64-column panel of a 128-row tile (16 KB)
 constexpr int TILE = 2 * PANEL;      // bytes of a [128 x 128] bf16 tile (32 KB)
 constexpr int THREADS = 512;         // warp groups {TMA, MMA, -, -}, A, B, loaders; registers 56, 200, 200, 56 (= 4 x 128)
@@ -45,7 +47,7 @@ constexpr uint32_t P_COL = 128, O_COL = 256;      // S at 0, P_X at 128 + 64 X, 
 constexpr float RESCALE_LOG2 = 8.0f;
 
 struct Smem {
-  uint64_t k_full[STAGES], v_full[STAGES], k_empty[STAGES], v_empty[STAGES];
+  uint64_t k_full[KST], k_empty[KST], v_full[VST], v_empty[VST];
   uint64_t s_full[2], p_ready[2];    // per query tile: scores written (commit) / P written (128 arrivals)
   uint64_t s_free;                   // the score buffer has been read (128 arrivals of whichever tile used it)
   uint64_t o_done[2];                // per query tile: P V of a key tile complete (commit)
@@ -53,9 +55,10 @@ struct Smem {
   uint64_t q_full, q_empty;          // Q tiles of an item gathered (128 arrivals) / no longer needed (commit)
   uint32_t tmem_base;
   int abort_flag;
-  int qinfo[4][IM];                  // [item % 4][row]: 2 * in-head position + (query has a single block), -1 for padding rows
 };
-constexpr size_t SMEM_BYTES = 1024 /*alignment slack*/ + 2 * TILE /*Q*/ + 2 * STAGES * TILE + sizeof(Smem) + 32;
+// no alignment slack: the kernel checks that its dynamic shared memory starts on a 1024-byte boundary
+constexpr size_t SMEM_BYTES = (2 /*Q*/ + KST + VST) * TILE + sizeof(Smem) + 32;
+static_assert(SMEM_BYTES <= 232448, "wide forward: shared memory");
 
 struct Params {
   const __nv_bfloat16* q;
@@ -160,11 +163,15 @@ __global__ void __launch_bounds__(THREADS, 1)
 attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                      const __grid_constant__ CUtensorMap tmQ, const Params p) {
   extern __shared__ uint8_t smem_raw[];
-  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sQ = base;                      // [2 query tiles][TILE]
-  uint8_t* sK = base + 2 * TILE;           // [STAGES][TILE]
-  uint8_t* sV = sK + STAGES * TILE;        // [STAGES][TILE]
-  Smem* sm = reinterpret_cast<Smem*>(sV + STAGES * TILE);
+  // the swizzled tiles need 1024-byte alignment and there is no room for alignment slack
+  if ((smem_u32(smem_raw) & 1023u) != 0) {
+    if (threadIdx.x == 0) set_status(p.status, VMOBA_ERR_CUDA);
+    return;
+  }
+  uint8_t* sQ = smem_raw;                  // [2 query tiles][TILE]
+  uint8_t* sK = sQ + 2 * TILE;             // [KST][TILE]
+  uint8_t* sV = sK + KST * TILE;           // [VST][TILE]
+  Smem* sm = reinterpret_cast<Smem*>(sV + VST * TILE);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &sm->abort_flag;
   // diagnostics: cycles one representative thread per role spends in each section
@@ -186,10 +193,8 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
   };
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
-      mbar_init(&sm->k_full[s], 1); mbar_init(&sm->v_full[s], 1);
-      mbar_init(&sm->k_empty[s], 1); mbar_init(&sm->v_empty[s], 1);
-    }
+    for (int s = 0; s < KST; ++s) { mbar_init(&sm->k_full[s], 1); mbar_init(&sm->k_empty[s], 1); }
+    for (int s = 0; s < VST; ++s) { mbar_init(&sm->v_full[s], 1); mbar_init(&sm->v_empty[s], 1); }
     for (int x = 0; x < 2; ++x) {
       mbar_init(&sm->s_full[x], 1); mbar_init(&sm->p_ready[x], 128);
       mbar_init(&sm->o_done[x], 1); mbar_init(&sm->o_free[x], 128);
@@ -216,32 +221,29 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
-      uint32_t fills = 0;
+      uint32_t ks = 0, kp = 1, vs = 0, vp = 1;       // ring slots and the parities of their `empty` waits (the first pass at once)
       for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
         const FwdItem it = decode_item<DENSE>(p, item);
         const int row0 = (int)it.head_off + it.key_begin;
-        for (int t = 0; t < it.ntiles; ++t, ++fills) {
-          const int s = fills % STAGES;
-          const uint32_t par = ((fills / STAGES) - 1) & 1;
+        for (int t = 0; t < it.ntiles; ++t) {
           const int y = row0 + t * BN;
           // a K stage is free once both query tiles' Q K^T of the key tile have run, a V stage only
           // after both P V
-          if (fills >= STAGES) mbar_wait(&sm->k_empty[s], par, abort_flag, p.status);
-          mbar_expect_tx(&sm->k_full[s], TILE);
-          tma_load_2d(sK + s * TILE, &tmK, &sm->k_full[s], 0, y);
-          tma_load_2d(sK + s * TILE + PANEL, &tmK, &sm->k_full[s], 64, y);
-          if (fills >= STAGES) mbar_wait(&sm->v_empty[s], par, abort_flag, p.status);
-          mbar_expect_tx(&sm->v_full[s], TILE);
-          tma_load_2d(sV + s * TILE, &tmV, &sm->v_full[s], 0, y);
-          tma_load_2d(sV + s * TILE + PANEL, &tmV, &sm->v_full[s], 64, y);
-        }
-      }
-      // drain: every issued load must have landed before the CTA may exit (only matters after a timeout)
-      if (*abort_flag) {
-        const uint32_t first = fills > STAGES ? fills - STAGES : 0;
-        for (uint32_t f = first; f < fills; ++f) {
-          mbar_wait(&sm->k_full[f % STAGES], (f / STAGES) & 1, abort_flag, p.status);
-          mbar_wait(&sm->v_full[f % STAGES], (f / STAGES) & 1, abort_flag, p.status);
+          mbar_wait(&sm->k_empty[ks], kp, abort_flag, p.status);
+          mbar_expect_tx(&sm->k_full[ks], TILE);
+          tma_load_2d(sK + ks * TILE, &tmK, &sm->k_full[ks], 0, y);
+          tma_load_2d(sK + ks * TILE + PANEL, &tmK, &sm->k_full[ks], 64, y);
+          mbar_wait(&sm->v_empty[vs], vp, abort_flag, p.status);
+          mbar_expect_tx(&sm->v_full[vs], TILE);
+          tma_load_2d(sV + vs * TILE, &tmV, &sm->v_full[vs], 0, y);
+          tma_load_2d(sV + vs * TILE + PANEL, &tmV, &sm->v_full[vs], 64, y);
+          // drain: every issued load must have landed before the CTA may exit (only matters after a timeout)
+          if (*abort_flag) {
+            mbar_wait(&sm->k_full[ks], kp ^ 1, abort_flag, p.status);
+            mbar_wait(&sm->v_full[vs], vp ^ 1, abort_flag, p.status);
+          }
+          if (++ks == KST) { ks = 0; kp ^= 1; }
+          if (++vs == VST) { vs = 0; vp ^= 1; }
         }
       }
     }
@@ -251,81 +253,111 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     {
       const bool leader = elect_one();
       const int n_items_u = __reduce_max_sync(0xffffffffu, n_items);
-      uint32_t fills = 0;              // key tiles consumed so far (ring position of K and of V)
-      uint32_t n = 0;                  // items done so far
-      uint32_t uses = 0;               // uses of the score buffer so far (phase of s_free)
-      uint32_t tcnt[2] = {0, 0};       // key tiles done per query tile (phase of p_ready)
-      uint32_t ecnt[2] = {0, 0};       // items done per query tile (phase of o_free)
-      const uint64_t dQ[2] = {make_smem_desc(smem_u32(sQ), 16, 1024), make_smem_desc(smem_u32(sQ + TILE), 16, 1024)};
+      // A look at a barrier takes this warp some 300 cycles while the tensor pipe streams its operands out of shared
+      // memory, whether it has completed or not, and two or three barriers stand before every product.  So the lanes look
+      // at different barriers of an operation in one instruction, and they look before the operation ahead of it is issued
+      // (one look after the other took 2050 of the 4400 cycles per pair of tiles).
+      struct Wait { uint32_t bar, par; };                              // what this lane looks at
+      auto wait_set = [&](uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, bool third, uint64_t* b2, uint32_t p2) -> Wait {
+        const int which = lane & 3;
+        Wait w{smem_u32(b0), p0};
+        if (which == 1) w = Wait{smem_u32(b1), p1};
+        if (which == 2 && third) w = Wait{smem_u32(b2), p2};
+        return w;
+      };
+      auto finish = [&](const Wait& w, bool seen) {
+        if (!__all_sync(0xffffffffu, seen)) mbar_wait_lanes(w.bar, w.par, abort_flag, p.status);
+        __syncwarp();
+      };
+      uint32_t n = 0;                               // items done so far
+      uint32_t uses = 0;                            // uses of the score buffer so far (phase of s_free)
+      uint32_t k_slot = 0, k_par = 0;               // K ring position of the next key tile
+      struct Tile { uint32_t v_slot, v_par;         // V ring position of the next P V
+                    uint32_t tcnt, ecnt; };         // P V and items done (phases of p_ready and o_free)
+      Tile ta{0, 0, 0, 0}, tb{0, 0, 0, 0};
+      const uint64_t dQ0 = make_smem_desc(smem_u32(sQ), 16, 1024);
       for (int item = blockIdx.x; item < n_items_u; item += gridDim.x, ++n) {
         FwdItem it = decode_item<DENSE>(p, item);
         it.nx = __reduce_max_sync(0xffffffffu, it.nx);
-        lap(5);
-        mbar_wait_warp(&sm->q_full, n & 1, abort_flag, p.status);
-        lap(0);
-        tc_fence_after();
-        auto qk = [&](int x, int t, int s) {
-          lap(5);
-          if (uses >= 1) mbar_wait_warp(&sm->s_free, (uses - 1) & 1, abort_flag, p.status);
-          lap(4);
-          ++uses;
+        const int nx = it.nx, ntiles = it.ntiles;
+        // The score buffer has been read (its first use waits for a phase before the first: passes at once), the K tile is there
+        auto qk_set = [&]() { return wait_set(&sm->s_free, (uses + 1) & 1, &sm->k_full[k_slot], k_par, false, nullptr, 0u); };
+        // P has been written, the V tile is there, the epilogue of the tile's previous item has read the accumulator
+        auto pv_set = [&](int x, int t) {
+          const Tile q = x ? tb : ta;
+          return wait_set(&sm->p_ready[x], q.tcnt & 1, &sm->v_full[q.v_slot], q.v_par, t == 0, &sm->o_free[x], (q.ecnt + 1) & 1);
+        };
+        auto qk = [&](int x, int t, uint32_t slot) {
           tc_fence_after();
           const int n_mma = (min(BN, it.n_keys - t * BN) + 15) & ~15;
           const uint32_t idesc = make_idesc_bf16(BM, n_mma, false, false);
-          const uint64_t dK0 = make_smem_desc(smem_u32(sK + s * TILE), 16, 1024);
+          const uint64_t dK0 = make_smem_desc(smem_u32(sK + slot * TILE), 16, 1024);
 #pragma unroll
           for (int ks = 0; ks < DH / 16; ++ks)
-            if (leader) mma_ss(tmem, dQ[x] + koff(ks), dK0 + koff(ks), idesc, ks > 0 ? 1u : 0u);
+            if (leader) mma_ss(tmem, dQ0 + (x ? (uint32_t)(TILE >> 4) : 0u) + koff(ks), dK0 + koff(ks), idesc, ks > 0 ? 1u : 0u);
           if (leader) mma_commit(&sm->s_full[x]);
+          if (x == nx - 1) {
+            if (leader) mma_commit(&sm->k_empty[slot]);
+            if (leader && t == ntiles - 1) mma_commit(&sm->q_empty);
+          }
         };
-        auto pv = [&](int x, int t, uint32_t f) {
-          const int s = f % STAGES;
-          lap(5);
-          mbar_wait_warp(&sm->p_ready[x], tcnt[x] & 1, abort_flag, p.status);
-          lap(2);
-          mbar_wait_warp(&sm->v_full[s], (f / STAGES) & 1, abort_flag, p.status);
-          // the accumulator was last used by the previous item on this query tile: its epilogue must have read it
-          if (t == 0 && ecnt[x] >= 1) mbar_wait_warp(&sm->o_free[x], (ecnt[x] - 1) & 1, abort_flag, p.status);
-          lap(3);
+        auto pv = [&](int x, int t, uint32_t slot) {
           tc_fence_after();
           const int ksteps = (min(BN, it.n_keys - t * BN) + 15) >> 4;
-          const uint64_t mV0 = make_smem_desc(smem_u32(sV + s * TILE), PANEL, 1024);
+          const uint64_t mV0 = make_smem_desc(smem_u32(sV + slot * TILE), PANEL, 1024);
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks)
             if (leader && ks < ksteps)   // P of keys 16 ks .. 16 ks + 15 sits in columns 8 ks .. of the tile's P buffer
               mma_ts(tmem + O_COL + x * 128, tmem + P_COL + x * 64 + ks * 8, mV0 + mnoff(ks), IDESC_PV, (t > 0 || ks > 0) ? 1u : 0u);
           if (leader) mma_commit(&sm->o_done[x]);
-          if (leader && x == it.nx - 1) mma_commit(&sm->v_empty[s]);
-          tcnt[x] += 1;
+          if (leader && x == nx - 1) mma_commit(&sm->v_empty[slot]);
         };
-        // A tile's P V(t-1) goes out behind its Q K^T(t): by then the other tile has had its turn on the score buffer
-        for (int t = 0; t < it.ntiles; ++t) {
-          const uint32_t f = fills + t;
-          const int s = f % STAGES;
-          lap(5);
-          mbar_wait_warp(&sm->k_full[s], (f / STAGES) & 1, abort_flag, p.status);
-          lap(1);
-          qk(0, t, s);
-          if (it.nx == 1) {
-            if (leader) mma_commit(&sm->k_empty[s]);
-            if (leader && t == it.ntiles - 1) mma_commit(&sm->q_empty);
-          }
-          if (t > 0) pv(0, t - 1, f - 1);
-          if (it.nx == 2) {
-            qk(1, t, s);
-            if (leader) mma_commit(&sm->k_empty[s]);
-            if (leader && t == it.ntiles - 1) mma_commit(&sm->q_empty);
-            if (t > 0) pv(1, t - 1, f - 1);
+        // Order: Q K^T(x, t), P V(x, t - 1) for x = A, B: a tile's P V goes out behind its next Q K^T, by then the other
+        // tile has had its turn on the score buffer.
+        lap(5);
+        mbar_wait_warp(&sm->q_full, n & 1, abort_flag, p.status);
+        lap(0);
+        Wait next = qk_set();
+        bool seen = mbar_test(next.bar, next.par);
+        for (int t = 0; t <= ntiles; ++t) {
+          const uint32_t slot_k = k_slot;
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            if (x >= nx) continue;
+            auto after = [&]() {                    // what comes behind step (x, t)
+              const bool to_b = x == 0 && nx == 2;
+              const int t_next = to_b ? t : t + 1;
+              return t_next < ntiles ? qk_set() : pv_set(to_b, ntiles - 1);
+            };
+            if (t < ntiles) {
+              lap(5);
+              finish(next, seen);
+              lap(1);
+              ++uses;
+              if (x == nx - 1 && ++k_slot == KST) { k_slot = 0; k_par ^= 1; }
+              next = t > 0 ? pv_set(x, t - 1) : after();
+              seen = mbar_test(next.bar, next.par);
+              qk(x, t, slot_k);
+            }
+            if (t > 0) {
+              lap(5);
+              finish(next, seen);
+              lap(2);
+              Tile& q = x ? tb : ta;
+              const uint32_t slot_v = q.v_slot;
+              q.tcnt += 1;
+              if (++q.v_slot == VST) { q.v_slot = 0; q.v_par ^= 1; }
+              if (nx == 1) { tb.v_slot = ta.v_slot; tb.v_par = ta.v_par; }
+              if (t < ntiles || x < nx - 1) {
+                next = after();
+                seen = mbar_test(next.bar, next.par);
+              }
+              pv(x, t - 1, slot_v);
+            }
           }
         }
-        {
-          const uint32_t f = fills + it.ntiles - 1;
-          pv(0, it.ntiles - 1, f);
-          if (it.nx == 2) pv(1, it.ntiles - 1, f);
-        }
-        fills += it.ntiles;
-        ecnt[0] += 1;
-        if (it.nx == 2) ecnt[1] += 1;
+        ta.ecnt += 1;
+        if (nx == 2) tb.ecnt += 1;
       }
       lap(5);
       if (leader) tflush(8);
@@ -340,27 +372,8 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     uint32_t n = 0;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
       const FwdItem it = decode_item<DENSE>(p, item);
-      int info[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int row = h * BM + lt;
-        info[h] = -1;
-        if (row < it.n_rows) {
-          const int qp = DENSE ? it.list_lo + row : checked_index(__ldg(p.q_idx + it.list_lo + row), p.S, p.status);
-          bool direct = true;
-          if (!DENSE) {
-            const long long G_ = it.head_off + qp;
-            direct = __ldg(p.q_ptr + G_ + 1) - __ldg(p.q_ptr + G_) == 1;
-          }
-          info[h] = 2 * qp + (direct ? 1 : 0);
-        }
-      }
       if constexpr (DENSE) {
         if (n >= 1) mbar_wait(&sm->q_empty, (n - 1) & 1, abort_flag, p.status);
-        // Four bookkeeping slots: the softmax warps read slot n % 4 in the epilogue of item n, and the
-        // loaders can be at most two items ahead of an epilogue.
-        sm->qinfo[n & 3][lt] = info[0];
-        sm->qinfo[n & 3][BM + lt] = info[1];
         if (lt == 0) {
           mbar_expect_tx(&sm->q_full, it.nx * TILE);
           for (int x = 0; x < it.nx; ++x) {
@@ -389,8 +402,6 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         }
         // both Q tiles are free once the previous item's last Q K^T has run
         if (n >= 1) mbar_wait(&sm->q_empty, (n - 1) & 1, abort_flag, p.status);
-        sm->qinfo[n & 3][lt] = info[0];
-        sm->qinfo[n & 3][BM + lt] = info[1];
         const uint32_t dst = smem_u32(sQ) + r0 * 128 + ((chunk ^ (r0 & 7)) << 4);
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
@@ -417,11 +428,16 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     const uint32_t s_tmem = tmem + lane_addr;
     const uint32_t p_tmem = tmem + lane_addr + P_COL + x * 64;
     const uint32_t o_tmem = tmem + lane_addr + O_COL + x * 128;
-    uint32_t tc = 0, n = 0;                          // key tiles done on this query tile; items seen
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
+    uint32_t tc = 0;                                 // key tiles done on this query tile
+    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
       const FwdItem it = decode_item<DENSE>(p, item);
       if (x >= it.nx) continue;
       float m_used = -INFINITY, l = 0.f, l_r = 0.f;   // l: exact sum (for LSE); l_r: sum of the bf16-rounded weights
+      // where this thread's row goes; the list entry is asked for now, what hangs on it during the first key tile
+      const int row = x * BM + r;
+      const bool row_ok = row < it.n_rows;
+      const int qpos = !row_ok ? 0 : DENSE ? it.list_lo + row : checked_index(__ldg(p.q_idx + it.list_lo + row), p.S, p.status);
+      int n_pairs = 1;
       for (int t = 0; t < it.ntiles; ++t, ++tc) {
         lap(3);
         mbar_wait(&sm->s_full[x], tc & 1, abort_flag, p.status);
@@ -459,29 +475,41 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
           m_used = mx;
           need = true;
         }
-        // P V of the tile before must be complete before P is overwritten and before O is rescaled
-        if (t > 0) {
-          mbar_wait(&sm->o_done[x], (tc - 1) & 1, abort_flag, p.status);
-          tc_fence_after();
-          if (__any_sync(0xffffffffu, need)) {
+        auto rescale_o = [&]() {                     // P V of the tile before is complete
 #pragma unroll 1
-            for (int c = 0; c < 8; ++c) {
-              uint32_t ov[16];
-              tmem_ld16(o_tmem + c * 16, ov);
-              tmem_ld_wait();
+          for (int c = 0; c < 8; ++c) {
+            uint32_t ov[16];
+            tmem_ld16(o_tmem + c * 16, ov);
+            tmem_ld_wait();
 #pragma unroll
-              for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * factor);
-              tmem_st16(o_tmem + c * 16, ov);
-            }
-            l *= factor;
-            l_r *= factor;
+            for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * factor);
+            tmem_st16(o_tmem + c * 16, ov);
           }
-        }
-        lap(2);
+        };
+        if (!DENSE && t == 0) n_pairs = __ldg(p.q_ptr + it.head_off + qpos + 1) - __ldg(p.q_ptr + it.head_off + qpos);
         float s0 = 0.f, s1 = 0.f, r0 = 0.f, r1 = 0.f;
         const float neg_m = -m_used;
+        {
+          // the first half's weights stay in registers until P V of the tile before has read the P buffer
+          uint32_t pk[2][16];
+          exp_pack32(sv, p.scale_log2, neg_m, pk[0], s0, s1, r0, r1);
+          if (valid > 32) exp_pack32(sv + 32, p.scale_log2, neg_m, pk[1], s0, s1, r0, r1);
+          lap(3);
+          if (t > 0) {
+            mbar_wait(&sm->o_done[x], (tc - 1) & 1, abort_flag, p.status);
+            tc_fence_after();
+            if (__any_sync(0xffffffffu, need)) {
+              rescale_o();
+              l *= factor;
+              l_r *= factor;
+            }
+          }
+          lap(2);
+          tmem_st16(p_tmem, pk[0]);
+          tmem_st16(p_tmem + 16, pk[1]);             // (whatever it holds where valid <= 32: P V does not read it)
+        }
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
+        for (int c = 2; c < 4; ++c) {
           if (32 * c < valid) {                      // (uniform; P V takes the keys up to `valid` only)
             uint32_t pk[16];
             exp_pack32(sv + 32 * c, p.scale_log2, neg_m, pk, s0, s1, r0, r1);
@@ -498,11 +526,7 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
       lap(3);
       mbar_wait(&sm->o_done[x], (tc - 1) & 1, abort_flag, p.status);
       tc_fence_after();
-      const int row = x * BM + r;
-      const int info = sm->qinfo[n & 3][row];
-      const bool row_ok = info >= 0;
-      const int qpos = row_ok ? info >> 1 : 0;
-      const bool direct = (info & 1) != 0;
+      const bool direct = n_pairs == 1;           // the query has a single block: final result
       const float inv = 1.0f / l_r;
       const float row_lse = (m_used + log2f(l)) * 0.6931471805599453f;
       const long long G_ = it.head_off + qpos;

@@ -73,6 +73,39 @@ __device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, v
   __syncwarp();
 }
 
+// One look at a barrier (shared-memory address), without suspending: has the phase of this parity completed?  Only
+// meaningful when the phase before it is known to have completed.
+__device__ __forceinline__ bool mbar_test(uint32_t bar_addr, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar_addr), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bounded wait of a whole warp whose lanes look at different barriers: returns when every lane's phase has completed.
+__device__ __forceinline__ void mbar_wait_lanes(uint32_t bar_addr, uint32_t parity, volatile int* abort_flag, int32_t* status) {
+  constexpr uint32_t kPolls = 1u << 22;
+  const uint32_t limit = __reduce_max_sync(0xffffffffu, *abort_flag ? 16u : kPolls);
+  for (uint32_t i = 0; i < limit; ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar_addr), "r"(parity)
+        : "memory");
+    if (__all_sync(0xffffffffu, ok != 0)) return;
+    if (i > 4096) __nanosleep(64);
+  }
+  *abort_flag = 1;
+  set_status(status, VMOBA_ERR_TIMEOUT);
+}
+
 // ---------------------------------------------------------------- fences
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
