@@ -106,9 +106,6 @@ __device__ __forceinline__ FwdItem decode_item(const Params& p, int item) {
   return it;
 }
 
-__device__ __forceinline__ constexpr uint32_t koff(int ks) { return (uint32_t)(((ks >> 2) * PANEL + (ks & 3) * 32) >> 4); }
-__device__ __forceinline__ constexpr uint32_t mnoff(int ks) { return (uint32_t)((ks * 2048) >> 4); }
-
 // p = 2^(s * scale - m) for 32 scores; bf16 pairs (keys 2i, 2i+1 -> word i); s0/s1 collect the exact
 // weights, r0/r1 the bf16-rounded ones (the tensor core multiplies the ROUNDED weights: O is
 // normalised by their sum, so that the rounding perturbs the weights but never their total).
@@ -255,8 +252,8 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
       const int n_items_u = __reduce_max_sync(0xffffffffu, n_items);
       // A look at a barrier takes this warp some 300 cycles while the tensor pipe streams its operands out of shared
       // memory, whether it has completed or not, and two or three barriers stand before every product.  So the lanes look
-      // at different barriers of an operation in one instruction, and they look before the operation ahead of it is issued
-      // (one look after the other took 2050 of the 4400 cycles per pair of tiles).
+      // at different barriers of an operation in one instruction, and the look is under way while the operation ahead of it
+      // is issued (one look after the other took 2050 of the 4400 cycles per pair of tiles).
       struct Wait { uint32_t bar, par; };                              // what this lane looks at
       auto wait_set = [&](uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, bool third, uint64_t* b2, uint32_t p2) -> Wait {
         const int which = lane & 3;
@@ -275,7 +272,7 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
       struct Tile { uint32_t v_slot, v_par;         // V ring position of the next P V
                     uint32_t tcnt, ecnt; };         // P V and items done (phases of p_ready and o_free)
       Tile ta{0, 0, 0, 0}, tb{0, 0, 0, 0};
-      const uint64_t dQ0 = make_smem_desc(smem_u32(sQ), 16, 1024);
+      const uint32_t lo_q = desc_lo(smem_u32(sQ), 16), lo_k = desc_lo(smem_u32(sK), 16), lo_v = desc_lo(smem_u32(sV), PANEL);
       for (int item = blockIdx.x; item < n_items_u; item += gridDim.x, ++n) {
         FwdItem it = decode_item<DENSE>(p, item);
         it.nx = __reduce_max_sync(0xffffffffu, it.nx);
@@ -287,30 +284,28 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
           const Tile q = x ? tb : ta;
           return wait_set(&sm->p_ready[x], q.tcnt & 1, &sm->v_full[q.v_slot], q.v_par, t == 0, &sm->o_free[x], (q.ecnt + 1) & 1);
         };
-        auto qk = [&](int x, int t, uint32_t slot) {
+        auto qk = [&](int x, int t, uint32_t slot, const Wait& w) -> bool {
           tc_fence_after();
           const int n_mma = (min(BN, it.n_keys - t * BN) + 15) & ~15;
           const uint32_t idesc = make_idesc_bf16(BM, n_mma, false, false);
-          const uint64_t dK0 = make_smem_desc(smem_u32(sK + slot * TILE), 16, 1024);
-#pragma unroll
-          for (int ks = 0; ks < DH / 16; ++ks)
-            if (leader) mma_ss(tmem, dQ0 + (x ? (uint32_t)(TILE >> 4) : 0u) + koff(ks), dK0 + koff(ks), idesc, ks > 0 ? 1u : 0u);
+          const bool seen_ = mma8_ss_test<OffK128, OffK128>(tmem, lo_q + (x ? (uint32_t)(TILE >> 4) : 0u), lo_k + slot * (TILE >> 4), idesc,
+                                                            leader, DH / 16, 0u, w.bar, w.par);
           if (leader) mma_commit(&sm->s_full[x]);
           if (x == nx - 1) {
             if (leader) mma_commit(&sm->k_empty[slot]);
             if (leader && t == ntiles - 1) mma_commit(&sm->q_empty);
           }
+          return seen_;
         };
-        auto pv = [&](int x, int t, uint32_t slot) {
+        auto pv = [&](int x, int t, uint32_t slot, const Wait& w) -> bool {
           tc_fence_after();
           const int ksteps = (min(BN, it.n_keys - t * BN) + 15) >> 4;
-          const uint64_t mV0 = make_smem_desc(smem_u32(sV + slot * TILE), PANEL, 1024);
-#pragma unroll
-          for (int ks = 0; ks < 8; ++ks)
-            if (leader && ks < ksteps)   // P of keys 16 ks .. 16 ks + 15 sits in columns 8 ks .. of the tile's P buffer
-              mma_ts(tmem + O_COL + x * 128, tmem + P_COL + x * 64 + ks * 8, mV0 + mnoff(ks), IDESC_PV, (t > 0 || ks > 0) ? 1u : 0u);
+          // P of keys 16 ks .. 16 ks + 15 sits in columns 8 ks .. of the tile's P buffer
+          const bool seen_ = mma8_ts_test<OffTmem8, OffMN>(tmem + O_COL + x * 128, tmem + P_COL + x * 64, lo_v + slot * (TILE >> 4), IDESC_PV,
+                                                           leader, ksteps, t > 0 ? 1u : 0u, w.bar, w.par);
           if (leader) mma_commit(&sm->o_done[x]);
           if (leader && x == nx - 1) mma_commit(&sm->v_empty[slot]);
+          return seen_;
         };
         // Order: Q K^T(x, t), P V(x, t - 1) for x = A, B: a tile's P V goes out behind its next Q K^T, by then the other
         // tile has had its turn on the score buffer.
@@ -336,8 +331,7 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
               ++uses;
               if (x == nx - 1 && ++k_slot == KST) { k_slot = 0; k_par ^= 1; }
               next = t > 0 ? pv_set(x, t - 1) : after();
-              seen = mbar_test(next.bar, next.par);
-              qk(x, t, slot_k);
+              seen = qk(x, t, slot_k, next);
             }
             if (t > 0) {
               lap(5);
@@ -348,11 +342,8 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
               q.tcnt += 1;
               if (++q.v_slot == VST) { q.v_slot = 0; q.v_par ^= 1; }
               if (nx == 1) { tb.v_slot = ta.v_slot; tb.v_par = ta.v_par; }
-              if (t < ntiles || x < nx - 1) {
-                next = after();
-                seen = mbar_test(next.bar, next.par);
-              }
-              pv(x, t - 1, slot_v);
+              if (t < ntiles || x < nx - 1) next = after();
+              seen = pv(x, t - 1, slot_v, next);
             }
           }
         }
