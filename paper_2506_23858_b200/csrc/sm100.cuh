@@ -73,19 +73,6 @@ __device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, v
   __syncwarp();
 }
 
-// One look at a barrier (shared-memory address), without suspending: has the phase of this parity completed?  Only
-// meaningful when the phase before it is known to have completed.
-__device__ __forceinline__ bool mbar_test(uint32_t bar_addr, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar_addr), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
 // Bounded wait of a whole warp whose lanes look at different barriers: returns when every lane's phase has completed.
 __device__ __forceinline__ void mbar_wait_lanes(uint32_t bar_addr, uint32_t parity, volatile int* abort_flag, int32_t* status) {
   constexpr uint32_t kPolls = 1u << 22;
@@ -224,61 +211,6 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
       "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
-// A k-loop of up to eight MMAs with a look at a barrier (mbar_test) in flight behind it: the look takes about 300 cycles
-// next to a busy tensor pipe, and an instruction that used its outcome ahead of the MMAs would hold them up.  Operands are
-// the low words of descriptors that share the high word DESC_HI_SW128 (or TMEM columns for A); step ks adds a_off(ks),
-// b_off(ks).  nk: steps to issue; leader: the one lane that issues; acc0: whether the first step accumulates.  Returns the
-// outcome of the look.
-constexpr uint32_t DESC_HI_SW128 = (1024u >> 4) | (1u << 14) | (2u << 29);   // 1024 bytes between groups of 8 rows, version 1, 128-byte swizzle
-__device__ __forceinline__ uint32_t desc_lo(uint32_t smem_addr, uint32_t lbo_bytes) {
-  return ((smem_addr & 0x3ffffu) >> 4) | ((lbo_bytes >> 4) << 16);
-}
-struct OffK128 {      // K-major [128 rows x 128] tile: two panels of 64 columns
-  __host__ __device__ static constexpr uint32_t at(int ks) { return (uint32_t)(((ks >> 2) * 16384 + (ks & 3) * 32) >> 4); }
-};
-struct OffMN {        // MN-major tile: 16 rows of 128 bytes per step
-  __host__ __device__ static constexpr uint32_t at(int ks) { return (uint32_t)((ks * 2048) >> 4); }
-};
-struct OffTmem8 {     // bf16 A operand in TMEM: 8 columns per step
-  __host__ __device__ static constexpr uint32_t at(int ks) { return (uint32_t)(ks * 8); }
-};
-struct OffTmemHalves {    // the same, 64 columns apart for the two halves of eight steps
-  __host__ __device__ static constexpr uint32_t at(int ks) { return (uint32_t)((ks >> 2) * 64 + (ks & 3) * 8); }
-};
-#define VMOBA_SS_STEP(ks, ao, bo)                                                                                      \
-  "setp.gt.s32 pk, %6, " #ks ";\n\tadd.u32 al, %2, " ao ";\n\tadd.u32 bl, %3, " bo ";\n\t"                            \
-  "mov.b64 da, {al, %5};\n\tmov.b64 db, {bl, %5};\n\t"                                                                \
-  "@pk tcgen05.mma.cta_group::1.kind::f16 [%1], da, db, %4, pa;\n\tsetp.eq.u32 pa, 0, 0;\n\t"
-#define VMOBA_TS_STEP(ks, ao, bo)                                                                                      \
-  "setp.gt.s32 pk, %6, " #ks ";\n\tadd.u32 al, %2, " ao ";\n\tadd.u32 bl, %3, " bo ";\n\t"                            \
-  "mov.b64 db, {bl, %5};\n\t"                                                                                          \
-  "@pk tcgen05.mma.cta_group::1.kind::f16 [%1], [al], db, %4, pa;\n\tsetp.eq.u32 pa, 0, 0;\n\t"
-#define VMOBA_MMA8(NAME, STEP, DECL)                                                                                   \
-  template <typename AOff, typename BOff>                                                                              \
-  __device__ __forceinline__ bool NAME(uint32_t d_tmem, uint32_t a, uint32_t b, uint32_t idesc, bool leader, int nk, \
-                                       uint32_t acc0, uint32_t bar, uint32_t parity) {                                                \
-    uint32_t seen;                                                                                                     \
-    asm volatile("{\n\t.reg .pred pw, pk, pa, pl;\n\t.reg .b32 al, bl;\n\t" DECL                                           \
-                 "mbarrier.test_wait.parity.shared::cta.b64 pw, [%8], %9;\n\tsetp.ne.b32 pa, %7, 0;\n\t"               \
-                 "setp.eq.u32 pl, %26, 0;\n\t@pl bra SKIP;\n\t"                                                        \
-                 STEP(0, "%10", "%18") STEP(1, "%11", "%19") STEP(2, "%12", "%20") STEP(3, "%13", "%21")               \
-                 STEP(4, "%14", "%22") STEP(5, "%15", "%23") STEP(6, "%16", "%24") STEP(7, "%17", "%25")               \
-                 "SKIP:\n\tselp.u32 %0, 1, 0, pw;\n\t}"                                                                         \
-                 : "=r"(seen)                                                                                          \
-                 : "r"(d_tmem), "r"(a), "r"(b), "r"(idesc), "r"(DESC_HI_SW128), "r"(nk), "r"(acc0), "r"(bar), "r"(parity), \
-                   "n"(AOff::at(0)), "n"(AOff::at(1)), "n"(AOff::at(2)), "n"(AOff::at(3)), "n"(AOff::at(4)),           \
-                   "n"(AOff::at(5)), "n"(AOff::at(6)), "n"(AOff::at(7)), "n"(BOff::at(0)), "n"(BOff::at(1)),           \
-                   "n"(BOff::at(2)), "n"(BOff::at(3)), "n"(BOff::at(4)), "n"(BOff::at(5)), "n"(BOff::at(6)),           \
-                   "n"(BOff::at(7)), "r"((uint32_t)leader)                                                             \
-                 : "memory");                                                                                          \
-    return seen != 0;                                                                                                  \
-  }
-VMOBA_MMA8(mma8_ss_test, VMOBA_SS_STEP, ".reg .b64 da, db;\n\t")     // A and B from shared memory
-VMOBA_MMA8(mma8_ts_test, VMOBA_TS_STEP, ".reg .b64 db;\n\t")         // A from TMEM
-#undef VMOBA_MMA8
-#undef VMOBA_SS_STEP
-#undef VMOBA_TS_STEP
-
 // Arrive on an mbarrier when all MMAs issued so far by this thread have completed.
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
