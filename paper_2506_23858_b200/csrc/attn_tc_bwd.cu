@@ -173,32 +173,10 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
-// All operand tiles have 128-byte rows, 128-byte swizzle and 1024 bytes between groups of eight rows: their descriptors
-// share the high word, and the low word is the address (16-byte units) plus the stride to the next 64 columns.  Only
-// 32-bit arithmetic on the low word is left to the issuing warp.
-constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
-__device__ __forceinline__ uint32_t lo_k(uint32_t tile_addr) { return ((tile_addr & 0x3ffffu) >> 4) | (1u << 16); }
-__device__ __forceinline__ uint32_t lo_mn(uint32_t tile_addr) { return ((tile_addr & 0x3ffffu) >> 4) | ((uint32_t)(PANEL >> 4) << 16); }
+__device__ __forceinline__ uint32_t lo_k(uint32_t tile_addr) { return desc_lo(tile_addr, 16); }
+__device__ __forceinline__ uint32_t lo_mn(uint32_t tile_addr) { return desc_lo(tile_addr, PANEL); }
 __device__ __forceinline__ constexpr uint32_t koff(int ks) { return (uint32_t)(((ks >> 2) * PANEL + (ks & 3) * 32) >> 4); }
 __device__ __forceinline__ constexpr uint32_t mnoff(int ks) { return (uint32_t)((ks * 2048) >> 4); }
-__device__ __forceinline__ void mma_ss_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "mov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(DESC_HI)
-      : "memory");
-}
-__device__ __forceinline__ void mma_ts_lo(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
-      "mov.b64 db, {%2, %5};\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n\t}" ::"r"(d_tmem),
-      "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(DESC_HI)
-      : "memory");
-}
 
 // Fragment shapes.  16x256b: of 16 TMEM lanes x 8 columns per repetition j, thread l holds lane l / 4 (registers 4j,
 // 4j+1) and lane l / 4 + 8 (4j+2, 4j+3), columns 8j + 2 (l % 4) and the next.  16x128b: lane l / 4 (2j) and l / 4 + 8

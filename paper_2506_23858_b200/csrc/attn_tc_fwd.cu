@@ -8,7 +8,7 @@
 // query tiles (A and B) that share each K/V tile, which halves the bytes per MMA.
 //
 //   warp 0        TMA producer: K and V tiles into two 2-stage rings
-//   warp 1        MMA issuer (the whole warp walks the loop, one elected lane issues); warp 2 waits for its operands
+//   warps 1, 2    MMA issuers: Q K^T, P V
 //   warps 4-7     softmax of tile A: thread = one query row, all 128 keys of the tile
 //   warps 8-11    softmax of tile B
 //   warps 12-15   loaders: gather the 256 Q rows of the NEXT item
@@ -39,10 +39,9 @@ constexpr int DH = 128;              // head dim
 // K and V ring depths.  A V tile is needed by A and, half a period later, by B, and is reloaded after that: with two
 // stages the MMA warp waited for V tiles (700 of 4550 cycles per pair of tiles).
 constexpr int KST = 2, VST = 3;
-constexpr int LAG2 = 2;              // with two query tiles: P V(u - 2) behind Q K^T(u)
 constexpr int PANEL = BM * 128;      // bytes of one 64-column panel of a 128-row tile (16 KB)
 constexpr int TILE = 2 * PANEL;      // bytes of a [128 x 128] bf16 tile (32 KB)
-constexpr int THREADS = 512;         // warp groups {TMA, MMA, waits, -}, A, B, loaders; registers 56, 200, 200, 56 (= 4 x 128)
+constexpr int THREADS = 512;         // warp groups {TMA, MMA, MMA, -}, A, B, loaders; registers 56, 200, 200, 56 (= 4 x 128)
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t P_COL = 128, O_COL = 256;      // S at 0, P_X at 128 + 64 X, O_X at 256 + 128 X
 constexpr float RESCALE_LOG2 = 8.0f;
@@ -109,20 +108,6 @@ __device__ __forceinline__ FwdItem decode_item(const Params& p, int item) {
 
 __device__ __forceinline__ constexpr uint32_t koff(int ks) { return (uint32_t)(((ks >> 2) * PANEL + (ks & 3) * 32) >> 4); }
 __device__ __forceinline__ constexpr uint32_t mnoff(int ks) { return (uint32_t)((ks * 2048) >> 4); }
-
-// Order of the matrix products of an item: uses of the score buffer u = A(0), B(0), A(1), ..., each Q K^T(u) followed by
-// P V(u - lag).
-struct OpOrder {
-  int nx, n_uses, lag;
-  __device__ __forceinline__ OpOrder(int nx_, int ntiles) : nx(nx_), n_uses(nx_ * ntiles), lag(nx_ == 2 ? LAG2 : 1) {}
-  __device__ __forceinline__ int x_of(int u) const { return nx == 2 ? u & 1 : 0; }
-  __device__ __forceinline__ int t_of(int u) const { return nx == 2 ? u >> 1 : u; }
-};
-
-// Operation `op` may be issued: from the waiting warp to the MMA warp through one of four hardware barriers.  The waiting
-// warp cannot be four operations ahead: an operation's own conditions hang on the one two uses of the score buffer before.
-__device__ __forceinline__ void hand_over(uint32_t op) { asm volatile("bar.sync %0, 64;" ::"r"(1 + (op & 3)) : "memory"); }
-__device__ __forceinline__ void hand_over_arrive(uint32_t op) { asm volatile("bar.arrive %0, 64;" ::"r"(1 + (op & 3)) : "memory"); }
 
 // p = 2^(s * scale - m) for 32 scores; bf16 pairs (keys 2i, 2i+1 -> word i); s0/s1 collect the exact
 // weights, r0/r1 the bf16-rounded ones (the tensor core multiplies the ROUNDED weights: O is
@@ -262,108 +247,82 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         }
       }
     }
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer: the whole warp walks the loop, one
-    // elected lane issues (warp-uniform control flow; see elect_one).  It looks at no mbarrier itself: a look takes some 300
-    // cycles next to a tensor pipe that streams its operands out of shared memory, seven of them per pair of tiles were
-    // half of the tensor pipe's time, and instructions that keep one under way behind the MMAs made the MMAs themselves
-    // slower to issue (92 instead of 66 cycles).  Warp 2 looks for it and hands over through hardware barriers.
+  } else if (warp <= 2) {
+    // ------------------------------------------------------------------ MMA issuers: warp 1 the Q K^T, warp 2 the P V; the
+    // whole warp walks the loop, one elected lane issues (warp-uniform control flow; see elect_one).
+    // Two of them, because one does not keep the tensor pipe busy: next to the softmax warps of its sub-partition a warp
+    // gets an MMA out every 105 cycles (64 is the pipe's rate), and a look at a barrier takes it some 300 cycles while the
+    // pipe streams its operands out of shared memory.  The lanes look at an operation's barriers at once.
     const bool leader = elect_one();
     const int n_items_u = __reduce_max_sync(0xffffffffu, n_items);
-    uint32_t op = 0;                              // operations so far
-    uint32_t k_slot = 0, va_slot = 0, vb_slot = 0;      // K ring position; V ring position per query tile
-    const uint64_t dQ0 = make_smem_desc(smem_u32(sQ), 16, 1024), dK0 = make_smem_desc(smem_u32(sK), 16, 1024);
-    const uint64_t mV0 = make_smem_desc(smem_u32(sV), PANEL, 1024);
-    for (int item = blockIdx.x; item < n_items_u; item += gridDim.x) {
-      FwdItem it = decode_item<DENSE>(p, item);
-      it.nx = __reduce_max_sync(0xffffffffu, it.nx);
-      const OpOrder order(it.nx, it.ntiles);
-      for (int u = 0; u < order.n_uses + order.lag; ++u) {
-        const int v = u - order.lag;
-        if (u < order.n_uses) {
-          const int x = order.x_of(u), t = order.t_of(u);
-          lap(5);
-          hand_over(op++);
-          lap(0);
-          tc_fence_after();
-          const int n_mma = (min(BN, it.n_keys - t * BN) + 15) & ~15;
-          const uint32_t idesc = make_idesc_bf16(BM, n_mma, false, false);
-          const uint64_t dq = dQ0 + (x ? (uint32_t)(TILE >> 4) : 0u), dk = dK0 + k_slot * (uint32_t)(TILE >> 4);
-#pragma unroll
-          for (int ks = 0; ks < DH / 16; ++ks)
-            if (leader) mma_ss(tmem, dq + koff(ks), dk + koff(ks), idesc, ks > 0 ? 1u : 0u);
-          if (leader) mma_commit(&sm->s_full[x]);
-          if (x == it.nx - 1) {
-            if (leader) mma_commit(&sm->k_empty[k_slot]);
-            if (leader && t == it.ntiles - 1) mma_commit(&sm->q_empty);
-            if (++k_slot == KST) k_slot = 0;
-          }
-        }
-        if (v >= 0) {
-          const int x = order.x_of(v), t = order.t_of(v);
-          uint32_t slot = x ? vb_slot : va_slot;
-          lap(5);
-          hand_over(op++);
-          lap(2);
-          tc_fence_after();
-          const int ksteps = (min(BN, it.n_keys - t * BN) + 15) >> 4;
-          const uint64_t mv = mV0 + slot * (uint32_t)(TILE >> 4);
-#pragma unroll
-          for (int ks = 0; ks < 8; ++ks)
-            if (leader && ks < ksteps)   // P of keys 16 ks .. 16 ks + 15 sits in columns 8 ks .. of the tile's P buffer
-              mma_ts(tmem + O_COL + x * 128, tmem + P_COL + x * 64 + ks * 8, mv + mnoff(ks), IDESC_PV, (t > 0 || ks > 0) ? 1u : 0u);
-          if (leader) mma_commit(&sm->o_done[x]);
-          if (leader && x == it.nx - 1) mma_commit(&sm->v_empty[slot]);
-          if (++slot == VST) slot = 0;
-          if (x) vb_slot = slot; else va_slot = slot;
-          if (it.nx == 1) vb_slot = va_slot;
-        }
-      }
-    }
-    lap(5);
-    if (leader) tflush(8);
-  } else if (warp == 2) {
-    // ------------------------------------------------------------------ waits on behalf of the MMA warp, in the order of its
-    // operations; the lanes look at an operation's barriers at once
-    uint32_t op = 0, uses = 0, n = 0;
-    uint32_t k_slot = 0, k_par = 0;
-    struct Tile { uint32_t v_slot, v_par, tcnt, ecnt; };     // V ring position of the next P V; P V and items done
-    Tile ta{0, 0, 0, 0}, tb{0, 0, 0, 0};
     auto wait3 = [&](uint64_t* b0, uint32_t p0, uint64_t* b1, uint32_t p1, bool third, uint64_t* b2, uint32_t p2) {
       const int which = lane & 3;
       uint32_t bar = smem_u32(b0), par = p0;
       if (which == 1) { bar = smem_u32(b1); par = p1; }
       if (which == 2 && third) { bar = smem_u32(b2); par = p2; }
+      lap(5);
       mbar_wait_lanes(bar, par, abort_flag, p.status);
       __syncwarp();
-      // once any wait of this CTA has given up, conditions may hold early: in step with the MMA warp from here on
-      if (__any_sync(0xffffffffu, *abort_flag != 0)) hand_over(op++); else hand_over_arrive(op++);
+      lap(0);
+      tc_fence_after();
     };
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
-      const FwdItem it = decode_item<DENSE>(p, item);
-      const OpOrder order(it.nx, it.ntiles);
-      for (int u = 0; u < order.n_uses + order.lag; ++u) {
-        const int v = u - order.lag;
-        if (u < order.n_uses) {
-          // the score buffer has been read (its first use waits for a phase before the first: passes at once), the K tile
-          // is there, and the item's Q tiles
-          wait3(&sm->s_free, (uses + 1) & 1, &sm->k_full[k_slot], k_par, u == 0, &sm->q_full, n & 1);
-          ++uses;
-          if (order.x_of(u) == it.nx - 1 && ++k_slot == KST) { k_slot = 0; k_par ^= 1; }
-        }
-        if (v >= 0) {
-          // P has been written, the V tile is there, the epilogue of the tile's previous item has read the accumulator
-          const int x = order.x_of(v);
-          Tile q = x ? tb : ta;
-          wait3(&sm->p_ready[x], q.tcnt & 1, &sm->v_full[q.v_slot], q.v_par, order.t_of(v) == 0, &sm->o_free[x], (q.ecnt + 1) & 1);
-          q.tcnt += 1;
-          if (++q.v_slot == VST) { q.v_slot = 0; q.v_par ^= 1; }
-          if (x) tb = q; else ta = q;
-          if (it.nx == 1) { tb.v_slot = ta.v_slot; tb.v_par = ta.v_par; }
+    if (warp == 1) {
+      uint32_t uses = 0, n = 0, slot = 0, par = 0;      // uses of the score buffer, items, K ring position
+      const uint32_t lo_q = desc_lo(smem_u32(sQ), 16), lo_k = desc_lo(smem_u32(sK), 16);
+      for (int item = blockIdx.x; item < n_items_u; item += gridDim.x, ++n) {
+        FwdItem it = decode_item<DENSE>(p, item);
+        it.nx = __reduce_max_sync(0xffffffffu, it.nx);
+        for (int t = 0; t < it.ntiles; ++t) {
+          const int n_mma = (min(BN, it.n_keys - t * BN) + 15) & ~15;
+          const uint32_t idesc = make_idesc_bf16(BM, n_mma, false, false);
+          const uint32_t dk = lo_k + slot * (uint32_t)(TILE >> 4);
+          for (int x = 0; x < it.nx; ++x) {
+            // the score buffer has been read (its first use waits for a phase before the first: passes at once), the K tile
+            // is there, and the item's Q tiles
+            wait3(&sm->s_free, (uses + 1) & 1, &sm->k_full[slot], par, t == 0 && x == 0, &sm->q_full, n & 1);
+            ++uses;
+            const uint32_t dq = lo_q + x * (uint32_t)(TILE >> 4);
+#pragma unroll
+            for (int ks = 0; ks < DH / 16; ++ks)
+              if (leader) mma_ss_lo(tmem, dq + koff(ks), dk + koff(ks), idesc, ks > 0 ? 1u : 0u);
+            if (leader) mma_commit(&sm->s_full[x]);
+          }
+          if (leader) mma_commit(&sm->k_empty[slot]);
+          if (leader && t == it.ntiles - 1) mma_commit(&sm->q_empty);
+          if (++slot == KST) { slot = 0; par ^= 1; }
         }
       }
-      ta.ecnt += 1;
-      if (it.nx == 2) tb.ecnt += 1;
+      lap(5);
+      if (leader) tflush(8);
+    } else {
+      uint32_t tcnt[2] = {0, 0}, ecnt[2] = {0, 0}, slot = 0, par = 0;      // per query tile: P V and items done; V ring position
+      const uint32_t lo_v = desc_lo(smem_u32(sV), PANEL);
+      for (int item = blockIdx.x; item < n_items_u; item += gridDim.x) {
+        FwdItem it = decode_item<DENSE>(p, item);
+        it.nx = __reduce_max_sync(0xffffffffu, it.nx);
+        for (int t = 0; t < it.ntiles; ++t) {
+          const int ksteps = (min(BN, it.n_keys - t * BN) + 15) >> 4;
+          const uint32_t mv = lo_v + slot * (uint32_t)(TILE >> 4);
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            if (x >= it.nx) continue;
+            // P has been written, the V tile is there, the epilogue of the tile's previous item has read the accumulator
+            wait3(&sm->p_ready[x], tcnt[x] & 1, &sm->v_full[slot], par, t == 0, &sm->o_free[x], (ecnt[x] + 1) & 1);
+            tcnt[x] += 1;
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)
+              if (leader && ks < ksteps)   // P of keys 16 ks .. 16 ks + 15 sits in columns 8 ks .. of the tile's P buffer
+                mma_ts_lo(tmem + O_COL + x * 128, tmem + P_COL + x * 64 + ks * 8, mv + mnoff(ks), IDESC_PV, (t > 0 || ks > 0) ? 1u : 0u);
+            if (leader) mma_commit(&sm->o_done[x]);
+          }
+          if (leader) mma_commit(&sm->v_empty[slot]);
+          if (++slot == VST) { slot = 0; par ^= 1; }
+        }
+        ecnt[0] += 1;
+        if (it.nx == 2) ecnt[1] += 1;
+      }
+      lap(5);
+      if (PROF && leader) { atomicAdd(p.prof + 10, wp[0]); atomicAdd(p.prof + 11, wp[5]); }
     }
   } else if (warp >= 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
