@@ -136,7 +136,7 @@ __device__ __forceinline__ void exp_pack64(const uint32_t (&sv)[64], float scale
     p1 = ex2(p1);
     add2(s0, s1, s0, s1, p0, p1);
     pk[i] = pack_bf16(p0, p1);
-    add2(r0, r1, r0, r1, __uint_as_float(pk[i] << 16), __uint_as_float(pk[i] & 0xffff0000u));
+    add_bf16_pair(r0, r1, pk[i]);
   }
 }
 

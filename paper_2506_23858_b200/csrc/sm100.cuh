@@ -323,6 +323,12 @@ __device__ __forceinline__ void mul2(float& d0, float& d1, float a0, float a1, f
       : "=f"(d0), "=f"(d1)
       : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
 }
+// r0 += the low, r1 += the high bf16 of a packed pair (sm_100: fp32 plus bf16 in one instruction, no unpacking)
+__device__ __forceinline__ void add_bf16_pair(float& r0, float& r1, uint32_t pair) {
+  asm("{\n\t.reg .b16 l, h;\n\tmov.b32 {l, h}, %2;\n\tadd.rn.f32.bf16 %0, l, %0;\n\tadd.rn.f32.bf16 %1, h, %1;\n\t}"
+      : "+f"(r0), "+f"(r1)
+      : "r"(pair));
+}
 // 32-byte store (sm_100): one full sector per thread, so that row-per-thread output loops write whole
 // sectors with every instruction.  The address must be 32-byte aligned.
 __device__ __forceinline__ void st_global_v8(float* p, float a0, float a1, float a2, float a3, float a4, float a5, float a6, float a7) {
