@@ -11,7 +11,7 @@
 //   warps 1, 2    MMA issuers: Q K^T, P V
 //   warps 4-7     softmax of tile A: thread = one query row, all 128 keys of the tile
 //   warps 8-11    softmax of tile B
-//   warps 12-15   loaders: gather the 256 Q rows of the NEXT item
+//   warps 12-15   gather the 256 Q rows of the NEXT item and write the rows of o of the one before
 //
 // TMEM: ONE score buffer S (128 columns) that A and B use in turn, P_A and P_B (64 columns each, bf16), the accumulators
 // O_A and O_B (128 columns each).  A softmax thread (200 registers) takes its whole row of 128 scores out of S at once and
@@ -51,10 +51,12 @@ struct Smem {
   uint64_t s_full[2], p_ready[2];    // per query tile: scores written (commit) / P written (128 arrivals)
   uint64_t s_free;                   // the score buffer has been read (128 arrivals of whichever tile used it)
   uint64_t o_done[2];                // per query tile: P V of a key tile complete (commit)
-  uint64_t o_free[2];                // per query tile: epilogue has read the accumulator (128 arrivals)
+  uint64_t ep_ready[2];              // per query tile: an item's normalisers are in ep_inv / ep_lse (128 softmax arrivals)
+  uint64_t o_free[2];                // per query tile: epilogue has read them and the accumulator (128 arrivals)
   uint64_t q_full, q_empty;          // Q tiles of an item gathered (128 arrivals) / no longer needed (commit)
   uint32_t tmem_base;
   int abort_flag;
+  float ep_inv[2][BM], ep_lse[2][BM];   // 1 / sum of the rounded weights, natural-log lse
 };
 // no alignment slack: the kernel checks that its dynamic shared memory starts on a 1024-byte boundary
 constexpr size_t SMEM_BYTES = (2 /*Q*/ + KST + VST) * TILE + sizeof(Smem) + 32;
@@ -137,23 +139,17 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// N (8 or 16) consecutive outputs as bf16 (one 16- or 32-byte store) and, if asked for, their rounding
-// residuals bf16(v - bf16(v)), computed in registers.
-template <int N>
-__device__ __forceinline__ void store_resid(__nv_bfloat16* dst, __nv_bfloat16* rdst, const float (&v)[N]) {
-  uint32_t h[N / 2], r[N / 2];
+// Eight consecutive outputs as bf16 (one 16-byte store) and, if asked for, their rounding residuals bf16(v - bf16(v)),
+// computed in registers.
+__device__ __forceinline__ void store8_resid(__nv_bfloat16* dst, __nv_bfloat16* rdst, const float (&v)[8]) {
+  uint32_t h[4], r[4];
 #pragma unroll
-  for (int k = 0; k < N / 2; ++k) {
+  for (int k = 0; k < 4; ++k) {
     h[k] = pack_bf16(v[2 * k], v[2 * k + 1]);
     r[k] = pack_bf16(v[2 * k] - __uint_as_float(h[k] << 16), v[2 * k + 1] - __uint_as_float(h[k] & 0xffff0000u));
   }
-  if constexpr (N == 16) {
-    st_global_v8(dst, h[0], h[1], h[2], h[3], h[4], h[5], h[6], h[7]);
-    if (rdst) st_global_v8(rdst, r[0], r[1], r[2], r[3], r[4], r[5], r[6], r[7]);
-  } else {
-    *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
-    if (rdst) *reinterpret_cast<uint4*>(rdst) = make_uint4(r[0], r[1], r[2], r[3]);
-  }
+  *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+  if (rdst) *reinterpret_cast<uint4*>(rdst) = make_uint4(r[0], r[1], r[2], r[3]);
 }
 
 // RASTER: the directly written rows of o go through p.o_map (a kernel of its own: with the map's address
@@ -197,7 +193,7 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     for (int s = 0; s < VST; ++s) { mbar_init(&sm->v_full[s], 1); mbar_init(&sm->v_empty[s], 1); }
     for (int x = 0; x < 2; ++x) {
       mbar_init(&sm->s_full[x], 1); mbar_init(&sm->p_ready[x], 128);
-      mbar_init(&sm->o_done[x], 1); mbar_init(&sm->o_free[x], 128);
+      mbar_init(&sm->o_done[x], 1); mbar_init(&sm->o_free[x], 128); mbar_init(&sm->ep_ready[x], 128);
     }
     mbar_init(&sm->s_free, 128);
     mbar_init(&sm->q_full, 128); mbar_init(&sm->q_empty, 1);
@@ -326,12 +322,95 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     }
   } else if (warp >= 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-    // ------------------------------------------------------------------ loaders: Q rows of the next item
-    // Sparse: asynchronous 16-byte copies, eight threads per 128-byte half row, asked for in the L2 ahead of time; dense:
+    // ------------------------------------------------------------------ loaders and epilogue: the Q rows of item n, then the
+    // rows of o of item n - 1 (while the softmax warps are at work on item n: an epilogue takes about as long as one and a
+    // half key tiles, a third of an item of three)
+    // Q, sparse: asynchronous 16-byte copies, eight threads per 128-byte half row, asked for in the L2 ahead of time; dense:
     // consecutive rows, TMA tiles.
     const int lt = (warp - 12) * 32 + lane;   // 0..127
-    const int r0 = lt >> 3, chunk = lt & 7;   // rows r0 + 16 k
+    const int r0 = lt >> 3, chunk = lt & 7;   // Q rows r0 + 16 k
     uint32_t n = 0;
+    uint32_t tcs[2] = {0, 0}, eps[2] = {0, 0};        // per query tile: P V and items done
+    auto epilogue = [&](const FwdItem& it) {
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        if (x >= it.nx) continue;
+        const uint32_t o_tmem = tmem + ((uint32_t)((warp & 3) * 32) << 16) + O_COL + x * 128;
+        const int row = x * BM + lt;                  // thread = query row
+        const bool row_ok = row < it.n_rows;
+        const int qpos = !row_ok ? 0 : DENSE ? it.list_lo + row : checked_index(__ldg(p.q_idx + it.list_lo + row), p.S, p.status);
+        const long long G_ = it.head_off + qpos;
+        // the query has a single block: final result
+        const bool direct = DENSE || __ldg(p.q_ptr + G_ + 1) - __ldg(p.q_ptr + G_) == 1;
+        const long long o_row_off = RASTER ? ((row_ok && direct) ? p.o_map.off(G_, DH) : 0) : G_ * DH;
+        const long long pos = (long long)it.list_lo + row;
+        tcs[x] += it.ntiles;
+        mbar_wait(&sm->ep_ready[x], eps[x] & 1, abort_flag, p.status);
+        eps[x] += 1;
+        const float inv = sm->ep_inv[x][lt], row_lse = sm->ep_lse[x][lt];
+        mbar_wait(&sm->o_done[x], (tcs[x] - 1) & 1, abort_flag, p.status);
+        tc_fence_after();
+        // a partial row goes out as fp16 times a power of two: find the row's largest magnitude first
+        float mul = inv, row_scale = 1.0f;
+        if constexpr (!DENSE) {
+          const bool partial = row_ok && !direct;
+          if (__any_sync(0xffffffffu, partial)) {
+            float amax = 0.f;
+#pragma unroll 1
+            for (int c = 0; c < 8; ++c) {
+              uint32_t ov[16];
+              tmem_ld16(o_tmem + c * 16, ov);
+              tmem_ld_wait();
+#pragma unroll
+              for (int i = 0; i < 16; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(ov[i])));
+            }
+            if (partial) {
+              row_scale = pow2_at_or_above(amax * inv);
+              mul = inv / row_scale;
+            }
+          }
+        }
+#pragma unroll 1
+        for (int c = 0; c < 8; ++c) {
+          uint32_t ov[16];
+          tmem_ld16(o_tmem + c * 16, ov);
+          tmem_ld_wait();
+          if (c == 7) {
+            tc_fence_before();
+            mbar_arrive(&sm->o_free[x]);
+          }
+          if (row_ok) {
+            const int col = 16 * c;
+            if (direct) {
+              __nv_bfloat16* dst = p.o + o_row_off + col;
+              __nv_bfloat16* rdst = p.o_resid ? p.o_resid + G_ * DH + col : nullptr;
+#pragma unroll
+              for (int i = 0; i < 16; i += 8) {
+                float v8[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v8[k] = __uint_as_float(ov[i + k]) * inv;
+                store8_resid(dst + i, rdst ? rdst + i : nullptr, v8);
+              }
+            } else {
+              __half* dst = p.part_o + pos * DH + col;
+              uint32_t h[8];
+#pragma unroll
+              for (int k = 0; k < 8; ++k) h[k] = pack_half2(__uint_as_float(ov[2 * k]) * mul, __uint_as_float(ov[2 * k + 1]) * mul);
+              if (p.part_o_32) {       // one 32-byte store, else two of 16 bytes
+                st_global_v8(dst, h[0], h[1], h[2], h[3], h[4], h[5], h[6], h[7]);
+              } else {
+                reinterpret_cast<uint4*>(dst)[0] = make_uint4(h[0], h[1], h[2], h[3]);
+                reinterpret_cast<uint4*>(dst)[1] = make_uint4(h[4], h[5], h[6], h[7]);
+              }
+            }
+          }
+        }
+        if (row_ok) {
+          if (direct) p.lse[G_] = row_lse; else { p.part_lse[pos] = row_lse; p.part_scale[pos] = row_scale; }
+        }
+      }
+    };
+    FwdItem before;
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
       const FwdItem it = decode_item<DENSE>(p, item);
       if constexpr (DENSE) {
@@ -379,10 +458,13 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         fence_async_proxy();
         mbar_arrive(&sm->q_full);
       }
+      if (n >= 1) epilogue(before);
+      before = it;
     }
+    if (n >= 1) epilogue(before);
   } else if (warp >= 4) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
-    // ------------------------------------------------------------------ softmax + epilogue of one query tile
+    // ------------------------------------------------------------------ softmax of one query tile
     const int x = (warp - 4) >> 2;                  // query tile of this warp group
     const int quad = warp & 3;                      // TMEM lane quarter this warp may access
     const int r = quad * 32 + lane;                 // query row inside the tile
@@ -390,16 +472,11 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     const uint32_t s_tmem = tmem + lane_addr;
     const uint32_t p_tmem = tmem + lane_addr + P_COL + x * 64;
     const uint32_t o_tmem = tmem + lane_addr + O_COL + x * 128;
-    uint32_t tc = 0;                                 // key tiles done on this query tile
+    uint32_t tc = 0, items = 0;                      // key tiles and items done on this query tile
     for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
       const FwdItem it = decode_item<DENSE>(p, item);
       if (x >= it.nx) continue;
       float m_used = -INFINITY, l = 0.f, l_r = 0.f;   // l: exact sum (for LSE); l_r: sum of the bf16-rounded weights
-      // where this thread's row goes; the list entry is asked for now, what hangs on it during the first key tile
-      const int row = x * BM + r;
-      const bool row_ok = row < it.n_rows;
-      const int qpos = !row_ok ? 0 : DENSE ? it.list_lo + row : checked_index(__ldg(p.q_idx + it.list_lo + row), p.S, p.status);
-      int n_pairs = 1;
       for (int t = 0; t < it.ntiles; ++t, ++tc) {
         lap(3);
         mbar_wait(&sm->s_full[x], tc & 1, abort_flag, p.status);
@@ -448,7 +525,6 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
             tmem_st16(o_tmem + c * 16, ov);
           }
         };
-        if (!DENSE && t == 0) n_pairs = __ldg(p.q_ptr + it.head_off + qpos + 1) - __ldg(p.q_ptr + it.head_off + qpos);
         float s0 = 0.f, s1 = 0.f, r0 = 0.f, r1 = 0.f;
         const float neg_m = -m_used;
         {
@@ -457,10 +533,10 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
           exp_pack32(sv, p.scale_log2, neg_m, pk[0], s0, s1, r0, r1);
           if (valid > 32) exp_pack32(sv + 32, p.scale_log2, neg_m, pk[1], s0, s1, r0, r1);
           lap(3);
-          if (t > 0) {
+          if (tc > 0) {                              // (of the item before, where t is 0)
             mbar_wait(&sm->o_done[x], (tc - 1) & 1, abort_flag, p.status);
             tc_fence_after();
-            if (__any_sync(0xffffffffu, need)) {
+            if (t > 0 && __any_sync(0xffffffffu, need)) {
               rescale_o();
               l *= factor;
               l_r *= factor;
@@ -484,76 +560,13 @@ attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
         tc_fence_before();
         mbar_arrive(&sm->p_ready[x]);
       }
-      // ---- epilogue: wait for the last P V, normalise, write the row
+      // ---- hand the row's normalisers to the epilogue warps, once they are through with the tile's previous item, and go on
       lap(3);
-      mbar_wait(&sm->o_done[x], (tc - 1) & 1, abort_flag, p.status);
-      tc_fence_after();
-      const bool direct = n_pairs == 1;           // the query has a single block: final result
-      const float inv = 1.0f / l_r;
-      const float row_lse = (m_used + log2f(l)) * 0.6931471805599453f;
-      const long long G_ = it.head_off + qpos;
-      const long long o_row_off = RASTER ? ((row_ok && direct) ? p.o_map.off(G_, DH) : 0) : G_ * DH;
-      const long long pos = (long long)it.list_lo + row;
-      // a partial row goes out as fp16 times a power of two: find the row's largest magnitude first
-      float mul = inv, row_scale = 1.0f;
-      if constexpr (!DENSE) {
-        const bool partial = row_ok && !direct;
-        if (__any_sync(0xffffffffu, partial)) {
-          float amax = 0.f;
-#pragma unroll 1
-          for (int c = 0; c < 4; ++c) {
-            uint32_t ov[32];
-            tmem_ld32(o_tmem + c * 32, ov);
-            tmem_ld_wait();
-#pragma unroll
-            for (int i = 0; i < 32; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(ov[i])));
-          }
-          if (partial) {
-            row_scale = pow2_at_or_above(amax * inv);
-            mul = inv / row_scale;
-          }
-        }
-      }
-#pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        uint32_t ov[32];
-        tmem_ld32(o_tmem + c * 32, ov);
-        tmem_ld_wait();
-        if (row_ok) {
-          const int col = 32 * c;
-          if (direct) {
-            __nv_bfloat16* dst = p.o + o_row_off + col;
-            __nv_bfloat16* rdst = p.o_resid ? p.o_resid + G_ * DH + col : nullptr;
-#pragma unroll
-            for (int i = 0; i < 32; i += 8) {     // 16-byte stores (32-byte ones were slower here: more values live at once)
-              float v8[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k) v8[k] = __uint_as_float(ov[i + k]) * inv;
-              store_resid<8>(dst + i, rdst ? rdst + i : nullptr, v8);
-            }
-          } else {
-            __half* dst = p.part_o + pos * DH + col;
-#pragma unroll
-            for (int i = 0; i < 32; i += 16) {
-              uint32_t h[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k)
-                h[k] = pack_half2(__uint_as_float(ov[i + 2 * k]) * mul, __uint_as_float(ov[i + 2 * k + 1]) * mul);
-              if (p.part_o_32) {       // one 32-byte store, else two of 16 bytes
-                st_global_v8(dst + i, h[0], h[1], h[2], h[3], h[4], h[5], h[6], h[7]);
-              } else {
-                reinterpret_cast<uint4*>(dst + i)[0] = make_uint4(h[0], h[1], h[2], h[3]);
-                reinterpret_cast<uint4*>(dst + i)[1] = make_uint4(h[4], h[5], h[6], h[7]);
-              }
-            }
-          }
-        }
-      }
-      if (row_ok) {
-        if (direct) p.lse[G_] = row_lse; else { p.part_lse[pos] = row_lse; p.part_scale[pos] = row_scale; }
-      }
-      tc_fence_before();
-      mbar_arrive(&sm->o_free[x]);
+      if (items >= 1) mbar_wait(&sm->o_free[x], (items - 1) & 1, abort_flag, p.status);
+      sm->ep_inv[x][r] = 1.0f / l_r;
+      sm->ep_lse[x][r] = (m_used + log2f(l)) * 0.6931471805599453f;
+      mbar_arrive(&sm->ep_ready[x]);
+      ++items;
       lap(4);
     }
     if (warp == 4 && lane == 0) tflush(0);
