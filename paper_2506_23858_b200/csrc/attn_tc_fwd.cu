@@ -599,18 +599,18 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
                          int32_t* status, int* item_ptr, int* item_tab, long long max_items, float* part_o,
                          float* part_lse, float* part_scale, cudaStream_t st, const RowMap& o_map);   // attn_tc_fwd_narrow.cu
 
-// Forward over the work lists (bf16, head_dim 128).  Key blocks of up to thirteen 128-key tiles go to the narrow
-// kernel (two CTAs of one query tile per SM), longer ones to the wide kernel of this file.  Returns
-// VMOBA_ERR_CUDA if the tensor maps or the launch fail.
+// Forward over the work lists (bf16, head_dim 128).  Key blocks of up to two 128-key tiles go to the narrow kernel (two
+// CTAs of one query tile per SM), longer ones to the wide kernel of this file.  Returns VMOBA_ERR_CUDA if the tensor maps
+// or the launch fail.
 int tc_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, const int* kb_ptr, const int* q_idx,
                        const int* q_ptr, const int* q_pairs, long long cap, void* o, void* o_resid, float* lse,
                        int32_t* status, int* item_ptr, int* item_tab, long long max_items, float* part_o,
                        float* part_lse, float* part_scale, cudaStream_t st, const RowMap& o_map) {
   using namespace tcw;
-  // Measured: with blocks of 234 to 1638 keys the narrow kernel is 4 to 14 % faster; from about 1900 keys on the
-  // two run level, and the narrow one reads every K / V tile twice as often from the L2, which costs a
-  // power-capped step more clock than the forward gains.
-  if (D.sb <= 13 * BN)
+  // Measured (forward stage, wide against narrow): 13 tiles and lists of thousands 1.91 against 2.40 ms, 6 tiles 1.19
+  // against 1.46, 3 tiles 0.82 against 1.02; two tiles with lists of 200 queries (33K tokens, 3D blocks of 234 keys)
+  // 0.400 against 0.365: a 256-row item is then over before its two halves have fallen into step.
+  if (D.sb <= 2 * BN)
     return tc_sparse_fwd_narrow(D, q, k, v, kb_ptr, q_idx, q_ptr, q_pairs, cap, o, o_resid, lse, status, item_ptr, item_tab,
                                 max_items, part_o, part_lse, part_scale, st, o_map);
   const long long n_kb = (long long)D.BH * D.Nb;

@@ -1,19 +1,17 @@
-// Tensor-core attention forward for short and medium key blocks (bf16, head_dim 128; Step 3 of VMoBA): written for
-// key blocks of a few 128-key tiles, where a work item is over after two or three tiles, and used up to thirteen.
+// Tensor-core attention forward for short key blocks (bf16, head_dim 128; Step 3 of VMoBA): up to two 128-key tiles, where
+// a work item is over after one or two tiles.
 //
-// The wide kernel (attn_tc_fwd.cu) keeps the tensor pipe busy by running two query tiles of one item in opposite
-// phase; that phase needs many key tiles to establish itself.  On a 270-key block both tiles run their softmax at
-// the same time, the tensor pipe waits for both, and the item's fixed costs (finding its list, gathering 256 query
-// rows into a single buffer, the epilogue's stores) are paid with nothing else in flight.  Here the overlap comes
-// from the hardware instead: an item is ONE 128-row query tile, a CTA needs 100 KB of shared memory, 256 TMEM
-// columns and 256 threads of 128 registers, and TWO CTAs share an SM.  While one of them gathers, waits for a key tile or
-// writes its rows, the other one has the tensor pipe and the exponential unit.
+// The wide kernel (attn_tc_fwd.cu) works two query tiles of an item against each other.  On a key block of one or two tiles
+// there is little to set against each other, and lists are often shorter than its 256 rows.  Here the overlap comes from
+// the hardware instead: an item is ONE 128-row query tile, a CTA needs 100 KB of shared memory and 256 TMEM columns, and
+// TWO CTAs share an SM.  While one of them gathers, waits for a key tile or writes its rows, the other one has the tensor
+// pipe and the exponential unit.
 //
 //   warp 0        TMA producer: K and V tiles, one stage each (a K tile is reloaded as soon as its Q K^T has run)
 //   warp 1        MMA issuer (all lanes walk the loop, one elected lane issues)
-//   warps 4-7     softmax (+ epilogue, unless warps 8-11 exist): thread = one query row
+//   warps 4-7     softmax: thread = one query row
 //   warps 2,3     loaders: gather the 128 Q rows (and per-row output bookkeeping) of the NEXT item
-//   warps 8-11    (key blocks of up to four tiles only) epilogue: read the accumulator, write the rows
+//   warps 8-11    epilogue: read the accumulator, write the rows
 //
 // Rows of queries with a single block are final and go to o; the others are partial results that the merge pass
 // combines: fp16 values times a power of two per row, beside the row's lse.
@@ -40,8 +38,7 @@ constexpr int BN = 128;              // keys per tile
 constexpr int DH = 128;              // head dim
 constexpr int PANEL = BM * 128;      // bytes of one 64-column panel of a 128-row tile (16 KB)
 constexpr int TILE = 2 * PANEL;      // bytes of a [128 x 128] bf16 tile (32 KB)
-constexpr int THREADS = 256;
-constexpr int THREADS_SPLIT = 384;   // with four epilogue warps
+constexpr int THREADS = 384;
 constexpr uint32_t TMEM_COLS = 256;
 constexpr uint32_t O_COL = 128;      // S at 0, P at 64, O at 128
 constexpr float RESCALE_LOG2 = 8.0f;
@@ -51,11 +48,11 @@ struct Smem {
   uint64_t s_full, p_ready;          // scores written (commit) / P written (128 arrivals)
   uint64_t o_done;                   // P V of a key tile complete (commit)
   uint64_t q_full, q_empty;          // Q tile of an item gathered (64 arrivals) / no longer needed (commit)
-  uint64_t ep_ready;                 // SPLIT: an item's normalisers are in ep_inv / ep_lse (128 softmax arrivals)
-  uint64_t o_free;                   // SPLIT: the epilogue warps have read the accumulator (128 arrivals)
+  uint64_t ep_ready;                 // an item's normalisers are in ep_inv / ep_lse (128 softmax arrivals)
+  uint64_t o_free;                   // the epilogue warps have read the accumulator (128 arrivals)
   uint32_t tmem_base;
   int abort_flag;
-  float ep_inv[2][BM], ep_lse[2][BM];   // SPLIT, [item % 2][row]: 1 / sum of the rounded weights, natural-log lse
+  float ep_inv[2][BM], ep_lse[2][BM];   // [item % 2][row]: 1 / sum of the rounded weights, natural-log lse
   int qinfo[4][BM];                  // [item % 4][row]: 2 * in-head position + (query has a single block), -1 for padding rows
 };
 // two CTAs per SM: each may use half of the SM's shared memory
@@ -175,13 +172,13 @@ __device__ __forceinline__ void store8_resid(__nv_bfloat16* dst, __nv_bfloat16* 
 }
 
 // RASTER: the directly written rows of o go through p.o_map.
-// SPLIT: four more warps (8-11) take the epilogue: they read the accumulator and write the rows while the softmax
-// warps are already on the next item's first tile.  With 384 threads two CTAs leave 80 registers per thread, so the
-// warp groups trade registers at the start: the softmax group takes 128, the first group keeps 72, the epilogue
-// group 40.  Its loaders then have no room to hold rows in registers: they ask the L2 for an item's rows ahead of
-// time and, once the Q tile is free, bring them in as asynchronous 16-byte copies straight into the swizzled tile.
-template <bool RASTER, bool SPLIT>
-__global__ void __launch_bounds__(SPLIT ? THREADS_SPLIT : THREADS, 2)
+// Warps 8-11 read the accumulator and write the rows while the softmax warps are already on the next item's first tile.
+// With 384 threads two CTAs leave 80 registers per thread, so the warp groups trade registers at the start: the softmax
+// group takes 128, the first group keeps 72, the epilogue group 40.  The loaders then have no room to hold rows in
+// registers: they ask the L2 for an item's rows ahead of time and, once the Q tile is free, bring them in as asynchronous
+// 16-byte copies straight into the swizzled tile.
+template <bool RASTER>
+__global__ void __launch_bounds__(THREADS, 2)
 attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -241,9 +238,9 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     return item_from_desc(p, d);
   };
 
-  // SPLIT: every role starts by taking or giving back registers (the whole warp group executes the same one)
+  // every role starts by taking or giving back registers (the whole warp group executes the same one)
   if (warp < 4) {
-    if constexpr (SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
   }
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
@@ -312,11 +309,9 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         lap(2);
         mbar_wait_warp(&sm->v_full, f & 1, abort_flag, p.status);
         lap(3);
-        if constexpr (SPLIT) {
-          // the accumulator still holds the item before until the epilogue warps have read it
-          if (t == 0 && n >= 1) mbar_wait_warp(&sm->o_free, (n - 1) & 1, abort_flag, p.status);
-          lap(4);
-        }
+        // the accumulator still holds the item before until the epilogue warps have read it
+        if (t == 0 && n >= 1) mbar_wait_warp(&sm->o_free, (n - 1) & 1, abort_flag, p.status);
+        lap(4);
         tc_fence_after();
         {
           const int ksteps = (keys + 15) >> 4;
@@ -343,7 +338,7 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
       // Four bookkeeping slots: the softmax warps read slot n % 4 in the epilogue of item n, and the loaders can be
       // at most two items ahead of an epilogue.
       int info[2];
-      if constexpr (SPLIT) {
+      {
         if ((chunk & 7) == 0) {       // one L2 request per 128-byte line of every row of the item
 #pragma unroll 4
           for (int i = 0; i < BM / 4; ++i) {
@@ -378,61 +373,14 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         asm volatile("cp.async.commit_group;" ::: "memory");
         asm volatile("cp.async.wait_group 0;" ::: "memory");
       }
-      // without epilogue warps the loaders have 128 registers: two rounds of 64 rows that wait in registers
-      constexpr int RR = 64;
-      constexpr int NI = RR / 4;
-      if constexpr (!SPLIT)
-      for (int rnd = 0; rnd < BM / RR; ++rnd) {
-        uint4 v[NI];
-#pragma unroll
-        for (int i = 0; i < NI; ++i) {
-          const int row = rnd * RR + (lt >> 4) + 4 * i;
-          v[i] = make_uint4(0u, 0u, 0u, 0u);
-          if (row < it.n_rows) {
-            const int qp = checked_index(__ldg(p.q_idx + it.list_lo + row), p.S, p.status);
-            v[i] = __ldg(reinterpret_cast<const uint4*>(qh + (long long)qp * DH) + chunk);
-          }
-        }
-        if (rnd == 0) {
-          // per-row bookkeeping of rows lt and 64 + lt, fetched while the rows are in flight
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            info[h] = -1;
-            if (h * 64 + lt < it.n_rows) {
-              const int qp = checked_index(__ldg(p.q_idx + it.list_lo + h * 64 + lt), p.S, p.status);
-              const long long G_ = it.head_off + qp;
-              info[h] = 2 * qp + ((p.q_ptr[G_ + 1] - p.q_ptr[G_]) == 1 ? 1 : 0);
-            }
-          }
-          // the later rounds' rows are fetched only after this round has been stored: ask the L2 for them now
-          // (one request per 128-byte line)
-          if ((chunk & 7) == 0) {
-#pragma unroll 4
-            for (int i = 0; i < (BM - RR) / 4; ++i) {
-              const int row = RR + (lt >> 4) + 4 * i;
-              if (row < it.n_rows) {
-                const int qp = checked_index(__ldg(p.q_idx + it.list_lo + row), p.S, p.status);
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(qh + (long long)qp * DH + chunk * 8));
-              }
-            }
-          }
-          // the Q tile is free once the previous item's last Q K^T has run
-          if (n >= 1) mbar_wait(&sm->q_empty, (n - 1) & 1, abort_flag, p.status);
-        }
-#pragma unroll
-        for (int i = 0; i < NI; ++i) {
-          const int row = rnd * RR + (lt >> 4) + 4 * i;
-          *reinterpret_cast<uint4*>(sQ + panel * PANEL + row * 128 + ((cc ^ (row & 7)) << 4)) = v[i];
-        }
-      }
       sm->qinfo[n & 3][lt] = info[0];
       sm->qinfo[n & 3][64 + lt] = info[1];
       fence_async_proxy();
       mbar_arrive(&sm->q_full);
     }
-  } else if (SPLIT && warp >= 8) {
-    // ------------------------------------------------------------------ epilogue warps (SPLIT): thread = one query row
-    if constexpr (SPLIT) asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+  } else if (warp >= 8) {
+    // ------------------------------------------------------------------ epilogue warps: thread = one query row
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     const int quad = warp & 3;
     const int r = quad * 32 + lane;
     const uint32_t o_tmem = tmem + ((uint32_t)(quad * 32) << 16) + O_COL;
@@ -505,7 +453,7 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     }
   } else {
     // ------------------------------------------------------------------ softmax + epilogue
-    if constexpr (SPLIT) asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
     const int quad = warp & 3;                      // TMEM lane quarter this warp may access
     const int r = quad * 32 + lane;                 // query row inside the tile
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
@@ -584,80 +532,10 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         tc_fence_before();
         mbar_arrive(&sm->p_ready);
       }
-      if constexpr (SPLIT) {
-        // hand the row's normalisers to the epilogue warps and go on with the next item
-        sm->ep_inv[n & 1][r] = 1.0f / l_r;
-        sm->ep_lse[n & 1][r] = (m_used + log2f(l)) * 0.6931471805599453f;
-        mbar_arrive(&sm->ep_ready);
-        lap(4);
-        continue;
-      }
-      // ---- epilogue: wait for the last P V, normalise, write the row
-      lap(3);
-      mbar_wait(&sm->o_done, (tc - 1) & 1, abort_flag, p.status);
-      tc_fence_after();
-      const int info = sm->qinfo[n & 3][r];
-      const bool row_ok = info >= 0;
-      const int qpos = row_ok ? info >> 1 : 0;
-      const bool direct = (info & 1) != 0;
-      const float inv = 1.0f / l_r;
-      const float row_lse = (m_used + log2f(l)) * 0.6931471805599453f;
-      const long long G_ = it.head_off + qpos;
-      const long long o_row_off = RASTER ? ((row_ok && direct) ? p.o_map.off(G_, DH) : 0) : G_ * DH;
-      const long long pos = (long long)it.list_lo + r;
-      const bool partial = row_ok && !direct;
-      // a partial row goes out as fp16 times a power of two: find the row's largest magnitude first
-      float mul = inv, row_scale = 1.0f;
-      if (__any_sync(0xffffffffu, partial)) {
-        float amax = 0.f;
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          uint32_t ov[32];
-          tmem_ld32(o_tmem + c * 32, ov);
-          tmem_ld_wait();
-#pragma unroll
-          for (int i = 0; i < 32; ++i) amax = fmaxf(amax, fabsf(__uint_as_float(ov[i])));
-        }
-        if (partial) {
-          row_scale = pow2_at_or_above(amax * inv);
-          mul = inv / row_scale;
-        }
-      }
-#pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        uint32_t ov[32];
-        tmem_ld32(o_tmem + c * 32, ov);
-        tmem_ld_wait();
-        if (row_ok) {
-          const int col = 32 * c;
-          if (direct) {
-            __nv_bfloat16* dst = p.o + o_row_off + col;
-            __nv_bfloat16* rdst = p.o_resid ? p.o_resid + G_ * DH + col : nullptr;
-#pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              float v8[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k) v8[k] = __uint_as_float(ov[i + k]) * inv;
-              store8_resid(dst + i, rdst ? rdst + i : nullptr, v8);
-            }
-          } else {
-#pragma unroll
-            for (int i = 0; i < 32; i += 16) {
-              uint32_t h[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k)
-                h[k] = pack_half2(__uint_as_float(ov[i + 2 * k]) * mul, __uint_as_float(ov[i + 2 * k + 1]) * mul);
-              store_part16(p.part_o + pos * DH + col + i, h, p.part_o_32);
-            }
-          }
-        }
-      }
-      if (row_ok) {
-        if (direct) p.lse[G_] = row_lse; else { p.part_lse[pos] = row_lse; p.part_scale[pos] = row_scale; }
-      }
-      // No barrier tells the MMA warp that the accumulator has been read: the next thing it waits for from these
-      // threads is the P of the next item's first tile, which they write after this point.
-      tc_fence_before();
+      // hand the row's normalisers to the epilogue warps and go on with the next item
+      sm->ep_inv[n & 1][r] = 1.0f / l_r;
+      sm->ep_lse[n & 1][r] = (m_used + log2f(l)) * 0.6931471805599453f;
+      mbar_arrive(&sm->ep_ready);
       lap(4);
     }
     if (warp == 4 && lane == 0) tflush(0);
@@ -695,20 +573,9 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
   p.part_o_32 = (reinterpret_cast<uintptr_t>(part_o) % 32) == 0;
   p.o_map = o_map;
   const long long items = std::max<long long>(1, std::min<long long>(cap / BM + n_kb, 2LL * sm_count()));
-  // Epilogue warps pay when an item is a few tiles long and its epilogue a quarter of it (C4 forward stage 0.42 ->
-  // 0.37 ms, C2 0.212 -> 0.190 ms, 3D layer of C5 with 4 heads 0.84 -> 0.81 ms); on key blocks of 1560 and 1638
-  // keys the plain variant is 2 % faster.
-  const bool split_mode = D.sb <= 4 * BN;
-  if (o_map.perm) {
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(attn_fwd_narrow_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    attn_fwd_narrow_kernel<true, false><<<(int)items, THREADS, SMEM_BYTES, st>>>(tmK, tmV, p);
-  } else if (split_mode) {
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(attn_fwd_narrow_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    attn_fwd_narrow_kernel<false, true><<<(int)items, THREADS_SPLIT, SMEM_BYTES, st>>>(tmK, tmV, p);
-  } else {
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(attn_fwd_narrow_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-    attn_fwd_narrow_kernel<false, false><<<(int)items, THREADS, SMEM_BYTES, st>>>(tmK, tmV, p);
-  }
+  auto kernel = o_map.perm ? attn_fwd_narrow_kernel<true> : attn_fwd_narrow_kernel<false>;
+  VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+  kernel<<<(int)items, THREADS, SMEM_BYTES, st>>>(tmK, tmV, p);
   const long long nq = (long long)D.BH * D.S;
   simt::merge_batched_kernel<__nv_bfloat16, __half><<<(int)std::min<long long>((nq + 255) / 256, sm_count() * 8), 256, 0, st>>>(
       q_ptr, q_pairs, nq, p.part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o, (__nv_bfloat16*)o_resid, lse, o_map);
