@@ -287,39 +287,41 @@ merge_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pairs, lon
   }
 }
 
-// The same merge for head_dim 128 and fp32 partials, 32 consecutive queries per warp and trip.  With one
-// query per warp the four dependent loads of a query (list bounds, pair positions, partial lse, rows) are
-// paid one after the other for every query; here lane l reads the bounds, the first kInLane pair positions
-// and their lse of query g0 + l, works out the weights on its own, and the warp then walks the queries that
-// need a row written, fetching all rows of a query at once.  Queries with more pairs than a lane keeps take
-// the warp-wide loop of merge_kernel.
+// The same merge for the tensor-core path (head_dim 128).  A partial row is stored as fp16 values times a power of two
+// (part_scale, one per row; the row's largest magnitude rounded up), which halves the bytes the forward writes and this
+// pass reads; a value is then off by at most 2^-11 of its row's largest one.  The scale is folded into the row's merge
+// weight.
 //
-// PT = __half: a partial row is stored as fp16 values times a power of two (part_scale, one per row; the row's
-// largest magnitude rounded up), which halves the bytes the forward writes and this pass reads; a value is then off
-// by at most 2^-11 of its row's largest one.  The scale is folded into the row's merge weight.
+// Bound by the latency of its loads: a query takes four that depend on one another (list bounds, pair positions, partial
+// lse, rows).  A warp takes 32 consecutive queries at a time.  Queries of up to kInLane pairs: lane l works out the weights
+// of query l on its own, then the warp walks the queries that need a row.  Longer ones: the weights are worked out by the
+// half-warp that adds up the rows.  Either way two queries are walked at once, one per half-warp: sixteen lanes of 16 bytes
+// fetch a row, and kBatch rows of each are in flight.  Nine pairs per query (907,200 queries, 2.3 GB) 536 us, 32 pairs
+// (393,120 queries) 826, two to six pairs 62 to 207: with a warp per query at a time and eight bytes per lane 714, 962 and
+// 72 to 255; 64 registers (four CTAs per SM) beat 80 by a tenth, kBatch = 4 loses a tenth.
 constexpr int kInLane = 8;
-template <typename PT>
-__device__ __forceinline__ float4 load_part4(const PT* p);
-template <>
-__device__ __forceinline__ float4 load_part4<float>(const float* p) { return *reinterpret_cast<const float4*>(p); }
-template <>
-__device__ __forceinline__ float4 load_part4<__half>(const __half* p) {
-  const uint2 u = *reinterpret_cast<const uint2*>(p);
-  const float2 a = __half22float2(*reinterpret_cast<const __half2*>(&u.x));
-  const float2 b = __half22float2(*reinterpret_cast<const __half2*>(&u.y));
-  return make_float4(a.x, a.y, b.x, b.y);
+constexpr int kBatch = 8;
+__device__ __forceinline__ void add_half8(float (&acc)[8], const uint4& v, float w) {
+  const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&u[i]));
+    acc[2 * i] = fmaf(w, f.x, acc[2 * i]);
+    acc[2 * i + 1] = fmaf(w, f.y, acc[2 * i + 1]);
+  }
 }
-template <typename T, typename PT>
-__global__ void __launch_bounds__(256)
+static __global__ void __launch_bounds__(256, 4)
 merge_batched_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pairs, long long n_queries,
-                     const PT* __restrict__ part_o, const float* __restrict__ part_lse,
-                     const float* __restrict__ part_scale, long long capacity,
-                     T* __restrict__ o, T* __restrict__ o_resid, float* __restrict__ lse, const RowMap o_map = RowMap()) {
+                     const __half* __restrict__ part_o, const float* __restrict__ part_lse,
+                     const float* __restrict__ part_scale, long long capacity, __nv_bfloat16* __restrict__ o,
+                     __nv_bfloat16* __restrict__ o_resid, float* __restrict__ lse, const RowMap o_map) {
   constexpr int DH = 128;
-  const int lane = threadIdx.x & 31;
+  constexpr uint32_t FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, hl = lane & 15, half = lane >> 4;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
   const int last = (int)(capacity - 1);
+  const uint4* rows = reinterpret_cast<const uint4*>(part_o) + hl;
   for (long long g0 = warp * 32; g0 < n_queries; g0 += nwarps * 32) {
     const long long g = g0 + lane;
     int lo = 0, n = 1, n_raw = 1;        // lanes beyond the last query behave like a directly written row
@@ -331,102 +333,124 @@ merge_batched_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pa
       if (n < 0) n = 0;
     }
     const bool direct = n == 1 && n_raw == 1;
-    int pos[kInLane];
-    float w[kInLane], sc[kInLane];
-    float out_lse = -INFINITY;
-    if (!direct && n > 0 && n <= kInLane) {
-      float mx = -INFINITY;
+    auto write_row = [&](int b, float (&acc)[8], float row_lse) {       // (b < 0: no query for this half-warp)
+      if (b < 0) return;
+      const long long gq = g0 + b;
+      uint32_t h[4], r[4];
 #pragma unroll
-      for (int k = 0; k < kInLane; ++k) {
-        pos[k] = 0; w[k] = -INFINITY;
-        if (k < n) pos[k] = min(max(q_pairs[lo + k], 0), last);
+      for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 x = __floats2bfloat162_rn(acc[2 * i], acc[2 * i + 1]);
+        h[i] = *reinterpret_cast<const uint32_t*>(&x);
+        const __nv_bfloat162 y = __floats2bfloat162_rn(acc[2 * i] - __uint_as_float(h[i] << 16), acc[2 * i + 1] - __uint_as_float(h[i] & 0xffff0000u));
+        r[i] = *reinterpret_cast<const uint32_t*>(&y);
       }
-#pragma unroll
-      for (int k = 0; k < kInLane; ++k) {
-        sc[k] = 1.0f;
-        if (k < n) {
-          w[k] = part_lse[pos[k]];
-          if (part_scale) sc[k] = part_scale[pos[k]];
-          mx = fmaxf(mx, w[k]);
-        }
-      }
-      float tot = 0.f;
-#pragma unroll
-      for (int k = 0; k < kInLane; ++k) {
-        w[k] = k < n ? expf(w[k] - mx) : 0.f;
-        tot += w[k];
-      }
-      const float inv = 1.0f / tot;
-#pragma unroll
-      for (int k = 0; k < kInLane; ++k) w[k] *= inv * sc[k];
-      out_lse = mx + logf(tot);
-    } else {
+      *reinterpret_cast<uint4*>(o + o_map.off(gq, DH) + hl * 8) = make_uint4(h[0], h[1], h[2], h[3]);
+      if (o_resid) *reinterpret_cast<uint4*>(o_resid + gq * DH + hl * 8) = make_uint4(r[0], r[1], r[2], r[3]);
+      if (hl == 0) lse[gq] = row_lse;
+    };
+    auto next_two = [&](uint32_t& todo) {          // this half-warp's query among the next two
+      const int b1 = __ffs(todo) - 1;
+      todo &= todo - 1;
+      const int b2 = todo ? __ffs(todo) - 1 : -1;
+      todo &= todo - 1;
+      return half ? b2 : b1;
+    };
+    // ---- queries without a pair and queries of up to kInLane pairs
+    uint32_t todo = __ballot_sync(FULL, !direct && n <= kInLane);
+    if (todo) {
+      int pos[kInLane];
+      float w[kInLane];
+      float out_lse = -INFINITY;
 #pragma unroll
       for (int k = 0; k < kInLane; ++k) { pos[k] = 0; w[k] = 0.f; }
-    }
-    uint32_t todo = __ballot_sync(0xffffffffu, !direct);
-    while (todo) {
-      const int b = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const long long gq = g0 + b;
-      const int nb = __shfl_sync(0xffffffffu, n, b);
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-      float row_lse = __shfl_sync(0xffffffffu, out_lse, b);
-      if (nb <= kInLane) {
-        float4 v[kInLane];
+      if (!direct && n > 0 && n <= kInLane) {
+        float sc[kInLane];
+        float mx = -INFINITY, tot = 0.f;
+#pragma unroll
+        for (int k = 0; k < kInLane; ++k)
+          if (k < n) pos[k] = min(max(q_pairs[lo + k], 0), last);
+#pragma unroll
+        for (int k = 0; k < kInLane; ++k) {
+          sc[k] = 0.f;
+          if (k < n) { w[k] = part_lse[pos[k]]; sc[k] = part_scale[pos[k]]; mx = fmaxf(mx, w[k]); }
+        }
+#pragma unroll
+        for (int k = 0; k < kInLane; ++k) { w[k] = k < n ? expf(w[k] - mx) : 0.f; tot += w[k]; }
+        const float inv = 1.0f / tot;
+#pragma unroll
+        for (int k = 0; k < kInLane; ++k) w[k] *= inv * sc[k];
+        out_lse = mx + logf(tot);
+      }
+      while (todo) {
+        const int b = next_two(todo), from = max(b, 0);
+        const int nq = __shfl_sync(FULL, n, from), nb = b < 0 ? 0 : nq;
+        const float row_lse = __shfl_sync(FULL, out_lse, from);
+        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        uint4 v[kInLane];
         float wk[kInLane];
 #pragma unroll
         for (int k = 0; k < kInLane; ++k) {
-          const int pk = __shfl_sync(0xffffffffu, pos[k], b);
-          wk[k] = __shfl_sync(0xffffffffu, w[k], b);
-          v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (k < nb) v[k] = load_part4<PT>(part_o + (long long)pk * DH + lane * 4);
+          const int pk = __shfl_sync(FULL, pos[k], from);
+          wk[k] = __shfl_sync(FULL, w[k], from);
+          v[k] = make_uint4(0u, 0u, 0u, 0u);
+          if (k < nb) v[k] = rows[(long long)pk * (DH / 8)];
         }
 #pragma unroll
-        for (int k = 0; k < kInLane; ++k) {
-          acc.x = fmaf(wk[k], v[k].x, acc.x); acc.y = fmaf(wk[k], v[k].y, acc.y);
-          acc.z = fmaf(wk[k], v[k].z, acc.z); acc.w = fmaf(wk[k], v[k].w, acc.w);
-        }
-      } else {
-        // many pairs: lane i of each group of 32 pairs fetches position and lse of pair i, the weights travel by shuffle
-        const long long qlo = __shfl_sync(0xffffffffu, lo, b), qhi = qlo + nb;
-        float mx = -INFINITY;
-        for (long long i0 = qlo; i0 < qhi; i0 += 32) {
-          const long long i = i0 + lane;
-          mx = fmaxf(mx, i < qhi ? part_lse[min(max(q_pairs[i], 0), last)] : -INFINITY);
-        }
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, s));
-        float tot = 0.f;
-        for (long long i0 = qlo; i0 < qhi; i0 += 32) {
-          const long long i = i0 + lane;
-          int my_pos = 0;
-          float my_w = 0.f, my_ws = 0.f;
-          if (i < qhi) {
-            my_pos = min(max(q_pairs[i], 0), last);
-            my_w = expf(part_lse[my_pos] - mx);
-            my_ws = part_scale ? my_w * part_scale[my_pos] : my_w;
-          }
-          tot += my_w;
-          const int m = (int)min((long long)32, qhi - i0);
-#pragma unroll 4
-          for (int k = 0; k < m; ++k) {
-            const long long pk = __shfl_sync(0xffffffffu, my_pos, k);
-            const float wgt = __shfl_sync(0xffffffffu, my_ws, k);
-            const float4 v = load_part4<PT>(part_o + pk * DH + lane * 4);
-            acc.x = fmaf(wgt, v.x, acc.x); acc.y = fmaf(wgt, v.y, acc.y);
-            acc.z = fmaf(wgt, v.z, acc.z); acc.w = fmaf(wgt, v.w, acc.w);
-          }
-        }
-#pragma unroll
-        for (int s = 16; s > 0; s >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, s);
-        const float inv = 1.0f / tot;
-        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
-        row_lse = mx + logf(tot);
+        for (int k = 0; k < kInLane; ++k) add_half8(acc, v[k], wk[k]);
+        write_row(b, acc, row_lse);
       }
-      T* o_row = o + o_map.off(gq, DH);
-      store4_resid(o_row + lane * 4, o_resid ? o_resid + gq * DH + lane * 4 : nullptr, acc);
-      if (lane == 0) lse[gq] = row_lse;
+    }
+    // ---- longer ones
+    todo = __ballot_sync(FULL, n > kInLane);
+    while (todo) {
+      const int b = next_two(todo), from = max(b, 0);
+      const int qlo = __shfl_sync(FULL, lo, from), nq = __shfl_sync(FULL, n, from);
+      const int nb = b < 0 ? 0 : nq;
+      const int n_max = max(__shfl_sync(FULL, nb, 0), __shfl_sync(FULL, nb, 16));
+      // largest lse of the query; the first sixteen pairs' positions and lse stay in registers
+      int pos0 = 0;
+      float l0 = -INFINITY;
+      if (hl < nb) { pos0 = min(max(q_pairs[qlo + hl], 0), last); l0 = part_lse[pos0]; }
+      float mx = l0;
+      for (int i = hl + 16; i < nb; i += 16) mx = fmaxf(mx, part_lse[min(max(q_pairs[qlo + i], 0), last)]);
+#pragma unroll
+      for (int s = 8; s > 0; s >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, s));
+      float tot = 0.f;
+      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+      for (int c0 = 0; c0 < n_max; c0 += 16) {
+        if (c0 > 0) {
+          pos0 = 0; l0 = -INFINITY;
+          if (c0 + hl < nb) { pos0 = min(max(q_pairs[qlo + c0 + hl], 0), last); l0 = part_lse[pos0]; }
+        }
+        float w0 = 0.f;
+        if (c0 + hl < nb) {
+          w0 = expf(l0 - mx);
+          tot += w0;
+          w0 *= part_scale[pos0];
+        }
+#pragma unroll
+        for (int k0 = 0; k0 < 16; k0 += kBatch) {
+          if (c0 + k0 >= n_max) break;
+          uint4 v[kBatch];
+          float wk[kBatch];
+#pragma unroll
+          for (int k = 0; k < kBatch; ++k) {
+            const int at = (lane & 16) + k0 + k;
+            const int pk = __shfl_sync(FULL, pos0, at);
+            wk[k] = __shfl_sync(FULL, w0, at);
+            v[k] = make_uint4(0u, 0u, 0u, 0u);
+            if (c0 + k0 + k < nb) v[k] = rows[(long long)pk * (DH / 8)];
+          }
+#pragma unroll
+          for (int k = 0; k < kBatch; ++k) add_half8(acc, v[k], wk[k]);
+        }
+      }
+#pragma unroll
+      for (int s = 8; s > 0; s >>= 1) tot += __shfl_xor_sync(FULL, tot, s);
+      const float inv = 1.0f / tot;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i] *= inv;
+      write_row(b, acc, mx + logf(tot));
     }
   }
 }

@@ -577,7 +577,7 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
   kernel<<<(int)items, THREADS, SMEM_BYTES, st>>>(tmK, tmV, p);
   const long long nq = (long long)D.BH * D.S;
-  simt::merge_batched_kernel<__nv_bfloat16, __half><<<(int)std::min<long long>((nq + 255) / 256, sm_count() * 8), 256, 0, st>>>(
+  simt::merge_batched_kernel<<<(int)std::min<long long>((nq + 255) / 256, sm_count() * 8), 256, 0, st>>>(
       q_ptr, q_pairs, nq, p.part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o, (__nv_bfloat16*)o_resid, lse, o_map);
   VMOBA_LAUNCH_OK(4);
   return VMOBA_OK;
