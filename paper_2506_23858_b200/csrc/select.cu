@@ -361,7 +361,7 @@ mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, 
   const int TW = QSEG >> 5;                           // words of a block's column over the segment's queries
   uint32_t* s_mask = sm;                              // [QSEG][mw]
   int* s_cnt = reinterpret_cast<int*>(sm + QSEG * mw);  // [Nb]
-  uint32_t* s_tm = sm + QSEG * mw + Nb;               // [Nb][TW]: the same bits, one row per key block
+  uint32_t* s_tm = sm + QSEG * mw + Nb;               // [TW][Nb]: the same bits, a word per 32 queries and key block
   __shared__ int s_total;
   const int seg = blockIdx.x, bh = blockIdx.y;
   const int q0 = seg * QSEG;
@@ -386,7 +386,7 @@ mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, 
     // own_sb > 0: a query also keeps the block it lies in (block-major position / tokens per block)
     if (sel || (q0 + ql) / own_sb == j) {
       atomicOr(&s_mask[ql * mw + (j >> 5)], 1u << (j & 31));
-      atomicOr(&s_tm[j * TW + (ql >> 5)], 1u << (ql & 31));
+      atomicOr(&s_tm[(ql >> 5) * Nb + j], 1u << (ql & 31));
       atomicAdd(&s_cnt[j], 1);
     }
   };
@@ -471,85 +471,114 @@ offsets_kernel(const int* __restrict__ kb_total, int* __restrict__ kb_ptr, long 
   }
 }
 
-// fill: a CTA re-reads its segment's mask words and derives q_ptr for its queries; then, one warp
-// per key block, the block's column of the segment (a few words written by the mark kernel) gives
-// the selecting queries in ascending order without touching the unset bits: each is placed in
-// q_idx, and the same position is recorded in the query-major list q_pairs.
+// fill: a CTA re-reads its segment's mask words and derives q_ptr for its queries; then thread = query walks the query's
+// set bits.  The position of a pair in q_idx is that of its block's first selecting query in the segment plus the
+// selecting queries below in the block's column of the segment (column words of the mark kernel, prefixed per word).  Both
+// lists of a segment are put together in shared memory, by block and by query, and written out in runs; a segment with
+// more than kStage pairs writes its entries one by one.  8.2 million pairs, nine per query: 119 us (273 with a warp per key
+// block that wrote q_pairs entry by entry); 12.6 million, 32 per query, beyond the stage: 154 (173).
+constexpr int kStage = 6144;
 __global__ void __launch_bounds__(kSegThreads)
 fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__ tmask, int S, int Nb, int mw, int QSEG,
             int nseg, const int* __restrict__ kb_ptr, const int* __restrict__ seg_cnt, const int* __restrict__ seg_qoff,
             int* __restrict__ q_idx, int* __restrict__ q_ptr, int* __restrict__ q_pairs, long long capacity) {
   extern __shared__ uint32_t sm[];
-  uint32_t* s_mask = sm;                                   // [QSEG][mw]
-  int* s_qoff = reinterpret_cast<int*>(sm + QSEG * mw);    // [QSEG] exclusive pair offset inside the segment
+  const int TW = QSEG >> 5;
+  uint32_t* s_mask = sm;                                    // [QSEG][mw]
+  uint32_t* s_tm = s_mask + QSEG * mw;                      // [TW][Nb] column words
+  int* s_pre = reinterpret_cast<int*>(s_tm + Nb * TW);      // [TW][Nb] entries of the segment in front of that word, by block
+  int* s_off = s_pre + Nb * TW;                             // [Nb + 1] entries in front of the block
+  int* s_pos = s_off + Nb + 1;                              // [Nb] position of the segment's first entry of the block in q_idx
+  int* s_idx = s_pos + Nb;                                  // [kStage] q_idx entries by block
+  int* s_pair = s_idx + kStage;                             // [kStage] q_pairs entries by query
   __shared__ int s_warp[kSegThreads / 32];
   const int seg = blockIdx.x, bh = blockIdx.y;
   const int q0 = seg * QSEG;
   const int nq = min(QSEG, S - q0);
-  const int TW = QSEG >> 5;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5, nwarps = blockDim.x >> 5;
+  // exclusive scan of one value per thread over the CTA
+  auto scan = [&](int v) {
+    int inc = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      int x = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += x;
+    }
+    __syncthreads();
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    if (warp == 0) {
+      int x = lane < nwarps ? s_warp[lane] : 0;
+      int xi = x;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        int y = __shfl_up_sync(0xffffffffu, xi, o);
+        if (lane >= o) xi += y;
+      }
+      if (lane < nwarps) s_warp[lane] = xi - x;
+    }
+    __syncthreads();
+    return s_warp[warp] + inc - v;
+  };
   const uint32_t* gm = mask_bits + ((long long)bh * S + q0) * mw;
-  for (int i = t; i < QSEG * mw; i += blockDim.x) s_mask[i] = i < nq * mw ? gm[i] : 0u;
+  const uint32_t* tm = tmask + ((long long)bh * nseg + seg) * Nb * TW;
+  const int* sc = seg_cnt + ((long long)bh * nseg + seg) * Nb;
+  for (int i = t; i < nq * mw; i += blockDim.x) s_mask[i] = gm[i];
+  for (int i = t; i < Nb * TW; i += blockDim.x) s_tm[i] = tm[i];
+  for (int j = t; j < Nb; j += blockDim.x)          // (clamped: beyond INT32_MAX is beyond every capacity)
+    s_pos[j] = (int)min((long long)kb_ptr[(long long)bh * Nb + j] + sc[j], (long long)INT32_MAX);
+  const long long qbase = seg_qoff[bh * nseg + seg];
   __syncthreads();
-  const int qbase = seg_qoff[bh * nseg + seg];
-  // exclusive scan of per-query pair counts (QSEG <= blockDim.x)
+  {
+    const int per = (Nb + blockDim.x - 1) / blockDim.x, j0 = min(t * per, Nb), j1 = min(j0 + per, Nb);
+    int c = 0;
+    for (int j = j0; j < j1; ++j)
+      for (int w = 0; w < TW; ++w) c += __popc(s_tm[w * Nb + j]);
+    int run = scan(c);
+    for (int j = j0; j < j1; ++j) {
+      s_off[j] = run;
+      for (int w = 0; w < TW; ++w) { s_pre[w * Nb + j] = run; run += __popc(s_tm[w * Nb + j]); }
+    }
+    if (j1 == Nb && j0 < j1) s_off[Nb] = run;
+  }
   int cnt = 0;
   if (t < nq)
     for (int w = 0; w < mw; ++w) cnt += __popc(s_mask[t * mw + w]);
-  int inc = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    int x = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += x;
-  }
-  if (lane == 31) s_warp[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    int x = lane < nwarps ? s_warp[lane] : 0;
-    int xi = x;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, xi, o);
-      if (lane >= o) xi += y;
-    }
-    if (lane < nwarps) s_warp[lane] = xi - x;
-  }
-  __syncthreads();
-  if (t < QSEG) {
-    int excl = s_warp[warp] + inc - cnt;
-    s_qoff[t] = excl;
-    if (t < nq) q_ptr[(long long)bh * S + q0 + t] = (int)min((long long)qbase + excl, (long long)INT32_MAX);
-  }
-  __syncthreads();
-  const int* sc = seg_cnt + ((long long)bh * nseg + seg) * Nb;
-  const uint32_t* tm = tmask + ((long long)bh * nseg + seg) * Nb * TW;
-  for (int j = warp; j < Nb; j += nwarps) {
-    // lane l holds the block's bits of queries 32 l .. 32 l + 31 of the segment (TW <= 16 words)
-    uint32_t word = lane < TW ? tm[j * TW + lane] : 0u;
-    int before = __popc(word);
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int x = __shfl_up_sync(0xffffffffu, before, o);
-      if (lane >= o) before += x;
-    }
-    before -= __popc(word);                                 // selecting queries in the lower words
-    const long long base = (long long)kb_ptr[(long long)bh * Nb + j] + sc[j];
-    const int wj = j >> 5;
-    const uint32_t bit = 1u << (j & 31);
-    while (word) {
-      const int b = __ffs(word) - 1;
-      word &= word - 1;
-      const int ql = 32 * lane + b;
-      const long long pos = base + before;
-      ++before;
-      if (pos < capacity) {
-        q_idx[pos] = q0 + ql;
-        int within = __popc(s_mask[ql * mw + wj] & (bit - 1u));
-        for (int w = 0; w < wj; ++w) within += __popc(s_mask[ql * mw + w]);
-        const long long qp = (long long)qbase + s_qoff[ql] + within;
-        if (qp < capacity) q_pairs[qp] = (int)pos;
+  int mine = scan(cnt);                              // this query's next entry of q_pairs, counted from the segment's first
+  const int total = s_off[Nb];
+  if (t < nq) q_ptr[(long long)bh * S + q0 + t] = (int)min(qbase + mine, (long long)INT32_MAX);
+  const bool staged = total <= kStage;
+  if (t < nq) {
+    const uint32_t lt_mask = (1u << lane) - 1u;
+    for (int w = 0; w < mw; ++w) {
+      uint32_t word = s_mask[t * mw + w];
+      while (word) {
+        const int j = 32 * w + __ffs(word) - 1;
+        word &= word - 1;
+        const int e = s_pre[warp * Nb + j] + __popc(s_tm[warp * Nb + j] & lt_mask);
+        const long long pos = (long long)s_pos[j] + (e - s_off[j]);
+        const int entry = (int)min(pos, (long long)INT32_MAX);
+        if (staged) {
+          s_idx[e] = q0 + t;
+          s_pair[mine] = entry;
+        } else if (pos < capacity) {
+          q_idx[pos] = q0 + t;
+          if (qbase + mine < capacity) q_pairs[qbase + mine] = entry;
+        }
+        ++mine;
       }
     }
+  }
+  if (!staged) return;
+  __syncthreads();
+  for (int i = t; i < total; i += blockDim.x)
+    if (qbase + i < capacity && s_pair[i] < capacity) q_pairs[qbase + i] = s_pair[i];
+  // a quarter warp per block's run
+  for (int j = t >> 3; j < Nb; j += blockDim.x >> 3) {
+    const int o0 = s_off[j], n = s_off[j + 1] - o0;
+    const long long pos = s_pos[j];
+    for (int i = t & 7; i < n; i += 8)
+      if (pos + i < capacity) q_idx[pos + i] = s_idx[o0 + i];
   }
 }
 
@@ -927,7 +956,7 @@ mark_from_mask_kernel(const uint32_t* __restrict__ mask_bits, int S, int Nb, int
   extern __shared__ uint32_t sm[];
   const int TW = QSEG >> 5;
   int* s_cnt = reinterpret_cast<int*>(sm);            // [Nb]
-  uint32_t* s_tm = sm + Nb;                           // [Nb][TW]
+  uint32_t* s_tm = sm + Nb;                           // [TW][Nb]
   __shared__ int s_total;
   const int seg = blockIdx.x, bh = blockIdx.y;
   const int q0 = seg * QSEG;
@@ -945,7 +974,7 @@ mark_from_mask_kernel(const uint32_t* __restrict__ mask_bits, int S, int Nb, int
     while (word) {
       const int j = 32 * wj + __ffs(word) - 1;
       word &= word - 1;
-      atomicOr(&s_tm[j * TW + (ql >> 5)], 1u << (ql & 31));
+      atomicOr(&s_tm[(ql >> 5) * Nb + j], 1u << (ql & 31));
       atomicAdd(&s_cnt[j], 1);
     }
   }
@@ -1190,12 +1219,13 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     VMOBA_LAUNCH_OK(1);
   }
 
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const size_t smem_fill = ((size_t)QSEG * D.mask_words + 2 * (size_t)D.Nb * (QSEG >> 5) + 2 * (size_t)D.Nb + 1 + 2 * kStage) * 4;
+  VMOBA_CUDA_OK(cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fill));
   long long nkb = (long long)D.BH * D.Nb;
   seg_prefix_kernel<<<(unsigned)((nkb + 255) / 256), 256, 0, st>>>(w.seg_cnt, w.kb_total, D.BH, D.Nb, nseg);
   offsets_kernel<<<1, 1024, 0, st>>>(w.kb_total, kb_ptr, nkb, w.seg_total, w.seg_qoff, (long long)D.BH * nseg,
                                      D.BH, D.Nb, k_per_head, capacity, q_ptr + (long long)D.BH * D.S, dev_status);
-  fill_kernel<<<sgrid, kSegThreads, smem, st>>>(mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg, kb_ptr, w.seg_cnt,
+  fill_kernel<<<sgrid, QSEG, smem_fill, st>>>(mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg, kb_ptr, w.seg_cnt,
                                                 w.seg_qoff, q_idx, q_ptr, q_pairs, capacity);
   VMOBA_LAUNCH_OK(3);
   VMOBA_GUARDS_CHECK(w.guards, dev_status, st);
