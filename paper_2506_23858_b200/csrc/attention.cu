@@ -71,14 +71,14 @@ static int simt_sparse_fwd(const Dims& D, const void* q, const void* k, const vo
   FwdWs w = carve_fwd(D, cap, ws);
   VMOBA_GUARDS_ARM(w.guards, st);
   const long long n_kb = (long long)D.BH * D.Nb;
-  simt::item_ptr_kernel<<<1, 1024, 0, st>>>(kb_ptr, n_kb, simt::kRows, cap, w.item_ptr);
+  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr);
   long long max_items = cap / simt::kRows + n_kb;
-  simt::attn_fwd_kernel<T, DH, false><<<grid_for(max_items, 8), simt::kThreads, 0, st>>>(
-      (const T*)q, (const T*)k, (const T*)v, kb_ptr, q_idx, q_ptr, w.item_ptr, (int)n_kb, D.S, D.Nb, D.sb, D.BH,
-      D.scale, (T*)o, (T*)o_resid, lse, w.part_o, w.part_lse, cap);
+  launch_kernel(simt::attn_fwd_kernel<T, DH, false>, grid_for(max_items, 8), simt::kThreads, 0, st, (const T*)q,
+                (const T*)k, (const T*)v, kb_ptr, q_idx, q_ptr, w.item_ptr, (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale,
+                (T*)o, (T*)o_resid, lse, w.part_o, w.part_lse, cap);
   long long nq = (long long)D.BH * D.S;
-  simt::merge_kernel<T, DH, float><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>(
-      q_ptr, q_pairs, nq, w.part_o, w.part_lse, cap, (T*)o, (T*)o_resid, lse);
+  launch_kernel(early_rows(D), simt::merge_kernel<T, DH, float>, grid_for((nq + 7) / 8, 16), 256, 0, st, q_ptr,
+                q_pairs, nq, w.part_o, w.part_lse, cap, (T*)o, (T*)o_resid, lse, RowMap());
   VMOBA_LAUNCH_OK(3);
   VMOBA_GUARDS_CHECK(w.guards, status, st);
   return VMOBA_OK;
@@ -98,29 +98,31 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
   if (use_tensor_cores(D)) {
     // the backward kernel adds every dQ contribution into the fp32 accumulator: the row-dot pass also clears the
     // rows of all selecting queries; they are converted afterwards (rows of queries without a block become zero)
-    simt::rowdot_kernel<T, DH><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>(
-        (const T*)o, (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, o_map, w.dq_acc, q_ptr);
+    launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
+                  (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, o_map, w.dq_acc, q_ptr);
     count_launches(1);
     int rc = tc_sparse_bwd(D, q, k, v, d_o, lse, w.Dv, kb_ptr, q_idx, cap, w.dq_acc, dk, dv, status, st, out_map, do_map);
     if (rc) return rc;
-    simt::cast_rows_kernel<T><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>(w.dq_acc, (T*)dq, q_ptr, nq, out_map);
+    launch_kernel(early_rows(D), simt::cast_rows_kernel<T>, grid_for((nq + 7) / 8, 16), 256, 0, st, w.dq_acc, (T*)dq,
+                  q_ptr, nq, out_map);
     VMOBA_LAUNCH_OK(1);
     VMOBA_GUARDS_CHECK(w.guards, status, st);
     return VMOBA_OK;
   }
-  simt::rowdot_kernel<T, DH><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>((const T*)o, (const T*)o_resid,
-                                                                        (const T*)d_o, nq, w.Dv, do_map);
+  launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
+                (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), nullptr, nullptr);
   count_launches(1);
   VMOBA_CUDA_OK(cudaMemsetAsync(w.dq_acc, 0, (size_t)nq * DH * sizeof(float), st));
-  simt::item_ptr_kernel<<<1, 1024, 0, st>>>(kb_ptr, n_kb, simt::kRows, cap, w.item_ptr);
+  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr);
   long long tiles = (D.sb + simt::kRows - 1) / simt::kRows;
-  simt::attn_bwd_dkdv_kernel<T, DH, false><<<grid_for(n_kb * tiles, 4), simt::kThreads, 0, st>>>(
-      (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb, D.BH,
-      D.scale, cap, (T*)dk, (T*)dv);
-  simt::attn_bwd_dq_kernel<T, DH, false><<<grid_for(nq / simt::kRows * D.Nb + n_kb, 4), simt::kThreads, 0, st>>>(
-      (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, w.item_ptr, (int)n_kb, D.S,
-      D.Nb, D.sb, D.BH, D.scale, cap, w.dq_acc, (T*)dq);
-  simt::cast_kernel<T><<<grid_for((nq * DH / 4 + 255) / 256, 16), 256, 0, st>>>(w.dq_acc, (T*)dq, nq * DH / 4);
+  launch_kernel(simt::attn_bwd_dkdv_kernel<T, DH, false>, grid_for(n_kb * tiles, 4), simt::kThreads, 0, st,
+                (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb, D.BH,
+                D.scale, cap, (T*)dk, (T*)dv);
+  launch_kernel(simt::attn_bwd_dq_kernel<T, DH, false>, grid_for(nq / simt::kRows * D.Nb + n_kb, 4), simt::kThreads,
+                0, st, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, w.item_ptr,
+                (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale, cap, w.dq_acc, (T*)dq);
+  launch_kernel(early_rows(D), simt::cast_kernel<T>, grid_for((nq * DH / 4 + 255) / 256, 16), 256, 0, st, w.dq_acc,
+                (T*)dq, nq * DH / 4);
   VMOBA_LAUNCH_OK(4);
   VMOBA_GUARDS_CHECK(w.guards, status, st);
   return VMOBA_OK;
@@ -136,29 +138,30 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
     int rc = tc_dense_fwd(D, q, k, v, o, d_o ? w.o_resid : nullptr, lse, status, st);
     if (rc) return rc;
   } else {
-    simt::attn_fwd_kernel<T, DH, true><<<grid_for(D.BH * tiles, 8), simt::kThreads, 0, st>>>(
-        (const T*)q, (const T*)k, (const T*)v, nullptr, nullptr, nullptr, nullptr, 0, D.S, 1, D.S, D.BH, D.scale,
-        (T*)o, d_o ? (T*)w.o_resid : nullptr, lse, nullptr, nullptr, 0);
+    launch_kernel(simt::attn_fwd_kernel<T, DH, true>, grid_for(D.BH * tiles, 8), simt::kThreads, 0, st, (const T*)q,
+                  (const T*)k, (const T*)v, nullptr, nullptr, nullptr, nullptr, 0, D.S, 1, D.S, D.BH, D.scale, (T*)o,
+                  d_o ? (T*)w.o_resid : nullptr, lse, nullptr, nullptr, 0);
     count_launches(1);
   }
   if (d_o) {
     // (the tensor-core backward adds dQ into the fp32 accumulator, cleared in the same pass; null on the other path)
-    simt::rowdot_kernel<T, DH><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>((const T*)o, (const T*)w.o_resid,
-                                                                          (const T*)d_o, nq, w.Dv, RowMap(), RowMap(), w.dq_acc);
+    launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
+                  (const T*)w.o_resid, (const T*)d_o, nq, w.Dv, RowMap(), RowMap(), w.dq_acc, nullptr);
     if (use_tensor_cores(D)) {
       VMOBA_LAUNCH_OK(1);
       int rc = tc_dense_bwd(D, q, k, v, d_o, lse, w.Dv, w.dq_acc, dk, dv, status, st);
       if (rc) return rc;
-      simt::cast_rows_kernel<T><<<grid_for((nq + 7) / 8, 16), 256, 0, st>>>(w.dq_acc, (T*)dq, nullptr, nq, RowMap());
+      launch_kernel(early_rows(D), simt::cast_rows_kernel<T>, grid_for((nq + 7) / 8, 16), 256, 0, st, w.dq_acc,
+                    (T*)dq, nullptr, nq, RowMap());
       VMOBA_LAUNCH_OK(1);
       return VMOBA_OK;
     }
-    simt::attn_bwd_dkdv_kernel<T, DH, true><<<grid_for(D.BH * tiles, 4), simt::kThreads, 0, st>>>(
-        (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, D.S, 1, D.S, D.BH,
-        D.scale, 0, (T*)dk, (T*)dv);
-    simt::attn_bwd_dq_kernel<T, DH, true><<<grid_for(D.BH * tiles, 4), simt::kThreads, 0, st>>>(
-        (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, nullptr, 0, D.S, 1, D.S,
-        D.BH, D.scale, 0, nullptr, (T*)dq);
+    launch_kernel(simt::attn_bwd_dkdv_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, 0, st,
+                  (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, D.S, 1, D.S,
+                  D.BH, D.scale, 0, (T*)dk, (T*)dv);
+    launch_kernel(simt::attn_bwd_dq_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, 0, st,
+                  (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, nullptr, 0, D.S,
+                  1, D.S, D.BH, D.scale, 0, nullptr, (T*)dq);
   }
   VMOBA_LAUNCH_OK(d_o ? 3 : 0);
   return VMOBA_OK;

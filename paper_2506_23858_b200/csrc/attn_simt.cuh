@@ -25,6 +25,7 @@ constexpr int kThreads = 256;  // 4 threads per row, each owning head_dim/4 chan
 static __global__ void __launch_bounds__(1024)
 item_ptr_kernel(const int* __restrict__ kb_ptr, long long n_kb, int rows, long long capacity,
                 int* __restrict__ item_ptr) {
+  if (!grid_begin()) return;
   __shared__ long long total;
   block_exclusive_scan(
       [&](long long i) {
@@ -39,6 +40,7 @@ item_ptr_kernel(const int* __restrict__ kb_ptr, long long n_kb, int rows, long l
 static __global__ void __launch_bounds__(256)
 item_desc_kernel(const int* __restrict__ item_ptr, const int* __restrict__ kb_ptr, long long n_kb, long long max_items,
                  long long capacity, int rows_per_item, int4* __restrict__ desc) {
+  if (!grid_begin()) return;
   const int lane = threadIdx.x & 31;
   const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n_kb; i += n_warps) {
@@ -108,6 +110,7 @@ attn_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
                 const int* __restrict__ item_ptr, int n_kb, int S, int Nb, int sb, int BH, float scale,
                 T* __restrict__ o, T* __restrict__ o_resid, float* __restrict__ lse, float* __restrict__ part_o,
                 float* __restrict__ part_lse, long long capacity) {
+  if (!grid_begin()) return;
   constexpr int DP = DH / 4;   // channels per thread
   constexpr int G = DP / 4;    // float4 groups per thread
   __shared__ __align__(16) float Ks[kTile * DH];
@@ -213,7 +216,8 @@ template <typename T, int DH, typename PT>
 __global__ void __launch_bounds__(256)
 merge_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pairs, long long n_queries,
              const PT* __restrict__ part_o, const float* __restrict__ part_lse, long long capacity,
-             T* __restrict__ o, T* __restrict__ o_resid, float* __restrict__ lse, const RowMap o_map = RowMap()) {
+             T* __restrict__ o, T* __restrict__ o_resid, float* __restrict__ lse, const RowMap o_map) {
+  if (!grid_begin()) return;
   constexpr int C = DH / 32;   // channels per lane
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -315,6 +319,7 @@ merge_batched_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pa
                      const __half* __restrict__ part_o, const float* __restrict__ part_lse,
                      const float* __restrict__ part_scale, long long capacity, __nv_bfloat16* __restrict__ o,
                      __nv_bfloat16* __restrict__ o_resid, float* __restrict__ lse, const RowMap o_map) {
+  if (!grid_begin()) return;
   constexpr int DH = 128;
   constexpr uint32_t FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31, hl = lane & 15, half = lane >> 4;
@@ -463,8 +468,9 @@ merge_batched_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pa
 template <typename T, int DH>
 __global__ void __launch_bounds__(256)
 rowdot_kernel(const T* __restrict__ o, const T* __restrict__ o_resid, const T* __restrict__ d_o, long long n_queries,
-              float* __restrict__ Dv, const RowMap do_map = RowMap(), const RowMap o_map = RowMap(),
-              float* __restrict__ zero_acc = nullptr, const int* __restrict__ q_ptr = nullptr) {
+              float* __restrict__ Dv, const RowMap do_map, const RowMap o_map,
+              float* __restrict__ zero_acc, const int* __restrict__ q_ptr) {
+  if (!grid_begin()) return;
   constexpr int C = DH / 32;
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -544,6 +550,7 @@ attn_bwd_dkdv_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
                      const T* __restrict__ d_o, const float* __restrict__ lse, const float* __restrict__ Dv,
                      const int* __restrict__ kb_ptr, const int* __restrict__ q_idx, int S, int Nb, int sb, int BH,
                      float scale, long long capacity, T* __restrict__ dk, T* __restrict__ dv) {
+  if (!grid_begin()) return;
   constexpr int DP = DH / 4, G = DP / 4;
   __shared__ __align__(16) float Qs[kTile * DH];
   __shared__ __align__(16) float dOs[kTile * DH];
@@ -639,6 +646,7 @@ attn_bwd_dq_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
                    const int* __restrict__ kb_ptr, const int* __restrict__ q_idx, const int* __restrict__ item_ptr,
                    int n_kb, int S, int Nb, int sb, int BH, float scale, long long capacity,
                    float* __restrict__ dq_acc, T* __restrict__ dq) {
+  if (!grid_begin()) return;
   constexpr int DP = DH / 4, G = DP / 4;
   __shared__ __align__(16) float Ks[kTile * DH];
   __shared__ __align__(16) float Vs[kTile * DH];
@@ -727,6 +735,7 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 cast_rows_kernel(const float* __restrict__ src, T* __restrict__ dst, const int* __restrict__ q_ptr, long long n_queries,
                  const RowMap map) {
+  if (!grid_begin()) return;
   constexpr int DH = 128;
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -765,6 +774,7 @@ cast_rows_kernel(const float* __restrict__ src, T* __restrict__ dst, const int* 
 template <typename T>
 __global__ void __launch_bounds__(256)
 cast_kernel(const float* __restrict__ src, T* __restrict__ dst, long long n4) {
+  if (!grid_begin()) return;
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x)
     store4(dst + 4 * i, *reinterpret_cast<const float4*>(src + 4 * i));
 }

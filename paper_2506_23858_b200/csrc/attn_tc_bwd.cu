@@ -217,6 +217,7 @@ template <bool DENSE, bool PROF>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmO, const KvParams p) {
+  if (!grid_begin()) return;
   extern __shared__ uint8_t smem_raw[];
   // the swizzled tiles need 1024-byte alignment and there is no room for alignment slack
   if ((smem_u32(smem_raw) & 1023u) != 0) {
@@ -713,7 +714,7 @@ static int launch(const Dims& D, const void* k, const void* v, KvParams& kp, cud
   const int grid = (int)std::max<long long>(1, std::min<long long>(items, sm_count()));
   auto kernel = kp.prof ? attn_bwd_fused_kernel<DENSE, true> : attn_bwd_fused_kernel<DENSE, false>;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-  kernel<<<grid, THREADS, SMEM_BYTES, st>>>(tmK, tmV, tmQ, tmO, kp);
+  launch_kernel(early_rows(D), kernel, grid, THREADS, SMEM_BYTES, st, tmK, tmV, tmQ, tmO, kp);
   VMOBA_LAUNCH_OK(1);
   return VMOBA_OK;
 }

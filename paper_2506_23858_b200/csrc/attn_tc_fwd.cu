@@ -158,6 +158,7 @@ template <bool DENSE, bool RASTER, bool PROF>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_fwd_wide_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                      const __grid_constant__ CUtensorMap tmQ, const Params p) {
+  if (!grid_begin()) return;
   extern __shared__ uint8_t smem_raw[];
   // the swizzled tiles need 1024-byte alignment and there is no room for alignment slack
   if ((smem_u32(smem_raw) & 1023u) != 0) {
@@ -587,7 +588,7 @@ static int launch_wide(const Dims& D, const void* q, const void* k, const void* 
     return VMOBA_ERR_CUDA;
   auto kernel = p.prof ? attn_fwd_wide_kernel<DENSE, RASTER, true> : attn_fwd_wide_kernel<DENSE, RASTER, false>;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-  kernel<<<grid, THREADS, SMEM_BYTES, st>>>(tmK, tmV, tmQ, p);
+  launch_kernel(kernel, grid, THREADS, SMEM_BYTES, st, tmK, tmV, tmQ, p);
   VMOBA_LAUNCH_OK(1);
   return VMOBA_OK;
 }
@@ -614,9 +615,9 @@ int tc_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, co
     return tc_sparse_fwd_narrow(D, q, k, v, kb_ptr, q_idx, q_ptr, q_pairs, cap, o, o_resid, lse, status, item_ptr, item_tab,
                                 max_items, part_o, part_lse, part_scale, st, o_map);
   const long long n_kb = (long long)D.BH * D.Nb;
-  simt::item_ptr_kernel<<<1, 1024, 0, st>>>(kb_ptr, n_kb, IM, cap, item_ptr);
-  simt::item_desc_kernel<<<(int)std::min<long long>((n_kb + 7) / 8, sm_count() * 8), 256, 0, st>>>(
-      item_ptr, kb_ptr, n_kb, max_items, cap, IM, reinterpret_cast<int4*>(item_tab));
+  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, IM, cap, item_ptr);
+  launch_kernel(simt::item_desc_kernel, (int)std::min<long long>((n_kb + 7) / 8, sm_count() * 8), 256, 0, st,
+                item_ptr, kb_ptr, n_kb, max_items, cap, IM, reinterpret_cast<int4*>(item_tab));
   Params p;
   p.q = (const __nv_bfloat16*)q; p.q_idx = q_idx; p.q_ptr = q_ptr; p.item_ptr = item_ptr;
   p.item_desc = reinterpret_cast<const int4*>(item_tab);
@@ -633,8 +634,9 @@ int tc_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, co
     if (int rc = launch_wide<false, false>(D, q, k, v, p, grid_items(cap / IM + n_kb), st)) return rc;
   }
   const long long nq = (long long)D.BH * D.S;
-  simt::merge_batched_kernel<<<(int)std::min<long long>((nq + 255) / 256, sm_count() * 8), 256, 0, st>>>(
-      q_ptr, q_pairs, nq, p.part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o, (__nv_bfloat16*)o_resid, lse, o_map);
+  launch_kernel(early_rows(D), simt::merge_batched_kernel, (int)std::min<long long>((nq + 255) / 256, sm_count() * 8),
+                256, 0, st, q_ptr, q_pairs, nq, p.part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o,
+                (__nv_bfloat16*)o_resid, lse, o_map);
   VMOBA_LAUNCH_OK(3);
   return VMOBA_OK;
 }

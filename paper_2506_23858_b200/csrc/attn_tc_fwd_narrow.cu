@@ -180,6 +180,7 @@ __device__ __forceinline__ void store8_resid(__nv_bfloat16* dst, __nv_bfloat16* 
 template <bool RASTER>
 __global__ void __launch_bounds__(THREADS, 2)
 attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const Params p) {
+  if (!grid_begin()) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = base;
@@ -559,9 +560,9 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
   if (!sm100::make_tmap_bf16_rows(&tmK, k, rows, DH, BN) || !sm100::make_tmap_bf16_rows(&tmV, v, rows, DH, BN))
     return VMOBA_ERR_CUDA;
   const long long n_kb = (long long)D.BH * D.Nb;
-  simt::item_ptr_kernel<<<1, 1024, 0, st>>>(kb_ptr, n_kb, BM, cap, item_ptr);
-  simt::item_desc_kernel<<<(int)std::min<long long>((n_kb + 7) / 8, sm_count() * 8), 256, 0, st>>>(
-      item_ptr, kb_ptr, n_kb, max_items, cap, BM, reinterpret_cast<int4*>(item_tab));
+  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, BM, cap, item_ptr);
+  launch_kernel(simt::item_desc_kernel, (int)std::min<long long>((n_kb + 7) / 8, sm_count() * 8), 256, 0, st,
+                item_ptr, kb_ptr, n_kb, max_items, cap, BM, reinterpret_cast<int4*>(item_tab));
   Params p;
   p.q = (const __nv_bfloat16*)q; p.q_idx = q_idx; p.q_ptr = q_ptr; p.item_ptr = item_ptr;
   p.item_desc = reinterpret_cast<const int4*>(item_tab);
@@ -575,10 +576,11 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
   const long long items = std::max<long long>(1, std::min<long long>(cap / BM + n_kb, 2LL * sm_count()));
   auto kernel = o_map.perm ? attn_fwd_narrow_kernel<true> : attn_fwd_narrow_kernel<false>;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
-  kernel<<<(int)items, THREADS, SMEM_BYTES, st>>>(tmK, tmV, p);
+  launch_kernel(kernel, (int)items, THREADS, SMEM_BYTES, st, tmK, tmV, p);
   const long long nq = (long long)D.BH * D.S;
-  simt::merge_batched_kernel<<<(int)std::min<long long>((nq + 255) / 256, sm_count() * 8), 256, 0, st>>>(
-      q_ptr, q_pairs, nq, p.part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o, (__nv_bfloat16*)o_resid, lse, o_map);
+  launch_kernel(early_rows(D), simt::merge_batched_kernel, (int)std::min<long long>((nq + 255) / 256, sm_count() * 8),
+                256, 0, st, q_ptr, q_pairs, nq, p.part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o,
+                (__nv_bfloat16*)o_resid, lse, o_map);
   VMOBA_LAUNCH_OK(4);
   return VMOBA_OK;
 }

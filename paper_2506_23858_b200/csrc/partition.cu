@@ -21,6 +21,7 @@ __device__ __forceinline__ int perm_of(const PermGeom& g, int p) {
 }
 
 __global__ void perm_table_kernel(PermGeom g, int S, int32_t* __restrict__ perm, int32_t* __restrict__ inv_perm) {
+  if (!grid_begin()) return;
   int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= S) return;
   int r = perm_of(g, p);
@@ -37,6 +38,7 @@ __global__ void __launch_bounds__(256)
 partition_kernel(PermGeom g, int S, int heads, long long n_rows, int inverse,
                  const uint4* __restrict__ src, uint4* __restrict__ dst,
                  long long rs_b, long long rs_s, long long rs_h /* raster strides in 16-byte vectors */) {
+  if (!grid_begin()) return;
   constexpr int ROWS_PER_PASS = 32 / VEC_PER_ROW > 0 ? 32 / VEC_PER_ROW : 1;
   constexpr int PASSES = 32 / ROWS_PER_PASS;        // passes to cover 32 rows
   constexpr int VITER = VEC_PER_ROW > 32 ? VEC_PER_ROW / 32 : 1;
@@ -85,9 +87,9 @@ static int launch_partition(const Dims& D, const PermGeom& g, int inverse, const
   long long cap = (long long)sm_count() * 8 * 4;
   if (blocks > cap) blocks = cap;
   long long per_vec = 16 / D.es;
-  partition_kernel<V><<<(unsigned)blocks, 256, 0, st>>>(
-      g, D.S, D.heads, n_rows, inverse, static_cast<const uint4*>(src), static_cast<uint4*>(dst),
-      rs[0] / per_vec, rs[1] / per_vec, rs[2] / per_vec);
+  launch_kernel(early_rows(D), partition_kernel<V>, (unsigned)blocks, 256, 0, st, g, D.S, D.heads, n_rows, inverse,
+                static_cast<const uint4*>(src), static_cast<uint4*>(dst), rs[0] / per_vec, rs[1] / per_vec,
+                rs[2] / per_vec);
   VMOBA_LAUNCH_OK(1);
   return VMOBA_OK;
 }
@@ -110,7 +112,7 @@ extern "C" int vmoba_partition(const vmoba_shape* shape, int inverse, const void
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   PermGeom g{D.H, D.W, D.bT, D.bH, D.bW, D.nH, D.nW, D.sb};
   if (perm_or_null || inv_perm_or_null) {
-    perm_table_kernel<<<(D.S + 255) / 256, 256, 0, st>>>(g, D.S, perm_or_null, inv_perm_or_null);
+    launch_kernel(perm_table_kernel, (D.S + 255) / 256, 256, 0, st, g, D.S, perm_or_null, inv_perm_or_null);
     VMOBA_LAUNCH_OK(1);
   }
   int V = D.d * D.es / 16;

@@ -24,6 +24,7 @@ size_t scores_ws_bytes(const Dims& D) {
 template <typename T, int DH>
 __global__ void __launch_bounds__(256)
 centroid_kernel(const T* __restrict__ k_bm, float* __restrict__ cent, int sb) {
+  if (!grid_begin()) return;
   constexpr int V = DH / 4;            // float4 columns per row
   constexpr int RL = 256 / V;          // row lanes
   __shared__ float4 red[RL][V];
@@ -55,6 +56,7 @@ template <typename T, int DH>
 __global__ void __launch_bounds__(256)
 scores_kernel(const T* __restrict__ q_bm, const float* __restrict__ cent, float* __restrict__ scores,
               int S, int Nb) {
+  if (!grid_begin()) return;
   extern __shared__ float smem[];
   constexpr int LD = 64 + 4;
   float* qT = smem;                 // [DH][LD]
@@ -119,11 +121,13 @@ scores_kernel(const T* __restrict__ q_bm, const float* __restrict__ cent, float*
 
 // Smallest and largest score of each head (the paths whose scores kernel does not take them on the way).
 __global__ void range_init_kernel(float* __restrict__ range, int BH) {
+  if (!grid_begin()) return;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < BH) { range[2 * i] = INFINITY; range[2 * i + 1] = -INFINITY; }
 }
 __global__ void __launch_bounds__(256)
 range_kernel(const float* __restrict__ scores, long long P, float* __restrict__ range) {
+  if (!grid_begin()) return;
   const int bh = blockIdx.y;
   const float* base = scores + (long long)bh * P;
   float lo = INFINITY, hi = -INFINITY;
@@ -142,19 +146,19 @@ range_kernel(const float* __restrict__ scores, long long P, float* __restrict__ 
 template <typename T, int DH>
 static int run_scores(const Dims& D, const void* q, const void* k, float* cent, float* scores, float* range, void* ws,
                       int32_t* status, cudaStream_t st) {
-  centroid_kernel<T, DH><<<D.BH * D.Nb, 256, 0, st>>>(static_cast<const T*>(k), cent, D.sb);
+  launch_kernel(centroid_kernel<T, DH>, D.BH * D.Nb, 256, 0, st, static_cast<const T*>(k), cent, D.sb);
   VMOBA_LAUNCH_OK(1);
   if (D.dtype == VMOBA_BF16 && DH == 128) return scores_tc(D, q, cent, scores, range, ws, status, st);
   size_t smem = 2 * DH * (64 + 4) * sizeof(float);
   VMOBA_CUDA_OK(cudaFuncSetAttribute(scores_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid((D.S + 63) / 64, 1, D.BH);
-  scores_kernel<T, DH><<<grid, 256, smem, st>>>(static_cast<const T*>(q), cent, scores, D.S, D.Nb);
+  launch_kernel(scores_kernel<T, DH>, grid, 256, smem, st, static_cast<const T*>(q), cent, scores, D.S, D.Nb);
   VMOBA_LAUNCH_OK(1);
   if (range) {
     const long long P = (long long)D.S * D.Nb;
-    range_init_kernel<<<(D.BH + 127) / 128, 128, 0, st>>>(range, D.BH);
+    launch_kernel(range_init_kernel, (D.BH + 127) / 128, 128, 0, st, range, D.BH);
     const int gx = (int)std::min<long long>(std::max<long long>(P / 2048, 1), std::max(1, sm_count() * 8 / D.BH));
-    range_kernel<<<dim3(gx, D.BH), 256, 0, st>>>(scores, P, range);
+    launch_kernel(range_kernel, dim3(gx, D.BH), 256, 0, st, scores, P, range);
     VMOBA_LAUNCH_OK(2);
   }
   return VMOBA_OK;

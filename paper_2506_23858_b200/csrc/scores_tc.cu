@@ -55,6 +55,7 @@ struct Params {
 __global__ void __launch_bounds__(256)
 split_centroids_kernel(const float* __restrict__ cent, __nv_bfloat16* __restrict__ parts, int Nb, int Nb_pad, int BH,
                        float* __restrict__ range) {
+  if (!grid_begin()) return;
   const long long n = (long long)BH * Nb_pad * DH;
   if (range) {     // the scores kernel that follows takes minima / maxima into these words
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -81,6 +82,7 @@ split_centroids_kernel(const float* __restrict__ cent, __nv_bfloat16* __restrict
 __global__ void __launch_bounds__(THREADS, 1)
 scores_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmS, const Params p) {
+  if (!grid_begin()) return;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = base;                    // [2][TILE]
@@ -302,7 +304,8 @@ int scores_tc(const Dims& D, const void* q_bm, const float* cent, float* scores,
   const int rows_pass = ((Nb_pad + n_pass - 1) / n_pass + 31) / 32 * 32;
   __nv_bfloat16* parts = reinterpret_cast<__nv_bfloat16*>((reinterpret_cast<uintptr_t>(ws) + 1023) & ~uintptr_t(1023));
   const long long n = (long long)D.BH * Nb_pad * DH;
-  split_centroids_kernel<<<(int)std::min<long long>((n + 255) / 256, sm_count() * 8), 256, 0, st>>>(cent, parts, D.Nb, Nb_pad, D.BH, range);
+  launch_kernel(split_centroids_kernel, (int)std::min<long long>((n + 255) / 256, sm_count() * 8), 256, 0, st, cent,
+                parts, D.Nb, Nb_pad, D.BH, range);
   CUtensorMap tmQ, tmB, tmS;
   const int tma_store = (D.Nb % 4 == 0) && (reinterpret_cast<uintptr_t>(scores) % 16 == 0);
   if (tma_store) {
@@ -320,7 +323,8 @@ int scores_tc(const Dims& D, const void* q_bm, const float* cent, float* scores,
   p.status = status;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(scores_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
   const long long items = (long long)D.BH * n_pass * ((D.S + BM - 1) / BM);
-  scores_tc_kernel<<<(int)std::max<long long>(1, std::min<long long>(items, sm_count())), THREADS, SMEM_BYTES, st>>>(tmQ, tmB, tmS, p);
+  launch_kernel(scores_tc_kernel, (int)std::max<long long>(1, std::min<long long>(items, sm_count())), THREADS,
+                SMEM_BYTES, st, tmQ, tmB, tmS, p);
   VMOBA_LAUNCH_OK(2);
   return VMOBA_OK;
 }

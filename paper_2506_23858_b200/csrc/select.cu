@@ -96,6 +96,7 @@ __device__ __forceinline__ void for_each_score(const float* __restrict__ base, l
 
 __global__ void __launch_bounds__(256)
 minmax_kernel(const float* __restrict__ scores, long long P, HeadState* __restrict__ st) {
+  if (!grid_begin()) return;
   const int bh = blockIdx.y;
   uint32_t kmin = 0xffffffffu, kmax = 0u;
   for_each_score(scores + (long long)bh * P, P, [&](float s) {
@@ -118,6 +119,7 @@ minmax_kernel(const float* __restrict__ scores, long long P, HeadState* __restri
 __global__ void init_state_kernel(HeadState* st, int BH, const float* __restrict__ range, unsigned int* __restrict__ g_cnt,
                                   double* __restrict__ g_w, uint32_t* __restrict__ g_minkey,
                                   uint32_t* __restrict__ g_maxkey) {
+  if (!grid_begin()) return;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (g_cnt && i < (long long)BH * kBins) { g_cnt[i] = 0u; g_w[i] = 0.0; g_minkey[i] = 0xffffffffu; g_maxkey[i] = 0u; }
   if (i >= BH) return;
@@ -147,6 +149,7 @@ __global__ void __launch_bounds__(256)
 hist_kernel(const float* __restrict__ scores, long long P, const HeadState* __restrict__ st, float sigma, int unit_w,
             unsigned int* __restrict__ g_cnt, double* __restrict__ g_w, uint32_t* __restrict__ g_minkey,
             uint32_t* __restrict__ g_maxkey, float* __restrict__ cand, long long ccap, unsigned int* __restrict__ cand_cnt) {
+  if (!grid_begin()) return;
   __shared__ unsigned int s_cnt[kBins];
   __shared__ float s_w[kBins];
   __shared__ uint32_t s_min[kBins];
@@ -200,6 +203,7 @@ constexpr int kRep = 32;
 __global__ void __launch_bounds__(512)
 hist0_kernel(const float* __restrict__ scores, long long P, const HeadState* __restrict__ st, float sigma, int unit_w,
              double* __restrict__ g_w) {
+  if (!grid_begin()) return;
   extern __shared__ float s_wr[];   // [kBins0][kRep]
   const int bh = blockIdx.y;
   const HeadState hs = st[bh];
@@ -227,6 +231,7 @@ scan_kernel(HeadState* __restrict__ st, float tau, double count_target, unsigned
             double* __restrict__ g_w,
             uint32_t* __restrict__ g_minkey, uint32_t* __restrict__ g_maxkey, int64_t* __restrict__ k_per_head,
             float* __restrict__ cutoff_per_head, long long ccap) {
+  if (!grid_begin()) return;
   __shared__ double s_wsum[32];
   __shared__ unsigned long long s_csum[32];
   __shared__ int s_cross;
@@ -341,6 +346,7 @@ scan_kernel(HeadState* __restrict__ st, float tau, double count_target, unsigned
 
 // After minmax: level-0 anchors.
 __global__ void setup_level0_kernel(HeadState* st, int BH) {
+  if (!grid_begin()) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= BH) return;
   float lo = key_float(st[i].min_key), hi = key_float(st[i].max_key);
@@ -357,6 +363,7 @@ __global__ void __launch_bounds__(kSegThreads)
 mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, int S, int Nb, int mw, int QSEG,
             int nseg, int own_sb, uint32_t* __restrict__ mask_bits, int* __restrict__ seg_cnt,
             int* __restrict__ seg_total, uint32_t* __restrict__ tmask) {
+  if (!grid_begin()) return;
   extern __shared__ uint32_t sm[];
   const int TW = QSEG >> 5;                           // words of a block's column over the segment's queries
   uint32_t* s_mask = sm;                              // [QSEG][mw]
@@ -434,6 +441,7 @@ mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, 
 // offsets A: per (head, block) turn the per-segment counts into exclusive prefixes along the
 // segments and record the block's total.
 __global__ void seg_prefix_kernel(int* __restrict__ seg_cnt, int* __restrict__ kb_total, int BH, int Nb, int nseg) {
+  if (!grid_begin()) return;
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (long long)BH * Nb) return;
   int bh = (int)(i / Nb), j = (int)(i % Nb);
@@ -456,6 +464,7 @@ offsets_kernel(const int* __restrict__ kb_total, int* __restrict__ kb_ptr, long 
                const int* __restrict__ seg_total, int* __restrict__ seg_qoff, long long n_seg,
                int BH, int Nb, int64_t* __restrict__ k_per_head, long long capacity,
                int* __restrict__ q_ptr_last, int32_t* __restrict__ dev_status) {
+  if (!grid_begin()) return;
   __shared__ long long total_a, total_b;
   block_exclusive_scan([&](long long i) { return kb_total[i]; }, kb_ptr, n_kb, &total_a);
   block_exclusive_scan([&](long long i) { return seg_total[i]; }, seg_qoff, n_seg, &total_b);
@@ -482,6 +491,7 @@ __global__ void __launch_bounds__(kSegThreads)
 fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__ tmask, int S, int Nb, int mw, int QSEG,
             int nseg, const int* __restrict__ kb_ptr, const int* __restrict__ seg_cnt, const int* __restrict__ seg_qoff,
             int* __restrict__ q_idx, int* __restrict__ q_ptr, int* __restrict__ q_pairs, long long capacity) {
+  if (!grid_begin()) return;
   extern __shared__ uint32_t sm[];
   const int TW = QSEG >> 5;
   uint32_t* s_mask = sm;                                    // [QSEG][mw]
@@ -626,6 +636,7 @@ template <int MW>
 __global__ void __launch_bounds__(256)
 select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int k, int own_sb,
                    uint32_t* __restrict__ mask_bits, HeadState* __restrict__ st, long long n_rows) {
+  if (!grid_begin()) return;
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -741,6 +752,7 @@ template <int N>     // N_b rounded up
 __global__ void __launch_bounds__(kTopkRowThreads)
 select_topk_rows_kernel(const float* __restrict__ scores, int S, int Nb, int k, int own_sb,
                         uint32_t* __restrict__ mask_bits, HeadState* __restrict__ st, long long n_rows) {
+  if (!grid_begin()) return;
   __shared__ float tile[kTopkRowThreads * (N | 1)];
   const int pitch = Nb | 1;
   const float inv_nb = 1.0f / (float)Nb;
@@ -813,6 +825,7 @@ template <int MW>
 __global__ void __launch_bounds__(256)
 select_threshold_local_kernel(const float* __restrict__ scores, int S, int Nb, int mw, float sigma, float tau, int own_sb,
                               uint32_t* __restrict__ mask_bits, HeadState* __restrict__ st, long long n_rows) {
+  if (!grid_begin()) return;
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -944,6 +957,7 @@ select_threshold_local_kernel(const float* __restrict__ scores, int S, int Nb, i
 }
 
 __global__ void local_cutoff_kernel(const HeadState* __restrict__ st, float* __restrict__ cutoff_per_head, int BH) {
+  if (!grid_begin()) return;
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < BH) cutoff_per_head[i] = key_float(st[i].cutoff_key);
 }
@@ -953,6 +967,7 @@ __global__ void local_cutoff_kernel(const HeadState* __restrict__ st, float* __r
 __global__ void __launch_bounds__(kSegThreads)
 mark_from_mask_kernel(const uint32_t* __restrict__ mask_bits, int S, int Nb, int mw, int QSEG, int nseg,
                       int* __restrict__ seg_cnt, int* __restrict__ seg_total, uint32_t* __restrict__ tmask) {
+  if (!grid_begin()) return;
   extern __shared__ uint32_t sm[];
   const int TW = QSEG >> 5;
   int* s_cnt = reinterpret_cast<int*>(sm);            // [Nb]
@@ -993,6 +1008,7 @@ mark_from_mask_kernel(const uint32_t* __restrict__ mask_bits, int S, int Nb, int
 // warp per query row; the head-wide quantile search then runs on `out` with unit temperature.
 __global__ void __launch_bounds__(256)
 rownorm_kernel(const float* __restrict__ scores, float* __restrict__ out, int Nb, float sigma, long long n_rows) {
+  if (!grid_begin()) return;
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
@@ -1113,7 +1129,8 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     // search on the row-normalised log-probabilities with unit temperature
     float* lp = reinterpret_cast<float*>(static_cast<char*>(ws) + ((w.bytes + 255) / 256) * 256);
     const long long n_rows = (long long)D.BH * D.S;
-    rownorm_kernel<<<(int)std::min<long long>((n_rows + 7) / 8, sm_count() * 8), 256, 0, st>>>(scores, lp, D.Nb, D.scale, n_rows);
+    launch_kernel(rownorm_kernel, (int)std::min<long long>((n_rows + 7) / 8, sm_count() * 8), 256, 0, st, scores, lp,
+                  D.Nb, D.scale, n_rows);
     VMOBA_LAUNCH_OK(1);
     scores = lp;
     sigma = 1.0f;
@@ -1126,22 +1143,25 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
   const dim3 sgrid(nseg, D.BH);
 
   if (local) {
-    init_state_kernel<<<(D.BH + 127) / 128, 128, 0, st>>>(w.state, D.BH, nullptr, nullptr, nullptr, nullptr, nullptr);
+    launch_kernel(init_state_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, D.BH, nullptr, nullptr, nullptr,
+                  nullptr, nullptr);
     // per-query rules: the mask comes straight from the rows; cutoff_key collects the smallest selected key
     const long long n_rows = (long long)D.BH * D.S;
     const int blocks = (int)std::min<long long>((n_rows + 7) / 8, sm_count() * 8);
     const int mw = D.mask_words;
     const int k = std::min(topk, D.Nb);
     auto topk_words = [&](auto tag) {
-      select_topk_kernel<decltype(tag)::value><<<blocks, 256, 0, st>>>(scores, D.S, D.Nb, mw, k, own_sb, mask_bits, w.state, n_rows);
+      launch_kernel(select_topk_kernel<decltype(tag)::value>, blocks, 256, 0, st, scores, D.S, D.Nb, mw, k, own_sb,
+                    mask_bits, w.state, n_rows);
     };
     auto topk_rows = [&](auto tag) {
       const int g = (int)std::min<long long>((n_rows + kTopkRowThreads - 1) / kTopkRowThreads, sm_count() * 32LL);
-      select_topk_rows_kernel<decltype(tag)::value><<<g, kTopkRowThreads, 0, st>>>(scores, D.S, D.Nb, k, own_sb, mask_bits, w.state, n_rows);
+      launch_kernel(select_topk_rows_kernel<decltype(tag)::value>, g, kTopkRowThreads, 0, st, scores, D.S, D.Nb, k,
+                    own_sb, mask_bits, w.state, n_rows);
     };
     auto threshold_words = [&](auto tag) {
-      select_threshold_local_kernel<decltype(tag)::value><<<blocks, 256, 0, st>>>(scores, D.S, D.Nb, mw, D.scale, tau, own_sb,
-                                                                                 mask_bits, w.state, n_rows);
+      launch_kernel(select_threshold_local_kernel<decltype(tag)::value>, blocks, 256, 0, st, scores, D.S, D.Nb, mw,
+                    D.scale, tau, own_sb, mask_bits, w.state, n_rows);
     };
 #define VMOBA_INT(n) std::integral_constant<int, n>()
     if (by_topk) {
@@ -1170,10 +1190,10 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
       else threshold_words(VMOBA_INT(kLocalMaxWords));
     }
 #undef VMOBA_INT
-    local_cutoff_kernel<<<(D.BH + 127) / 128, 128, 0, st>>>(w.state, cutoff_per_head, D.BH);
+    launch_kernel(local_cutoff_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, cutoff_per_head, D.BH);
     VMOBA_CUDA_OK(cudaFuncSetAttribute(mark_from_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    mark_from_mask_kernel<<<sgrid, kSegThreads, smem, st>>>(mask_bits, D.S, D.Nb, D.mask_words, QSEG, nseg, w.seg_cnt,
-                                                            w.seg_total, w.tmask);
+    launch_kernel(mark_from_mask_kernel, sgrid, kSegThreads, smem, st, mask_bits, D.S, D.Nb, D.mask_words, QSEG, nseg,
+                  w.seg_cnt, w.seg_total, w.tmask);
     VMOBA_LAUNCH_OK(4);
   } else {
     // head-wide rules: weighted quantile of the pool (unit weights and a pair budget for top-k)
@@ -1183,16 +1203,16 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
       tau = count_target >= (double)P ? 1.0f : 0.5f;      // tau only tells the scan whether everything is taken
     }
     const int unit_w = by_topk ? 1 : 0;
-    init_state_kernel<<<(unsigned)(((long long)D.BH * kBins + 255) / 256), 256, 0, st>>>(w.state, D.BH, range, w.g_cnt, w.g_w,
-                                                                                        w.g_minkey, w.g_maxkey);
+    launch_kernel(init_state_kernel, (unsigned)(((long long)D.BH * kBins + 255) / 256), 256, 0, st, w.state, D.BH,
+                  range, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey);
 
     // enough CTAs per head to fill the machine, few enough that the per-CTA flush stays small
     long long per_head = (P / 4 + 255) / 256;
     int gx = (int)std::min<long long>(std::max<long long>(per_head / 8, 1), std::max(1, sm_count() * 8 / D.BH));
     dim3 grid(gx, D.BH);
     if (!range) {
-      minmax_kernel<<<grid, 256, 0, st>>>(scores, P, w.state);
-      setup_level0_kernel<<<(D.BH + 127) / 128, 128, 0, st>>>(w.state, D.BH);
+      launch_kernel(minmax_kernel, grid, 256, 0, st, scores, P, w.state);
+      launch_kernel(setup_level0_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, D.BH);
       count_launches(2);
     }
     {
@@ -1200,33 +1220,35 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
       VMOBA_CUDA_OK(cudaFuncSetAttribute(hist0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem0));
       // three 512-thread CTAs per SM hold their replicated bins side by side
       int gx0 = (int)std::min<long long>(std::max<long long>(per_head / 16, 1), std::max(1, sm_count() * 3 / D.BH));
-      hist0_kernel<<<dim3(gx0, D.BH), 512, smem0, st>>>(scores, P, w.state, sigma, unit_w, w.g_w);
+      launch_kernel(early_rows(D), hist0_kernel, dim3(gx0, D.BH), 512, smem0, st, scores, P, w.state, sigma, unit_w,
+                    w.g_w);
     }
-    scan_kernel<0><<<D.BH, 1024, 0, st>>>(w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey, k_per_head,
-                                         cutoff_per_head, w.ccap);
-    hist_kernel<1><<<grid, 256, 0, st>>>(scores, P, w.state, sigma, unit_w, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey, w.cand,
-                                        w.ccap, &w.state->cand_cnt);
-    scan_kernel<1><<<D.BH, 1024, 0, st>>>(w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey, k_per_head,
-                                         cutoff_per_head, w.ccap);
-    hist_kernel<2><<<grid, 256, 0, st>>>(scores, P, w.state, sigma, unit_w, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey, w.cand,
-                                        w.ccap, &w.state->cand_cnt);
-    scan_kernel<2><<<D.BH, 1024, 0, st>>>(w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey, k_per_head,
-                                         cutoff_per_head, w.ccap);
+    launch_kernel(scan_kernel<0>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
+                  w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
+    launch_kernel(hist_kernel<1>, grid, 256, 0, st, scores, P, w.state, sigma, unit_w, w.g_cnt, w.g_w, w.g_minkey,
+                  w.g_maxkey, w.cand, w.ccap, &w.state->cand_cnt);
+    launch_kernel(scan_kernel<1>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
+                  w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
+    launch_kernel(hist_kernel<2>, grid, 256, 0, st, scores, P, w.state, sigma, unit_w, w.g_cnt, w.g_w, w.g_minkey,
+                  w.g_maxkey, w.cand, w.ccap, &w.state->cand_cnt);
+    launch_kernel(scan_kernel<2>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
+                  w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
     VMOBA_LAUNCH_OK(7);
     VMOBA_CUDA_OK(cudaFuncSetAttribute(mark_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    mark_kernel<<<sgrid, kSegThreads, smem, st>>>(scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg, own_sb, mask_bits,
-                                                  w.seg_cnt, w.seg_total, w.tmask);
+    launch_kernel(mark_kernel, sgrid, kSegThreads, smem, st, scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg,
+                  own_sb, mask_bits, w.seg_cnt, w.seg_total, w.tmask);
     VMOBA_LAUNCH_OK(1);
   }
 
   const size_t smem_fill = ((size_t)QSEG * D.mask_words + 2 * (size_t)D.Nb * (QSEG >> 5) + 2 * (size_t)D.Nb + 1 + 2 * kStage) * 4;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fill));
   long long nkb = (long long)D.BH * D.Nb;
-  seg_prefix_kernel<<<(unsigned)((nkb + 255) / 256), 256, 0, st>>>(w.seg_cnt, w.kb_total, D.BH, D.Nb, nseg);
-  offsets_kernel<<<1, 1024, 0, st>>>(w.kb_total, kb_ptr, nkb, w.seg_total, w.seg_qoff, (long long)D.BH * nseg,
-                                     D.BH, D.Nb, k_per_head, capacity, q_ptr + (long long)D.BH * D.S, dev_status);
-  fill_kernel<<<sgrid, QSEG, smem_fill, st>>>(mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg, kb_ptr, w.seg_cnt,
-                                                w.seg_qoff, q_idx, q_ptr, q_pairs, capacity);
+  launch_kernel(seg_prefix_kernel, (unsigned)((nkb + 255) / 256), 256, 0, st, w.seg_cnt, w.kb_total, D.BH, D.Nb,
+                nseg);
+  launch_kernel(offsets_kernel, 1, 1024, 0, st, w.kb_total, kb_ptr, nkb, w.seg_total, w.seg_qoff,
+                (long long)D.BH * nseg, D.BH, D.Nb, k_per_head, capacity, q_ptr + (long long)D.BH * D.S, dev_status);
+  launch_kernel(fill_kernel, sgrid, QSEG, smem_fill, st, mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg,
+                kb_ptr, w.seg_cnt, w.seg_qoff, q_idx, q_ptr, q_pairs, capacity);
   VMOBA_LAUNCH_OK(3);
   VMOBA_GUARDS_CHECK(w.guards, dev_status, st);
   return VMOBA_OK;
