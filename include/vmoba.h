@@ -103,6 +103,12 @@ int vmoba_partition(const vmoba_shape* shape, int inverse, const void* src, void
                     const int64_t raster_strides_bsh[3], int32_t* perm_or_null,
                     int32_t* inv_perm_or_null, void* stream);
 
+/* vmoba_partition of n (1 .. 4) tensors of the same shape in one launch (q, k and v of a layer): host arrays of n
+ * pointers and n stride triples. */
+int vmoba_partition_many(const vmoba_shape* shape, int inverse, int32_t n, const void* const* src, void* const* dst,
+                         const int64_t (*raster_strides_bsh)[3], int32_t* perm_or_null, int32_t* inv_perm_or_null,
+                         void* stream);
+
 /*
  * Step 1 + Step 2a, Eq. 2 and the similarity map of Section 3.3:
  *   centroids [B, heads, N_b, head_dim] fp32 = mean of each key block,

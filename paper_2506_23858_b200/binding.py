@@ -18,7 +18,8 @@ F32, BF16 = 0, 1
 STAGE_SCORES, STAGE_SELECT, STAGE_ATTN_FWD, STAGE_ATTN_BWD, STAGE_FULL_FWD, STAGE_FULL_BWD, STAGE_SELECT_ROWNORM = range(7)
 
 EXPORTS = (
-    "vmoba_status_string", "vmoba_kernel_launches", "vmoba_workspace_bytes", "vmoba_partition", "vmoba_block_scores",
+    "vmoba_status_string", "vmoba_kernel_launches", "vmoba_workspace_bytes", "vmoba_partition",
+    "vmoba_partition_many", "vmoba_block_scores",
     "vmoba_block_scores_range", "vmoba_select", "vmoba_select_rule_apply", "vmoba_select_ranged", "vmoba_select_static", "vmoba_select_static_scratch_bytes", "vmoba_attn_fwd",
     "vmoba_attn_fwd_raster", "vmoba_attn_bwd", "vmoba_attn_bwd_raster", "vmoba_full_attn",
     "vmoba_debug_wait_profile", "vmoba_debug_wait_timeout",
@@ -96,6 +97,8 @@ def lib():
     L.vmoba_workspace_bytes.argtypes = [sp, ctypes.c_int, i64]
     L.vmoba_partition.restype = ctypes.c_int
     L.vmoba_partition.argtypes = [sp, ctypes.c_int, vp, vp, ctypes.POINTER(i64), vp, vp, vp]
+    L.vmoba_partition_many.restype = ctypes.c_int
+    L.vmoba_partition_many.argtypes = [sp, ctypes.c_int, ctypes.c_int32, vp, vp, vp, vp, vp, vp]
     L.vmoba_block_scores.restype = ctypes.c_int
     L.vmoba_block_scores.argtypes = [sp, vp, vp, vp, vp, vp, vp, sz, vp]
     L.vmoba_block_scores_range.restype = ctypes.c_int
@@ -170,6 +173,16 @@ def vmoba_partition(shape, inverse, src, dst, raster_strides_bsh, perm=None, inv
     strides = (ctypes.c_int64 * 3)(*[int(x) for x in raster_strides_bsh])
     _check(lib().vmoba_partition(ctypes.byref(shape), int(inverse), _ptr(src), _ptr(dst), strides, _ptr(perm),
                                  _ptr(inv_perm), _stream(stream)), "vmoba_partition")
+
+
+def vmoba_partition_many(shape, inverse, srcs, dsts, raster_strides_bsh, perm=None, inv_perm=None, stream=None):
+    """vmoba_partition of up to four tensors in one launch; raster_strides_bsh: one (batch, token, head) triple each."""
+    n = len(srcs)
+    strides = (ctypes.c_int64 * (3 * n))(*[x for t in raster_strides_bsh for x in t])
+    src = (ctypes.c_void_p * n)(*[t.data_ptr() for t in srcs])
+    dst = (ctypes.c_void_p * n)(*[t.data_ptr() for t in dsts])
+    _check(lib().vmoba_partition_many(ctypes.byref(shape), inverse, n, src, dst, strides, _ptr(perm), _ptr(inv_perm),
+                                      _stream(stream)), "vmoba_partition_many")
 
 
 def vmoba_block_scores(shape, q_bm, k_bm, centroids, scores, dev_status, ws, stream=None):

@@ -73,6 +73,16 @@ class VmobaLayer:
         src, dst = (bm, raster) if inverse else (raster, bm)
         vb.vmoba_partition(self.shape, int(inverse), src, dst, self.raster_strides(raster), perm, inv_perm)
 
+    def partition_many(self, rasters, bms, perm=None):
+        """Up to four tensors of the layer's shape into block-major order, and the permutation table, in one launch."""
+        vb.vmoba_partition_many(self.shape, 0, rasters, bms, [self.raster_strides(x) for x in rasters], perm=perm)
+
+    def partitions(self, raster) -> bool:
+        """Whether partition() takes this tensor as it lies: the layer's type, 16-byte rows on 16-byte boundaries."""
+        e = 16 // raster.element_size()
+        return (raster.dtype == self.q_bm.dtype and raster.stride(3) == 1 and raster.data_ptr() % 16 == 0
+                and all(x % e == 0 for x in raster.stride()[:3]))
+
     def block_scores(self, with_range=True):
         """Centroids and scores; with_range: the scores kernel also takes each head's smallest and largest score,
         which lets select() skip its own pass for them (valid until self.scores is overwritten by other means)."""
@@ -156,9 +166,7 @@ class VmobaLayer:
         fold_o: let the forward kernels write o in raster order themselves (bf16, head_dim 128) instead of an inverse
         partition pass; off by default (measured on B200: the scattered 256-byte row writes cost the attention kernel
         more than the pass they save, at 12 heads as at 40).  o_out must then stay alive and unchanged until backward()."""
-        self.partition(q, self.q_bm, perm=self.perm)
-        self.partition(k, self.k_bm)
-        self.partition(v, self.v_bm)
+        self.partition_many((q, k, v), (self.q_bm, self.k_bm, self.v_bm), perm=self.perm)
         self.block_scores()
         self.select(tau)
         if fold_o:
@@ -223,11 +231,16 @@ class SteppedAttention:
     def forward(self, step: int, q, k, v, o_out) -> str:
         """Runs step `step`; returns which path ran ("dense" or "sparse")."""
         if self.schedule[step]:
-            # the dense kernels take [B, heads, S, d] in any one token order
-            qd, kd, vd = (x.permute(0, 2, 1, 3).contiguous() for x in (q, k, v))
-            od = torch.empty_like(qd)
-            vb.vmoba_full_attn(self.layer.shape, qd, kd, vd, od, self._lse, dev_status=self.layer.dev_status)
-            o_out.copy_(od.permute(0, 2, 1, 3))
+            # the dense kernels take [B, heads, S, d] in any one token order: block-major will do
+            L = self.layer
+            q, k, v = (x if L.partitions(x) else x.contiguous() for x in (q, k, v))
+            qd, kd, vd, od = (torch.empty_like(L.q_bm) for _ in range(4))
+            L.partition_many((q, k, v), (qd, kd, vd))
+            vb.vmoba_full_attn(L.shape, qd, kd, vd, od, self._lse, dev_status=L.dev_status)
+            o = o_out if L.partitions(o_out) else torch.empty(o_out.shape, dtype=L.q_bm.dtype, device=L.device)
+            L.partition(o, od, inverse=True)
+            if o is not o_out:
+                o_out.copy_(o)
             return "dense"
         self.layer.forward(q, k, v, self.tau, o_out)
         return "sparse"
