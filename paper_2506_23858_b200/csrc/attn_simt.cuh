@@ -303,6 +303,8 @@ merge_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pairs, lon
 // fetch a row, and kBatch rows of each are in flight.  Nine pairs per query (907,200 queries, 2.3 GB) 536 us, 32 pairs
 // (393,120 queries) 826, two to six pairs 62 to 207: with a warp per query at a time and eight bytes per lane 714, 962 and
 // 72 to 255; 64 registers (four CTAs per SM) beat 80 by a tenth, kBatch = 4 loses a tenth.
+//
+// span (a power of two up to 32): queries a warp takes at a time, see merge_batched().
 constexpr int kInLane = 8;
 constexpr int kBatch = 8;
 __device__ __forceinline__ void add_half8(float (&acc)[8], const uint4& v, float w) {
@@ -318,7 +320,7 @@ static __global__ void __launch_bounds__(256, 4)
 merge_batched_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pairs, long long n_queries,
                      const __half* __restrict__ part_o, const float* __restrict__ part_lse,
                      const float* __restrict__ part_scale, long long capacity, __nv_bfloat16* __restrict__ o,
-                     __nv_bfloat16* __restrict__ o_resid, float* __restrict__ lse, const RowMap o_map) {
+                     __nv_bfloat16* __restrict__ o_resid, float* __restrict__ lse, const RowMap o_map, int span) {
   if (!grid_begin()) return;
   constexpr int DH = 128;
   constexpr uint32_t FULL = 0xffffffffu;
@@ -327,10 +329,10 @@ merge_batched_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pa
   const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
   const int last = (int)(capacity - 1);
   const uint4* rows = reinterpret_cast<const uint4*>(part_o) + hl;
-  for (long long g0 = warp * 32; g0 < n_queries; g0 += nwarps * 32) {
+  for (long long g0 = warp * span; g0 < n_queries; g0 += nwarps * span) {
     const long long g = g0 + lane;
-    int lo = 0, n = 1, n_raw = 1;        // lanes beyond the last query behave like a directly written row
-    if (g < n_queries) {
+    int lo = 0, n = 1, n_raw = 1;        // lanes beyond the span or the last query behave like a directly written row
+    if (lane < span && g < n_queries) {
       lo = q_ptr[g];
       const int hi_raw = q_ptr[g + 1];
       n_raw = hi_raw - lo;
@@ -458,6 +460,19 @@ merge_batched_kernel(const int* __restrict__ q_ptr, const int* __restrict__ q_pa
       write_row(b, acc, mx + logf(tot));
     }
   }
+}
+
+// Fewer than 32 queries at a time where 32 would leave the SMs short of the 32 warps each holds: the walk through a warp's
+// queries is a chain of loads, two queries after two (22,464 queries of 3 to 40 pairs: 23 us with 32).
+static void merge_batched(const Dims& D, const int* q_ptr, const int* q_pairs, const __half* part_o, const float* part_lse,
+                          const float* part_scale, long long cap, void* o, void* o_resid, float* lse, const RowMap& o_map,
+                          cudaStream_t st) {
+  const long long nq = (long long)D.BH * D.S;
+  int span = 32;
+  while (span > 2 && nq < (long long)sm_count() * 32 * span) span /= 2;
+  launch_kernel(early_rows(D), merge_batched_kernel, (int)std::min<long long>((nq + 8 * span - 1) / (8 * span), sm_count() * 8),
+                256, 0, st, q_ptr, q_pairs, nq, part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o,
+                (__nv_bfloat16*)o_resid, lse, o_map, span);
 }
 
 // ------------------------------------------------------------------------------ backward

@@ -633,10 +633,7 @@ int tc_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, co
   } else {
     if (int rc = launch_wide<false, false>(D, q, k, v, p, grid_items(cap / IM + n_kb), st)) return rc;
   }
-  const long long nq = (long long)D.BH * D.S;
-  launch_kernel(early_rows(D), simt::merge_batched_kernel, (int)std::min<long long>((nq + 255) / 256, sm_count() * 8),
-                256, 0, st, q_ptr, q_pairs, nq, p.part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o,
-                (__nv_bfloat16*)o_resid, lse, o_map);
+  simt::merge_batched(D, q_ptr, q_pairs, p.part_o, part_lse, part_scale, cap, o, o_resid, lse, o_map, st);
   VMOBA_LAUNCH_OK(3);
   return VMOBA_OK;
 }

@@ -577,10 +577,7 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
   auto kernel = o_map.perm ? attn_fwd_narrow_kernel<true> : attn_fwd_narrow_kernel<false>;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
   launch_kernel(kernel, (int)items, THREADS, SMEM_BYTES, st, tmK, tmV, p);
-  const long long nq = (long long)D.BH * D.S;
-  launch_kernel(early_rows(D), simt::merge_batched_kernel, (int)std::min<long long>((nq + 255) / 256, sm_count() * 8),
-                256, 0, st, q_ptr, q_pairs, nq, p.part_o, part_lse, part_scale, cap, (__nv_bfloat16*)o,
-                (__nv_bfloat16*)o_resid, lse, o_map);
+  simt::merge_batched(D, q_ptr, q_pairs, p.part_o, part_lse, part_scale, cap, o, o_resid, lse, o_map, st);
   VMOBA_LAUNCH_OK(4);
   return VMOBA_OK;
 }
