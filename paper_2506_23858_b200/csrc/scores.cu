@@ -20,34 +20,65 @@ size_t scores_ws_bytes(const Dims& D) {
   return (D.dtype == VMOBA_BF16 && D.d == 128) ? scores_tc_ws_bytes(D) : 256;
 }
 
-// One CTA per (batch, head, block): 256 threads = (256 / V) row lanes x V float4-column lanes.
-template <typename T, int DH>
-__global__ void __launch_bounds__(256)
-centroid_kernel(const T* __restrict__ k_bm, float* __restrict__ cent, int sb) {
+// Eq. 2.  A CTA sums DH / SPLIT columns of one (batch, head, block) with 1024 / DH row lanes, each over every (1024 / DH)-th
+// row in order, then adds the row lanes' sums in order: the result does not depend on SPLIT.  Bound by HBM bandwidth, with
+// few blocks by the latency of a thread's chain of loads, hence the many in flight.
+// The blocks are taken from the last position of every head to the first: the partition of k, in token order over all heads,
+// ends there, and what it wrote last is still in L2.
+template <typename T, int DH, int SPLIT>
+__global__ void __launch_bounds__((1024 / DH) * (DH * (int)sizeof(T) / 16 / SPLIT))
+centroid_kernel(const T* __restrict__ k_bm, float* __restrict__ cent, int sb, int BH, int Nb) {
   if (!grid_begin()) return;
-  constexpr int V = DH / 4;            // float4 columns per row
-  constexpr int RL = 256 / V;          // row lanes
-  __shared__ float4 red[RL][V];
-  const long long blk = blockIdx.x;    // (b*heads + head) * Nb + j : blocks are contiguous in block-major order
-  const T* base = k_bm + blk * (long long)sb * DH;
+  constexpr int W = 16 / sizeof(T);          // columns per thread
+  constexpr int V = DH / W / SPLIT;          // threads per row
+  constexpr int RL = 1024 / DH;              // row lanes
+  constexpr int U = SPLIT > 1 ? 32 : 8;      // 16-byte loads of a thread in flight
+  __shared__ float red[RL][V * W];
+  const unsigned i = gridDim.x - 1 - blockIdx.x;
+  const int part = i % SPLIT, j = (int)(i / SPLIT / BH), bh = (int)(i / SPLIT - (unsigned)j * BH);
+  const long long blk = (long long)bh * Nb + j;
   const int col = threadIdx.x % V, rl = threadIdx.x / V;
-  float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int r = rl; r < sb; r += RL) {
-    float4 x = load4(base + (long long)r * DH + col * 4);
-    acc.x += x.x; acc.y += x.y; acc.z += x.z; acc.w += x.w;
-  }
-  red[rl][col] = acc;
-  __syncthreads();
-  if (rl == 0) {
-    float4 s = red[0][col];
-    for (int i = 1; i < RL; ++i) {
-      float4 x = red[i][col];
-      s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+  const uint4* base = reinterpret_cast<const uint4*>(k_bm + blk * (long long)sb * DH) + part * V + col;
+  float acc[W];
+#pragma unroll
+  for (int c = 0; c < W; ++c) acc[c] = 0.f;
+  for (int r0 = rl; r0 < sb; r0 += RL * U) {
+    uint4 x[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (r0 + u * RL < sb) x[u] = __ldg(base + (long long)(r0 + u * RL) * (DH / W));
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (r0 + u * RL >= sb) break;
+      const uint32_t w[4] = {x[u].x, x[u].y, x[u].z, x[u].w};
+#pragma unroll
+      for (int c = 0; c < W; ++c) {
+        if constexpr (W == 4) acc[c] += __uint_as_float(w[c]);
+        else acc[c] += __uint_as_float(c & 1 ? w[c >> 1] & 0xffff0000u : w[c >> 1] << 16);
+      }
     }
-    float inv = 1.0f / (float)sb;
-    s.x *= inv; s.y *= inv; s.z *= inv; s.w *= inv;
-    store4(cent + blk * DH + col * 4, s);
   }
+#pragma unroll
+  for (int c = 0; c < W; ++c) red[rl][col * W + c] = acc[c];
+  __syncthreads();
+  const float inv = 1.0f / (float)sb;
+  for (int c = threadIdx.x; c < V * W; c += RL * V) {
+    float s = red[0][c];
+    for (int r = 1; r < RL; ++r) s += red[r][c];
+    cent[blk * DH + part * V * W + c] = s * inv;
+  }
+}
+
+template <typename T, int DH>
+static void run_centroids(const Dims& D, const T* k, float* cent, cudaStream_t st) {
+  constexpr int THREADS = (1024 / DH) * (DH * (int)sizeof(T) / 16);
+  const long long n = (long long)D.BH * D.Nb;
+  // Four CTAs per block where one would not give every SM four.  12 heads: 24 blocks of 1,400 keys 41 us with one, 24 with
+  // four; 16 blocks of 840 keys 20 and 8; 140 blocks of 234 keys 15 with one.
+  if (n < sm_count() * 4ll)
+    launch_kernel(centroid_kernel<T, DH, 4>, (unsigned)(4 * n), THREADS / 4, 0, st, k, cent, D.sb, D.BH, D.Nb);
+  else
+    launch_kernel(centroid_kernel<T, DH, 1>, (unsigned)n, THREADS, 0, st, k, cent, D.sb, D.BH, D.Nb);
 }
 
 // fp32 tile GEMM: a CTA computes 64 queries x 64 blocks with the whole head_dim in shared
@@ -146,7 +177,7 @@ range_kernel(const float* __restrict__ scores, long long P, float* __restrict__ 
 template <typename T, int DH>
 static int run_scores(const Dims& D, const void* q, const void* k, float* cent, float* scores, float* range, void* ws,
                       int32_t* status, cudaStream_t st) {
-  launch_kernel(centroid_kernel<T, DH>, D.BH * D.Nb, 256, 0, st, static_cast<const T*>(k), cent, D.sb);
+  run_centroids<T, DH>(D, static_cast<const T*>(k), cent, st);
   VMOBA_LAUNCH_OK(1);
   if (D.dtype == VMOBA_BF16 && DH == 128) return scores_tc(D, q, cent, scores, range, ws, status, st);
   size_t smem = 2 * DH * (64 + 4) * sizeof(float);

@@ -68,8 +68,9 @@ __device__ __forceinline__ int bin_at(const HeadState& hs, int L, float s) {
   return b;
 }
 
-// Streams the P scores of one head through f(value); blockIdx.x strides over chunks.
-template <typename F>
+// Streams the P scores of one head through f(value); blockIdx.x strides over chunks.  DOWN: from the end of the head to
+// its start, which finds in L2 what the pass before read or wrote last.
+template <bool DOWN, typename F>
 __device__ __forceinline__ void for_each_score(const float* __restrict__ base, long long P, F f) {
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const long long nth = (long long)gridDim.x * blockDim.x;
@@ -80,12 +81,12 @@ __device__ __forceinline__ void for_each_score(const float* __restrict__ base, l
     for (; i + 3 * nth < P4; i += 4 * nth) {     // four independent 16-byte loads in flight
       float4 x[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] = __ldg(b4 + i + j * nth);
+      for (int j = 0; j < 4; ++j) x[j] = __ldg(b4 + (DOWN ? P4 - 1 - (i + j * nth) : i + j * nth));
 #pragma unroll
       for (int j = 0; j < 4; ++j) { f(x[j].x); f(x[j].y); f(x[j].z); f(x[j].w); }
     }
     for (; i < P4; i += nth) {
-      float4 x = __ldg(b4 + i);
+      float4 x = __ldg(b4 + (DOWN ? P4 - 1 - i : i));
       f(x.x); f(x.y); f(x.z); f(x.w);
     }
     for (long long i = (P4 << 2) + tid; i < P; i += nth) f(__ldg(base + i));
@@ -99,7 +100,7 @@ minmax_kernel(const float* __restrict__ scores, long long P, HeadState* __restri
   if (!grid_begin()) return;
   const int bh = blockIdx.y;
   uint32_t kmin = 0xffffffffu, kmax = 0u;
-  for_each_score(scores + (long long)bh * P, P, [&](float s) {
+  for_each_score<false>(scores + (long long)bh * P, P, [&](float s) {
     uint32_t k = float_key(s);
     kmin = min(kmin, k);
     kmax = max(kmax, k);
@@ -170,7 +171,7 @@ hist_kernel(const float* __restrict__ scores, long long P, const HeadState* __re
   const bool from_list = L == 2 && hs.cand_ok;
   const float* src = from_list ? list : scores + (long long)bh * P;
   const long long n_src = from_list ? (long long)hs.cand_cnt : P;
-  for_each_score(src, n_src, [&](float s) {
+  for_each_score<L == 1>(src, n_src, [&](float s) {
     if (L >= 1 && bin_at(hs, 0, s) != hs.bin[0]) return;
     if (L == 1 && list) {
       const unsigned int pos = atomicAdd(cand_cnt + bh * (sizeof(HeadState) / sizeof(unsigned int)), 1u);
@@ -211,7 +212,7 @@ hist0_kernel(const float* __restrict__ scores, long long P, const HeadState* __r
   __syncthreads();
   const float smax = key_float(hs.max_key);
   const int rep = threadIdx.x & (kRep - 1);
-  for_each_score(scores + (long long)bh * P, P, [&](float s) {
+  for_each_score<false>(scores + (long long)bh * P, P, [&](float s) {
     atomicAdd(&s_wr[bin_at(hs, 0, s) * kRep + rep], unit_w ? 1.0f : pair_weight(sigma, s, smax));
   });
   __syncthreads();
@@ -370,7 +371,9 @@ mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, 
   int* s_cnt = reinterpret_cast<int*>(sm + QSEG * mw);  // [Nb]
   uint32_t* s_tm = sm + QSEG * mw + Nb;               // [TW][Nb]: the same bits, a word per 32 queries and key block
   __shared__ int s_total;
-  const int seg = blockIdx.x, bh = blockIdx.y;
+  // segments in token order over all heads: the histogram pass before ended at every head's start, which is still in L2
+  const unsigned id = blockIdx.y * gridDim.x + blockIdx.x;
+  const int seg = (int)(id / gridDim.y), bh = (int)(id - (unsigned)seg * gridDim.y);
   const int q0 = seg * QSEG;
   const int nq = min(QSEG, S - q0);
   const uint32_t cutoff = st[bh].cutoff_key;

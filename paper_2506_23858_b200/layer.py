@@ -166,7 +166,8 @@ class VmobaLayer:
         fold_o: let the forward kernels write o in raster order themselves (bf16, head_dim 128) instead of an inverse
         partition pass; off by default (measured on B200: the scattered 256-byte row writes cost the attention kernel
         more than the pass they save, at 12 heads as at 40).  o_out must then stay alive and unchanged until backward()."""
-        self.partition_many((q, k, v), (self.q_bm, self.k_bm, self.v_bm), perm=self.perm)
+        # k last: the centroids, computed next, find the end of it in L2
+        self.partition_many((v, q, k), (self.v_bm, self.q_bm, self.k_bm), perm=self.perm)
         self.block_scores()
         self.select(tau)
         if fold_o:
