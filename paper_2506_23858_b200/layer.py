@@ -73,9 +73,11 @@ class VmobaLayer:
         src, dst = (bm, raster) if inverse else (raster, bm)
         vb.vmoba_partition(self.shape, int(inverse), src, dst, self.raster_strides(raster), perm, inv_perm)
 
-    def partition_many(self, rasters, bms, perm=None):
-        """Up to four tensors of the layer's shape into block-major order, and the permutation table, in one launch."""
-        vb.vmoba_partition_many(self.shape, 0, rasters, bms, [self.raster_strides(x) for x in rasters], perm=perm)
+    def partition_many(self, rasters, bms, inverse=False, perm=None):
+        """Up to four tensors of the layer's shape into block-major order (inverse: back), and the permutation table, in
+        one launch."""
+        srcs, dsts = (bms, rasters) if inverse else (rasters, bms)
+        vb.vmoba_partition_many(self.shape, int(inverse), srcs, dsts, [self.raster_strides(x) for x in rasters], perm=perm)
 
     def partitions(self, raster) -> bool:
         """Whether partition() takes this tensor as it lies: the layer's type, 16-byte rows on 16-byte boundaries."""
@@ -194,9 +196,7 @@ class VmobaLayer:
         if self.o_raster is not None:      # the block-major backward reads o_bm, which the raster forward did not write
             self.partition(self.o_raster, self.o_bm)
         self.attn_bwd()
-        self.partition(dq_out, self.dq_bm, inverse=True)
-        self.partition(dk_out, self.dk_bm, inverse=True)
-        self.partition(dv_out, self.dv_bm, inverse=True)
+        self.partition_many((dq_out, dk_out, dv_out), (self.dq_bm, self.dk_bm, self.dv_bm), inverse=True)
 
     def check_status(self):
         code = int(self.dev_status.item())
