@@ -26,6 +26,7 @@ namespace vmoba {
 constexpr int kBins = 2048;
 constexpr int kBins0 = 512;    // level 0 uses fewer bins, each replicated once per lane
 constexpr int kSegThreads = 512;
+constexpr int kCandStage = 1024;      // pairs of the crossing bin that a CTA of the level-1 pass gathers
 
 struct HeadState {
   uint32_t min_key, max_key;   // order-preserving keys of the head's extreme scores
@@ -155,6 +156,8 @@ hist_kernel(const float* __restrict__ scores, long long P, const HeadState* __re
   __shared__ float s_w[kBins];
   __shared__ uint32_t s_min[kBins];
   __shared__ uint32_t s_max[L == 1 ? kBins : 1];
+  __shared__ float s_cand[L == 1 ? kCandStage : 1];
+  __shared__ unsigned int s_cand_n, s_cand_at;
   const int bh = blockIdx.y;
   const HeadState hs = st[bh];
   if (L == 2 && hs.resolved) return;     // level 1 already pinned the cutoff: nothing to refine
@@ -163,10 +166,13 @@ hist_kernel(const float* __restrict__ scores, long long P, const HeadState* __re
     s_min[i] = 0xffffffffu;
     if (L == 1) s_max[i] = 0u;
   }
+  if (threadIdx.x == 0) s_cand_n = 0u;
   __syncthreads();
   const float smax = key_float(hs.max_key);
   // level 1 copies the pairs of the level-0 crossing bin (one bin of 512: few) to the head's list; level 2 reads
-  // the list instead of the matrix if all of them found room
+  // the list instead of the matrix if all of them found room.  They are gathered in shared memory and get their places
+  // with one atomic per CTA: with one each, a warp waits for the answer at every pair (white inputs, 55 million pairs:
+  // 142 us against 68).
   float* list = cand ? cand + (long long)bh * ccap : nullptr;
   const bool from_list = L == 2 && hs.cand_ok;
   const float* src = from_list ? list : scores + (long long)bh * P;
@@ -174,8 +180,12 @@ hist_kernel(const float* __restrict__ scores, long long P, const HeadState* __re
   for_each_score<L == 1>(src, n_src, [&](float s) {
     if (L >= 1 && bin_at(hs, 0, s) != hs.bin[0]) return;
     if (L == 1 && list) {
-      const unsigned int pos = atomicAdd(cand_cnt + bh * (sizeof(HeadState) / sizeof(unsigned int)), 1u);
-      if (pos < ccap) list[pos] = s;
+      unsigned int pos = atomicAdd(&s_cand_n, 1u);
+      if (pos < kCandStage) s_cand[pos] = s;
+      else {
+        pos = atomicAdd(cand_cnt + bh * (sizeof(HeadState) / sizeof(unsigned int)), 1u);
+        if (pos < ccap) list[pos] = s;
+      }
     }
     if (L >= 2 && bin_at(hs, 1, s) != hs.bin[1]) return;
     int b = bin_at(hs, L, s);
@@ -185,6 +195,14 @@ hist_kernel(const float* __restrict__ scores, long long P, const HeadState* __re
     if (L == 1) atomicMax(&s_max[b], float_key(s));
   });
   __syncthreads();
+  if (L == 1 && list) {
+    const unsigned int n = min(s_cand_n, (unsigned int)kCandStage);
+    if (n && threadIdx.x == 0)
+      s_cand_at = atomicAdd(cand_cnt + bh * (sizeof(HeadState) / sizeof(unsigned int)), n);
+    __syncthreads();
+    for (unsigned int k = threadIdx.x; k < n; k += blockDim.x)
+      if (s_cand_at + k < ccap) list[s_cand_at + k] = s_cand[k];
+  }
   for (int i = threadIdx.x; i < kBins; i += blockDim.x) {
     unsigned int c = s_cnt[i];
     if (c) {
@@ -442,24 +460,38 @@ mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, 
 }
 
 // offsets A: per (head, block) turn the per-segment counts into exclusive prefixes along the
-// segments and record the block's total.
-__global__ void seg_prefix_kernel(int* __restrict__ seg_cnt, int* __restrict__ kb_total, int BH, int Nb, int nseg) {
+// segments and record the block's total.  A CTA takes 32 blocks of a head (lane: block), a warp a run of about eight of their
+// segments.  Bound by the latency of its loads: 1,680 blocks x 64 segments 3.3 us, 3,360 x 169 3.5; with a thread per block,
+// eight segments after eight, 7.3 and 12.2.
+__global__ void __launch_bounds__(1024)
+seg_prefix_kernel(int* __restrict__ seg_cnt, int* __restrict__ kb_total, int Nb, int nseg) {
   if (!grid_begin()) return;
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long long)BH * Nb) return;
-  int bh = (int)(i / Nb), j = (int)(i % Nb);
+  __shared__ int s_sum[32][32];              // [run][block]
+  const int groups = (Nb + 31) / 32, bh = blockIdx.x / groups;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_runs = blockDim.x >> 5;
+  const int j = (blockIdx.x - bh * groups) * 32 + lane, per = (nseg + n_runs - 1) / n_runs;
+  const int s0 = min(nseg, warp * per), s1 = j < Nb ? min(nseg, s0 + per) : s0;
+  int* col = seg_cnt + (long long)bh * nseg * Nb + j;
   int run = 0;
+  if (n_runs > 1) {
+    int sum = 0;
+#pragma unroll 8
+    for (int s = s0; s < s1; ++s) sum += col[(long long)s * Nb];
+    s_sum[warp][lane] = sum;
+    __syncthreads();
+#pragma unroll 8
+    for (int w = 0; w < warp; ++w) run += s_sum[w][lane];
+  }
   // eight segments per trip: their loads go out together (the stores of a trip would otherwise order them)
-  for (int s0 = 0; s0 < nseg; s0 += 8) {
-    int* p = seg_cnt + ((long long)bh * nseg + s0) * Nb + j;
+  for (int s = s0; s < s1; s += 8) {
     int c[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) c[k] = s0 + k < nseg ? p[(long long)k * Nb] : 0;
+    for (int k = 0; k < 8; ++k) c[k] = s + k < s1 ? col[(long long)(s + k) * Nb] : 0;
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-      if (s0 + k < nseg) { p[(long long)k * Nb] = run; run += c[k]; }
+      if (s + k < s1) { col[(long long)(s + k) * Nb] = run; run += c[k]; }
   }
-  kb_total[i] = run;
+  if (warp == n_runs - 1 && j < Nb) kb_total[(long long)bh * Nb + j] = run;
 }
 
 __global__ void __launch_bounds__(1024)
@@ -472,10 +504,13 @@ offsets_kernel(const int* __restrict__ kb_total, int* __restrict__ kb_ptr, long 
   block_exclusive_scan([&](long long i) { return kb_total[i]; }, kb_ptr, n_kb, &total_a);
   block_exclusive_scan([&](long long i) { return seg_total[i]; }, seg_qoff, n_seg, &total_b);
   __syncthreads();
-  for (int bh = threadIdx.x; bh < BH; bh += blockDim.x) {
+  // a warp per head
+  for (int bh = threadIdx.x >> 5; bh < BH; bh += blockDim.x >> 5) {
     long long a = 0;
-    for (int j = 0; j < Nb; ++j) a += kb_total[(long long)bh * Nb + j];
-    k_per_head[bh] = a;
+    for (int j = threadIdx.x & 31; j < Nb; j += 32) a += kb_total[(long long)bh * Nb + j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if ((threadIdx.x & 31) == 0) k_per_head[bh] = a;
   }
   if (threadIdx.x == 0) {
     *q_ptr_last = (int)min(total_a, (long long)INT32_MAX);
@@ -1246,8 +1281,8 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
   const size_t smem_fill = ((size_t)QSEG * D.mask_words + 2 * (size_t)D.Nb * (QSEG >> 5) + 2 * (size_t)D.Nb + 1 + 2 * kStage) * 4;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fill));
   long long nkb = (long long)D.BH * D.Nb;
-  launch_kernel(seg_prefix_kernel, (unsigned)((nkb + 255) / 256), 256, 0, st, w.seg_cnt, w.kb_total, D.BH, D.Nb,
-                nseg);
+  launch_kernel(seg_prefix_kernel, (unsigned)(D.BH * ((D.Nb + 31) / 32)), 32 * std::min(32, (nseg + 7) / 8), 0, st,
+                w.seg_cnt, w.kb_total, D.Nb, nseg);
   launch_kernel(offsets_kernel, 1, 1024, 0, st, w.kb_total, kb_ptr, nkb, w.seg_total, w.seg_qoff,
                 (long long)D.BH * nseg, D.BH, D.Nb, k_per_head, capacity, q_ptr + (long long)D.BH * D.S, dev_status);
   launch_kernel(fill_kernel, sgrid, QSEG, smem_fill, st, mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg,
