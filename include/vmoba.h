@@ -298,6 +298,17 @@ int vmoba_attn_bwd_raster(const vmoba_shape* shape, const void* q_bm, const void
                           size_t ws_bytes, void* stream);
 
 /*
+ * vmoba_attn_bwd_raster that also leaves d_o (raster order, strides required) in do_bm [B, heads, S, head_dim],
+ * block-major, on the way: the attention kernel reads that copy, and dO needs no partition pass of its own.
+ */
+int vmoba_attn_bwd_raster_do(const vmoba_shape* shape, const void* q_bm, const void* k_bm, const void* v_bm,
+                             const void* o, const int64_t o_strides_bsh[3], const void* o_resid_or_null, const float* lse,
+                             const void* d_o, const int64_t do_strides_bsh[3], void* do_bm, const int32_t* kb_ptr,
+                             const int32_t* q_idx, const int32_t* q_ptr, int64_t capacity, void* dq, void* dk, void* dv,
+                             const int64_t grad_strides_bsh[3], const int32_t* perm, int32_t* dev_status, void* ws,
+                             size_t ws_bytes, void* stream);
+
+/*
  * Dense softmax attention over all S keys: the tau = 1 limit of the layer and the speed-up
  * denominator (the "Full Attention" baseline of Section 4.1).  Tensors are [B, heads, S, head_dim]
  * in any one token order.  If do_or_null is given, also computes dq, dk, dv.

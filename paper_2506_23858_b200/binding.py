@@ -21,7 +21,8 @@ EXPORTS = (
     "vmoba_status_string", "vmoba_kernel_launches", "vmoba_workspace_bytes", "vmoba_partition",
     "vmoba_partition_many", "vmoba_block_scores",
     "vmoba_block_scores_range", "vmoba_select", "vmoba_select_rule_apply", "vmoba_select_ranged", "vmoba_select_static", "vmoba_select_static_scratch_bytes", "vmoba_attn_fwd",
-    "vmoba_attn_fwd_raster", "vmoba_attn_bwd", "vmoba_attn_bwd_raster", "vmoba_full_attn",
+    "vmoba_attn_fwd_raster", "vmoba_attn_bwd", "vmoba_attn_bwd_raster",
+    "vmoba_attn_bwd_raster_do", "vmoba_full_attn",
     "vmoba_debug_wait_profile", "vmoba_debug_wait_timeout",
 )
 
@@ -123,6 +124,9 @@ def lib():
     p64 = ctypes.POINTER(ctypes.c_int64)
     L.vmoba_attn_bwd_raster.argtypes = [sp, vp, vp, vp, vp, p64, vp, vp, vp, p64, vp, vp, vp, i64,
                                         vp, vp, vp, p64, vp, vp, vp, sz, vp]
+    L.vmoba_attn_bwd_raster_do.restype = ctypes.c_int
+    L.vmoba_attn_bwd_raster_do.argtypes = [sp, vp, vp, vp, vp, p64, vp, vp, vp, p64, vp, vp, vp, vp, i64,
+                                           vp, vp, vp, p64, vp, vp, vp, sz, vp]
     L.vmoba_attn_fwd_raster.restype = ctypes.c_int
     L.vmoba_attn_fwd_raster.argtypes = [sp, vp, vp, vp, vp, vp, vp, vp, i64, vp, p64, vp, vp, vp, vp, vp, sz, vp]
     L.vmoba_debug_wait_timeout.restype = ctypes.c_int
@@ -271,11 +275,19 @@ def vmoba_attn_fwd_raster(shape, q_bm, k_bm, v_bm, kb_ptr, q_idx, q_ptr, q_pairs
 
 
 def vmoba_attn_bwd_raster(shape, q_bm, k_bm, v_bm, o, o_strides_bsh, o_resid, lse, d_o, do_strides_bsh, kb_ptr, q_idx,
-                          q_ptr, capacity, dq, dk, dv, grad_strides_bsh, perm, dev_status, ws, stream=None):
+                          q_ptr, capacity, dq, dk, dv, grad_strides_bsh, perm, dev_status, ws, stream=None, do_bm=None):
+    """do_bm: with a raster-order d_o, a block-major tensor that takes a copy of it on the way."""
     p, n = _ws_args(ws)
     dos = None if do_strides_bsh is None else (ctypes.c_int64 * 3)(*[int(x) for x in do_strides_bsh])
     os_ = None if o_strides_bsh is None else (ctypes.c_int64 * 3)(*[int(x) for x in o_strides_bsh])
     gs = (ctypes.c_int64 * 3)(*[int(x) for x in grad_strides_bsh])
+    if do_bm is not None:
+        _check(lib().vmoba_attn_bwd_raster_do(ctypes.byref(shape), _ptr(q_bm), _ptr(k_bm), _ptr(v_bm), _ptr(o), os_,
+                                              _ptr(o_resid), _ptr(lse), _ptr(d_o), dos, _ptr(do_bm), _ptr(kb_ptr),
+                                              _ptr(q_idx), _ptr(q_ptr), int(capacity), _ptr(dq), _ptr(dk), _ptr(dv), gs,
+                                              _ptr(perm), _ptr(dev_status), p, n, _stream(stream)),
+               "vmoba_attn_bwd_raster_do")
+        return
     _check(lib().vmoba_attn_bwd_raster(ctypes.byref(shape), _ptr(q_bm), _ptr(k_bm), _ptr(v_bm), _ptr(o), os_,
                                        _ptr(o_resid), _ptr(lse), _ptr(d_o), dos, _ptr(kb_ptr), _ptr(q_idx),
                                        _ptr(q_ptr), int(capacity), _ptr(dq), _ptr(dk), _ptr(dv), gs, _ptr(perm),

@@ -88,7 +88,7 @@ template <typename T, int DH>
 static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const void* v, const void* o,
                            const void* o_resid, const float* lse, const void* d_o, const int* kb_ptr, const int* q_idx,
                            const int* q_ptr, long long cap, void* dq, void* dk, void* dv, int32_t* status, void* ws,
-                           cudaStream_t st, const RowMap& out_map, const RowMap& do_map, const RowMap& o_map) {
+                           cudaStream_t st, const RowMap& out_map, const RowMap& do_map, const RowMap& o_map, void* do_bm) {
   // raster-order o / dO / gradients (perm set) are handled by the tensor-core kernels only
   if ((out_map.perm || do_map.perm || o_map.perm) && !use_tensor_cores(D)) return VMOBA_ERR_NOT_IMPLEMENTED;
   BwdWs w = carve_bwd(D, false, ws, cap);
@@ -99,9 +99,10 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
     // the backward kernel adds every dQ contribution into the fp32 accumulator: the row-dot pass also clears the
     // rows of all selecting queries; they are converted afterwards (rows of queries without a block become zero)
     launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
-                  (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, o_map, w.dq_acc, q_ptr);
+                  (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, o_map, w.dq_acc, q_ptr, (T*)do_bm);
     count_launches(1);
-    int rc = tc_sparse_bwd(D, q, k, v, d_o, lse, w.Dv, kb_ptr, q_idx, cap, w.dq_acc, dk, dv, status, st, out_map, do_map);
+    int rc = tc_sparse_bwd(D, q, k, v, do_bm ? do_bm : d_o, lse, w.Dv, kb_ptr, q_idx, cap, w.dq_acc, dk, dv, status, st,
+                           out_map, do_bm ? RowMap() : do_map);
     if (rc) return rc;
     launch_kernel(early_rows(D), simt::cast_rows_kernel<T>, grid_for((nq + 7) / 8, 16), 256, 0, st, w.dq_acc, (T*)dq,
                   q_ptr, nq, out_map);
@@ -110,7 +111,7 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
     return VMOBA_OK;
   }
   launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
-                (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), nullptr, nullptr);
+                (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), nullptr, nullptr, (T*)nullptr);
   count_launches(1);
   VMOBA_CUDA_OK(cudaMemsetAsync(w.dq_acc, 0, (size_t)nq * DH * sizeof(float), st));
   launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr);
@@ -146,7 +147,7 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
   if (d_o) {
     // (the tensor-core backward adds dQ into the fp32 accumulator, cleared in the same pass; null on the other path)
     launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
-                  (const T*)w.o_resid, (const T*)d_o, nq, w.Dv, RowMap(), RowMap(), w.dq_acc, nullptr);
+                  (const T*)w.o_resid, (const T*)d_o, nq, w.Dv, RowMap(), RowMap(), w.dq_acc, nullptr, (T*)nullptr);
     if (use_tensor_cores(D)) {
       VMOBA_LAUNCH_OK(1);
       int rc = tc_dense_bwd(D, q, k, v, d_o, lse, w.Dv, w.dq_acc, dk, dv, status, st);
@@ -263,7 +264,7 @@ extern "C" int vmoba_attn_bwd(const vmoba_shape* shape, const void* q_bm, const 
   if (D.dtype != VMOBA_BF16) o_resid_or_null = nullptr;
   if (!aligned16(o_resid_or_null)) return VMOBA_ERR_ARG;
   VMOBA_DISPATCH(simt_sparse_bwd, D, q_bm, k_bm, v_bm, o_bm, o_resid_or_null, lse, do_bm, kb_ptr, q_idx, q_ptr,
-                 capacity, dq_bm, dk_bm, dv_bm, dev_status, ws, st, RowMap(), RowMap(), RowMap());
+                 capacity, dq_bm, dk_bm, dv_bm, dev_status, ws, st, RowMap(), RowMap(), RowMap(), nullptr);
 }
 
 extern "C" int vmoba_attn_fwd_raster(const vmoba_shape* shape, const void* q_bm, const void* k_bm, const void* v_bm,
@@ -298,9 +299,9 @@ extern "C" int vmoba_attn_fwd_raster(const vmoba_shape* shape, const void* q_bm,
   return rc;
 }
 
-extern "C" int vmoba_attn_bwd_raster(const vmoba_shape* shape, const void* q_bm, const void* k_bm, const void* v_bm,
+static int attn_bwd_raster_impl(const vmoba_shape* shape, const void* q_bm, const void* k_bm, const void* v_bm,
                                      const void* o_bm, const int64_t o_strides_bsh[3], const void* o_resid_or_null,
-                                     const float* lse, const void* d_o, const int64_t do_strides_bsh[3],
+                                     const float* lse, const void* d_o, const int64_t do_strides_bsh[3], void* do_bm,
                                      const int32_t* kb_ptr,
                                      const int32_t* q_idx, const int32_t* q_ptr, int64_t capacity, void* dq, void* dk,
                                      void* dv, const int64_t grad_strides_bsh[3], const int32_t* perm,
@@ -325,7 +326,7 @@ extern "C" int vmoba_attn_bwd_raster(const vmoba_shape* shape, const void* q_bm,
   if (ws_bytes < carve_bwd(D, false, nullptr, capacity).bytes) return VMOBA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (D.dtype != VMOBA_BF16) o_resid_or_null = nullptr;
-  if (!aligned16(o_resid_or_null)) return VMOBA_ERR_ARG;
+  if (!aligned16(o_resid_or_null) || !aligned16(do_bm)) return VMOBA_ERR_ARG;
   RowMap out_map, do_map, o_map;
   out_map.perm = perm;
   out_map.heads = do_map.heads = o_map.heads = D.heads;
@@ -340,7 +341,30 @@ extern "C" int vmoba_attn_bwd_raster(const vmoba_shape* shape, const void* q_bm,
     do_map.sb = do_strides_bsh[0]; do_map.st = do_strides_bsh[1]; do_map.sh = do_strides_bsh[2];
   }
   VMOBA_DISPATCH(simt_sparse_bwd, D, q_bm, k_bm, v_bm, o_bm, o_resid_or_null, lse, d_o, kb_ptr, q_idx, q_ptr,
-                 capacity, dq, dk, dv, dev_status, ws, st, out_map, do_map, o_map);
+                 capacity, dq, dk, dv, dev_status, ws, st, out_map, do_map, o_map, do_bm);
+}
+
+extern "C" int vmoba_attn_bwd_raster(const vmoba_shape* shape, const void* q_bm, const void* k_bm, const void* v_bm,
+                                     const void* o_bm, const int64_t o_strides_bsh[3], const void* o_resid_or_null,
+                                     const float* lse, const void* d_o, const int64_t do_strides_bsh[3],
+                                     const int32_t* kb_ptr,
+                                     const int32_t* q_idx, const int32_t* q_ptr, int64_t capacity, void* dq, void* dk,
+                                     void* dv, const int64_t grad_strides_bsh[3], const int32_t* perm,
+                                     int32_t* dev_status, void* ws, size_t ws_bytes, void* stream) {
+  return attn_bwd_raster_impl(shape, q_bm, k_bm, v_bm, o_bm, o_strides_bsh, o_resid_or_null, lse, d_o, do_strides_bsh, nullptr, kb_ptr, q_idx, q_ptr,
+                              capacity, dq, dk, dv, grad_strides_bsh, perm, dev_status, ws, ws_bytes, stream);
+}
+
+extern "C" int vmoba_attn_bwd_raster_do(const vmoba_shape* shape, const void* q_bm, const void* k_bm, const void* v_bm,
+                                     const void* o_bm, const int64_t o_strides_bsh[3], const void* o_resid_or_null,
+                                     const float* lse, const void* d_o, const int64_t do_strides_bsh[3], void* do_bm,
+                                     const int32_t* kb_ptr,
+                                     const int32_t* q_idx, const int32_t* q_ptr, int64_t capacity, void* dq, void* dk,
+                                     void* dv, const int64_t grad_strides_bsh[3], const int32_t* perm,
+                                     int32_t* dev_status, void* ws, size_t ws_bytes, void* stream) {
+  if (!do_strides_bsh || !do_bm || do_bm == d_o) return VMOBA_ERR_ARG;
+  return attn_bwd_raster_impl(shape, q_bm, k_bm, v_bm, o_bm, o_strides_bsh, o_resid_or_null, lse, d_o, do_strides_bsh, do_bm, kb_ptr, q_idx, q_ptr,
+                              capacity, dq, dk, dv, grad_strides_bsh, perm, dev_status, ws, ws_bytes, stream);
 }
 
 extern "C" int vmoba_full_attn(const vmoba_shape* shape, const void* q, const void* k, const void* v, void* o,

@@ -149,9 +149,10 @@ class VmobaLayer:
                                  self.o_resid, self.lse, self.dev_status, self.ws)
         self.o_raster = o_out
 
-    def attn_bwd_raster(self, do_raster_or_none, dq_out, dk_out, dv_out):
+    def attn_bwd_raster(self, do_raster_or_none, dq_out, dk_out, dv_out, keep_do=False):
         """Backward writing dq, dk, dv in raster order (needs self.perm from the forward's partition of q); dO is
-        read in raster order too if given, else from self.do_bm; o is read from the raster-order tensor the last
+        read in raster order too if given, else from self.do_bm; keep_do: the pass that reads it first leaves it in
+        self.do_bm and the attention kernel reads it there; o is read from the raster-order tensor the last
         attn_fwd_raster wrote, else from self.o_bm."""
         do = self.do_bm if do_raster_or_none is None else do_raster_or_none
         dos = None if do_raster_or_none is None else self.raster_strides(do)
@@ -159,7 +160,8 @@ class VmobaLayer:
         os_ = None if self.o_raster is None else self.raster_strides(o)
         vb.vmoba_attn_bwd_raster(self.shape, self.q_bm, self.k_bm, self.v_bm, o, os_, self.o_resid, self.lse, do,
                                  dos, self.kb_ptr, self.q_idx, self.q_ptr, self.capacity, dq_out,
-                                 dk_out, dv_out, self.raster_strides(dq_out), self.perm, self.dev_status, self.ws)
+                                 dk_out, dv_out, self.raster_strides(dq_out), self.perm, self.dev_status, self.ws,
+                                 do_bm=self.do_bm if keep_do else None)
 
     # ---- whole layer --------------------------------------------------------------------
     def forward(self, q, k, v, tau, o_out, fold_o=None):
@@ -183,16 +185,17 @@ class VmobaLayer:
 
         fold_inverse: let the backward kernels write dq, dk, dv in raster order themselves (bf16, head_dim 128,
         outputs with equal strides) instead of three inverse partition passes; default: whenever possible.
-        fold_do: also let them read dO in raster order instead of partitioning it first (pays with few heads)."""
+        fold_do: also let the attention kernel read dO in raster order; by default the pass before it, which reads dO
+        for its own purpose, leaves a block-major copy."""
         if fold_inverse is None:
             fold_inverse = self.can_fold_inverse(dq_out, dk_out, dv_out)
         if fold_inverse and fold_do:
             self.attn_bwd_raster(do, dq_out, dk_out, dv_out)
             return
-        self.partition(do, self.do_bm)
         if fold_inverse:
-            self.attn_bwd_raster(None, dq_out, dk_out, dv_out)
+            self.attn_bwd_raster(do, dq_out, dk_out, dv_out, keep_do=True)
             return
+        self.partition(do, self.do_bm)
         if self.o_raster is not None:      # the block-major backward reads o_bm, which the raster forward did not write
             self.partition(self.o_raster, self.o_bm)
         self.attn_bwd()
