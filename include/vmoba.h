@@ -325,14 +325,12 @@ int vmoba_full_attn(const vmoba_shape* shape, const void* q, const void* k, cons
  * synchronising, and keeps it alive until it is cleared here.  Process-wide, not thread-safe; kernels run a
  * little slower while a buffer is registered, and their results do not change.
  *   forward kernel:  [0] softmax thread waiting for scores, [1] score read + row maximum, [2] accumulator
- *     rescale, [3] exponentials + P written, [4] epilogue (wait for the last P V, normalise, write), [6] its
- *     total; MMA warp: [8] wait for Q, [9] for K, [10] for P, [11] for V, [12] for a free accumulator,
- *     [13] issuing, [14] its total.
- *   backward kernel: [0] TMA warp waiting for free K / V buffers; [1] the TMA warp's total plus the writer
- *     warp's staging and reductions (one slot); MMA warp: [2] wait for K / V, [3] for a gathered chunk, [4] for
- *     P^T / dS^T, [5] for free accumulators or the dQ^T buffer, [6] its total; loaders: [7] wait for a free
- *     chunk, [8] total; compute warps: [10] wait for a chunk, [11] for S^T / dP^T, [12] for the dK / dV hand-off,
- *     [13] total; writer warp: [9] wait for dQ^T, [14] reading it from TMEM, [15] waiting at the staging barrier.
+ *     rescale, [3] exponentials + P written, [4] handing over the normalisers of an item, [6] its total;
+ *     Q K^T warp: [8] waiting, [13] issuing, [14] its total; P V warp: [10] waiting, [11] issuing.
+ *   backward kernel: [0] TMA warp waiting for free K / V buffers, [1] its total; MMA warp: [2] wait for K / V, [3] for
+ *     gathered rows, [4] for P^T / dS^T, [5] for the dQ^T columns or the accumulators, [6] its total; Q loaders: [7] wait
+ *     for a free tile, [8] total; compute warps: [9] wait for Q rows, [10] for S^T, [11] for dP^T, [12] for the dV / dK
+ *     hand-off, [13] total; dQ writers: [14] wait for dQ^T, [15] total.
  */
 void vmoba_debug_wait_profile(void* dev_counters16);
 
