@@ -35,7 +35,7 @@ static FwdWs carve_fwd(const Dims& D, long long cap, void* ws) {
   Carver c(ws);
   FwdWs w;
   w.item_ptr = c.take<int>((size_t)D.BH * D.Nb + 1);
-  w.item_tab = c.take<int>(4 * (size_t)max_items_128(D, cap));   // one int per item, or a 16-byte descriptor
+  w.item_tab = c.take<int>(4 * (size_t)max_items_128(D, cap));   // a 16-byte record per item
   w.part_lse = c.take<float>((size_t)cap);
   w.part_scale = c.take<float>((size_t)cap);     // per partial row: the power of two its fp16 values are scaled by
   // fp32 rows on the CUDA-core path, fp16 rows (scaled per row) on the tensor-core path
@@ -45,12 +45,11 @@ static FwdWs carve_fwd(const Dims& D, long long cap, void* ws) {
   return w;
 }
 
-struct BwdWs { int* item_ptr; int* item_tab; float* Dv; float* dq_acc; void* o_resid; size_t bytes; Guards guards; };
-static BwdWs carve_bwd(const Dims& D, bool dense, void* ws, long long cap = 0) {
+struct BwdWs { int* item_ptr; float* Dv; float* dq_acc; void* o_resid; size_t bytes; Guards guards; };
+static BwdWs carve_bwd(const Dims& D, bool dense, void* ws) {
   Carver c(ws);
   BwdWs w;
   w.item_ptr = c.take<int>((size_t)D.BH * D.Nb + 1);
-  w.item_tab = dense ? nullptr : c.take<int>((size_t)max_items_128(D, cap));
   w.Dv = c.take<float>((size_t)D.BH * D.S);
   w.dq_acc = dense && !use_tensor_cores(D) ? nullptr : c.take<float>((size_t)D.BH * D.S * D.d);
   w.o_resid = (dense && D.dtype == VMOBA_BF16) ? c.take<__nv_bfloat16>((size_t)D.BH * D.S * D.d) : nullptr;
@@ -91,7 +90,7 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
                            cudaStream_t st, const RowMap& out_map, const RowMap& do_map, const RowMap& o_map, void* do_bm) {
   // raster-order o / dO / gradients (perm set) are handled by the tensor-core kernels only
   if ((out_map.perm || do_map.perm || o_map.perm) && !use_tensor_cores(D)) return VMOBA_ERR_NOT_IMPLEMENTED;
-  BwdWs w = carve_bwd(D, false, ws, cap);
+  BwdWs w = carve_bwd(D, false, ws);
   VMOBA_GUARDS_ARM(w.guards, st);
   const long long n_kb = (long long)D.BH * D.Nb;
   const long long nq = (long long)D.BH * D.S;
@@ -208,7 +207,7 @@ extern "C" size_t vmoba_workspace_bytes(const vmoba_shape* shape, int stage, int
     case VMOBA_STAGE_SELECT: return select_ws_bytes(D);
     case VMOBA_STAGE_SELECT_ROWNORM: return select_rownorm_ws_bytes(D);
     case VMOBA_STAGE_ATTN_FWD: return carve_fwd(D, capacity, nullptr).bytes;
-    case VMOBA_STAGE_ATTN_BWD: return carve_bwd(D, false, nullptr, capacity).bytes;
+    case VMOBA_STAGE_ATTN_BWD: return carve_bwd(D, false, nullptr).bytes;
     case VMOBA_STAGE_FULL_FWD: return 256;
     case VMOBA_STAGE_FULL_BWD: return carve_bwd(D, true, nullptr).bytes;
     default: return 0;
@@ -259,7 +258,7 @@ extern "C" int vmoba_attn_bwd(const vmoba_shape* shape, const void* q_bm, const 
       !aligned16(dq_bm) || !aligned16(dk_bm) || !aligned16(dv_bm) || !aligned16(ws))
     return VMOBA_ERR_ARG;
   if (capacity <= 0 || capacity > (int64_t)INT32_MAX) return VMOBA_ERR_ARG;
-  if (ws_bytes < carve_bwd(D, false, nullptr, capacity).bytes) return VMOBA_ERR_WORKSPACE;
+  if (ws_bytes < carve_bwd(D, false, nullptr).bytes) return VMOBA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (D.dtype != VMOBA_BF16) o_resid_or_null = nullptr;
   if (!aligned16(o_resid_or_null)) return VMOBA_ERR_ARG;
@@ -323,7 +322,7 @@ static int attn_bwd_raster_impl(const vmoba_shape* shape, const void* q_bm, cons
     if (o_strides_bsh && (o_strides_bsh[i] < 0 || o_strides_bsh[i] % per16)) return VMOBA_ERR_ARG;
   }
   if (capacity <= 0 || capacity > (int64_t)INT32_MAX) return VMOBA_ERR_ARG;
-  if (ws_bytes < carve_bwd(D, false, nullptr, capacity).bytes) return VMOBA_ERR_WORKSPACE;
+  if (ws_bytes < carve_bwd(D, false, nullptr).bytes) return VMOBA_ERR_WORKSPACE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (D.dtype != VMOBA_BF16) o_resid_or_null = nullptr;
   if (!aligned16(o_resid_or_null) || !aligned16(do_bm)) return VMOBA_ERR_ARG;
