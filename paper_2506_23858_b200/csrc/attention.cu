@@ -70,7 +70,7 @@ static int simt_sparse_fwd(const Dims& D, const void* q, const void* k, const vo
   FwdWs w = carve_fwd(D, cap, ws);
   VMOBA_GUARDS_ARM(w.guards, st);
   const long long n_kb = (long long)D.BH * D.Nb;
-  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr);
+  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
   long long max_items = cap / simt::kRows + n_kb;
   launch_kernel(simt::attn_fwd_kernel<T, DH, false>, grid_for(max_items, 8), simt::kThreads, 0, st, (const T*)q,
                 (const T*)k, (const T*)v, kb_ptr, q_idx, q_ptr, w.item_ptr, (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale,
@@ -113,7 +113,7 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
                 (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), nullptr, nullptr, (T*)nullptr);
   count_launches(1);
   VMOBA_CUDA_OK(cudaMemsetAsync(w.dq_acc, 0, (size_t)nq * DH * sizeof(float), st));
-  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr);
+  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
   long long tiles = (D.sb + simt::kRows - 1) / simt::kRows;
   launch_kernel(simt::attn_bwd_dkdv_kernel<T, DH, false>, grid_for(n_kb * tiles, 4), simt::kThreads, 0, st,
                 (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb, D.BH,

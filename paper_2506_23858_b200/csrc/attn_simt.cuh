@@ -9,6 +9,8 @@
 // directly, queries with none are zero-filled by the merge kernel.
 #pragma once
 
+#include <algorithm>
+
 #include <cuda_fp16.h>
 
 #include "common.cuh"
@@ -20,11 +22,27 @@ constexpr int kRows = 64;      // rows (queries, or keys in the dK/dV kernel) pe
 constexpr int kTile = 32;      // rows of the streamed operand per shared-memory tile
 constexpr int kThreads = 256;  // 4 threads per row, each owning head_dim/4 channels
 
+// item_desc[item] = {index of the (batch, head, key block) list, first list position, rows (<= rows_per_item), 0}; a warp
+// per list (a thread per list took 13 us for 240 lists of 77 items, bound by the latency of its loop).
+__device__ __forceinline__ void write_item_desc(const int* item_ptr, const int* __restrict__ kb_ptr, long long n_kb,
+                                                long long max_items, long long capacity, int rows_per_item,
+                                                int4* __restrict__ desc, long long warp, long long n_warps) {
+  const int lane = threadIdx.x & 31;
+  for (long long i = warp; i < n_kb; i += n_warps) {
+    const long long t0 = item_ptr[i], t1 = min((long long)item_ptr[i + 1], max_items);
+    const long long lo = min((long long)kb_ptr[i], capacity), hi = min((long long)kb_ptr[i + 1], capacity);
+    for (long long t = t0 + lane; t < t1; t += 32) {
+      const long long l = lo + (t - t0) * rows_per_item;
+      desc[t] = make_int4((int)i, (int)l, (int)min((long long)rows_per_item, hi - l), 0);
+    }
+  }
+}
+
 // chunk-count prefix over the (batch, head, key block) lists: item_ptr[i] = number of work
 // items before list i when every list is cut into chunks of `rows` queries.
 static __global__ void __launch_bounds__(1024)
 item_ptr_kernel(const int* __restrict__ kb_ptr, long long n_kb, int rows, long long capacity,
-                int* __restrict__ item_ptr) {
+                int* item_ptr, int4* desc, long long max_items) {
   if (!grid_begin()) return;
   __shared__ long long total;
   block_exclusive_scan(
@@ -33,24 +51,27 @@ item_ptr_kernel(const int* __restrict__ kb_ptr, long long n_kb, int rows, long l
         return (hi - lo + rows - 1) / rows;
       },
       item_ptr, n_kb, &total);
+  if (desc) write_item_desc(item_ptr, kb_ptr, n_kb, max_items, capacity, rows, desc, threadIdx.x >> 5, blockDim.x >> 5);
 }
 
-// item_desc[item] = {index of the (batch, head, key block) list, first list position, rows (<= rows_per_item), 0}; a warp
-// per list (a thread per list took 13 us for 240 lists of 77 items, bound by the latency of its loop).
 static __global__ void __launch_bounds__(256)
 item_desc_kernel(const int* __restrict__ item_ptr, const int* __restrict__ kb_ptr, long long n_kb, long long max_items,
                  long long capacity, int rows_per_item, int4* __restrict__ desc) {
   if (!grid_begin()) return;
-  const int lane = threadIdx.x & 31;
-  const long long n_warps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n_kb; i += n_warps) {
-    const long long t0 = item_ptr[i], t1 = min((long long)item_ptr[i + 1], max_items);
-    const long long lo = min((long long)kb_ptr[i], capacity), hi = min((long long)kb_ptr[i + 1], capacity);
-    for (long long t = t0 + lane; t < t1; t += 32) {
-      const long long l = lo + (t - t0) * rows_per_item;
-      desc[t] = make_int4((int)i, (int)l, (int)min((long long)rows_per_item, hi - l), 0);
-    }
-  }
+  write_item_desc(item_ptr, kb_ptr, n_kb, max_items, capacity, rows_per_item, desc,
+                  (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), (long long)gridDim.x * (blockDim.x >> 5));
+}
+
+// Offsets of the lists' items and the items' records.  One CTA does both where the lists are one trip of its scan and the
+// items few (a launch less: forward and backward of 1.9K tokens 122.7 -> 119.6 us); else the records are spread over the chip.
+static void make_items(const int* kb_ptr, long long n_kb, int rows, long long cap, long long max_items, int* item_ptr,
+                       int4* desc, cudaStream_t st) {
+  const bool one = n_kb <= 1024 && max_items <= 4096;
+  launch_kernel(item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, rows, cap, item_ptr, one ? desc : nullptr, max_items);
+  if (!one)
+    launch_kernel(item_desc_kernel, (int)std::min<long long>((n_kb + 7) / 8, sm_count() * 8), 256, 0, st, item_ptr, kb_ptr,
+                  n_kb, max_items, cap, rows, desc);
+  count_launches(one ? 1 : 2);
 }
 
 struct Item {

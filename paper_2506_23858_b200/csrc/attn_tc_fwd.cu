@@ -615,9 +615,7 @@ int tc_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, co
     return tc_sparse_fwd_narrow(D, q, k, v, kb_ptr, q_idx, q_ptr, q_pairs, cap, o, o_resid, lse, status, item_ptr, item_tab,
                                 max_items, part_o, part_lse, part_scale, st, o_map);
   const long long n_kb = (long long)D.BH * D.Nb;
-  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, IM, cap, item_ptr);
-  launch_kernel(simt::item_desc_kernel, (int)std::min<long long>((n_kb + 7) / 8, sm_count() * 8), 256, 0, st,
-                item_ptr, kb_ptr, n_kb, max_items, cap, IM, reinterpret_cast<int4*>(item_tab));
+  simt::make_items(kb_ptr, n_kb, IM, cap, max_items, item_ptr, reinterpret_cast<int4*>(item_tab), st);
   Params p;
   p.q = (const __nv_bfloat16*)q; p.q_idx = q_idx; p.q_ptr = q_ptr; p.item_ptr = item_ptr;
   p.item_desc = reinterpret_cast<const int4*>(item_tab);
@@ -634,7 +632,7 @@ int tc_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, co
     if (int rc = launch_wide<false, false>(D, q, k, v, p, grid_items(cap / IM + n_kb), st)) return rc;
   }
   simt::merge_batched(D, q_ptr, q_pairs, p.part_o, part_lse, part_scale, cap, o, o_resid, lse, o_map, st);
-  VMOBA_LAUNCH_OK(3);
+  VMOBA_LAUNCH_OK(1);
   return VMOBA_OK;
 }
 

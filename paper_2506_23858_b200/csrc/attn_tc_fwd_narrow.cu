@@ -560,9 +560,7 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
   if (!sm100::make_tmap_bf16_rows(&tmK, k, rows, DH, BN) || !sm100::make_tmap_bf16_rows(&tmV, v, rows, DH, BN))
     return VMOBA_ERR_CUDA;
   const long long n_kb = (long long)D.BH * D.Nb;
-  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, BM, cap, item_ptr);
-  launch_kernel(simt::item_desc_kernel, (int)std::min<long long>((n_kb + 7) / 8, sm_count() * 8), 256, 0, st,
-                item_ptr, kb_ptr, n_kb, max_items, cap, BM, reinterpret_cast<int4*>(item_tab));
+  simt::make_items(kb_ptr, n_kb, BM, cap, max_items, item_ptr, reinterpret_cast<int4*>(item_tab), st);
   Params p;
   p.q = (const __nv_bfloat16*)q; p.q_idx = q_idx; p.q_ptr = q_ptr; p.item_ptr = item_ptr;
   p.item_desc = reinterpret_cast<const int4*>(item_tab);
@@ -578,7 +576,7 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
   launch_kernel(kernel, (int)items, THREADS, SMEM_BYTES, st, tmK, tmV, p);
   simt::merge_batched(D, q_ptr, q_pairs, p.part_o, part_lse, part_scale, cap, o, o_resid, lse, o_map, st);
-  VMOBA_LAUNCH_OK(4);
+  VMOBA_LAUNCH_OK(2);
   return VMOBA_OK;
 }
 
