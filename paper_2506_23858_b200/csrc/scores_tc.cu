@@ -168,7 +168,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         if (++s == nq) { s = 0; ph ^= 1; }
       }
       if (*abort_flag) {
-        // the newest load of every slot: in this round of the ring for slots below s, in the one before for the others
+        // the newest load of every slot: in this lap of the ring for slots below s, in the one before for the others
         for (int f = 0; f < filled; ++f) mbar_wait(&sm->q_full[f], (f < s ? ph : ph ^ 1) ^ 1, abort_flag, p.status);
         if (bn > 0) mbar_wait(&sm->b_full, (bn - 1) & 1, abort_flag, p.status);
       }
