@@ -49,7 +49,7 @@ struct Smem {
   uint64_t o_done;                   // P V of a key tile complete (commit)
   uint64_t q_full, q_empty;          // Q tile of an item gathered (64 arrivals) / no longer needed (commit)
   uint64_t ep_ready;                 // an item's normalisers are in ep_inv / ep_lse (128 softmax arrivals)
-  uint64_t o_free;                   // the epilogue warps have read the accumulator (128 arrivals)
+  uint64_t o_free;                   // the epilogue warps have read them and the accumulator (128 arrivals)
   uint32_t tmem_base;
   int abort_flag;
   float ep_inv[2][BM], ep_lse[2][BM];   // [item % 2][row]: 1 / sum of the rounded weights, natural-log lse
@@ -304,8 +304,7 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
           if (leader && t == ntiles - 1) mma_commit(&sm->q_empty);
         }
         lap(5);
-        // P of this tile; it also says that the softmax threads have left the epilogue of the item before, i.e.
-        // that its accumulator has been read
+        // P of this tile
         mbar_wait_warp(&sm->p_ready, f & 1, abort_flag, p.status);
         lap(2);
         mbar_wait_warp(&sm->v_full, f & 1, abort_flag, p.status);
@@ -336,8 +335,7 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     for (int item = blockIdx.x; item < n_items; item += gridDim.x, ++n) {
       const Item it = get_item(item);
       const __nv_bfloat16* qh = p.q + it.head_off * DH;
-      // Four bookkeeping slots: the softmax warps read slot n % 4 in the epilogue of item n, and the loaders can be
-      // at most two items ahead of an epilogue.
+      // Four bookkeeping slots: the epilogue of item n reads slot n % 4, and the loaders can be at most two items ahead of it.
       int info[2];
       {
         if ((chunk & 7) == 0) {       // one L2 request per 128-byte line of every row of the item
@@ -453,7 +451,7 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
       }
     }
   } else {
-    // ------------------------------------------------------------------ softmax + epilogue
+    // ------------------------------------------------------------------ softmax
     asm volatile("setmaxnreg.inc.sync.aligned.u32 128;");
     const int quad = warp & 3;                      // TMEM lane quarter this warp may access
     const int r = quad * 32 + lane;                 // query row inside the tile
@@ -533,7 +531,11 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
         tc_fence_before();
         mbar_arrive(&sm->p_ready);
       }
-      // hand the row's normalisers to the epilogue warps and go on with the next item
+      // Hand the row's normalisers to the epilogue warps, once they are through with the item before, and go on.  Without
+      // the wait ep_ready could complete two phases while an epilogue warp, held up by its stores, has yet to look at the
+      // first: with one key tile per item nothing else stands in between (with two, the second Q K^T follows a P V that has
+      // waited for o_free), and the epilogue would wait for a phase that needs its own arrival.
+      if (n >= 1) mbar_wait(&sm->o_free, (n - 1) & 1, abort_flag, p.status);
       sm->ep_inv[n & 1][r] = 1.0f / l_r;
       sm->ep_lse[n & 1][r] = (m_used + log2f(l)) * 0.6931471805599453f;
       mbar_arrive(&sm->ep_ready);
