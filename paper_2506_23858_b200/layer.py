@@ -231,18 +231,22 @@ class SteppedAttention:
         self.schedule = dense_step_schedule(n_steps, dense_fraction)
         s = layer.shape
         self._lse = torch.empty(s.B * s.heads * s.S, dtype=torch.float32, device=layer.device)
+        # the grid as one block: the partition into it keeps the raster order of the tokens
+        self._one_block = vb.Shape.from_buffer_copy(s)
+        self._one_block.bT, self._one_block.bH, self._one_block.bW = s.T, s.H, s.W
 
     def forward(self, step: int, q, k, v, o_out) -> str:
         """Runs step `step`; returns which path ran ("dense" or "sparse")."""
         if self.schedule[step]:
-            # the dense kernels take [B, heads, S, d] in any one token order: block-major will do
-            L = self.layer
+            # the dense kernels take [B, heads, S, d].  The tokens stay in raster order: the running maximum that a row's
+            # weights are rounded against, and with it the last bits of o, depends on the order of the keys.
+            L, one = self.layer, self._one_block
             q, k, v = (x if L.partitions(x) else x.contiguous() for x in (q, k, v))
             qd, kd, vd, od = (torch.empty_like(L.q_bm) for _ in range(4))
-            L.partition_many((q, k, v), (qd, kd, vd))
+            vb.vmoba_partition_many(one, 0, (q, k, v), (qd, kd, vd), [L.raster_strides(x) for x in (q, k, v)])
             vb.vmoba_full_attn(L.shape, qd, kd, vd, od, self._lse, dev_status=L.dev_status)
             o = o_out if L.partitions(o_out) else torch.empty(o_out.shape, dtype=L.q_bm.dtype, device=L.device)
-            L.partition(o, od, inverse=True)
+            vb.vmoba_partition(one, 1, od, o, L.raster_strides(o))
             if o is not o_out:
                 o_out.copy_(o)
             return "dense"

@@ -62,3 +62,20 @@ def test_dense_step_takes_any_strides():
     stepped.forward(0, *odd, o_odd)
     L.check_status()
     assert torch.equal(o, o_odd)
+
+
+@pytest.mark.parametrize("dtype, d", [("bf16", 128), ("f32", 64)])
+def test_dense_step_keeps_the_raster_order(dtype, d):
+    """Bit for bit full attention over the tokens in the caller's order: a row's weights are rounded against a running
+    maximum, so another order of the keys gives other last bits."""
+    shape = vb.make_shape(2, 2, d, (6, 12, 26), (3, 6, 13), dtype)
+    L = VmobaLayer(shape, 4096)
+    torch.manual_seed(8)
+    q, k, v = (2.0 * torch.randn(2, shape.S, 2, d, device="cuda").to(L.q_bm.dtype) for _ in range(3))
+    o = torch.empty_like(q)
+    assert SteppedAttention(L, 0.25, 1, 1.0).forward(0, q, k, v, o) == "dense"
+    qh, kh, vh = (x.permute(0, 2, 1, 3).contiguous() for x in (q, k, v))
+    ref, lse = torch.empty_like(qh), torch.empty(2 * 2 * shape.S, device="cuda")
+    vb.vmoba_full_attn(shape, qh, kh, vh, ref, lse, dev_status=L.dev_status)
+    L.check_status()
+    assert torch.equal(o, ref.permute(0, 2, 1, 3))
