@@ -663,6 +663,26 @@ __device__ __forceinline__ bool split_interval(float lo, float hi, float& mid) {
   return mid > lo && mid < hi;
 }
 
+// The searches below compare scores as floats, which gives a NaN no place; the rule does (a NaN's key lies beyond those of the
+// infinities), and every query keeps exactly k blocks.  Rows with a NaN are found by a maximum that hands NaN on, at the price
+// of one that does not, and are searched on the scores' keys.  These are made from words that are never floats: as a float
+// operation, setting a NaN's sign is free to return any NaN, and did.
+__device__ __forceinline__ uint32_t key_of_bits(uint32_t u) {
+  if (u == 0x80000000u) u = 0u;      // -0 ties with +0
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ uint32_t bits_of(float x) {
+  uint32_t u;
+  asm("mov.b32 %0, %1;" : "=r"(u) : "f"(x));
+  return u;
+}
+constexpr uint32_t kInfKey = 0xff800000u;      // key of +inf: a larger one is a NaN's
+
 // Top-k per query, one warp per row: lane l holds blocks l + 32 i.  Search over the row's score range for a threshold
 // that k scores reach; it usually ends early, on a threshold that exactly k scores reach, and otherwise on the k-th
 // score itself, whose ties are then taken in block order.  The first probe is the threshold of the row before (rows
@@ -685,10 +705,15 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
   if (row_begin >= row_end) return;
   int head = (int)(row_begin / S), pos = (int)(row_begin - (long long)head * S);
   float low = INFINITY;                 // smallest score this lane has selected in the head so far
+  int on_keys = 0, first = pos;         // rows of the head that were searched on keys; the run's first row in it
+  uint32_t low_key = 0xffffffffu;       // smallest cutoff of those
   auto flush = [&]() {
-    const uint32_t key = __reduce_min_sync(0xffffffffu, float_key(low));
+    uint32_t key = __reduce_min_sync(0xffffffffu, float_key(low));
+    if (on_keys > 0) key = on_keys < pos - first ? min(key, low_key) : low_key;
     if (lane == 0) atomicMin(&st[head].cutoff_key, key);
     low = INFINITY;
+    on_keys = first = 0;
+    low_key = 0xffffffffu;
   };
   float next[MW];
   auto load_row = [&](const float* sr) {
@@ -705,16 +730,17 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
 #pragma unroll
     for (int i = 0; i < MW; ++i) {
       x[i] = next[i];
-      mx = fmaxf(mx, x[i]);
+      mx = max_nan(mx, x[i]);
       if (lane + 32 * i < Nb) mn = fminf(mn, x[i]);
     }
     src += Nb;
     if (row + 1 < row_end) load_row(src);
     // invariant: at least k scores reach lo, fewer than k reach hi (or lo == hi)
     float lo = key_float(__reduce_min_sync(0xffffffffu, float_key(mn)));
-    float hi = key_float(__reduce_max_sync(0xffffffffu, float_key(mx)));
+    const uint32_t mx_bits = bits_of(mx), top = __reduce_max_sync(0xffffffffu, (mx_bits & 0x80000000u) ? ~mx_bits : (mx_bits | 0x80000000u));
+    float hi = key_float(top);
     bool exact = false;                 // exactly k scores reach lo
-    if (k < Nb) {
+    if (k < Nb && top <= kInfKey) {
       // (a block the row does not have counts as -inf, which no threshold above the row's minimum lets through)
       auto count_ge = [&](float c) {
         int n = 0;
@@ -746,7 +772,36 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
       }
     }
     uint32_t my_word = 0u;
-    if (exact) {
+    if (top > kInfKey) {
+      // the largest key that k blocks reach, bit by bit; blocks above it, and those at it in block order.  (The row is read
+      // again word by word: rare, and with the registers of the other search it would cost that one its warps.)
+      const uint32_t* sr = reinterpret_cast<const uint32_t*>(scores) + row * Nb + lane;
+      auto key_at = [&](int i) { return key_of_bits(__ldg(sr + 32 * i)); };
+      auto count_keys = [&](auto pred) {
+        int n = 0;
+#pragma unroll 1
+        for (int i = 0; lane + 32 * i < Nb; ++i) n += pred(key_at(i)) ? 1 : 0;
+        __syncwarp();
+        return __reduce_add_sync(0xffffffffu, n);
+      };
+      uint32_t c = 0u;
+#pragma unroll 1
+      for (uint32_t bit = 0x80000000u; bit; bit >>= 1)
+        if (count_keys([&](uint32_t key) { return key >= (c | bit); }) >= k) c |= bit;
+      int need = k - count_keys([&](uint32_t key) { return key > c; });
+#pragma unroll 1
+      for (int i = 0; i < mw; ++i) {
+        const bool in = lane + 32 * i < Nb;
+        const uint32_t key = in ? key_at(i) : 0u;
+        const uint32_t e = __ballot_sync(0xffffffffu, in && key == c);
+        const bool sel = in && (key > c || (key == c && __popc(e & lt_mask) < need));
+        need -= __popc(e);
+        const uint32_t word = __ballot_sync(0xffffffffu, sel);
+        if (lane == i) my_word = word;
+      }
+      low_key = min(low_key, c);
+      ++on_keys;
+    } else if (exact) {
 #pragma unroll
       for (int i = 0; i < MW; ++i) {
         const bool sel = x[i] >= lo;
@@ -809,7 +864,7 @@ select_topk_rows_kernel(const float* __restrict__ scores, int S, int Nb, int k, 
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       x[j] = (live && j < Nb) ? tile[threadIdx.x * pitch + j] : -INFINITY;
-      if (j < Nb) { lo = fminf(lo, x[j]); hi = fmaxf(hi, x[j]); }
+      if (j < Nb) { lo = fminf(lo, x[j]); hi = max_nan(hi, x[j]); }
     }
     auto count_ge = [&](float c) {
       int n = 0;
@@ -817,7 +872,8 @@ select_topk_rows_kernel(const float* __restrict__ scores, int S, int Nb, int k, 
       for (int j = 0; j < N; ++j) n += (j < Nb && x[j] >= c) ? 1 : 0;
       return n;
     };
-    if (live && k < Nb) {
+    const bool on_keys = live && hi != hi;
+    if (live && k < Nb && !on_keys) {
       float mid;
       if (count_ge(hi) >= k) lo = hi;
       while (split_interval(lo, hi, mid)) {
@@ -826,24 +882,45 @@ select_topk_rows_kernel(const float* __restrict__ scores, int S, int Nb, int k, 
         if (n == k) break;
       }
     }
-    int need = k;
+    uint32_t word = 0u, key = 0xffffffffu;      // selected blocks, smallest selected key
+    if (on_keys) {
+      auto key_at = [&](int j) { return key_of_bits(reinterpret_cast<const uint32_t*>(tile)[threadIdx.x * pitch + j]); };
+      uint32_t c = 0u;
+#pragma unroll 1
+      for (uint32_t bit = 0x80000000u; bit; bit >>= 1) {
+        int n = 0;
+#pragma unroll 1
+        for (int j = 0; j < Nb; ++j) n += key_at(j) >= (c | bit) ? 1 : 0;
+        if (n >= k) c |= bit;
+      }
+      int need = k;
+#pragma unroll 1
+      for (int j = 0; j < Nb; ++j) need -= key_at(j) > c ? 1 : 0;
+#pragma unroll 1
+      for (int j = 0; j < Nb; ++j) {
+        const uint32_t kj = key_at(j);
+        if (kj > c || (kj == c && need-- > 0)) word |= 1u << j;
+      }
+      key = c;
+    } else {
+      int need = k;
 #pragma unroll
-    for (int j = 0; j < N; ++j) need -= (j < Nb && x[j] > lo) ? 1 : 0;
-    uint32_t word = 0u;
-    float low = INFINITY;
+      for (int j = 0; j < N; ++j) need -= (j < Nb && x[j] > lo) ? 1 : 0;
+      float low = INFINITY;
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
-      const bool tie = x[j] == lo && need > 0;
-      const bool sel = j < Nb && (x[j] > lo || tie);
-      if (j < Nb && x[j] == lo) --need;
-      if (sel) { word |= 1u << j; low = fminf(low, x[j]); }
+      for (int j = 0; j < N; ++j) {
+        const bool tie = x[j] == lo && need > 0;
+        const bool sel = j < Nb && (x[j] > lo || tie);
+        if (j < Nb && x[j] == lo) --need;
+        if (sel) { word |= 1u << j; low = fminf(low, x[j]); }
+      }
+      if (live) key = float_key(low);
     }
     const long long row = row0 + threadIdx.x;
     if (live && own_sb > 0) word |= 1u << ((int)(row % S) / own_sb);
     if (live) mask_bits[row] = word;
     // smallest selected key: one atomic per warp unless its rows straddle two heads
     const int head = live ? (int)(row / S) : -1;
-    const uint32_t key = live ? float_key(low) : 0xffffffffu;
     const int head_lo = __reduce_min_sync(0xffffffffu, live ? head : INT32_MAX), head_hi = __reduce_max_sync(0xffffffffu, head);
     if (head_lo == head_hi) {
       const uint32_t m = __reduce_min_sync(0xffffffffu, key);
