@@ -271,7 +271,8 @@ int vmoba_attn_fwd_raster(const vmoba_shape* shape, const void* q_bm, const void
  * dq, dk, dv [B, heads, S, head_dim] (dtype) from do_bm, the forward's o_bm (+ o_resid) and lse.
  * Queries without a selected block get dq = 0.  The paper states no gradient formula; this is
  * the softmax-attention gradient restricted to the selected pairs.  `capacity` is the one given
- * to vmoba_select (list positions at or beyond it are never read).
+ * to vmoba_select (list positions at or beyond it are never read).  dk and dv repeat bit for bit; the blocks' parts of
+ * a row of dq are added in fp32 in any order.
  */
 int vmoba_attn_bwd(const vmoba_shape* shape, const void* q_bm, const void* k_bm, const void* v_bm,
                    const void* o_bm, const void* o_resid_or_null, const float* lse, const void* do_bm,
@@ -311,7 +312,10 @@ int vmoba_attn_bwd_raster_do(const vmoba_shape* shape, const void* q_bm, const v
 /*
  * Dense softmax attention over all S keys: the tau = 1 limit of the layer and the speed-up
  * denominator (the "Full Attention" baseline of Section 4.1).  Tensors are [B, heads, S, head_dim]
- * in any one token order.  If do_or_null is given, also computes dq, dk, dv.
+ * in any one token order.  If do_or_null is given, also computes dq, dk, dv.  The results repeat bit for bit.
+ * For the backward ws must hold vmoba_workspace_bytes(shape, VMOBA_STAGE_FULL_BWD, 0) bytes: 4 * B * heads * S, for bf16 the
+ * rounding residual of o (2 bytes per element of a tensor) and, for bf16 with head_dim 128, an fp32 accumulator of dq (4 bytes
+ * per element: 1.5 GB at 75,600 tokens and 40 heads).
  */
 int vmoba_full_attn(const vmoba_shape* shape, const void* q, const void* k, const void* v, void* o,
                     float* lse, const void* do_or_null, void* dq, void* dk, void* dv,
@@ -324,9 +328,11 @@ int vmoba_full_attn(const vmoba_shape* shape, const void* q, const void* k, cons
  * grid size (one CTA per SM) for cycles per CTA.  The caller zeroes the buffer before a launch, reads it after
  * synchronising, and keeps it alive until it is cleared here.  Process-wide, not thread-safe; kernels run a
  * little slower while a buffer is registered, and their results do not change.
- *   forward kernel:  [0] softmax thread waiting for scores, [1] score read + row maximum, [2] accumulator
+ *   forward kernels: [0] softmax thread waiting for scores, [1] score read + row maximum, [2] accumulator
  *     rescale, [3] exponentials + P written, [4] handing over the normalisers of an item, [6] its total;
- *     Q K^T warp: [8] waiting, [13] issuing, [14] its total; P V warp: [10] waiting, [11] issuing.
+ *     key blocks of more than 256 keys and dense: Q K^T warp [8] waiting, [13] issuing, [14] its total; P V warp [10] waiting,
+ *     [11] issuing; shorter key blocks: MMA warp [8] wait for Q, [9] for K, [10] for P, [11] for V, [12] for a free
+ *     accumulator, [13] issuing, [14] its total.
  *   backward kernel: [0] TMA warp waiting for free K / V buffers, [1] its total; MMA warp: [2] wait for K / V, [3] for
  *     gathered rows, [4] for P^T / dS^T, [5] for the dQ^T columns or the accumulators, [6] its total; Q loaders: [7] wait
  *     for a free tile, [8] total; compute warps: [9] wait for Q rows, [10] for S^T, [11] for dP^T, [12] for the dV / dK

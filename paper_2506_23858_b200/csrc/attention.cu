@@ -24,7 +24,8 @@ int tc_sparse_bwd(const Dims& D, const void* q, const void* k, const void* v, co
                   const float* Dv, const int* kb_ptr, const int* q_idx, long long cap, float* dq_acc, void* dk, void* dv,
                   int32_t* status, cudaStream_t st, const RowMap& out_map, const RowMap& do_map);
 int tc_dense_bwd(const Dims& D, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
-                 const float* Dv, float* dq_acc, void* dk, void* dv, int32_t* status, cudaStream_t st);
+                 const float* Dv, float* dq_acc, int* turns, void* dk, void* dv, int32_t* status, cudaStream_t st);
+long long tc_dense_bwd_turns(const Dims& D);
 
 static bool use_tensor_cores(const Dims& D) { return D.dtype == VMOBA_BF16 && D.d == 128; }
 
@@ -45,7 +46,7 @@ static FwdWs carve_fwd(const Dims& D, long long cap, void* ws) {
   return w;
 }
 
-struct BwdWs { int* item_ptr; float* Dv; float* dq_acc; void* o_resid; size_t bytes; Guards guards; };
+struct BwdWs { int* item_ptr; float* Dv; float* dq_acc; void* o_resid; int* turns; size_t bytes; Guards guards; };
 static BwdWs carve_bwd(const Dims& D, bool dense, void* ws) {
   Carver c(ws);
   BwdWs w;
@@ -53,6 +54,7 @@ static BwdWs carve_bwd(const Dims& D, bool dense, void* ws) {
   w.Dv = c.take<float>((size_t)D.BH * D.S);
   w.dq_acc = dense && !use_tensor_cores(D) ? nullptr : c.take<float>((size_t)D.BH * D.S * D.d);
   w.o_resid = (dense && D.dtype == VMOBA_BF16) ? c.take<__nv_bfloat16>((size_t)D.BH * D.S * D.d) : nullptr;
+  w.turns = dense && use_tensor_cores(D) ? c.take<int>((size_t)tc_dense_bwd_turns(D)) : nullptr;
   w.bytes = c.total();
   w.guards = c.guards;
   return w;
@@ -98,7 +100,7 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
     // the backward kernel adds every dQ contribution into the fp32 accumulator: the row-dot pass also clears the
     // rows of all selecting queries; they are converted afterwards (rows of queries without a block become zero)
     launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
-                  (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, o_map, w.dq_acc, q_ptr, (T*)do_bm);
+                  (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, o_map, w.dq_acc, q_ptr, (T*)do_bm, nullptr, 0);
     count_launches(1);
     int rc = tc_sparse_bwd(D, q, k, v, do_bm ? do_bm : d_o, lse, w.Dv, kb_ptr, q_idx, cap, w.dq_acc, dk, dv, status, st,
                            out_map, do_bm ? RowMap() : do_map);
@@ -110,7 +112,7 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
     return VMOBA_OK;
   }
   launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
-                (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), nullptr, nullptr, (T*)nullptr);
+                (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), nullptr, nullptr, (T*)nullptr, nullptr, 0);
   count_launches(1);
   VMOBA_CUDA_OK(cudaMemsetAsync(w.dq_acc, 0, (size_t)nq * DH * sizeof(float), st));
   launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
@@ -144,12 +146,13 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
     count_launches(1);
   }
   if (d_o) {
-    // (the tensor-core backward adds dQ into the fp32 accumulator, cleared in the same pass; null on the other path)
+    // (the tensor-core backward's turn counters are cleared in the same pass; null on the other path)
     launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
-                  (const T*)w.o_resid, (const T*)d_o, nq, w.Dv, RowMap(), RowMap(), w.dq_acc, nullptr, (T*)nullptr);
+                  (const T*)w.o_resid, (const T*)d_o, nq, w.Dv, RowMap(), RowMap(), nullptr, nullptr, (T*)nullptr, w.turns,
+                  w.turns ? tc_dense_bwd_turns(D) : 0);
     if (use_tensor_cores(D)) {
       VMOBA_LAUNCH_OK(1);
-      int rc = tc_dense_bwd(D, q, k, v, d_o, lse, w.Dv, w.dq_acc, dk, dv, status, st);
+      int rc = tc_dense_bwd(D, q, k, v, d_o, lse, w.Dv, w.dq_acc, w.turns, dk, dv, status, st);
       if (rc) return rc;
       launch_kernel(early_rows(D), simt::cast_rows_kernel<T>, grid_for((nq + 7) / 8, 16), 256, 0, st, w.dq_acc,
                     (T*)dq, nullptr, nq, RowMap());

@@ -500,7 +500,7 @@ static void merge_batched(const Dims& D, const int* q_ptr, const int* q_pairs, c
 // D = rowsum(dO * O), one warp per query; o and dO block-major or in raster order through their maps, the
 // rounding residual of o always block-major.  If zero_acc is given, the fp32 dQ accumulator rows of the queries
 // with at least one selected block (of every query without q_ptr) are cleared in the same pass: the only rows the
-// backward kernel adds into.
+// backward kernel adds into.  zero_words: n_words counters to clear on the way.
 // do_out: a block-major copy of dO is left there on the way, so that dO in raster order needs no pass of its own (two
 // batches of 32,760 queries x 12 heads: 166 us, 179 in two passes; 13,440 x 12: 41 and 43; 75,600 x 40: 761 and 783; small
 // calls save a launch).
@@ -508,8 +508,11 @@ template <typename T, int DH>
 __global__ void __launch_bounds__(256)
 rowdot_kernel(const T* __restrict__ o, const T* __restrict__ o_resid, const T* __restrict__ d_o, long long n_queries,
               float* __restrict__ Dv, const RowMap do_map, const RowMap o_map,
-              float* __restrict__ zero_acc, const int* __restrict__ q_ptr, T* __restrict__ do_out) {
+              float* __restrict__ zero_acc, const int* __restrict__ q_ptr, T* __restrict__ do_out,
+              int* __restrict__ zero_words, long long n_words) {
   if (!grid_begin()) return;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n_words; i += (long long)gridDim.x * blockDim.x)
+    zero_words[i] = 0;
   constexpr int C = DH / 32;
   const int lane = threadIdx.x & 31;
   const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);

@@ -13,7 +13,8 @@
 //                                                         lands in the dP^T columns)
 //   Every key belongs to exactly one item: dK and dV are written once, no atomics.  dQ^T is read out of TMEM by eight
 //   writer warps and added into an fp32 accumulator with red.global.add.v4.f32 (per warp instruction: complete 128-byte
-//   lines of four query rows).
+//   lines of four query rows).  Sparse: in whatever order the items come to it, so dQ is repeatable to rounding only.  Dense:
+//   key tile after key tile, see Turns below; the whole dense backward repeats bit for bit.
 //
 // What bounds it is the shared-memory port (128 bytes per cycle).  A shared-memory MMA with N = 128 fetches 8 KB of
 // operands in its 64 cycles, a TS one 4 KB; per 128 x 128 unit that is 2048 cycles of operands against 2560 cycles of
@@ -60,7 +61,9 @@ struct KvSmem {
   uint64_t dp_full, ds_ready;                                      // dP^T complete (commit) / dS^T written (256 arrivals)
   uint64_t dq_full, dq_free;                                       // dQ^T complete (commit) / read out of TMEM (256 arrivals)
   uint64_t acc_done, acc_free;                                     // dV / dK of an item complete (commit) / read (256 arrivals)
+  uint64_t turn_ok, rows_out, rows_seen;                           // dense: it is this tile's turn / its dQ is on the way (256 arrivals) / and noted
   uint32_t tmem_base;
+  int ticket;                                // dense: the CTA's item
   int abort_flag;
   alignas(16) float lse2[NQ][QU];            // lse * log2 e, with the Q rows of a unit
   alignas(16) float negD[2][QU];             // -rowsum(dO * O), with its dO rows
@@ -75,6 +78,17 @@ static_assert(SMEM_BYTES <= 232448, "backward: shared memory");
 constexpr int THREADS = 896;
 constexpr uint32_t IDESC_TN = make_idesc_bf16(128, 128, false, true);    // dV, dK: A from TMEM, B MN-major
 
+// Turns (dense).  Every unit of every head has a counter: the number of key tiles whose dQ has been added there.  Key tile t
+// adds to it when it stands at t (the first one stores, so nothing has to be cleared), so the sum is taken in one order
+// whatever the timing.  A CTA takes one item, by a ticket drawn when it starts: the tiles an item waits for belong to lower
+// tickets, which CTAs that are running hold, so the waiting ends whatever else occupies the device.  The key tiles of a head
+// follow one another about a unit apart; tickets go round `group` heads, so that a head's tiles start few units apart
+// (SMs / group) and come no faster than one per unit.  Two warps that have nothing else to do look at the counter and move it
+// on (a fence behind the reductions, a look at another CTA's word): the writers see shared-memory barriers only.
+// Measured, against reductions in any order and tiles that start at different units (forward and backward): 12 heads x 13,440
+// tokens 3946 -> 4024 us, x 8,000 1453 -> 1492, 4 heads x 32,760 7665 -> 8128.  Where the tiles of a head are most of what
+// there is to run, they wait for one another: 12 x 3,000 216 -> 275, 12 x 1,000 71 -> 100, 1 x 3,000 132 -> 224 (257, 377 and
+// 227 with dQ in a kernel of its own).  With the writers looking at the counters themselves 12 x 13,440 took 4798.
 struct KvParams {
   const __nv_bfloat16 *q, *d_o;
   const float *lse, *Dv;
@@ -86,31 +100,39 @@ struct KvParams {
   int dkv_32;                  // dk and dv are 32-byte aligned: rows go out with 32-byte stores
   RowMap out_map;              // where the dK / dV rows go (block-major, or raster order through perm)
   RowMap do_map;               // where the dO rows come from (likewise)
-  float* dq_acc;               // fp32 [queries][head_dim], zeroed rows of all selecting queries; columns in the order of the
+  float* dq_acc;               // fp32 [queries][head_dim]; sparse: zeroed rows of all selecting queries; columns in the order of the
                                // dQ writers: position 32 w + 4 r + a holds column 32 w + r + 8 a (r < 8, a < 4)
+  int* turns;                  // dense: [BH][units], then the ticket; zero at the start
+  int group;                   // dense: heads whose key tiles are taken in turn
   int32_t* status;
   unsigned long long* prof;    // optional wait-time counters (diagnostics), or null
 };
 
 struct KvItem {
-  int bh, key0, valid, n_list, n_units, first_unit;
+  int bh, key0, valid, n_list, n_units, tile;
   int list_lo, head_off;       // positions and rows fit 31 bits (capacity, B * heads * S <= 2^30)
 };
 
 template <bool DENSE>
 __device__ __forceinline__ KvItem kv_decode(const KvParams& p, int item, int tiles) {
   KvItem it;
-  const int kbi = item / tiles;
-  const int tile = item - kbi * tiles;
-  it.bh = DENSE ? kbi : kbi / p.Nb;
-  const int j = kbi - it.bh * (DENSE ? 1 : p.Nb);
-  it.key0 = (DENSE ? 0 : j * p.sb) + tile * BN;
-  it.valid = min(BN, (DENSE ? p.S : p.sb) - tile * BN);
-  it.head_off = it.bh * p.S;
   if constexpr (DENSE) {
+    // groups of heads; in a group, the first key tile of every head, then the second ones
+    const int per = p.group * tiles, first = item / per * p.group, heads = min(p.group, p.BH - first), r = item % per;
+    it.tile = r / heads;
+    it.bh = first + r - it.tile * heads;
+    it.key0 = it.tile * BN;
+    it.valid = min(BN, p.S - it.key0);
+    it.head_off = it.bh * p.S;
     it.list_lo = 0;
     it.n_list = p.S;
   } else {
+    const int kbi = item / tiles;
+    it.tile = item - kbi * tiles;
+    it.bh = kbi / p.Nb;
+    it.key0 = (kbi - it.bh * p.Nb) * p.sb + it.tile * BN;
+    it.valid = min(BN, p.sb - it.tile * BN);
+    it.head_off = it.bh * p.S;
     long long lo = min((long long)p.kb_ptr[kbi], p.capacity), hi = min((long long)p.kb_ptr[kbi + 1], p.capacity);
 #ifdef VMOBA_DEBUG
     if (lo < 0 || hi < lo) {      // offsets must be non-negative and ascending
@@ -122,17 +144,7 @@ __device__ __forceinline__ KvItem kv_decode(const KvParams& p, int item, int til
     it.n_list = (int)(hi - lo);
   }
   it.n_units = (it.n_list + QU - 1) / QU;
-  // Dense: the tiles of a head start at different units, so that their reductions do not meet in the same accumulator
-  // rows.  Sparse: tiles of a block walk its list in step, which keeps the gathered rows in the L2.
-  it.first_unit = DENSE ? (int)((long long)tile * it.n_units / tiles) : 0;
   return it;
-}
-// list unit worked on in step i of an item
-template <bool DENSE>
-__device__ __forceinline__ int unit_of(const KvItem& it, int i) {
-  if (!DENSE) return i;
-  const int u = it.first_unit + i;
-  return u >= it.n_units ? u - it.n_units : u;
 }
 
 // Walks the units of all items of this CTA, one per next().
@@ -140,8 +152,8 @@ template <bool DENSE>
 struct UnitWalk {
   KvItem it;
   int item, i, n_items, tiles, first, rows;
-  __device__ __forceinline__ UnitWalk(const KvParams& p, int n_items_, int tiles_)
-      : item((int)blockIdx.x - (int)gridDim.x), i(0), n_items(n_items_), tiles(tiles_), first(0), rows(0) { it.n_units = 0; }
+  __device__ __forceinline__ UnitWalk(int first_item, int n_items_, int tiles_)
+      : item(first_item - (int)gridDim.x), i(0), n_items(n_items_), tiles(tiles_), first(0), rows(0) { it.n_units = 0; }
   __device__ __forceinline__ bool next(const KvParams& p) {
     while (i >= it.n_units) {
       item += gridDim.x;
@@ -149,7 +161,7 @@ struct UnitWalk {
       it = kv_decode<DENSE>(p, item, tiles);
       i = 0;
     }
-    first = unit_of<DENSE>(it, i) * QU;
+    first = i * QU;
     rows = min(QU, it.n_list - first);
     ++i;
     return true;
@@ -171,6 +183,25 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 // 16-byte vector reduction into global memory (fp32 add)
 __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float c, float d) {
   asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+
+// Waits (bounded) until a turn counter has reached `turn`; the reductions of other threads follow a barrier.
+__device__ __forceinline__ void turn_wait(const int* addr, int turn, volatile int* abort_flag, int32_t* status) {
+  constexpr uint32_t kPolls = 1u << 22;
+  const uint32_t limit = *abort_flag ? 16u : kPolls;
+  for (uint32_t i = 0; i < limit; ++i) {
+    int at;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(at) : "l"(addr) : "memory");
+    if (at >= turn) return;
+    __nanosleep(32);
+  }
+  *abort_flag = 1;
+  set_status(status, VMOBA_ERR_TIMEOUT);
+}
+// Passes the turn on, at device scope: behind the reductions of the threads whose barrier this one has waited for.
+__device__ __forceinline__ void turn_pass(int* addr, int next) {
+  asm volatile("fence.acq_rel.gpu;" ::: "memory");
+  asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(addr), "r"(next) : "memory");
 }
 
 __device__ __forceinline__ uint32_t lo_k(uint32_t tile_addr) { return desc_lo(tile_addr, 16); }
@@ -260,7 +291,9 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     mbar_init(&sm->dp_full, 1); mbar_init(&sm->ds_ready, 256);
     mbar_init(&sm->dq_full, 1); mbar_init(&sm->dq_free, 256);
     mbar_init(&sm->acc_done, 1); mbar_init(&sm->acc_free, 256);
+    if constexpr (DENSE) { mbar_init(&sm->turn_ok, 1); mbar_init(&sm->rows_out, 256); mbar_init(&sm->rows_seen, 1); }
     sm->abort_flag = 0;
+    if constexpr (DENSE) sm->ticket = atomicAdd(p.turns + (long long)p.BH * ((p.S + QU - 1) / QU), 1);
     fence_barrier_init();
     prefetch_tmap(&tmK);
     prefetch_tmap(&tmV);
@@ -276,6 +309,9 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
 
   const int tiles = ((DENSE ? p.S : p.sb) + BN - 1) / BN;
   const int n_items = p.BH * (DENSE ? 1 : p.Nb) * tiles;
+  // dense: as many CTAs as items, one each
+  auto first_item = [&]() { return DENSE ? sm->ticket : (int)blockIdx.x; };
+  auto next_item = [&](int item) { return DENSE ? n_items : item + (int)gridDim.x; };
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
@@ -283,7 +319,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       // ---------------------------------------------------------------- TMA: K and V tiles, one pair per item
       if (lane == 0) {
         uint32_t n = 0;
-        for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+        for (int item = first_item(); item < n_items; item = next_item(item)) {
           const KvItem it = kv_decode<DENSE>(p, item, tiles);
           if (it.n_units == 0) continue;
           const int y = it.head_off + it.key0;
@@ -330,14 +366,14 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       const uint32_t kK = lo_k(smem_u32(sK)), kV = lo_k(smem_u32(sV)), mK = lo_mn(smem_u32(sK)), mS = lo_mn(smem_u32(sDS));
       const uint32_t kQ = lo_k(smem_u32(sQ)), kO = lo_k(smem_u32(sO)), mQ = lo_mn(smem_u32(sQ)), mO = lo_mn(smem_u32(sO));
       constexpr uint32_t STAGE = TILE >> 4;
-      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+      for (int item = first_item(); item < n_items; item = next_item(item)) {
         const KvItem it = kv_decode<DENSE>(p, item, tiles);
         // the list bounds come from memory: a warp reduction marks them as warp-uniform
         const int n_list = __reduce_max_sync(0xffffffffu, it.n_list);
         const int n_units = (n_list + QU - 1) / QU;
         if (n_units == 0) continue;
         const int key_steps = (it.valid + 15) >> 4;
-        auto rows16 = [&](int i) { return (min(QU, n_list - unit_of<DENSE>(it, i) * QU) + 15) >> 4; };   // 16-query steps of a unit
+        auto rows16 = [&](int i) { return (min(QU, n_list - i * QU) + 15) >> 4; };   // 16-query steps of a unit
         auto issue_s = [&](int i) {
           wwait(1, &sm->q_full[s_slot], s_par);
           tc_fence_after();
@@ -412,6 +448,22 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         ++n;
       }
       if (leader) tflush(2, 4);      // [2] k_full + v_full, [3] q_full + do_full, [4] p_ready + ds_ready, [5] dq_free + acc_free, [6] total
+    } else if (DENSE && lane == 0) {
+      // ---------------------------------------------------------------- turns: warp 3 waits for them, warp 2 passes them on.
+      // Warp 3 lets the writers go on only when warp 2 has noted the end of the unit before: no barrier gets a phase ahead.
+      const KvItem it = kv_decode<DENSE>(p, first_item(), tiles);
+      int* turn = p.turns + (long long)it.bh * it.n_units;
+      for (int i = 0; i < it.n_units; ++i) {
+        if (warp == 3) {
+          if (it.tile > 0) turn_wait(turn + i, it.tile, abort_flag, p.status);
+          if (i > 0) mbar_wait(&sm->rows_seen, (i - 1) & 1, abort_flag, p.status);
+          mbar_arrive(&sm->turn_ok);
+        } else {
+          mbar_wait(&sm->rows_out, i & 1, abort_flag, p.status);
+          mbar_arrive(&sm->rows_seen);
+          turn_pass(turn + i, it.tile + 1);
+        }
+      }
     }
   } else if (warp < 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
@@ -424,7 +476,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     // Dense: consecutive rows, TMA tiles requested by one of the threads that bring the scalars.
     const bool is_q = warp < 8;
     const int lt = threadIdx.x & 127, r0 = 4 * (warp & 3) + (lane >> 3), chunk = lane & 7;      // rows r0 + 16 k
-    UnitWalk<DENSE> walk(p, n_items, tiles);
+    UnitWalk<DENSE> walk(first_item(), n_items, tiles);
     const bool raster = !is_q && p.do_map.perm != nullptr;
     const long long stride = raster ? p.do_map.st : (long long)DH;
     const uint32_t tile0 = smem_u32(is_q ? sQ : sO);
@@ -508,11 +560,11 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const uint32_t dq_tmem = tmem + ((uint32_t)(quad * 32) << 16) + DPT_COL + 64 * qhalf;
     float* acc_col = p.dq_acc + quad * 32 + (lane & ~3);
     uint32_t g = 0;
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    for (int item = first_item(); item < n_items; item = next_item(item)) {
       const KvItem it = kv_decode<DENSE>(p, item, tiles);
       float* acc_head = acc_col + (long long)it.head_off * DH;
       for (int i = 0; i < it.n_units; ++i, ++g) {
-        const int first = unit_of<DENSE>(it, i) * QU + 64 * qhalf;
+        const int first = i * QU + 64 * qhalf;
         // accumulator rows of queries lane and 32 + lane of this half of the unit (-1 beyond the list)
         int row_lane[2];
 #pragma unroll
@@ -530,15 +582,28 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         tc_fence_before();
         mbar_arrive(&sm->dq_free);
         // A reduction holds its source registers until the load/store unit has taken them, so each has its own four.
+        auto write_rows = [&](auto put) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
+          for (int j = 0; j < 8; ++j)
 #pragma unroll
-          for (int e = 0; e < 2; ++e) {        // query 8 j + 2 (lane % 4) + e of this half
-            const int rw = __shfl_sync(0xffffffffu, row_lane[j >> 2], (8 * j + 2 * (lane & 3) + e) & 31);
-            if (rw >= 0)
-              red_add_v4(acc_head + (long long)rw * DH, __uint_as_float(x[0][4 * j + e]) * p.scale, __uint_as_float(x[0][4 * j + 2 + e]) * p.scale,
-                         __uint_as_float(x[1][4 * j + e]) * p.scale, __uint_as_float(x[1][4 * j + 2 + e]) * p.scale);
-          }
+            for (int e = 0; e < 2; ++e) {        // query 8 j + 2 (lane % 4) + e of this half
+              const int rw = __shfl_sync(0xffffffffu, row_lane[j >> 2], (8 * j + 2 * (lane & 3) + e) & 31);
+              if (rw >= 0)
+                put(acc_head + (long long)rw * DH, __uint_as_float(x[0][4 * j + e]) * p.scale, __uint_as_float(x[0][4 * j + 2 + e]) * p.scale,
+                    __uint_as_float(x[1][4 * j + e]) * p.scale, __uint_as_float(x[1][4 * j + 2 + e]) * p.scale);
+            }
+        };
+        auto add = [](float* to, float a, float b, float c, float d) { red_add_v4(to, a, b, c, d); };
+        if constexpr (DENSE) {
+          twait(1, &sm->turn_ok, g & 1);
+          if (it.tile == 0)
+            write_rows([](float* to, float a, float b, float c, float d) { *reinterpret_cast<float4*>(to) = make_float4(a, b, c, d); });
+          else
+            write_rows(add);
+          mbar_arrive(&sm->rows_out);
+        } else {
+          write_rows(add);
+        }
       }
     }
     if (warp == 20 && lane == 0) tflush(14, 1);     // [14] dq_full, [15] total
@@ -553,7 +618,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     const int mrow = quad * 32 + 8 * ((lane >> 3) & 1) + (lane & 7), mj = lane >> 4;
     const uint32_t ds_row = smem_u32(sDS) + half * PANEL + mrow * 128;
     uint32_t n = 0, g = 0, slot = 0, par = 0;        // items and units done; slot and parity of the Q ring
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    for (int item = first_item(); item < n_items; item = next_item(item)) {
       const KvItem it = kv_decode<DENSE>(p, item, tiles);
       if (it.n_units == 0) {
         // no query selected this block: its keys get zero gradients
@@ -711,7 +776,7 @@ static int launch(const Dims& D, const void* k, const void* v, KvParams& kp, cud
               (!kp.out_map.perm || (kp.out_map.sb % 16 == 0 && kp.out_map.st % 16 == 0 && kp.out_map.sh % 16 == 0));
   const long long items = (long long)D.BH * kp.Nb * ((kp.sb + BN - 1) / BN);
   if (items > (long long)INT32_MAX - 4096) return VMOBA_ERR_SHAPE;
-  const int grid = (int)std::max<long long>(1, std::min<long long>(items, sm_count()));
+  const int grid = DENSE ? (int)items : (int)std::max<long long>(1, std::min<long long>(items, sm_count()));
   auto kernel = kp.prof ? attn_bwd_fused_kernel<DENSE, true> : attn_bwd_fused_kernel<DENSE, false>;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
   launch_kernel(early_rows(D), kernel, grid, THREADS, SMEM_BYTES, st, tmK, tmV, tmQ, tmO, kp);
@@ -732,17 +797,23 @@ int tc_sparse_bwd(const Dims& D, const void* q, const void* k, const void* v, co
   kp.kb_ptr = kb_ptr; kp.q_idx = q_idx; kp.capacity = cap;
   kp.dk = (__nv_bfloat16*)dk; kp.dv = (__nv_bfloat16*)dv; kp.status = status;
   kp.dq_acc = dq_acc; kp.out_map = out_map; kp.do_map = do_map;
+  kp.turns = nullptr; kp.group = 1;
   return tcb::launch<false>(D, k, v, kp, st);
 }
 
-// Dense backward: every query of a head meets every key tile; dq_acc is zero everywhere.
+// Dense backward: every query of a head meets every key tile; turns holds tc_dense_bwd_turns() zeros, dq_acc anything.
+long long tc_dense_bwd_turns(const Dims& D) { return (long long)D.BH * ((D.S + tcb::QU - 1) / tcb::QU) + 1; }
 int tc_dense_bwd(const Dims& D, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
-                 const float* Dv, float* dq_acc, void* dk, void* dv, int32_t* status, cudaStream_t st) {
+                 const float* Dv, float* dq_acc, int* turns, void* dk, void* dv, int32_t* status, cudaStream_t st) {
   tcb::KvParams kp;
   kp.q = (const __nv_bfloat16*)q; kp.d_o = (const __nv_bfloat16*)d_o; kp.lse = lse; kp.Dv = Dv;
   kp.kb_ptr = nullptr; kp.q_idx = nullptr; kp.capacity = 0;
   kp.dk = (__nv_bfloat16*)dk; kp.dv = (__nv_bfloat16*)dv; kp.status = status;
-  kp.dq_acc = dq_acc;
+  kp.dq_acc = dq_acc; kp.turns = turns;
+  // Sixteen heads: their accumulators, Q and dO pass through the L2 once per SMs / 16 key tiles.  More where a head has so few
+  // units that its tiles would come too slowly for the SMs.
+  const int units = (D.S + tcb::QU - 1) / tcb::QU;
+  kp.group = std::min(D.BH, std::max(16, sm_count() / units));
   return tcb::launch<true>(D, k, v, kp, st);
 }
 
