@@ -241,11 +241,16 @@ class SteppedAttention:
             # the dense kernels take [B, heads, S, d].  The tokens stay in raster order: the running maximum that a row's
             # weights are rounded against, and with it the last bits of o, depends on the order of the keys.
             L, one = self.layer, self._one_block
-            q, k, v = (x if L.partitions(x) else x.contiguous() for x in (q, k, v))
+            # (a fresh tensor, not contiguous(): that returns a contiguous tensor as it is, whatever its address, the strides
+            # of its dimensions of size one and its type)
+            fresh = lambda x: torch.empty(x.shape, dtype=L.q_bm.dtype, device=L.device)
+            q, k, v = (x if L.partitions(x) else fresh(x).copy_(x) for x in (q, k, v))
             qd, kd, vd, od = (torch.empty_like(L.q_bm) for _ in range(4))
             vb.vmoba_partition_many(one, 0, (q, k, v), (qd, kd, vd), [L.raster_strides(x) for x in (q, k, v)])
             vb.vmoba_full_attn(L.shape, qd, kd, vd, od, self._lse, dev_status=L.dev_status)
-            o = o_out if L.partitions(o_out) else torch.empty(o_out.shape, dtype=L.q_bm.dtype, device=L.device)
+            # (an o_out whose elements share memory goes through copy_, which refuses it)
+            shared = any(st == 0 and n > 1 for st, n in zip(o_out.stride(), o_out.shape))
+            o = o_out if L.partitions(o_out) and not shared else fresh(o_out)
             vb.vmoba_partition(one, 1, od, o, L.raster_strides(o))
             if o is not o_out:
                 o_out.copy_(o)

@@ -79,3 +79,44 @@ def test_dense_step_keeps_the_raster_order(dtype, d):
     vb.vmoba_full_attn(shape, qh, kh, vh, ref, lse, dev_status=L.dev_status)
     L.check_status()
     assert torch.equal(o, ref.permute(0, 2, 1, 3))
+
+
+def _placed(x, how):
+    """The values of x in a tensor that lies in memory otherwise."""
+    if how == "offset":                                     # contiguous, one element off a 16-byte boundary
+        y = torch.empty(x.numel() + 1, dtype=x.dtype, device="cuda")[1:].view(x.shape)
+    elif how == "batch_stride":                             # one batch whose stride is no multiple of 16 bytes
+        y = torch.empty(x.numel(), dtype=x.dtype, device="cuda").as_strided(x.shape, (x.numel() + 3, *x.stride()[1:]))
+    else:
+        y = torch.empty(x.shape, dtype=how, device="cuda")
+    return y.copy_(x)
+
+
+@pytest.mark.parametrize("how", ["offset", "batch_stride", torch.float32, torch.bfloat16], ids=str)
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_dense_step_takes_any_placement_and_type(dtype, how):
+    shape = vb.make_shape(1, 2, 64, (2, 8, 8), (1, 4, 4), dtype)
+    L = VmobaLayer(shape, 4096)
+    stepped = SteppedAttention(L, 0.25, 1, 1.0)
+    torch.manual_seed(6)
+    qkv = [torch.randn(1, shape.S, 2, 64, device="cuda").to(torch.bfloat16).to(L.q_bm.dtype) for _ in range(3)]
+    o = torch.empty_like(qkv[0])
+    stepped.forward(0, *qkv, o)
+    o2 = _placed(torch.zeros_like(o), how)
+    stepped.forward(0, *[_placed(x, how) for x in qkv], o2)
+    L.check_status()
+    assert torch.equal(o2, o.to(o2.dtype))
+
+
+def test_dense_step_takes_expanded_inputs_and_refuses_an_expanded_output():
+    shape = vb.make_shape(2, 2, 64, (2, 8, 8), (1, 4, 4), "f32")
+    L = VmobaLayer(shape, 4096)
+    stepped = SteppedAttention(L, 0.25, 1, 1.0)
+    torch.manual_seed(6)
+    q, kv = torch.randn(2, shape.S, 2, 64, device="cuda"), torch.randn(1, shape.S, 2, 64, device="cuda")
+    o, want = torch.empty_like(q), torch.empty_like(q)
+    stepped.forward(0, q, kv.expand_as(q), kv.expand_as(q), o)
+    stepped.forward(0, q, kv.expand_as(q).clone(), kv.expand_as(q).clone(), want)
+    assert torch.equal(o, want)
+    with pytest.raises(RuntimeError):
+        stepped.forward(0, q, q, q, torch.empty(1, shape.S, 2, 64, device="cuda").expand_as(q))
