@@ -1362,7 +1362,11 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
                 w.seg_cnt, w.kb_total, D.Nb, nseg);
   launch_kernel(offsets_kernel, 1, 1024, 0, st, w.kb_total, kb_ptr, nkb, w.seg_total, w.seg_qoff,
                 (long long)D.BH * nseg, D.BH, D.Nb, k_per_head, capacity, q_ptr + (long long)D.BH * D.S, dev_status);
-  launch_kernel(fill_kernel, sgrid, QSEG, smem_fill, st, mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg,
+  // A thread per query of the segment; many blocks leave short segments (32 queries from 2,049 blocks on), whose columns and
+  // runs want the threads all the same: 2,100 blocks x 33,600 queries 1001 -> 432 us (whole selection, threshold rule), 8,192 x
+  // 16,384 3376 -> 1053.
+  const int fill_threads = QSEG >= 128 ? QSEG : kSegThreads;
+  launch_kernel(fill_kernel, sgrid, fill_threads, smem_fill, st, mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg,
                 kb_ptr, w.seg_cnt, w.seg_qoff, q_idx, q_ptr, q_pairs, capacity);
   VMOBA_LAUNCH_OK(3);
   VMOBA_GUARDS_CHECK(w.guards, dev_status, st);

@@ -43,6 +43,18 @@ def test_lists_match_the_mask(heads, S, nb):
     assert _check_lists(L) > 0
 
 
+@pytest.mark.parametrize("heads, S, nb", [(2, 2048, 1024), (2, 2050, 1025), (1, 4098, 2049), (1, 8192, 8192)])
+def test_lists_of_short_segments(heads, S, nb):
+    """So many blocks that a segment has fewer than 128 queries (from 1,025 on; 32 from 2,049 on): more threads than queries."""
+    shape = vb.make_shape(1, heads, 64, (nb, 1, S // nb), (1, 1, S // nb), "f32")
+    L = VmobaLayer(shape, heads * S * 64)
+    torch.manual_seed(nb)
+    for _ in range(2):
+        L.select_rule(vb.SELECT_TOPK_GLOBAL, topk=17, scores=torch.randn(L.scores.shape, device="cuda"))
+        L.check_status()
+        assert _check_lists(L) == heads * S * 17
+
+
 @pytest.mark.parametrize("spread", [1.0, 1e-2, 1e-4], ids=["spread", "few_bins", "one_bin"])
 def test_crowded_bins(spread):
     shape = vb.make_shape(1, 2, 128, (64, 1, 64), (1, 1, 64), "bf16")
