@@ -676,12 +676,17 @@ __device__ __forceinline__ float max_nan(float a, float b) {
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
   return d;
 }
-__device__ __forceinline__ uint32_t bits_of(float x) {
-  uint32_t u;
-  asm("mov.b32 %0, %1;" : "=r"(u) : "f"(x));
-  return u;
+// over a converged warp (sm_100: on floats as they are)
+__device__ __forceinline__ float warp_max_nan(float x) {
+  float d;
+  asm volatile("redux.sync.max.NaN.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(x));
+  return d;
 }
-constexpr uint32_t kInfKey = 0xff800000u;      // key of +inf: a larger one is a NaN's
+__device__ __forceinline__ float warp_min(float x) {
+  float d;
+  asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(x));
+  return d;
+}
 
 // Top-k per query, one warp per row: lane l holds blocks l + 32 i.  Search over the row's score range for a threshold
 // that k scores reach; it usually ends early, on a threshold that exactly k scores reach, and otherwise on the k-th
@@ -736,11 +741,10 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
     src += Nb;
     if (row + 1 < row_end) load_row(src);
     // invariant: at least k scores reach lo, fewer than k reach hi (or lo == hi)
-    float lo = key_float(__reduce_min_sync(0xffffffffu, float_key(mn)));
-    const uint32_t mx_bits = bits_of(mx), top = __reduce_max_sync(0xffffffffu, (mx_bits & 0x80000000u) ? ~mx_bits : (mx_bits | 0x80000000u));
-    float hi = key_float(top);
+    float lo = warp_min(mn), hi = warp_max_nan(mx);
+    const bool has_nan = hi != hi;
     bool exact = false;                 // exactly k scores reach lo
-    if (k < Nb && top <= kInfKey) {
+    if (k < Nb && !has_nan) {
       // (a block the row does not have counts as -inf, which no threshold above the row's minimum lets through)
       auto count_ge = [&](float c) {
         int n = 0;
@@ -752,7 +756,7 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
       bool below = false, above = false;
       if (!(mid > lo && mid < hi) && !split_interval(lo, hi, mid)) {
         lo = hi;                        // two neighbouring values at most: is the larger one the k-th?
-        if (count_ge(hi) < k) lo = key_float(__reduce_min_sync(0xffffffffu, float_key(mn)));
+        if (count_ge(hi) < k) lo = warp_min(mn);
       } else {
         for (;;) {
           const int n = count_ge(mid);
@@ -772,7 +776,7 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
       }
     }
     uint32_t my_word = 0u;
-    if (top > kInfKey) {
+    if (has_nan) {
       // the largest key that k blocks reach, bit by bit; blocks above it, and those at it in block order.  (The row is read
       // again word by word: rare, and with the registers of the other search it would cost that one its warps.)
       const uint32_t* sr = reinterpret_cast<const uint32_t*>(scores) + row * Nb + lane;
