@@ -65,6 +65,12 @@ static int grid_for(long long items, int per_sm) {
   return (int)std::max<long long>(g, 1);
 }
 
+// Whether the CUDA-core kernels are launched ahead of the end of the kernel before them.  Several of their CTAs share an SM, and
+// early ones go where that kernel has left room: two to an SM while others stay empty, which costs a long kernel more than the
+// launch it saves.  Dense forward and backward, early against not: 4 heads x 2,000 tokens (bf16, head_dim 64) 1842 / 1366 us,
+// 12 x 512 483 / 370; a sparse forward of 4 x 256 (three early launches) 31 / 39.  pairs: (query, key) pairs at most.
+static bool early_simt(const Dims& D, double pairs) { return pairs * D.d <= (double)(1 << 26); }
+
 template <typename T, int DH>
 static int simt_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, const int* kb_ptr,
                            const int* q_idx, const int* q_ptr, const int* q_pairs, long long cap, void* o,
@@ -74,7 +80,7 @@ static int simt_sparse_fwd(const Dims& D, const void* q, const void* k, const vo
   const long long n_kb = (long long)D.BH * D.Nb;
   launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
   long long max_items = cap / simt::kRows + n_kb;
-  launch_kernel(simt::attn_fwd_kernel<T, DH, false>, grid_for(max_items, 8), simt::kThreads, 0, st, (const T*)q,
+  launch_kernel(early_simt(D, (double)cap * D.sb), simt::attn_fwd_kernel<T, DH, false>, grid_for(max_items, 8), simt::kThreads, 0, st, (const T*)q,
                 (const T*)k, (const T*)v, kb_ptr, q_idx, q_ptr, w.item_ptr, (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale,
                 (T*)o, (T*)o_resid, lse, w.part_o, w.part_lse, cap);
   long long nq = (long long)D.BH * D.S;
@@ -117,10 +123,11 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
   VMOBA_CUDA_OK(cudaMemsetAsync(w.dq_acc, 0, (size_t)nq * DH * sizeof(float), st));
   launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
   long long tiles = (D.sb + simt::kRows - 1) / simt::kRows;
-  launch_kernel(simt::attn_bwd_dkdv_kernel<T, DH, false>, grid_for(n_kb * tiles, 4), simt::kThreads, 0, st,
+  const bool early = early_simt(D, (double)cap * D.sb);
+  launch_kernel(early, simt::attn_bwd_dkdv_kernel<T, DH, false>, grid_for(n_kb * tiles, 4), simt::kThreads, 0, st,
                 (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb, D.BH,
                 D.scale, cap, (T*)dk, (T*)dv);
-  launch_kernel(simt::attn_bwd_dq_kernel<T, DH, false>, grid_for(nq / simt::kRows * D.Nb + n_kb, 4), simt::kThreads,
+  launch_kernel(early, simt::attn_bwd_dq_kernel<T, DH, false>, grid_for(nq / simt::kRows * D.Nb + n_kb, 4), simt::kThreads,
                 0, st, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, w.item_ptr,
                 (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale, cap, w.dq_acc, (T*)dq);
   launch_kernel(early_rows(D), simt::cast_kernel<T>, grid_for((nq * DH / 4 + 255) / 256, 16), 256, 0, st, w.dq_acc,
@@ -136,11 +143,12 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
   const long long nq = (long long)D.BH * D.S;
   const long long tiles = (D.S + simt::kRows - 1) / simt::kRows;
   BwdWs w = carve_bwd(D, true, d_o ? ws : nullptr);
+  const bool early = early_simt(D, (double)D.BH * D.S * D.S);
   if (use_tensor_cores(D)) {
     int rc = tc_dense_fwd(D, q, k, v, o, d_o ? w.o_resid : nullptr, lse, status, st);
     if (rc) return rc;
   } else {
-    launch_kernel(simt::attn_fwd_kernel<T, DH, true>, grid_for(D.BH * tiles, 8), simt::kThreads, 0, st, (const T*)q,
+    launch_kernel(early, simt::attn_fwd_kernel<T, DH, true>, grid_for(D.BH * tiles, 8), simt::kThreads, 0, st, (const T*)q,
                   (const T*)k, (const T*)v, nullptr, nullptr, nullptr, nullptr, 0, D.S, 1, D.S, D.BH, D.scale, (T*)o,
                   d_o ? (T*)w.o_resid : nullptr, lse, nullptr, nullptr, 0);
     count_launches(1);
@@ -159,10 +167,10 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
       VMOBA_LAUNCH_OK(1);
       return VMOBA_OK;
     }
-    launch_kernel(simt::attn_bwd_dkdv_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, 0, st,
+    launch_kernel(early, simt::attn_bwd_dkdv_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, 0, st,
                   (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, D.S, 1, D.S,
                   D.BH, D.scale, 0, (T*)dk, (T*)dv);
-    launch_kernel(simt::attn_bwd_dq_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, 0, st,
+    launch_kernel(early, simt::attn_bwd_dq_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, 0, st,
                   (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, nullptr, 0, D.S,
                   1, D.S, D.BH, D.scale, 0, nullptr, (T*)dq);
   }
