@@ -55,3 +55,48 @@ def test_planted_out_of_range_entry_is_reported_by_the_range_checked_build():
     lines = dict(l.split() for l in r.stdout.strip().splitlines() if l.split()[0] in ("clean", "planted"))
     assert lines["clean"] == "0"
     assert lines["planted"] == "8"          # VMOBA_ERR_BOUNDS
+
+
+CHAIN = r"""
+import sys, torch
+from paper_2506_23858_b200 import binding as vb
+from paper_2506_23858_b200.layer import SteppedAttention, VmobaLayer
+out = []
+for dtype, grid, block, heads, d in (("f32", (1, 8, 8), (1, 4, 4), 2, 64), ("bf16", (4, 16, 16), (2, 4, 8), 3, 128),
+                                     ("bf16", (6, 12, 26), (3, 6, 13), 12, 128), ("bf16", (9, 32, 32), (3, 8, 16), 8, 128)):
+    shape = vb.make_shape(1, heads, d, grid, block, dtype)
+    L = VmobaLayer(shape, 4 * heads * shape.S, with_backward=True)
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    sets = [[torch.randn(1, shape.S, heads, d, device="cuda", generator=gen).to(L.q_bm.dtype) for _ in range(4)] for _ in range(2)]
+    for i in (0, 1, 0, 1):
+        q, k, v, do = sets[i]
+        o, dq, dk, dv, dense = (torch.empty_like(q) for _ in range(5))
+        # (the head-wide top-k counts pairs where the threshold rule adds weights in any order: the same kernels, and the
+        # same bits from run to run)
+        L.partition_many((v, q, k), (L.v_bm, L.q_bm, L.k_bm), perm=L.perm)
+        L.block_scores()
+        L.select_rule(vb.SELECT_TOPK_GLOBAL, topk=2)
+        L.attn_fwd()
+        L.partition(o, L.o_bm, inverse=True)
+        L.backward(do, dq, dk, dv)
+        n = int(L.k_per_head.sum())
+        out += [x.cpu() for x in (o, L.lse, dk, dv, L.mask_bits, L.kb_ptr, L.q_ptr, L.q_idx[:n], L.q_pairs[:n])]
+        L.select_rule(vb.SELECT_TOPK_LOCAL, topk=3)
+        SteppedAttention(L, 0.25, 1, 1.0).forward(0, q, k, v, dense)
+        out += [L.mask_bits.cpu(), dense.cpu()]
+    L.check_status()
+torch.save(out, sys.argv[1])
+"""
+
+
+def test_overlapped_launches_give_what_serialised_ones_give(tmp_path):
+    """The range-checked build launches every kernel after the end of the one before it; the library itself sets most of them
+    up while that one still runs.  Forward, backward, selections and dense step over two sets of inputs in turn: bit for bit
+    the same (dQ apart, whose parts come in any order)."""
+    import torch
+    for name, env in (("overlapped", dict(os.environ)), ("serialised", _debug_env())):
+        r = subprocess.run([sys.executable, "-c", CHAIN, str(tmp_path / name)], env=env, cwd=ROOT, capture_output=True, text=True,
+                           timeout=600)
+        assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-2000:]
+    a, b = (torch.load(tmp_path / n) for n in ("overlapped", "serialised"))
+    assert len(a) == len(b) and all(torch.equal(x, y) for x, y in zip(a, b))

@@ -1,5 +1,6 @@
-"""Forwards on both sides of the sizes (1,024 lists, 4,096 items) up to which one CTA writes the items' offsets and records,
-with lists of very different lengths: every query's result against plain softmax attention over its blocks."""
+"""Forwards on both sides of the sizes (1,024 lists; room for 4,096 items, which is capacity / 128 + lists + 1) up to which one
+CTA writes the items' offsets and records, with lists of very different lengths: every query's result against plain softmax
+attention over its blocks."""
 import pytest
 import torch
 
@@ -10,8 +11,10 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("heads, nb, sb, capacity", [(4, 256, 2, 300000), (4, 257, 2, 300000), (1, 8, 300, 8 * 2400),
-                                                     (1, 8, 300, 1 << 20), (2, 8, 400, 1 << 21)],
-                         ids=["1024_lists", "1028_lists", "few_items", "4105_items", "wide_8k_items"])
+                                                     (1, 8, 300, 4087 * 128), (1, 8, 300, 4088 * 128), (4, 40, 50, 3935 * 128),
+                                                     (4, 40, 50, 3936 * 128), (1, 8, 300, 1 << 20), (2, 8, 400, 1 << 21)],
+                         ids=["1024_lists", "1028_lists", "159_items", "4096_items", "4097_items", "narrow_4096_items",
+                              "narrow_4097_items", "8201_items", "16401_items"])
 def test_lists_of_any_length(heads, nb, sb, capacity):
     shape = vb.make_shape(1, heads, 128, (nb, sb, 1), (1, sb, 1), "bf16")
     S = shape.S
