@@ -62,6 +62,7 @@ struct KvSmem {
   uint64_t dq_full, dq_free;                                       // dQ^T complete (commit) / read out of TMEM (256 arrivals)
   uint64_t acc_done, acc_free;                                     // dV / dK of an item complete (commit) / read (256 arrivals)
   uint64_t turn_ok, rows_out, rows_seen;                           // dense: it is this tile's turn / its dQ is on the way (256 arrivals) / and noted
+  uint64_t drain;                                                  // (after a time-out only)
   uint32_t tmem_base;
   int ticket;                                // dense: the CTA's item
   int abort_flag;
@@ -269,10 +270,11 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   auto twait = [&](int site, uint64_t* bar, uint32_t parity) {
     if constexpr (PROF) {
       const long long t0 = clock64();
-      mbar_wait(bar, parity, abort_flag, p.status);
+      const bool ok = mbar_wait(bar, parity, abort_flag, p.status);
       wp[site] += (unsigned long long)(clock64() - t0);
+      return ok;
     } else {
-      mbar_wait(bar, parity, abort_flag, p.status);
+      return mbar_wait(bar, parity, abort_flag, p.status);
     }
   };
   auto tflush = [&](int base_site, int nsites) {
@@ -291,6 +293,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     mbar_init(&sm->dp_full, 1); mbar_init(&sm->ds_ready, 256);
     mbar_init(&sm->dq_full, 1); mbar_init(&sm->dq_free, 256);
     mbar_init(&sm->acc_done, 1); mbar_init(&sm->acc_free, 256);
+    mbar_init(&sm->drain, 1);
     if constexpr (DENSE) { mbar_init(&sm->turn_ok, 1); mbar_init(&sm->rows_out, 256); mbar_init(&sm->rows_seen, 1); }
     sm->abort_flag = 0;
     if constexpr (DENSE) sm->ticket = atomicAdd(p.turns + (long long)p.BH * ((p.S + QU - 1) / QU), 1);
@@ -319,16 +322,17 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       // ---------------------------------------------------------------- TMA: K and V tiles, one pair per item
       if (lane == 0) {
         uint32_t n = 0;
+        bool v_ahead = false;      // (nothing is loaded after a time-out)
         for (int item = first_item(); item < n_items; item = next_item(item)) {
           const KvItem it = kv_decode<DENSE>(p, item, tiles);
           if (it.n_units == 0) continue;
           const int y = it.head_off + it.key0;
           // V is free after the item's last dP^T, K only after its last dQ^T
-          if (n >= 1) twait(0, &sm->v_empty, (n - 1) & 1);
+          if (n >= 1 && !twait(0, &sm->v_empty, (n - 1) & 1)) break;
           mbar_expect_tx(&sm->v_full, TILE);
           tma_load_2d(sV, &tmV, &sm->v_full, 0, y);
           tma_load_2d(sV + PANEL, &tmV, &sm->v_full, 64, y);
-          if (n >= 1) twait(0, &sm->k_empty, (n - 1) & 1);
+          if (n >= 1 && !twait(0, &sm->k_empty, (n - 1) & 1)) { v_ahead = true; break; }
           mbar_expect_tx(&sm->k_full, TILE);
           tma_load_2d(sK, &tmK, &sm->k_full, 0, y);
           tma_load_2d(sK + PANEL, &tmK, &sm->k_full, 64, y);
@@ -346,7 +350,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         // drain: every issued load must have landed before the CTA may exit (only matters after a timeout)
         if (*abort_flag && n > 0) {
           mbar_wait(&sm->k_full, (n - 1) & 1, abort_flag, p.status);
-          mbar_wait(&sm->v_full, (n - 1) & 1, abort_flag, p.status);
+          mbar_wait(&sm->v_full, (n - (v_ahead ? 0 : 1)) & 1, abort_flag, p.status);
         }
         tflush(0, 1);      // [0] k_empty + v_empty, [1] total
       }
@@ -447,6 +451,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         g += n_units;
         ++n;
       }
+      if (leader && *abort_flag) mma_drain(&sm->drain);
       if (leader) tflush(2, 4);      // [2] k_full + v_full, [3] q_full + do_full, [4] p_ready + ds_ready, [5] dq_free + acc_free, [6] total
     } else if (DENSE && lane == 0) {
       // ---------------------------------------------------------------- turns: warp 3 waits for them, warp 2 passes them on.

@@ -50,6 +50,7 @@ struct Smem {
   uint64_t q_full, q_empty;          // Q tile of an item gathered (64 arrivals) / no longer needed (commit)
   uint64_t ep_ready;                 // an item's normalisers are in ep_inv / ep_lse (128 softmax arrivals)
   uint64_t o_free;                   // the epilogue warps have read them and the accumulator (128 arrivals)
+  uint64_t drain;                    // (after a time-out only)
   uint32_t tmem_base;
   int abort_flag;
   float ep_inv[2][BM], ep_lse[2][BM];   // [item % 2][row]: 1 / sum of the rounded weights, natural-log lse
@@ -214,6 +215,7 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     mbar_init(&sm->o_done, 1);
     mbar_init(&sm->q_full, 64); mbar_init(&sm->q_empty, 1);
     mbar_init(&sm->ep_ready, 128); mbar_init(&sm->o_free, 128);
+    mbar_init(&sm->drain, 1);
     sm->abort_flag = 0;
     fence_barrier_init();
     prefetch_tmap(&tmK);
@@ -247,27 +249,28 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     // ------------------------------------------------------------------ TMA producer
     if (lane == 0) {
       uint32_t fills = 0;
-      for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+      bool go = true, k_ahead = false;      // (nothing is loaded after a time-out)
+      for (int item = blockIdx.x; go && item < n_items; item += gridDim.x) {
         const Item it = get_item(item);
         const int row0 = (int)it.head_off + it.key_begin;
         for (int t = 0; t < it.ntiles; ++t, ++fills) {
           const uint32_t par = (fills - 1) & 1;
           const int y = row0 + t * BN;
           // the K stage is free once the Q K^T of the tile before has run, the V stage after its P V
-          if (fills >= 1) mbar_wait(&sm->k_empty, par, abort_flag, p.status);
+          if (fills >= 1 && !mbar_wait(&sm->k_empty, par, abort_flag, p.status)) { go = false; break; }
           mbar_expect_tx(&sm->k_full, TILE);
           tma_load_2d(sK, &tmK, &sm->k_full, 0, y);
           tma_load_2d(sK + PANEL, &tmK, &sm->k_full, 64, y);
-          if (fills >= 1) mbar_wait(&sm->v_empty, par, abort_flag, p.status);
+          if (fills >= 1 && !mbar_wait(&sm->v_empty, par, abort_flag, p.status)) { go = false; k_ahead = true; break; }
           mbar_expect_tx(&sm->v_full, TILE);
           tma_load_2d(sV, &tmV, &sm->v_full, 0, y);
           tma_load_2d(sV + PANEL, &tmV, &sm->v_full, 64, y);
         }
       }
       // drain: every issued load must have landed before the CTA may exit (only matters after a timeout)
-      if (*abort_flag && fills >= 1) {
-        mbar_wait(&sm->k_full, (fills - 1) & 1, abort_flag, p.status);
-        mbar_wait(&sm->v_full, (fills - 1) & 1, abort_flag, p.status);
+      if (*abort_flag) {
+        if (fills >= 1 || k_ahead) mbar_wait(&sm->k_full, (fills - (k_ahead ? 0 : 1)) & 1, abort_flag, p.status);
+        if (fills >= 1) mbar_wait(&sm->v_full, (fills - 1) & 1, abort_flag, p.status);
       }
     }
   } else if (warp == 1) {
@@ -327,6 +330,7 @@ attn_fwd_narrow_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_con
     }
     lap(5);
     if (leader) tflush(8);
+    if (leader && *abort_flag) mma_drain(&sm->drain);
   } else if (warp < 4) {
     // ------------------------------------------------------------------ loaders: Q rows of the next item
     const int lt = (warp - 2) * 32 + lane;   // 0..63

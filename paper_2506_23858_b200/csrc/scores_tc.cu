@@ -40,6 +40,7 @@ struct Smem {
   uint64_t q_full[NQ_MAX], q_empty[NQ_MAX];
   uint64_t b_full, b_empty;
   uint64_t acc_full[2], acc_empty[2];
+  uint64_t drain;                         // (after a time-out only)
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -111,6 +112,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     }
     mbar_init(&sm->b_full, 1);
     mbar_init(&sm->b_empty, 1);
+    mbar_init(&sm->drain, 1);
     sm->abort_flag = 0;
     fence_barrier_init();
     prefetch_tmap(&tmQ);
@@ -148,7 +150,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         const long long bh = group / p.n_pass;
         if (group != cur_group) {
           // new centroid range: wait until the MMAs that read the old one are done
-          if (bn > 0) mbar_wait(&sm->b_empty, (bn - 1) & 1, abort_flag, p.status);
+          if (bn > 0 && !mbar_wait(&sm->b_empty, (bn - 1) & 1, abort_flag, p.status)) break;      // (nothing is loaded after a time-out)
           const int y0 = (int)(bh * p.Nb_pad + (long long)pass * p.rows_pass);
           mbar_expect_tx(&sm->b_full, 3 * 2 * p.rows_pass * 128);
           for (int part = 0; part < 3; ++part) {
@@ -159,8 +161,8 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
           cur_group = group;
           ++bn;
         }
-        if (filled == nq) mbar_wait(&sm->q_empty[s], ph, abort_flag, p.status);
-        else ++filled;
+        if (filled < nq) ++filled;
+        else if (!mbar_wait(&sm->q_empty[s], ph, abort_flag, p.status)) break;
         const int y = (int)(bh * p.S) + tile * BM;
         mbar_expect_tx(&sm->q_full[s], TILE);
         tma_load_2d(sQ + s * TILE, &tmQ, &sm->q_full[s], 0, y);
@@ -211,6 +213,7 @@ scores_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         if (leader) mma_commit(&sm->acc_full[e]);
         if (++s == nq) { s = 0; ph ^= 1; }
       }
+      if (leader && *abort_flag) mma_drain(&sm->drain);
     }
   } else {
     // ------------------------------------------------------------------ epilogue: thread = query row

@@ -131,24 +131,6 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* map, int x, i
                "r"(y)
                : "memory");
 }
-// Row gather: four rows (given by their row coordinates) of a 2D tensor whose map has a one-row
-// box of 64 columns; the rows land in four consecutive 128-byte rows at smem_dst with the same
-// 128-byte swizzle a tiled load produces, so a 128-row operand tile is 32 of these per panel.
-__device__ __forceinline__ void tma_gather4(void* smem_dst, const CUtensorMap* map, uint64_t* bar, int col, int r0, int r1,
-                                            int r2, int r3) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, "
-      "%6, %7}], [%2];" ::"r"(smem_u32(smem_dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(col), "r"(r0), "r"(r1), "r"(r2), "r"(r3)
-      : "memory");
-}
-// One warp gathers a [128 x 128] bf16 tile (two 64-column panels of 16 KB): lane l fetches tile rows
-// 4l .. 4l+3.  rows[k] are absolute row coordinates of this lane's four rows.
-__device__ __forceinline__ void tma_gather_tile128(uint8_t* tile, const CUtensorMap* map, uint64_t* bar, int lane,
-                                                   const int (&rows)[4]) {
-  tma_gather4(tile + lane * 512, map, bar, 0, rows[0], rows[1], rows[2], rows[3]);
-  tma_gather4(tile + 16384 + lane * 512, map, bar, 64, rows[0], rows[1], rows[2], rows[3]);
-}
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
@@ -243,6 +225,14 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// After a time-out: what the tensor pipe was given by this thread has run (bounded) before the CTA frees its TMEM and exits.
+// bar: a barrier of one arrival that nothing else uses.
+__device__ __forceinline__ void mma_drain(uint64_t* bar) {
+  mma_commit(bar);
+  for (uint32_t i = 0; i < (1u << 16); ++i)
+    if (mbar_try_wait(bar, 0)) return;
+}
+
 // ---------------------------------------------------------------- TMEM <-> registers (warp-wide, lane = row)
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
   asm volatile(
@@ -264,11 +254,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr)
       : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(r[0]),
-               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
 }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
   asm volatile(
