@@ -3,9 +3,9 @@
 
 A step is one pass of the whole layer over one batch of synthetic video-DiT-shaped input:
 partition(q, k, v) -> centroids + scores -> global threshold selection -> sparse attention
-forward -> inverse partition(o), and for training workloads the backward:
-partition(dO) -> sparse attention backward writing dq, dk, dv in raster order (bf16, head_dim 128;
-otherwise the backward followed by the inverse partitions of the gradients).  Workloads with
+forward -> inverse partition(o), and for training workloads the backward, as the layer runs it: sparse
+attention backward reading dO and writing dq, dk, dv in raster order (bf16, head_dim 128; otherwise
+partition(dO), the backward and the inverse partitions of the gradients).  Workloads with
 several partitions (c3, c5) run the layer once per partition (1D, 2D, 3D) per step.
 
     python bench.py --gpus 1 --steps 20 --warmup 3                # default workload: c5
@@ -267,7 +267,7 @@ def main():
     ap.add_argument("--no-fold", action="store_true",
                     help="partition dO and inverse-partition dq, dk, dv in passes of their own (instead of the backward reading / writing raster order)")
     ap.add_argument("--fold-do", action="store_true",
-                    help="also let the backward read dO in raster order (pays with few heads: c4 yes, c5 no)")
+                    help="let the attention kernel itself read dO in raster order (by default the pass before it leaves a block-major copy)")
     ap.add_argument("--fold-o", action="store_true",
                     help="let the forward write o in raster order (saves the inverse partition pass of o; measured slower)")
     ap.add_argument("--heads", type=int, default=0, help="override the number of heads (small profiling runs)")
@@ -352,8 +352,7 @@ def main():
 
         for layer in L:
             mark("start")
-            layer.partition(dev["q"], layer.q_bm, perm=layer.perm); layer.partition(dev["k"], layer.k_bm)
-            layer.partition(dev["v"], layer.v_bm)
+            layer.partition_many((dev["v"], dev["q"], dev["k"]), (layer.v_bm, layer.q_bm, layer.k_bm), perm=layer.perm)
             mark("partition")
             layer.block_scores(); mark("scores")
             do_select(layer, layer_w[id(layer)], layer_pos[id(layer)]); mark("select")
@@ -367,16 +366,15 @@ def main():
                     # the backward kernels read dO and write dq, dk, dv in raster order themselves (Eq. 1 folded in)
                     layer.attn_bwd_raster(dev["do"], outs["dq"], outs["dk"], outs["dv"]); mark("attn_bwd")
                 elif fold:
-                    layer.partition(dev["do"], layer.do_bm); mark("partition")
-                    layer.attn_bwd_raster(None, outs["dq"], outs["dk"], outs["dv"]); mark("attn_bwd")
+                    # the pass that takes rowsum(dO * O) leaves dO in block-major order on the way
+                    layer.attn_bwd_raster(dev["do"], outs["dq"], outs["dk"], outs["dv"], keep_do=True); mark("attn_bwd")
                 else:
                     layer.partition(dev["do"], layer.do_bm); mark("partition")
                     if layer.o_raster is not None:
                         layer.partition(layer.o_raster, layer.o_bm)
                     layer.attn_bwd(); mark("attn_bwd")
-                    layer.partition(outs["dq"], layer.dq_bm, inverse=True)
-                    layer.partition(outs["dk"], layer.dk_bm, inverse=True)
-                    layer.partition(outs["dv"], layer.dv_bm, inverse=True)
+                    layer.partition_many((outs["dq"], outs["dk"], outs["dv"]), (layer.dq_bm, layer.dk_bm, layer.dv_bm),
+                                         inverse=True)
                     mark("partition")
         return evs
 
@@ -507,10 +505,9 @@ def main():
 
     es = 2 if w0.dtype == "bf16" else 4
     tensor_bytes = w0.B * w0.S * w0.heads * w0.head_dim * es
-    # partition passes of a step: q, k, v in; o out unless the forward writes raster order; dO in unless the backward
-    # reads raster order; dq, dk, dv out unless the backward writes raster order
-    n_part = len(layers) * (3 + (0 if fold_o else 1)
-                            + ((0 if (fold and args.fold_do) else 1) + (0 if fold else 3) if with_bwd else 0))
+    # partition passes of a step: q, k, v in; o out unless the forward writes raster order; dO in and dq, dk, dv out unless
+    # the backward reads and writes raster order
+    n_part = len(layers) * (3 + (0 if fold_o else 1) + (4 if with_bwd and not fold else 0))
     alg = {
         "partition": ("hbm", 2.0 * tensor_bytes * n_part),
         "scores": ("hbm", sum(2.0 * tensor_bytes + 4.0 * w.B * w.heads * (w.S * w.n_blocks + w.n_blocks * w.head_dim)

@@ -501,7 +501,7 @@ static void merge_batched(const Dims& D, const int* q_ptr, const int* q_pairs, c
 // rounding residual of o always block-major.  If zero_acc is given, the fp32 dQ accumulator rows of the queries
 // with at least one selected block (of every query without q_ptr) are cleared in the same pass: the only rows the
 // backward kernel adds into.  zero_words: n_words counters to clear on the way.
-// do_out: a block-major copy of dO is left there on the way, so that dO in raster order needs no pass of its own (two
+// do_out (bf16, head_dim 128): a block-major copy of dO is left there on the way, so that dO in raster order needs no pass of its own (two
 // batches of 32,760 queries x 12 heads: 166 us, 179 in two passes; 13,440 x 12: 41 and 43; 75,600 x 40: 761 and 783; small
 // calls save a launch).
 template <typename T, int DH>
@@ -568,8 +568,6 @@ rowdot_kernel(const T* __restrict__ o, const T* __restrict__ o_resid, const T* _
   for (long long g = warp; g < n_queries; g += nwarps) {
     float a = 0.f;
     const T* do_row = d_o + do_map.off(g, DH);
-    if (do_out)
-      for (int c = lane; c < DH; c += 32) do_out[g * DH + c] = do_row[c];
     const T* o_row = o + o_map.off(g, DH);
     if (zero_acc && (!q_ptr || __ldg(q_ptr + g + 1) - __ldg(q_ptr + g) >= 1)) {
       float4* row = reinterpret_cast<float4*>(zero_acc + g * DH);

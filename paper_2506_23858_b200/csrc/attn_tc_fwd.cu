@@ -7,7 +7,7 @@
 // cycles, and the L2-to-SM path, not the tensor pipe, sets the pace.  Here a CTA owns TWO 128-row
 // query tiles (A and B) that share each K/V tile, which halves the bytes per MMA.
 //
-//   warp 0        TMA producer: K and V tiles into two 2-stage rings
+//   warp 0        TMA producer: K tiles into a ring of two stages, V tiles into one of three
 //   warps 1, 2    MMA issuers: Q K^T, P V
 //   warps 4-7     softmax of tile A: thread = one query row, all 128 keys of the tile
 //   warps 8-11    softmax of tile B

@@ -160,10 +160,12 @@ inline void count_launches(int n) { g_kernel_launches.fetch_add((unsigned long l
     ::vmoba::count_launches(n);                             \
   } while (0)
 
-// Every kernel of the library begins with grid_begin() and is launched by launch_kernel(), `early` or not.  An early launch does
+// Every kernel of a call begins with grid_begin() and is launched by launch_kernel(), `early` or not (the guard kernels of the
+// range-checked build, where nothing is early, and the diagnostics' own kernel do neither).  An early launch does
 // not wait for the end of the kernel before it in the stream: its CTAs are set up while the other still runs, stop in
 // grid_begin() until that one has completed and its writes are visible, and then allow the same for the next.  A call is a
-// chain of up to twenty kernels, many of a few microseconds, and each early launch is worth 1.5 .. 3 us (forward of 33K tokens,
+// chain of some twenty kernels (23 in bf16 with the backward, 27 in fp32), many of a few microseconds, and each early launch
+// is worth 1.5 .. 3 us (forward of 33K tokens,
 // 12 heads: 659 -> 624 us; forward and backward of 1.9K tokens: 204 -> 171 us).
 //
 // Not early: a long kernel that lives by many loads in flight, after one with another shape.  CTAs that move in beside the
