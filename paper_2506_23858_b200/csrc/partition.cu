@@ -1,8 +1,6 @@
 // Step 1 of VMoBA (Eq. 1): reorder tokens of the T x H x W latent into 1D / 2D / 3D blocks,
 // and the inverse reordering.  A pure permutation of head_dim-wide rows, bound by HBM
 // bandwidth: every row is read once and written once with 16-byte vector accesses.
-#include <algorithm>
-
 #include "common.cuh"
 
 namespace vmoba {
@@ -30,9 +28,12 @@ struct PartTensors {
 };
 
 // Rows are enumerated as ((b * S + p) * heads + head): consecutive rows share a token, so the
-// raster side is touched in runs of heads * head_dim contiguous elements.  A warp takes ROWS rows
-// at a time: lane l derives the two offsets of row l once, then the warp streams the rows' 16-byte
-// vectors with the offsets broadcast by shuffle, up to eight passes' loads ahead of their stores.
+// raster side is touched in runs of heads * head_dim contiguous elements.  A warp takes ROWS rows:
+// lane l derives the two offsets of row l once, then the warp streams the rows' 16-byte vectors
+// with the offsets broadcast by shuffle, the loads of four passes ahead of their stores.  Bound by HBM.
+// Four passes and a CTA per 8 x ROWS rows: three tensors of 75,600 x 40 heads 733 us (6340 GB/s), of 32,760 x 12 x 2 197, of
+// 13,440 x 12 53.  Eight passes and at most 32 CTAs per SM, which walk on, took 808, 221 and 57, eight passes alone 820, 220 and
+// 58, two passes 757, 205 and 57 (one tensor after the other, as before, 770, 220 and 69).
 // blockIdx.y: tensor (one launch for up to four of them; the first one's CTAs also write the permutation tables).
 template <int VEC_PER_ROW, int ROWS>   // 16-byte vectors per row: head_dim * elem_size / 16
 __global__ void __launch_bounds__(256)
@@ -41,47 +42,46 @@ partition_kernel(PermGeom g, int S, int heads, int n_rows, int inverse, const __
   if (!grid_begin()) return;
   constexpr int ROWS_PER_PASS = 32 / VEC_PER_ROW > 0 ? 32 / VEC_PER_ROW : 1;
   constexpr int PASSES = ROWS / ROWS_PER_PASS;
-  constexpr int U = PASSES < 8 ? PASSES : 8;         // passes whose loads are in flight together
+  // passes whose loads are in flight together (few rows per warp: all of them)
+  constexpr int U = PASSES < 4 || ROWS < 32 ? PASSES : 4;
   const int lane = threadIdx.x & 31;
-  const int warp_id = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int n_warps = gridDim.x * (blockDim.x >> 5);
+  const long long base = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * ROWS;
+  if (base >= n_rows) return;
   const int k = blockIdx.y;
   const uint4* __restrict__ src = t.src[k];
   uint4* __restrict__ dst = t.dst[k];
   const int sub = lane / VEC_PER_ROW, vec = lane % VEC_PER_ROW;
-  for (long long base = (long long)warp_id * ROWS; base < n_rows; base += (long long)n_warps * ROWS) {
-    const long long row = base + lane;
-    long long off_r = 0, off_bm = 0;
-    if (lane < ROWS && row < n_rows) {
-      const unsigned bp = (unsigned)row / (unsigned)heads, head = (unsigned)row - bp * heads;
-      const unsigned b = bp / (unsigned)S;
-      const int p = (int)(bp - b * S);
-      const int r = perm_of(g, p);
-      off_r = b * t.rs_b[k] + (long long)r * t.rs_s[k] + head * t.rs_h[k];
-      off_bm = (((long long)b * heads + head) * S + p) * VEC_PER_ROW;
-      if (k == 0 && b == 0 && head == 0) {
-        if (perm) perm[p] = r;
-        if (inv_perm) inv_perm[r] = p;
-      }
+  const long long row = base + lane;
+  long long off_r = 0, off_bm = 0;
+  if (lane < ROWS && row < n_rows) {
+    const unsigned bp = (unsigned)row / (unsigned)heads, head = (unsigned)row - bp * heads;
+    const unsigned b = bp / (unsigned)S;
+    const int p = (int)(bp - b * S);
+    const int r = perm_of(g, p);
+    off_r = b * t.rs_b[k] + (long long)r * t.rs_s[k] + head * t.rs_h[k];
+    off_bm = (((long long)b * heads + head) * S + p) * VEC_PER_ROW;
+    if (k == 0 && b == 0 && head == 0) {
+      if (perm) perm[p] = r;
+      if (inv_perm) inv_perm[r] = p;
     }
-    const long long off_src = inverse ? off_bm : off_r;
-    const long long off_dst = inverse ? off_r : off_bm;
-    const int left = (int)min((long long)ROWS, n_rows - base);
+  }
+  const long long off_src = inverse ? off_bm : off_r;
+  const long long off_dst = inverse ? off_r : off_bm;
+  const int left = (int)min((long long)ROWS, n_rows - base);
 #pragma unroll 1
-    for (int p0 = 0; p0 < PASSES; p0 += U) {
-      uint4 v[U];
-      long long to[U];
+  for (int p0 = 0; p0 < PASSES; p0 += U) {
+    uint4 v[U];
+    long long to[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int from = (p0 + u) * ROWS_PER_PASS + sub;
-        const long long so = __shfl_sync(0xffffffffu, off_src, from);
-        to[u] = __shfl_sync(0xffffffffu, off_dst, from);
-        if (from < left) v[u] = __ldg(src + so + vec);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-        if ((p0 + u) * ROWS_PER_PASS + sub < left) dst[to[u] + vec] = v[u];
+    for (int u = 0; u < U; ++u) {
+      const int from = (p0 + u) * ROWS_PER_PASS + sub;
+      const long long so = __shfl_sync(0xffffffffu, off_src, from);
+      to[u] = __shfl_sync(0xffffffffu, off_dst, from);
+      if (from < left) v[u] = __ldg(src + so + vec);
     }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if ((p0 + u) * ROWS_PER_PASS + sub < left) dst[to[u] + vec] = v[u];
   }
 }
 
@@ -89,11 +89,9 @@ template <int V>
 static int launch_partition(const Dims& D, const PermGeom& g, int inverse, int n, const PartTensors& t, int32_t* perm,
                             int32_t* inv_perm, cudaStream_t st) {
   const long long n_rows = (long long)D.BH * D.S;
-  const long long cap = (long long)sm_count() * 8 * 4;
   auto go = [&](auto kernel, int rows) {
-    const long long blocks = std::min<long long>((n_rows + 8 * rows - 1) / (8 * rows), std::max<long long>(cap / n, 1));
-    launch_kernel(early_rows(D), kernel, dim3((unsigned)blocks, n), 256, 0, st, g, D.S, D.heads, (int)n_rows, inverse,
-                  t, perm, inv_perm);
+    launch_kernel(early_rows(D), kernel, dim3((unsigned)((n_rows + 8 * rows - 1) / (8 * rows)), n), 256, 0, st, g, D.S, D.heads,
+                  (int)n_rows, inverse, t, perm, inv_perm);
   };
   // 32 rows per warp once that gives every SM its 64 warps; below, 8 rows, for more warps to hide a pass's latency
   // (22,464 rows, bf16, head_dim 128: one tensor 9.1 us with 32, three tensors 7.5 us with 8)
