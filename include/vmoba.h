@@ -315,7 +315,7 @@ int vmoba_attn_bwd_raster_do(const vmoba_shape* shape, const void* q_bm, const v
  * in any one token order.  If do_or_null is given, also computes dq, dk, dv.  The results repeat bit for bit.
  * For the backward ws must hold vmoba_workspace_bytes(shape, VMOBA_STAGE_FULL_BWD, 0) bytes: 4 * B * heads * S, for bf16 the
  * rounding residual of o (2 bytes per element of a tensor) and, for bf16 with head_dim 128, an fp32 accumulator of dq (4 bytes
- * per element: 1.5 GB at 75,600 tokens and 40 heads).
+ * per element: 1.5 GB at 75,600 tokens and 40 heads; up to four of them where they fit 128 MB).
  */
 int vmoba_full_attn(const vmoba_shape* shape, const void* q, const void* k, const void* v, void* o,
                     float* lse, const void* do_or_null, void* dq, void* dk, void* dv,

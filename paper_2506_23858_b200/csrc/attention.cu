@@ -25,6 +25,7 @@ int tc_sparse_bwd(const Dims& D, const void* q, const void* k, const void* v, co
                   int32_t* status, cudaStream_t st, const RowMap& out_map, const RowMap& do_map);
 int tc_dense_bwd(const Dims& D, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
                  const float* Dv, float* dq_acc, int* turns, void* dk, void* dv, int32_t* status, cudaStream_t st);
+int tc_dense_bwd_parts(const Dims& D);           // accumulators of dQ
 long long tc_dense_bwd_turns(const Dims& D);
 
 static bool use_tensor_cores(const Dims& D) { return D.dtype == VMOBA_BF16 && D.d == 128; }
@@ -52,7 +53,7 @@ static BwdWs carve_bwd(const Dims& D, bool dense, void* ws) {
   BwdWs w;
   w.item_ptr = c.take<int>((size_t)D.BH * D.Nb + 1);
   w.Dv = c.take<float>((size_t)D.BH * D.S);
-  w.dq_acc = dense && !use_tensor_cores(D) ? nullptr : c.take<float>((size_t)D.BH * D.S * D.d);
+  w.dq_acc = dense && !use_tensor_cores(D) ? nullptr : c.take<float>((size_t)D.BH * D.S * D.d * (dense ? tc_dense_bwd_parts(D) : 1));
   w.o_resid = (dense && D.dtype == VMOBA_BF16) ? c.take<__nv_bfloat16>((size_t)D.BH * D.S * D.d) : nullptr;
   w.turns = dense && use_tensor_cores(D) ? c.take<int>((size_t)tc_dense_bwd_turns(D)) : nullptr;
   w.bytes = c.total();
@@ -112,7 +113,7 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
                            out_map, do_bm ? RowMap() : do_map);
     if (rc) return rc;
     launch_kernel(early_rows(D), simt::cast_rows_kernel<T>, grid_for((nq + 7) / 8, 16), 256, 0, st, w.dq_acc, (T*)dq,
-                  q_ptr, nq, out_map);
+                  q_ptr, nq, out_map, 1);
     VMOBA_LAUNCH_OK(1);
     VMOBA_GUARDS_CHECK(w.guards, status, st);
     return VMOBA_OK;
@@ -163,7 +164,7 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
       int rc = tc_dense_bwd(D, q, k, v, d_o, lse, w.Dv, w.dq_acc, w.turns, dk, dv, status, st);
       if (rc) return rc;
       launch_kernel(early_rows(D), simt::cast_rows_kernel<T>, grid_for((nq + 7) / 8, 16), 256, 0, st, w.dq_acc,
-                    (T*)dq, nullptr, nq, RowMap());
+                    (T*)dq, nullptr, nq, RowMap(), tc_dense_bwd_parts(D));
       VMOBA_LAUNCH_OK(1);
       return VMOBA_OK;
     }

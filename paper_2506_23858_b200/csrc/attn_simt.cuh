@@ -773,11 +773,11 @@ attn_bwd_dq_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __
 
 // Rows of the tensor-core backward's fp32 dQ accumulator -> output dtype.  The accumulator keeps its 128 columns in the
 // order that kernel reduces them in: position 32 w + 4 r + a holds column 32 w + r + 8 a.  Queries without a selected
-// block (q_ptr given) get zeros without a read.
+// block (q_ptr given) get zeros without a read.  parts: accumulators behind one another, added up in order.
 template <typename T>
 __global__ void __launch_bounds__(256)
 cast_rows_kernel(const float* __restrict__ src, T* __restrict__ dst, const int* __restrict__ q_ptr, long long n_queries,
-                 const RowMap map) {
+                 const RowMap map, int parts) {
   if (!grid_begin()) return;
   constexpr int DH = 128;
   const int lane = threadIdx.x & 31;
@@ -805,6 +805,13 @@ cast_rows_kernel(const float* __restrict__ src, T* __restrict__ dst, const int* 
       if (used[r]) {
         const float* row = src + min(g0 + r, n_queries - 1) * DH + at;
         v[r] = make_float4(__ldg(row), __ldg(row + 4), __ldg(row + 8), __ldg(row + 12));
+      }
+    }
+    for (int part = 1; part < parts; ++part) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const float* row = src + (part * n_queries + min(g0 + r, n_queries - 1)) * DH + at;
+        v[r].x += __ldg(row); v[r].y += __ldg(row + 4); v[r].z += __ldg(row + 8); v[r].w += __ldg(row + 12);
       }
     }
 #pragma unroll

@@ -86,10 +86,13 @@ constexpr uint32_t IDESC_TN = make_idesc_bf16(128, 128, false, true);    // dV, 
 // follow one another about a unit apart; tickets go round `group` heads, so that a head's tiles start few units apart
 // (SMs / group) and come no faster than one per unit.  Two warps that have nothing else to do look at the counter and move it
 // on (a fence behind the reductions, a look at another CTA's word): the writers see shared-memory barriers only.
+// Where the tiles of a head are most of what there is to run, waiting for one another takes as long as the work.  Up to four
+// accumulators with counters of their own, if they fit 128 MB, shorten the row: tile t adds to accumulator t % parts, and
+// cast_rows adds these up.
 // Measured, against reductions in any order and tiles that start at different units (forward and backward): 12 heads x 13,440
-// tokens 3946 -> 4024 us, x 8,000 1453 -> 1492, 4 heads x 32,760 7665 -> 8128.  Where the tiles of a head are most of what
-// there is to run, they wait for one another: 12 x 3,000 216 -> 275, 12 x 1,000 71 -> 100, 1 x 3,000 132 -> 224 (257, 377 and
-// 227 with dQ in a kernel of its own).  With the writers looking at the counters themselves 12 x 13,440 took 4798.
+// tokens 3796 -> 3912 us, x 8,000 1448 -> 1498, 4 heads x 32,760 7713 -> 8221 (one accumulator); 12 x 3,000 218 -> 252, 12 x 1,000
+// 71 -> 81, 1 x 3,000 132 -> 158 (four; with one 275, 100, 224; with dQ in a kernel of its own 376, 118, 227).  With the
+// writers looking at the counters themselves 12 x 13,440 took 4798.
 struct KvParams {
   const __nv_bfloat16 *q, *d_o;
   const float *lse, *Dv;
@@ -103,7 +106,8 @@ struct KvParams {
   RowMap do_map;               // where the dO rows come from (likewise)
   float* dq_acc;               // fp32 [queries][head_dim]; sparse: zeroed rows of all selecting queries; columns in the order of the
                                // dQ writers: position 32 w + 4 r + a holds column 32 w + r + 8 a (r < 8, a < 4)
-  int* turns;                  // dense: [BH][units], then the ticket; zero at the start
+  int parts;                   // dense: accumulators (dq_acc holds that many of [queries][head_dim])
+  int* turns;                  // dense: [parts][BH][units], then the ticket; zero at the start
   int group;                   // dense: heads whose key tiles are taken in turn
   int32_t* status;
   unsigned long long* prof;    // optional wait-time counters (diagnostics), or null
@@ -245,7 +249,8 @@ __device__ __forceinline__ void stmatrix_x4(uint32_t addr, uint32_t a, uint32_t 
                : "memory");
 }
 
-template <bool DENSE, bool PROF>
+// MULTI (dense): several accumulators (with p.parts read in the one kernel, the case of one ran 4 % slower).
+template <bool DENSE, bool MULTI, bool PROF>
 __global__ void __launch_bounds__(THREADS, 1)
 attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
                       const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmO, const KvParams p) {
@@ -296,7 +301,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     mbar_init(&sm->drain, 1);
     if constexpr (DENSE) { mbar_init(&sm->turn_ok, 1); mbar_init(&sm->rows_out, 256); mbar_init(&sm->rows_seen, 1); }
     sm->abort_flag = 0;
-    if constexpr (DENSE) sm->ticket = atomicAdd(p.turns + (long long)p.BH * ((p.S + QU - 1) / QU), 1);
+    if constexpr (DENSE) sm->ticket = atomicAdd(p.turns + (long long)(MULTI ? p.parts : 1) * p.BH * ((p.S + QU - 1) / QU), 1);
     fence_barrier_init();
     prefetch_tmap(&tmK);
     prefetch_tmap(&tmV);
@@ -310,6 +315,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   tc_fence_after();
   const uint32_t tmem = sm->tmem_base;
 
+  const int parts = MULTI ? p.parts : 1;
   const int tiles = ((DENSE ? p.S : p.sb) + BN - 1) / BN;
   const int n_items = p.BH * (DENSE ? 1 : p.Nb) * tiles;
   // dense: as many CTAs as items, one each
@@ -457,16 +463,17 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
       // ---------------------------------------------------------------- turns: warp 3 waits for them, warp 2 passes them on.
       // Warp 3 lets the writers go on only when warp 2 has noted the end of the unit before: no barrier gets a phase ahead.
       const KvItem it = kv_decode<DENSE>(p, first_item(), tiles);
-      int* turn = p.turns + (long long)it.bh * it.n_units;
+      const int rank = it.tile / parts;
+      int* turn = p.turns + ((long long)(it.tile - rank * parts) * p.BH + it.bh) * it.n_units;
       for (int i = 0; i < it.n_units; ++i) {
         if (warp == 3) {
-          if (it.tile > 0) turn_wait(turn + i, it.tile, abort_flag, p.status);
+          if (rank > 0) turn_wait(turn + i, rank, abort_flag, p.status);
           if (i > 0) mbar_wait(&sm->rows_seen, (i - 1) & 1, abort_flag, p.status);
           mbar_arrive(&sm->turn_ok);
         } else {
           mbar_wait(&sm->rows_out, i & 1, abort_flag, p.status);
           mbar_arrive(&sm->rows_seen);
-          turn_pass(turn + i, it.tile + 1);
+          turn_pass(turn + i, rank + 1);
         }
       }
     }
@@ -568,6 +575,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
     for (int item = first_item(); item < n_items; item = next_item(item)) {
       const KvItem it = kv_decode<DENSE>(p, item, tiles);
       float* acc_head = acc_col + (long long)it.head_off * DH;
+      if constexpr (MULTI) acc_head += (long long)(it.tile % parts) * p.BH * p.S * DH;
       for (int i = 0; i < it.n_units; ++i, ++g) {
         const int first = i * QU + 64 * qhalf;
         // accumulator rows of queries lane and 32 + lane of this half of the unit (-1 beyond the list)
@@ -601,7 +609,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
         auto add = [](float* to, float a, float b, float c, float d) { red_add_v4(to, a, b, c, d); };
         if constexpr (DENSE) {
           twait(1, &sm->turn_ok, g & 1);
-          if (it.tile == 0)
+          if (it.tile < parts)
             write_rows([](float* to, float a, float b, float c, float d) { *reinterpret_cast<float4*>(to) = make_float4(a, b, c, d); });
           else
             write_rows(add);
@@ -765,7 +773,7 @@ attn_bwd_fused_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_cons
   if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
 }
 
-template <bool DENSE>
+template <bool DENSE, bool MULTI>
 static int launch(const Dims& D, const void* k, const void* v, KvParams& kp, cudaStream_t st) {
   CUtensorMap tmK, tmV, tmQ, tmO;
   const uint64_t rows = (uint64_t)D.BH * D.S;
@@ -782,7 +790,7 @@ static int launch(const Dims& D, const void* k, const void* v, KvParams& kp, cud
   const long long items = (long long)D.BH * kp.Nb * ((kp.sb + BN - 1) / BN);
   if (items > (long long)INT32_MAX - 4096) return VMOBA_ERR_SHAPE;
   const int grid = DENSE ? (int)items : (int)std::max<long long>(1, std::min<long long>(items, sm_count()));
-  auto kernel = kp.prof ? attn_bwd_fused_kernel<DENSE, true> : attn_bwd_fused_kernel<DENSE, false>;
+  auto kernel = kp.prof ? attn_bwd_fused_kernel<DENSE, MULTI, true> : attn_bwd_fused_kernel<DENSE, MULTI, false>;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
   launch_kernel(early_rows(D), kernel, grid, THREADS, SMEM_BYTES, st, tmK, tmV, tmQ, tmO, kp);
   VMOBA_LAUNCH_OK(1);
@@ -802,24 +810,30 @@ int tc_sparse_bwd(const Dims& D, const void* q, const void* k, const void* v, co
   kp.kb_ptr = kb_ptr; kp.q_idx = q_idx; kp.capacity = cap;
   kp.dk = (__nv_bfloat16*)dk; kp.dv = (__nv_bfloat16*)dv; kp.status = status;
   kp.dq_acc = dq_acc; kp.out_map = out_map; kp.do_map = do_map;
-  kp.turns = nullptr; kp.group = 1;
-  return tcb::launch<false>(D, k, v, kp, st);
+  kp.turns = nullptr; kp.group = 1; kp.parts = 1;
+  return tcb::launch<false, false>(D, k, v, kp, st);
 }
 
 // Dense backward: every query of a head meets every key tile; turns holds tc_dense_bwd_turns() zeros, dq_acc anything.
-long long tc_dense_bwd_turns(const Dims& D) { return (long long)D.BH * ((D.S + tcb::QU - 1) / tcb::QU) + 1; }
+int tc_dense_bwd_parts(const Dims& D) {
+  const long long acc = (long long)D.BH * D.S * D.d * (long long)sizeof(float), tiles = (D.S + tcb::BN - 1) / tcb::BN;
+  return (int)std::max<long long>(1, std::min<long long>(std::min<long long>(4, tiles), (128ll << 20) / acc));
+}
+long long tc_dense_bwd_turns(const Dims& D) {
+  return (long long)tc_dense_bwd_parts(D) * D.BH * ((D.S + tcb::QU - 1) / tcb::QU) + 1;
+}
 int tc_dense_bwd(const Dims& D, const void* q, const void* k, const void* v, const void* d_o, const float* lse,
                  const float* Dv, float* dq_acc, int* turns, void* dk, void* dv, int32_t* status, cudaStream_t st) {
   tcb::KvParams kp;
   kp.q = (const __nv_bfloat16*)q; kp.d_o = (const __nv_bfloat16*)d_o; kp.lse = lse; kp.Dv = Dv;
   kp.kb_ptr = nullptr; kp.q_idx = nullptr; kp.capacity = 0;
   kp.dk = (__nv_bfloat16*)dk; kp.dv = (__nv_bfloat16*)dv; kp.status = status;
-  kp.dq_acc = dq_acc; kp.turns = turns;
+  kp.dq_acc = dq_acc; kp.turns = turns; kp.parts = tc_dense_bwd_parts(D);
   // Sixteen heads: their accumulators, Q and dO pass through the L2 once per SMs / 16 key tiles.  More where a head has so few
   // units that its tiles would come too slowly for the SMs.
   const int units = (D.S + tcb::QU - 1) / tcb::QU;
   kp.group = std::min(D.BH, std::max(16, sm_count() / units));
-  return tcb::launch<true>(D, k, v, kp, st);
+  return kp.parts > 1 ? tcb::launch<true, true>(D, k, v, kp, st) : tcb::launch<true, false>(D, k, v, kp, st);
 }
 
 // Registers (or clears, with null) a device buffer of 16 uint64 counters for the attention kernels'

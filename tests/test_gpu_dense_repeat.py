@@ -1,5 +1,6 @@
 """The dense backward adds the parts of dQ key tile after key tile: two runs agree bit for bit, whatever order the CTAs come
-in, and the sum is right at the edges of tiles and units, with one head and with more heads than are taken in turn."""
+in, and the sum is right at the edges of tiles and units, with one head and with more heads than are taken in turn, with one to
+four accumulators."""
 import pytest
 import torch
 
@@ -9,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("B, heads, S", [(1, 1, 1), (1, 2, 127), (1, 1, 129), (2, 3, 640), (1, 17, 300), (3, 50, 257), (1, 1, 20000),
-                                         (1, 12, 5000)])
+                                         (1, 12, 5000), (1, 20, 13440)])
 def test_dense_gradients_repeat(B, heads, S):
     shape = vb.make_shape(B, heads, 128, (S, 1, 1), (S, 1, 1), "bf16")
     torch.manual_seed(S)
