@@ -194,6 +194,28 @@ template <typename... P, typename... A>
 inline void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   launch_kernel(true, kernel, grid, block, smem, st, std::forward<A>(args)...);
 }
+// Early, in clusters of `cluster` consecutive CTAs.
+template <typename... P, typename... A>
+inline void launch_cluster(int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+#ifdef VMOBA_DEBUG
+  cfg.numAttrs = 1;
+#else
+  cfg.numAttrs = 2;
+#endif
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 // One tensor of at most 16 MB: a pass over a few of them takes about ten microseconds, of which an early launch saves two.
 inline bool early_rows(const Dims& D) { return (long long)D.BH * D.S * D.d * D.es <= (16ll << 20); }

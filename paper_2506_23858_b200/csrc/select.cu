@@ -16,8 +16,11 @@
 //   mark    : mask bits + per (segment, block) counts + per-segment pair totals
 //   offsets : CSR offsets by key block (kb_ptr) and by query (q_ptr)
 //   fill    : q_idx (queries of each key block, ascending) and q_pairs (pairs of each query)
+// Small pools take select_pool_kernel instead of everything before fill (pool_plan).
 #include <algorithm>
 #include <type_traits>
+
+#include <cooperative_groups.h>
 
 #include "common.cuh"
 
@@ -527,8 +530,9 @@ offsets_kernel(const int* __restrict__ kb_total, int* __restrict__ kb_ptr, long 
 constexpr int kStage = 6144;
 __global__ void __launch_bounds__(kSegThreads)
 fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__ tmask, int S, int Nb, int mw, int QSEG,
-            int nseg, const int* __restrict__ kb_ptr, const int* __restrict__ seg_cnt, const int* __restrict__ seg_qoff,
-            int* __restrict__ q_idx, int* __restrict__ q_ptr, int* __restrict__ q_pairs, long long capacity) {
+            int nseg, int* __restrict__ kb_ptr, const int* __restrict__ seg_cnt, const int* __restrict__ seg_qoff,
+            int* __restrict__ q_idx, int* __restrict__ q_ptr, int* __restrict__ q_pairs, long long capacity,
+            const int* __restrict__ kb_excl, const int64_t* __restrict__ k_per_head, int32_t* __restrict__ dev_status) {
   if (!grid_begin()) return;
   extern __shared__ uint32_t sm[];
   const int TW = QSEG >> 5;
@@ -573,9 +577,24 @@ fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__
   const int* sc = seg_cnt + ((long long)bh * nseg + seg) * Nb;
   for (int i = t; i < nq * mw; i += blockDim.x) s_mask[i] = gm[i];
   for (int i = t; i < Nb * TW; i += blockDim.x) s_tm[i] = tm[i];
-  for (int j = t; j < Nb; j += blockDim.x)          // (clamped: beyond INT32_MAX is beyond every capacity)
-    s_pos[j] = (int)min((long long)kb_ptr[(long long)bh * Nb + j] + sc[j], (long long)INT32_MAX);
-  const long long qbase = seg_qoff[bh * nseg + seg];
+  // kb_excl: the offsets so far are counted from the head's first pair, and this kernel adds the pairs of the heads before
+  long long base = 0;
+  if (kb_excl) {
+    for (int h = lane; h < bh; h += 32) base += k_per_head[h];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(0xffffffffu, base, o);
+  }
+  for (int j = t; j < Nb; j += blockDim.x) {        // (clamped: beyond INT32_MAX is beyond every capacity)
+    const long long first = kb_excl ? base + kb_excl[(long long)bh * (Nb + 1) + j] : (long long)kb_ptr[(long long)bh * Nb + j];
+    s_pos[j] = (int)min(first + sc[j], (long long)INT32_MAX);
+    if (kb_excl && seg == 0) kb_ptr[(long long)bh * Nb + j] = (int)min(first, (long long)INT32_MAX);
+  }
+  if (kb_excl && seg == 0 && bh == (int)gridDim.y - 1 && t == 0) {
+    const long long all = base + k_per_head[bh];
+    kb_ptr[(long long)gridDim.y * Nb] = q_ptr[(long long)gridDim.y * S] = (int)min(all, (long long)INT32_MAX);
+    if (all > capacity) set_status(dev_status, VMOBA_ERR_CAPACITY);
+  }
+  const long long qbase = base + seg_qoff[bh * nseg + seg];
   __syncthreads();
   {
     const int per = (Nb + blockDim.x - 1) / blockDim.x, j0 = min(t * per, Nb), j1 = min(j0 + per, Nb);
@@ -1122,6 +1141,437 @@ mark_from_mask_kernel(const uint32_t* __restrict__ mask_bits, int S, int Nb, int
   if (threadIdx.x == 0) seg_total[bh * nseg + seg] = s_total;
 }
 
+// ------------------------------------------------------------------------------------------
+// Small pools: one cluster of up to eight CTAs per head does the whole of the selection up to the offsets of its own pairs;
+// fill_kernel adds the pairs of the heads before.  Two launches take the place of eleven, each of which waited two to five
+// microseconds for the one before it: 12 heads x 1,872 queries x 8 blocks 40 -> 18 us, x 13,440 x 16 57 -> 38.  A CTA takes
+// whole segments of QSEG queries and keeps their scores in shared memory.  The search is the one of the kernels above in other
+// steps, bound by the latency of each:
+//   * 32 bins of the head's range, a set for every thread (one bank each, plain additions; with 512 bins shared by the
+//     CTA, the compare-and-swap loops that fp32 additions in shared memory are took 14 us for 27,000 scores);
+//   * the scores of the crossing bin, put together in a list, in a bin of it per thread (again, where they are alike);
+//   * the up to kPoolFinal scores of the crossing bin of those, each against all others.
+// What the CTAs of a cluster have to tell one another they write into each other's shared memory ahead of a barrier (the
+// finer bins are read from there), and all of them come to the same state.
+// SRC = kPoolMask: the per-query rules, whose mask words exist already.
+enum PoolSrc { kPoolScores, kPoolMask };
+constexpr int kPoolCtas = 8;                  // what every device schedules as one cluster
+constexpr int kPoolBins0 = 32, kPoolLevels = 3, kPoolFinal = 256;
+constexpr int kPoolSmemMax = 224 * 1024;
+// A second (fourth, eighth) CTA shares a head from more than 4,096 scores per CTA on, as long as all heads run at once: 12 heads x
+// 15,000 scores 19.0 us (one CTA 25), x 33,000 21.2 (16,384 per CTA 26; whole selection, 37.7 by the passes over the matrix).
+constexpr long long kPoolSlice = 4096;
+// Up to 2,048 scores a CTA has 256 threads, else 512: a step that every thread takes costs their number (x 1,024 scores 14.8
+// us with 256, 15.2 with 512, 16.7 with 1,024; x 15,000 in two CTAs 24.1, 21.6, 23.0).
+constexpr long long kPoolShort = 2048;
+// bytes of shared memory: the first bins of T threads; then, in their place, masses and counts of the levels' bins and the list
+constexpr int kPoolFront = kPoolBins0 * 4;      // (per thread)
+
+struct PoolArgs {
+  const float* scores;
+  const float* range;          // or null: looked for here
+  const HeadState* state;      // kPoolMask: smallest selected key of each head
+  int S, Nb, mw, QSEG, nseg, segs_per, own_sb, unit_w;
+  float sigma, tau;
+  double count_target;
+  uint32_t* mask_bits;
+  uint32_t* tmask;
+  int* seg_cnt;
+  int* seg_qoff;
+  int* kb_excl;                // [BH][Nb + 1] pairs of the head in front of each block
+  int64_t* k_per_head;
+  float* cutoff_per_head;
+};
+
+// exclusive sum over the threads of the CTA (s_warp: a word per warp; the caller keeps calls apart by barriers)
+template <typename T>
+__device__ __noinline__ T pool_exclusive(T x, T* s_warp) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  T inc = x;
+#pragma unroll 1
+  for (int o = 1; o < 32; o <<= 1) {
+    const T v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) s_warp[warp] = inc;
+  __syncthreads();
+  T before = lane < warp ? s_warp[lane] : T(0);
+#pragma unroll 1
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  return before + (inc - x);
+}
+
+template <PoolSrc SRC, int T>
+__global__ void __launch_bounds__(T, 1)
+select_pool_kernel(const PoolArgs a) {
+  if (!grid_begin()) return;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  // a barrier of the cluster (a head with one CTA: its own, at a third of the price)
+  auto meet = [&]() { if (cluster.num_blocks() > 1) cluster.sync(); else __syncthreads(); };
+  // before the first look into another CTA's shared memory: all of them have started
+  auto all_there = []() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); };
+  constexpr int kFront = SRC == kPoolScores ? kPoolFront * T : 0, kLevelBytes = 8 * T, kList = (kPoolFront * T - kPoolLevels * kLevelBytes) / 4;
+  extern __shared__ __align__(16) unsigned char pool_smem[];
+  __shared__ int s_pairs[kPoolCtas];
+  __shared__ int s_sum[32];
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), bh = (int)blockIdx.x / C;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int Nb = a.Nb, mw = a.mw, TW = a.QSEG >> 5;
+  const int seg0 = rank * a.segs_per, segs = max(0, min(a.segs_per, a.nseg - seg0));      // (none, for the last CTAs of some)
+  const int q0 = seg0 * a.QSEG, nq = max(0, min(a.S - q0, a.segs_per * a.QSEG));
+  const int n = nq * Nb;
+  int* s_tot = reinterpret_cast<int*>(pool_smem + kFront);      // [C][Nb] pairs of the CTAs
+  int* s_seg = s_tot + C * Nb;                                  // [segs_per][Nb]
+  int* s_segp = s_seg + a.segs_per * Nb;                        // [segs_per] pairs of a segment
+  for (int i = t; i < a.segs_per * (Nb + 1); i += T) s_seg[i] = 0;      // (s_segp follows)
+  uint32_t* gmask = a.mask_bits + ((long long)bh * a.S + q0) * mw;
+  uint32_t* gtm = a.tmask + ((long long)bh * a.nseg + seg0) * TW * Nb;      // [segs][TW][Nb]
+
+  uint32_t cutoff = 0u;
+  float* s_src = nullptr;
+  if constexpr (SRC == kPoolScores) {
+    __shared__ double s_w0[kPoolCtas][kPoolBins0], s_dsum[32], s_above;
+    __shared__ uint32_t s_key[kPoolCtas][2], s_final[kPoolFinal], s_best, s_least;
+    __shared__ int s_crossed, s_lowest, s_listed, s_n, s_at, s_k, s_cross[kPoolLevels];
+    __shared__ float s_anchor[kPoolLevels], s_inv[kPoolLevels];
+    s_src = reinterpret_cast<float*>(pool_smem + kFront + ((4 * (C * Nb + a.segs_per * (Nb + 1)) + 15) & ~15));
+    float* s_own = reinterpret_cast<float*>(pool_smem);        // [kPoolBins0][threads]
+#pragma unroll
+    for (int b = 0; b < kPoolBins0 / 4; ++b) reinterpret_cast<float4*>(s_own)[b * T + t] = make_float4(0.f, 0.f, 0.f, 0.f);
+    uint32_t min_key = 0xffffffffu, max_key = 0u;
+    if (a.range) { min_key = float_key(__ldg(a.range + 2 * bh)); max_key = float_key(__ldg(a.range + 2 * bh + 1)); }
+    {
+      const float* g_src = a.scores + ((long long)bh * a.S + q0) * Nb;
+      if ((reinterpret_cast<uintptr_t>(g_src) & 15u) == 0) {
+        const int n4 = n >> 2;
+#pragma unroll 8
+        for (int i = t; i < n4; i += T) reinterpret_cast<float4*>(s_src)[i] = __ldg(reinterpret_cast<const float4*>(g_src) + i);
+        if (t < n - (n4 << 2)) s_src[(n4 << 2) + t] = __ldg(g_src + (n4 << 2) + t);
+      } else {
+#pragma unroll 8
+        for (int i = t; i < n; i += T) s_src[i] = __ldg(g_src + i);
+      }
+    }
+    // smallest and largest of a value over the cluster
+    auto exchange = [&](uint32_t& lo, uint32_t& hi) {
+      if (t == 0) { s_least = 0xffffffffu; s_best = 0u; }
+      __syncthreads();
+      lo = __reduce_min_sync(0xffffffffu, lo);
+      hi = __reduce_max_sync(0xffffffffu, hi);
+      if (lane == 0) { atomicMin(&s_least, lo); atomicMax(&s_best, hi); }
+      __syncthreads();
+      if (t < C) {
+        uint32_t* to = cluster.map_shared_rank(s_key[rank], t);
+        to[0] = s_least; to[1] = s_best;
+      }
+      meet();
+      for (int c = 0; c < C; ++c) { lo = min(lo, s_key[c][0]); hi = max(hi, s_key[c][1]); }
+    };
+    all_there();
+    __syncthreads();
+    if (!a.range) {
+#pragma unroll 2
+      for (int i = t; i < n; i += T) {
+        const uint32_t key = float_key(s_src[i]);
+        min_key = min(min_key, key);
+        max_key = max(max_key, key);
+      }
+      exchange(min_key, max_key);
+    }
+    const float lo = key_float(min_key), smax = key_float(max_key), span = smax - lo;
+    const float inv0 = span > 0.f ? (float)kPoolBins0 / span : 0.f, off0 = -lo * inv0;
+    const bool unit_w = a.unit_w != 0;
+    auto weight = [&](float s) { return unit_w ? 1.0f : pair_weight(a.sigma, s, smax); };
+    // ---- the first bins: floor(s * inv0 + off0) by an addition that rounds down, NaN to bin 0
+#pragma unroll 4
+    for (int i = t; i < n; i += T) {
+      const float s = s_src[i], x = fminf(fmaxf(fmaf(s, inv0, off0), 0.f), (float)(kPoolBins0 - 1));
+      const int b = __float_as_int(__fadd_rd(x, 8388608.f)) & (kPoolBins0 - 1);
+      s_own[b * T + t] += weight(s);
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int b = warp; b < kPoolBins0; b += T / 32) {
+      float w = 0.f;
+#pragma unroll
+      for (int r = 0; r < T / 32; ++r) {
+        const float x = s_own[b * T + 32 * r + lane];
+        if (x > 0.f) w += x;
+      }
+      double x = (double)w;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      if (lane < C) cluster.map_shared_rank(s_w0[rank], lane)[b] = x;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 2 * kPoolLevels; ++i) reinterpret_cast<uint32_t*>(pool_smem)[i * T + t] = 0u;
+    meet();
+    double need;                           // mass still to be covered from the crossing bin down
+    int cross0;
+    {
+      double x = 0.0;                      // lane l: bin 31 - l
+      for (int c = 0; c < C; ++c) x += s_w0[c][kPoolBins0 - 1 - lane];
+      double inc = x;
+#pragma unroll 1
+      for (int o = 1; o < 32; o <<= 1) {
+        const double v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      const double total = __shfl_sync(0xffffffffu, inc, 31), excl = inc - x;
+      need = a.count_target >= 0.0 ? a.count_target : (double)a.tau * total;
+      const unsigned int hit = __ballot_sync(0xffffffffu, x > 0.0 && excl < need && inc >= need);
+      const unsigned int occupied = __ballot_sync(0xffffffffu, x > 0.0);
+      const int e = hit ? __ffs(hit) - 1 : occupied ? 31 - __clz(occupied) : kPoolBins0 - 1;
+      cross0 = kPoolBins0 - 1 - e;
+      need -= __shfl_sync(0xffffffffu, excl, e);
+    }
+    cutoff = min_key;                      // everything, where tau = 1
+    if (a.tau < 1.0f) {
+      // ---- the list of the crossing bin's scores (the last bin has no end), if it has room for them
+      const float y_lo = (float)cross0, y_hi = cross0 == kPoolBins0 - 1 ? NAN : (float)(cross0 + 1);
+      auto inside = [&](float s) {
+        const float y = fmaf(s, inv0, off0);
+        return (cross0 == 0 || y >= y_lo) && !(y >= y_hi);
+      };
+      float* s_list = reinterpret_cast<float*>(pool_smem + kPoolLevels * kLevelBytes);
+      int mine = 0;
+#pragma unroll 4
+      for (int i = t; i < n; i += T) mine += inside(s_src[i]) ? 1 : 0;
+      int at = pool_exclusive(mine, s_sum);
+      if (t == T - 1) s_listed = at + mine;
+      if (mine && at + mine <= kList)
+#pragma unroll 4
+        for (int i = t; i < n; i += T) {
+          const float s = s_src[i];
+          if (inside(s)) s_list[at++] = s;
+        }
+      if (t == 0) {
+        s_anchor[0] = inv0 > 0.f ? lo + (float)cross0 / inv0 : lo;
+        s_inv[0] = fminf(inv0 * (float)T, 1e30f);
+      }
+      __syncthreads();
+      const bool over = s_listed > kList;
+      const float* src = over ? s_src : s_list;
+      const int n_src = over ? n : s_listed;
+      auto bin_of = [&](int L, float s) {
+        const float x = (s - s_anchor[L]) * s_inv[L];
+        return x > 0.f ? (int)fminf(x, (float)(T - 1)) : 0;
+      };
+      auto each = [&](int levels, auto f) {          // the scores inside the crossing bins of so many levels
+#pragma unroll 1
+        for (int i = t; i < n_src; i += T) {
+          const float s = src[i];
+          bool in = !over || inside(s);
+#pragma unroll 1
+          for (int l = 0; l < levels; ++l) in = in && bin_of(l, s) == s_cross[l];
+          if (in) f(s);
+        }
+      };
+      // ---- a bin of it per thread; thread t looks after bin T - 1 - t
+#pragma unroll 1
+      for (int L = 0; L < kPoolLevels; ++L) {
+        float* w = reinterpret_cast<float*>(pool_smem + L * kLevelBytes);
+        unsigned int* cnt = reinterpret_cast<unsigned int*>(w + T);
+        each(L, [&](float s) {
+          const int b = bin_of(L, s);
+          // lanes that are at the same score go in one update: scores that are all alike would queue for one bin
+          const uint32_t key = float_key(s);
+          const unsigned int here = __activemask();
+          int lanes = 1;
+          if (__reduce_min_sync(here, key) == __reduce_max_sync(here, key)) {
+            if (lane != __ffs(here) - 1) return;
+            lanes = __popc(here);
+          }
+          atomicAdd(&cnt[b], (unsigned int)lanes);
+          atomicAdd(&w[b], (float)lanes * weight(s));
+        });
+        if (t == 0) { s_crossed = INT32_MAX; s_lowest = -1; s_k = 0; s_n = 0; s_best = 0u; s_least = 0xffffffffu; s_above = 0.0; }
+        meet();
+        const int b = T - 1 - t;
+        double x = 0.0;
+        int k = 0, before = 0;
+#pragma unroll
+        for (int c0 = 0; c0 < kPoolCtas; c0 += 4) {
+          if (c0 >= C) break;
+          unsigned int ks[4];
+          float ws[4];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const int from = min(c0 + c, C - 1);
+            ks[c] = *cluster.map_shared_rank(cnt + b, from);
+            ws[c] = *cluster.map_shared_rank(w + b, from);
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            if (c0 + c < C) {
+              x += (double)ws[c];
+              if (c0 + c < rank) before += (int)ks[c];
+              k += (int)ks[c];
+            }
+        }
+        const double excl = pool_exclusive(x, s_dsum);
+        if (k && excl < need && excl + x >= need) atomicMin(&s_crossed, t);
+        const unsigned int some = __ballot_sync(0xffffffffu, k != 0);
+        if (lane == 0 && some) atomicMax(&s_lowest, 32 * warp + 31 - __clz(some));      // where rounding keeps the sum below `need`
+        __syncthreads();
+        const int e = s_crossed != INT32_MAX ? s_crossed : s_lowest >= 0 ? s_lowest : T - 1;
+        if (t == e) {
+          s_above = excl; s_k = k; s_at = before; s_cross[L] = T - 1 - e;
+          if (L + 1 < kPoolLevels) {
+            s_anchor[L + 1] = s_inv[L] > 0.f ? s_anchor[L] + (float)(T - 1 - e) / s_inv[L] : s_anchor[L];
+            s_inv[L + 1] = fminf(s_inv[L] * (float)T, 1e30f);
+          }
+        }
+        __syncthreads();
+        need -= s_above;
+        const int K = s_k;
+        if (K <= kPoolFinal) {
+          // ---- the last few, each against all others: the largest key whose mass and that of those above reach the target
+          each(L + 1, [&](float s) {
+            const int to = s_at + atomicAdd(&s_n, 1);
+            const uint32_t key = float_key(s);
+            for (int c = 0; c < C; ++c) cluster.map_shared_rank(s_final, c)[to] = key;
+          });
+          meet();
+          int G = 32;                      // threads per score
+          while (G * K > T) G >>= 1;
+          const int i = t / G, r = t & (G - 1);
+          float mass = 0.f;
+          const uint32_t key = i < K ? s_final[i] : 0u;
+          if (i < K)
+#pragma unroll 1
+            for (int j = r; j < K; j += G) {
+              const uint32_t other = s_final[j];
+              if (other >= key) mass += weight(key_float(other));
+            }
+#pragma unroll 1
+          for (int o = G >> 1; o > 0; o >>= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
+          const uint32_t best = __reduce_max_sync(0xffffffffu, i < K && (double)mass >= need ? key : 0u);
+          const uint32_t least = __reduce_min_sync(0xffffffffu, i < K ? key : 0xffffffffu);
+          if (lane == 0) {
+            if (best) atomicMax(&s_best, best);
+            atomicMin(&s_least, least);
+          }
+          __syncthreads();
+          cutoff = s_best ? s_best : s_least;
+          break;
+        }
+        uint32_t kmin = 0xffffffffu, kmax = 0u;
+        each(L + 1, [&](float s) {
+          kmin = min(kmin, float_key(s));
+          kmax = max(kmax, float_key(s));
+        });
+        exchange(kmin, kmax);
+        cutoff = kmin;
+        if (kmin == kmax) break;
+      }
+    }
+    if (rank == 0 && t == 0) a.cutoff_per_head[bh] = key_float(cutoff);
+  } else {
+    if (rank == 0 && t == 0) a.cutoff_per_head[bh] = key_float(a.state[bh].cutoff_key);
+    __syncthreads();
+    all_there();
+  }
+
+  // ---- mark: a warp takes 32 queries x 32 blocks at a time.  Lane = query puts its mask word together (the lanes start at
+  // different blocks: rows a power of two apart would meet in a few banks); ballots of its bits are the column words.
+#pragma unroll 1
+  for (int sg = 0; sg < segs; ++sg)
+#pragma unroll 1
+    for (int g = sg * TW + ((warp - sg * TW) & (T / 32 - 1)); g < (sg + 1) * TW; g += T / 32) {
+      const int rows = nq - g * 32;         // (< 1 beyond the head's last query)
+      const bool live = lane < rows;
+#pragma unroll 1
+      for (int i = 0; i < mw; ++i) {
+        const int width = min(32, Nb - 32 * i);
+        uint32_t word = 0u, col = 0u;
+        uint32_t* to = gmask + (g * 32 + lane) * mw + i;
+        if constexpr (SRC == kPoolMask) {
+          if (live) word = *to;
+        } else {
+          if (live) {
+            const float* s = s_src + (g * 32 + lane) * Nb + 32 * i;
+            int j = lane & ((1 << (31 - __clz(width))) - 1);
+#pragma unroll 4
+            for (int r = 0; r < width; ++r) {
+              // (a NaN without a sign goes as -0, as it does in mark_kernel, whose key the compiler takes for a float operation)
+              const float x = s[j];
+              uint32_t key = float_key(x);
+              if (x != x && key > 0x80000000u) key = 0x7fffffffu;
+              if (key >= cutoff) word |= 1u << j;
+              if (++j == width) j = 0;
+            }
+            if (a.own_sb > 0) {             // the query's own block, if it is to be kept
+              const int own = (q0 + g * 32 + lane) / a.own_sb;
+              if ((own >> 5) == i) word |= 1u << (own & 31);
+            }
+            *to = word;
+          }
+          __syncwarp();
+        }
+#pragma unroll 4
+        for (int r = 0; r < width; ++r) {
+          const uint32_t c = __ballot_sync(0xffffffffu, (word >> r) & 1u);
+          if (lane == r) col = c;
+        }
+        if (lane < width) {
+          gtm[g * Nb + 32 * i + lane] = col;
+          if (col) atomicAdd(&s_seg[sg * Nb + 32 * i + lane], __popc(col));
+        }
+      }
+    }
+  __syncthreads();
+  // ---- places of the segments' pairs, from the head's first pair on: by key block, by query, and of the blocks
+  int pairs = 0;
+  for (int j = t; j < Nb; j += T) {
+    int sum = 0;
+    for (int sg = 0; sg < segs; ++sg) {
+      const int x = s_seg[sg * Nb + j];
+      if (x) atomicAdd(&s_segp[sg], x);
+      sum += x;
+    }
+    for (int c = 0; c < C; ++c) cluster.map_shared_rank(s_tot + rank * Nb, c)[j] = sum;
+    pairs += sum;
+  }
+  const int before = pool_exclusive(pairs, s_sum);
+  if (t == T - 1)
+    for (int c = 0; c < C; ++c) cluster.map_shared_rank(s_pairs, c)[rank] = before + pairs;
+  meet();      // (what is read from here on is the CTA's own: it may leave when it is done)
+  const int per = (Nb + T - 1) / T, j0 = min(t * per, Nb), j1 = min(j0 + per, Nb);
+  int run_all = 0;
+  for (int j = j0; j < j1; ++j) {
+    int run = 0;
+    for (int c = 0; c < C; ++c) {
+      const int x = s_tot[c * Nb + j];
+      if (c < rank) run += x;
+      run_all += x;
+    }
+    for (int sg = 0; sg < segs; ++sg) {
+      a.seg_cnt[((long long)bh * a.nseg + seg0 + sg) * Nb + j] = run;
+      run += s_seg[sg * Nb + j];
+    }
+  }
+  if (t == T - 1) {
+    int run = 0;
+    for (int c = 0; c < rank; ++c) run += s_pairs[c];
+    for (int sg = 0; sg < segs; ++sg) {
+      a.seg_qoff[bh * a.nseg + seg0 + sg] = run;
+      run += s_segp[sg];
+    }
+  }
+  if (rank == 0) {
+    int at = pool_exclusive(run_all, s_sum);
+    int* kb = a.kb_excl + (long long)bh * (Nb + 1);
+    for (int j = j0; j < j1; ++j) {
+      kb[j] = at;
+      for (int c = 0; c < C; ++c) at += s_tot[c * Nb + j];
+    }
+    if (t == T - 1) a.k_per_head[bh] = at;
+  }
+}
+
 // Row normalisation for the second reading of Eq. 4: out[i][j] = sigma * s[i][j] - logsumexp_j(sigma * s[i][:]),
 // the logarithm of S times the pair's probability when every query is normalised on its own.  One
 // warp per query row; the head-wide quantile search then runs on `out` with unit temperature.
@@ -1155,6 +1605,40 @@ static int seg_queries(int mw) {
   return q;
 }
 
+// How select_pool_kernel divides a head (C = 0: it does not take it, the passes over the matrix do).  It takes what runs in one
+// wave: 12 heads x 215,000 scores 56.6 -> 38.7 us, but 40 heads of them, in two and a half, 89.6 -> 103.7.
+struct PoolPlan { int C, T, QSEG, nseg, segs_per; size_t smem, smem_mask; };
+static PoolPlan pool_plan(const Dims& D) {
+  PoolPlan p = {};
+  const long long P = (long long)D.S * D.Nb;
+  if (P > kPoolCtas * (long long)kPoolSmemMax / 4 || D.Nb > 1024) return p;
+  auto divide = [&](int C) {
+    const int most = seg_queries(D.mask_words);
+    p.C = C;
+    p.segs_per = (int)(((long long)D.S + (long long)most * C - 1) / ((long long)most * C));
+    p.QSEG = (D.S + C * p.segs_per - 1) / (C * p.segs_per);
+    p.QSEG = (p.QSEG + 31) / 32 * 32;
+    p.nseg = (D.S + p.QSEG - 1) / p.QSEG;
+    p.segs_per = (p.nseg + C - 1) / C;
+    p.smem_mask = 4 * ((size_t)C * D.Nb + (size_t)p.segs_per * (D.Nb + 1)) + 16;
+    p.T = P / C <= kPoolShort ? 256 : 512;
+    p.smem = kPoolFront * p.T + p.smem_mask + 4 * (size_t)p.segs_per * p.QSEG * D.Nb;
+    return p.smem <= (size_t)kPoolSmemMax;
+  };
+  auto at_once = [&](int C) {
+    const long long per_sm = std::min<long long>((227 * 1024) / (long long)(p.smem + 5 * 1024), 2048 / p.T);
+    return (long long)D.BH * C <= sm_count() * per_sm;
+  };
+  int C = 1;
+  while (C < kPoolCtas && P / C > kPoolSlice && (long long)D.BH * 2 * C <= sm_count()) C *= 2;
+  while (!divide(C)) {
+    if (C == kPoolCtas) { p.C = 0; return p; }
+    C *= 2;
+  }
+  if (!at_once(C)) p.C = 0;
+  return p;
+}
+
 struct SelectWs {
   HeadState* state;
   unsigned int* g_cnt;
@@ -1165,7 +1649,9 @@ struct SelectWs {
   int* seg_cnt;
   int* seg_total;
   int* seg_qoff;
-  int* kb_total;
+  int* kb_total;        // pairs of a block; from select_pool_kernel: [BH][Nb + 1] pairs of the head in front of it
+  PoolPlan pool;
+  int QSEG, nseg;       // queries of a segment, segments of a head
   float* cand;          // [BH][ccap] scores copied aside by the level-0 pass (optional: the last slice)
   long long ccap;
   size_t base_bytes;    // without the candidate lists
@@ -1182,20 +1668,22 @@ static long long cand_capacity(const Dims& D) {
 static SelectWs carve_select(const Dims& D, void* ws) {
   SelectWs w;
   Carver c(ws);
-  int QSEG = seg_queries(D.mask_words);
-  long long nseg = (D.S + QSEG - 1) / QSEG;
+  w.pool = pool_plan(D);
+  const int QSEG = w.QSEG = w.pool.C ? w.pool.QSEG : seg_queries(D.mask_words);
+  const long long nseg = w.nseg = (D.S + QSEG - 1) / QSEG;
   w.state = c.take<HeadState>(D.BH);
-  w.g_cnt = c.take<unsigned int>((size_t)D.BH * kBins);
-  w.g_w = c.take<double>((size_t)D.BH * kBins);
-  w.g_minkey = c.take<uint32_t>((size_t)D.BH * kBins);
-  w.g_maxkey = c.take<uint32_t>((size_t)D.BH * kBins);
+  const size_t bins = w.pool.C ? 0 : (size_t)D.BH * kBins;      // (select_pool_kernel keeps its bins to itself)
+  w.g_cnt = c.take<unsigned int>(bins);
+  w.g_w = c.take<double>(bins);
+  w.g_minkey = c.take<uint32_t>(bins);
+  w.g_maxkey = c.take<uint32_t>(bins);
   w.tmask = c.take<uint32_t>((size_t)D.BH * nseg * D.Nb * (QSEG >> 5));
   w.seg_cnt = c.take<int>((size_t)D.BH * nseg * D.Nb);
   w.seg_total = c.take<int>((size_t)D.BH * nseg);
   w.seg_qoff = c.take<int>((size_t)D.BH * nseg + 1);
-  w.kb_total = c.take<int>((size_t)D.BH * D.Nb);
+  w.kb_total = c.take<int>((size_t)D.BH * (D.Nb + 1));
   w.base_bytes = c.total();
-  w.ccap = cand_capacity(D);
+  w.ccap = w.pool.C ? 0 : cand_capacity(D);
   w.cand = c.take<float>((size_t)D.BH * w.ccap);
   w.bytes = c.total();
   w.guards = c.guards;
@@ -1256,8 +1744,23 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     range = nullptr;      // the range of the raw scores says nothing about the transformed matrix
   }
   VMOBA_GUARDS_ARM(w.guards, st);
-  const int QSEG = seg_queries(D.mask_words);
-  const int nseg = (D.S + QSEG - 1) / QSEG;
+  const int QSEG = w.QSEG, nseg = w.nseg;
+  const bool pool = w.pool.C > 0;
+  auto pool_launch = [&](auto tag, const float* pool_range, int unit_w, double count_target) -> int {
+    const size_t pool_smem = decltype(tag)::value == kPoolMask ? w.pool.smem_mask : w.pool.smem;
+    PoolArgs a;
+    a.scores = scores; a.range = pool_range; a.state = w.state;
+    a.S = D.S; a.Nb = D.Nb; a.mw = D.mask_words; a.QSEG = QSEG; a.nseg = nseg; a.segs_per = w.pool.segs_per;
+    a.own_sb = own_sb; a.unit_w = unit_w; a.sigma = sigma; a.tau = tau; a.count_target = count_target;
+    a.mask_bits = mask_bits; a.tmask = w.tmask; a.seg_cnt = w.seg_cnt; a.seg_qoff = w.seg_qoff; a.kb_excl = w.kb_total;
+    a.k_per_head = k_per_head; a.cutoff_per_head = cutoff_per_head;
+    auto kernel = w.pool.T == 256 ? select_pool_kernel<decltype(tag)::value, 256> : select_pool_kernel<decltype(tag)::value, 512>;
+    VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pool_smem));
+    launch_cluster(w.pool.C, kernel, (unsigned)(D.BH * w.pool.C), w.pool.T, pool_smem, st, a);
+    VMOBA_LAUNCH_OK(1);
+    return VMOBA_OK;
+  };
+#define VMOBA_POOL(src) std::integral_constant<PoolSrc, src>()
   const size_t smem = (size_t)QSEG * D.mask_words * 4 + (size_t)std::max(D.Nb, QSEG) * 4 + (size_t)D.Nb * (QSEG >> 5) * 4;
   const dim3 sgrid(nseg, D.BH);
 
@@ -1309,11 +1812,16 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
       else threshold_words(VMOBA_INT(kLocalMaxWords));
     }
 #undef VMOBA_INT
+    VMOBA_LAUNCH_OK(2);
+    if (pool) {
+      if ((rc = pool_launch(VMOBA_POOL(kPoolMask), nullptr, 0, -1.0))) return rc;
+    } else {
     launch_kernel(local_cutoff_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, cutoff_per_head, D.BH);
     VMOBA_CUDA_OK(cudaFuncSetAttribute(mark_from_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     launch_kernel(mark_from_mask_kernel, sgrid, kSegThreads, smem, st, mask_bits, D.S, D.Nb, D.mask_words, QSEG, nseg,
                   w.seg_cnt, w.seg_total, w.tmask);
-    VMOBA_LAUNCH_OK(4);
+    VMOBA_LAUNCH_OK(2);
+    }
   } else {
     // head-wide rules: weighted quantile of the pool (unit weights and a pair budget for top-k)
     double count_target = -1.0;
@@ -1322,6 +1830,9 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
       tau = count_target >= (double)P ? 1.0f : 0.5f;      // tau only tells the scan whether everything is taken
     }
     const int unit_w = by_topk ? 1 : 0;
+    if (pool) {
+      if ((rc = pool_launch(VMOBA_POOL(kPoolScores), range, unit_w, count_target))) return rc;
+    } else {
     launch_kernel(init_state_kernel, (unsigned)(((long long)D.BH * kBins + 255) / 256), 256, 0, st, w.state, D.BH,
                   range, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey);
 
@@ -1357,22 +1868,28 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     launch_kernel(mark_kernel, sgrid, kSegThreads, smem, st, scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg,
                   own_sb, mask_bits, w.seg_cnt, w.seg_total, w.tmask);
     VMOBA_LAUNCH_OK(1);
+    }
   }
+#undef VMOBA_POOL
 
   const size_t smem_fill = ((size_t)QSEG * D.mask_words + 2 * (size_t)D.Nb * (QSEG >> 5) + 2 * (size_t)D.Nb + 1 + 2 * kStage) * 4;
   VMOBA_CUDA_OK(cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fill));
   long long nkb = (long long)D.BH * D.Nb;
-  launch_kernel(seg_prefix_kernel, (unsigned)(D.BH * ((D.Nb + 31) / 32)), 32 * std::min(32, (nseg + 7) / 8), 0, st,
-                w.seg_cnt, w.kb_total, D.Nb, nseg);
-  launch_kernel(offsets_kernel, 1, 1024, 0, st, w.kb_total, kb_ptr, nkb, w.seg_total, w.seg_qoff,
-                (long long)D.BH * nseg, D.BH, D.Nb, k_per_head, capacity, q_ptr + (long long)D.BH * D.S, dev_status);
+  if (!pool) {
+    launch_kernel(seg_prefix_kernel, (unsigned)(D.BH * ((D.Nb + 31) / 32)), 32 * std::min(32, (nseg + 7) / 8), 0, st,
+                  w.seg_cnt, w.kb_total, D.Nb, nseg);
+    launch_kernel(offsets_kernel, 1, 1024, 0, st, w.kb_total, kb_ptr, nkb, w.seg_total, w.seg_qoff,
+                  (long long)D.BH * nseg, D.BH, D.Nb, k_per_head, capacity, q_ptr + (long long)D.BH * D.S, dev_status);
+    VMOBA_LAUNCH_OK(2);
+  }
   // A thread per query of the segment; many blocks leave short segments (32 queries from 2,049 blocks on), whose columns and
   // runs want the threads all the same: 2,100 blocks x 33,600 queries 1001 -> 432 us (whole selection, threshold rule), 8,192 x
   // 16,384 3376 -> 1053.
   const int fill_threads = QSEG >= 128 ? QSEG : kSegThreads;
   launch_kernel(fill_kernel, sgrid, fill_threads, smem_fill, st, mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg,
-                kb_ptr, w.seg_cnt, w.seg_qoff, q_idx, q_ptr, q_pairs, capacity);
-  VMOBA_LAUNCH_OK(3);
+                kb_ptr, w.seg_cnt, w.seg_qoff, q_idx, q_ptr, q_pairs, capacity, pool ? w.kb_total : nullptr, k_per_head,
+                dev_status);
+  VMOBA_LAUNCH_OK(1);
   VMOBA_GUARDS_CHECK(w.guards, dev_status, st);
   return VMOBA_OK;
 }

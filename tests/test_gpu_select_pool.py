@@ -1,0 +1,157 @@
+"""Small pools (up to 2^20 scores per head): the whole of the selection up to the offsets is one kernel, a cluster per head.
+Larger ones go through the chain of passes over the score matrix, with which it is compared here: a pool of m copies of the same
+scores has m times the mass above any score, so the cutoff is the same and every copy keeps the same pairs."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2506_23858_b200 import binding as vb
+
+pytestmark = pytest.mark.gpu
+POOL_MAX = 1 << 20
+
+
+def _run(shape, scores, rule, tau=0.25, topk=1, score_range=None, capacity=None):
+    BH, S, Nb = shape.B * shape.heads, shape.S, shape.n_blocks
+    cap = capacity or BH * S * Nb
+    new = lambda n, dt=torch.int32: torch.full((n,), -7, dtype=dt, device="cuda")
+    out = dict(mask=new(BH * S * shape.mask_words), kb_ptr=new(BH * Nb + 1), q_idx=new(cap), q_ptr=new(BH * S + 1), q_pairs=new(cap),
+               k=new(BH, torch.int64), cutoff=torch.full((BH,), float("nan"), device="cuda"),
+               status=torch.zeros(1, dtype=torch.int32, device="cuda"))
+    ws = torch.full((vb.workspace_bytes(shape, vb.STAGE_SELECT, cap),), 0x5a, dtype=torch.uint8, device="cuda")
+    args = (out["mask"], out["kb_ptr"], out["q_idx"], out["q_ptr"], out["q_pairs"], cap, out["k"], out["cutoff"], out["status"], ws)
+    if score_range is None:
+        vb.vmoba_select_rule_apply(shape, scores, rule, tau, topk, *args)
+    else:
+        vb.vmoba_select_ranged(shape, scores, score_range, rule, tau, topk, *args)
+    torch.cuda.synchronize()
+    return out
+
+
+def _mask(shape, out):
+    BH, S, Nb = shape.B * shape.heads, shape.S, shape.n_blocks
+    w = out["mask"].cpu().numpy().view(np.uint32).reshape(BH, S, -1)
+    bits = ((w[..., None] >> np.arange(32, dtype=np.uint32)) & 1).astype(bool).reshape(BH, S, -1)
+    assert not bits[..., Nb:].any()
+    return bits[..., :Nb]
+
+
+def _check_lists(shape, out, m):
+    """kb_ptr, q_idx, q_ptr, q_pairs and the counts are those of the mask."""
+    BH, S, Nb = m.shape
+    assert out["k"].tolist() == m.sum((1, 2)).tolist()
+    per_block = m.sum(1).reshape(-1)
+    assert out["kb_ptr"].tolist() == [0] + np.cumsum(per_block).tolist()
+    assert out["q_ptr"].tolist() == [0] + np.cumsum(m.sum(2).reshape(-1)).tolist()
+    n = int(m.sum())
+    bh, j, q = np.nonzero(m.transpose(0, 2, 1))          # by block, then query
+    assert np.array_equal(out["q_idx"][:n].cpu().numpy(), q)
+    place = np.zeros(m.shape, dtype=np.int64)
+    place[bh, q, j] = np.arange(n)
+    assert np.array_equal(out["q_pairs"][:n].cpu().numpy(), place[m])
+
+
+def _shape(heads, grid, block):
+    return vb.make_shape(1, heads, 64, grid, block, "f32")
+
+
+# grid, block: one CTA; several, some of them without a segment; rows of an odd number of blocks (slices off 16-byte boundaries); short
+# rows; rows of several mask words; slices that stay in shared memory and, from 320K scores on, that do not
+SHAPES = [((1, 7, 9), (1, 1, 1)), ((4, 8, 8), (1, 8, 8)), ((3, 43, 8), (3, 43, 1)), ((5, 13, 11), (1, 13, 11)), ((2, 33, 37), (1, 3, 37)),
+          ((8, 24, 35), (2, 3, 35)), ((7, 40, 35), (7, 10, 5)), ((6, 40, 35), (3, 10, 5)), ((5, 25, 34), (5, 5, 2))]
+
+
+@pytest.mark.parametrize("grid,block", SHAPES)
+@pytest.mark.parametrize("rule,tau,topk", [(vb.SELECT_THRESHOLD_GLOBAL, 0.25, 0), (vb.SELECT_THRESHOLD_GLOBAL, 1.0, 0),
+                                           (vb.SELECT_TOPK_GLOBAL, 0.0, 3)])
+def test_pool_kernel_agrees_with_the_passes_over_the_matrix(grid, block, rule, tau, topk):
+    heads = 3
+    small = _shape(heads, grid, block)
+    S, Nb = small.S, small.n_blocks
+    assert S * Nb <= POOL_MAX
+    copies = POOL_MAX // (S * Nb) + 1
+    # the copies are further query rows: the same blocks per row, `copies` times the frames and the frames per block
+    large = _shape(heads, (grid[0] * copies, grid[1], grid[2]), (block[0] * copies, block[1], block[2]))
+    assert large.n_blocks == Nb and large.S * Nb > POOL_MAX
+    g = torch.Generator(device="cuda").manual_seed(S * Nb)
+    x = 4.0 * torch.randn((heads, S, Nb), generator=g, device="cuda")
+    y = x[:, None].expand(heads, copies, S, Nb).reshape(heads, copies * S, Nb).contiguous()
+    a = _run(small, x, rule, tau, topk)
+    ranged = _run(small, x, rule, tau, topk, score_range=torch.stack([x.amin((1, 2)), x.amax((1, 2))], 1).contiguous())
+    b = _run(large, y, rule, tau, topk, capacity=int(heads * large.S * Nb))
+    ma = _mask(small, a)
+    for out in (a, ranged):
+        _check_lists(small, out, _mask(small, out))
+        assert int(out["status"]) == 0
+    # the budget of the pair-count rule and, for masses, one pair at the cutoff: sums of up to 2^20 fp32 weights in any order
+    # are off by 1e-6 of the whole, less than a pair's weight at most cutoffs
+    mb = _mask(large, b).reshape(heads, copies, S, Nb)
+    for other in (_mask(small, ranged), mb[:, 0], mb[:, -1]):
+        assert (np.abs(other.sum((1, 2)) - ma.sum((1, 2))) <= (1 if rule == vb.SELECT_THRESHOLD_GLOBAL else 0)).all()
+        assert (other != ma).sum() <= heads
+    assert torch.allclose(a["cutoff"], b["cutoff"], atol=1e-2)
+
+
+@pytest.mark.parametrize("values", ["constant", "zeros", "two", "infinite", "nan"])
+@pytest.mark.parametrize("rule,tau,topk", [(vb.SELECT_THRESHOLD_GLOBAL, 0.3, 0), (vb.SELECT_TOPK_GLOBAL, 0.0, 2)])
+def test_pool_kernel_special_scores(values, rule, tau, topk):
+    """Ties, infinities and NaN come out as they do from the passes over the matrix (same copies as above)."""
+    heads, grid, block = 2, (4, 13, 11), (1, 13, 11)
+    small = _shape(heads, grid, block)
+    S, Nb = small.S, small.n_blocks
+    copies = POOL_MAX // (S * Nb) + 1
+    large = _shape(heads, (grid[0] * copies, grid[1], grid[2]), (block[0] * copies, block[1], block[2]))
+    g = torch.Generator(device="cuda").manual_seed(3)
+    x = torch.randn((heads, S, Nb), generator=g, device="cuda")
+    if values == "constant":
+        x.fill_(1.25)
+    elif values == "zeros":
+        x.zero_()
+        x[:, ::3] = -0.0
+    elif values == "two":
+        x = torch.where(x > 0, 2.0, -1.0)
+    elif values == "infinite":
+        x[:, ::50] = -float("inf")
+        x[0, 7, 1] = float("inf")
+    elif values == "nan":
+        x[0, 5] = float("nan")
+        x[1, 9, 2] = -float("nan")
+    y = x[:, None].expand(heads, copies, S, Nb).reshape(heads, copies * S, Nb).contiguous()
+    score_range = None
+    if values == "nan":          # (as the scores kernel leaves it: of the numbers)
+        score_range = torch.stack([x.nan_to_num(0.0).amin((1, 2)), x.nan_to_num(0.0).amax((1, 2))], 1).contiguous()
+    a = _run(small, x, rule, tau, topk, score_range)
+    b = _run(large, y, rule, tau, topk, score_range, capacity=int(heads * large.S * Nb))
+    ma, mb = _mask(small, a), _mask(large, b).reshape(heads, copies, S, Nb)
+    _check_lists(small, a, ma)
+    # a NaN takes the mass of the lowest bin of its CTA (there) or thread (here) with it: a few pairs of 600
+    assert (ma != mb[:, 0]).sum() <= (8 if values == "nan" else 0) and (mb[:, 0] == mb[:, -1]).all()
+    if values == "nan":
+        assert np.array_equal(ma[0, 5], mb[0, 0, 5]) and ma[1, 9, 2] == mb[1, 0, 9, 2]
+
+
+@pytest.mark.parametrize("rule,topk", [(vb.SELECT_TOPK_LOCAL, 3), (vb.SELECT_THRESHOLD_LOCAL, 0),
+                                       (vb.SELECT_THRESHOLD_GLOBAL | vb.SELECT_KEEP_OWN_BLOCK, 0)])
+@pytest.mark.parametrize("grid,block", SHAPES[1:])
+def test_lists_of_small_pools_follow_the_mask(grid, block, rule, topk):
+    shape = _shape(3, grid, block)
+    x = torch.randn((3, shape.S, shape.n_blocks), generator=torch.Generator(device="cuda").manual_seed(1), device="cuda")
+    out = _run(shape, x, rule, 0.3, topk)
+    m = _mask(shape, out)
+    _check_lists(shape, out, m)
+    if rule == vb.SELECT_TOPK_LOCAL:
+        want = torch.zeros_like(x, dtype=torch.bool).scatter_(2, x.topk(min(topk, shape.n_blocks), 2).indices, True)
+        assert np.array_equal(m, want.cpu().numpy())
+        assert torch.equal(out["cutoff"], torch.where(want, x, torch.inf).amin((1, 2)))
+    if rule & vb.SELECT_KEEP_OWN_BLOCK:
+        own = np.arange(shape.S) // (shape.S // shape.n_blocks)
+        assert m[:, np.arange(shape.S), own].all()
+
+
+def test_too_small_a_capacity_is_reported():
+    shape = _shape(2, (4, 8, 8), (1, 8, 8))
+    x = torch.randn((2, shape.S, shape.n_blocks), device="cuda")
+    out = _run(shape, x, vb.SELECT_TOPK_LOCAL, topk=2, capacity=700)
+    assert int(out["status"]) == vb.ERR_CAPACITY
+    out = _run(shape, x, vb.SELECT_TOPK_LOCAL, topk=2, capacity=1024)
+    assert int(out["status"]) == 0
