@@ -40,12 +40,28 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
+// A look that does not suspend the thread: 1 if the phase has completed.
+__device__ __forceinline__ uint32_t mbar_test_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  return ok;
+}
+
 // Bounded wait.  `abort_flag` (shared memory) is set on the first timeout of the CTA; once set,
 // later waits give up after a few polls so that the kernel drains quickly.
 __device__ __forceinline__ bool mbar_wait_polls(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int32_t* status,
                                                 uint32_t polls) {
+  // (the first look ahead of the abort flag, whose load is another trip to shared memory: dense forward and backward of 13,440
+  // tokens, 12 heads, 4.47 -> 4.31 ms, backward of 55K tokens 3.16 -> 3.09)
+  if (mbar_try_wait(bar, parity)) return true;
   const uint32_t limit = *abort_flag ? 16u : polls;
-  for (uint32_t i = 0; i < limit; ++i) {
+  for (uint32_t i = 1; i < limit; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if (i > 4096) __nanosleep(64);
   }
@@ -76,8 +92,7 @@ __device__ __forceinline__ void mbar_wait_warp(uint64_t* bar, uint32_t parity, v
 // Bounded wait of a whole warp whose lanes look at different barriers: returns when every lane's phase has completed.
 __device__ __forceinline__ void mbar_wait_lanes(uint32_t bar_addr, uint32_t parity, volatile int* abort_flag, int32_t* status) {
   constexpr uint32_t kPolls = 1u << 22;
-  const uint32_t limit = __reduce_max_sync(0xffffffffu, *abort_flag ? 16u : kPolls);
-  for (uint32_t i = 0; i < limit; ++i) {
+  auto look = [&]() {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
@@ -86,7 +101,12 @@ __device__ __forceinline__ void mbar_wait_lanes(uint32_t bar_addr, uint32_t pari
         : "=r"(ok)
         : "r"(bar_addr), "r"(parity)
         : "memory");
-    if (__all_sync(0xffffffffu, ok != 0)) return;
+    return __all_sync(0xffffffffu, ok != 0);
+  };
+  if (look()) return;
+  const uint32_t limit = __reduce_max_sync(0xffffffffu, *abort_flag ? 16u : kPolls);
+  for (uint32_t i = 1; i < limit; ++i) {
+    if (look()) return;
     if (i > 4096) __nanosleep(64);
   }
   *abort_flag = 1;
