@@ -194,9 +194,9 @@ template <typename... P, typename... A>
 inline void launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   launch_kernel(true, kernel, grid, block, smem, st, std::forward<A>(args)...);
 }
-// Early, in clusters of `cluster` consecutive CTAs.
+// In clusters of `cluster` consecutive CTAs.
 template <typename... P, typename... A>
-inline void launch_cluster(int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+inline void launch_cluster(bool early, int cluster, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -210,10 +210,9 @@ inline void launch_cluster(int cluster, void (*kernel)(P...), dim3 grid, dim3 bl
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
 #ifdef VMOBA_DEBUG
-  cfg.numAttrs = 1;
-#else
-  cfg.numAttrs = 2;
+  early = false;
 #endif
+  cfg.numAttrs = early ? 2 : 1;
   cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 

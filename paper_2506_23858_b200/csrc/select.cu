@@ -45,6 +45,7 @@ struct HeadState {
   unsigned int cand_cnt;       // pairs of the level-0 crossing bin, copied aside by the level-1 pass
   int cand_ok;                 // every one of them found room in the list: level 2 reads the list
   float bin0_off;              // -anchor[0] * inv[0]: the level-0 bin of s is floor(s * inv[0] + bin0_off)
+  float win_lo, win_hi;        // the window that a sample gives the cutoff
   uint32_t pad;
 };
 
@@ -1201,6 +1202,240 @@ __device__ __noinline__ T pool_exclusive(T x, T* s_warp) {
   return before + (inc - x);
 }
 
+// The search for a head's cutoff among the scores src[0 .. n) of every CTA of a cluster, which lie in [lo, lo + span] (shared or
+// global memory; I: a type that holds n).  target(total, need): the mass to be covered, given that of all these scores; false: they
+// cannot hold the cutoff, and the search ends.  front: kPoolFront * T bytes of shared memory.  WIDE: from global memory, sixteen bytes
+// per load.
+template <int T, bool WIDE, typename I, typename Meet, typename Weight, typename Target>
+__device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& cluster, Meet meet, unsigned char* front, const float* src,
+                                            I n, float lo, float span, Weight weight, Target target, uint32_t& cutoff) {
+  constexpr int kLevelBytes = 8 * T, kList = (kPoolFront * T - kPoolLevels * kLevelBytes) / 4;
+  __shared__ double s_w0[kPoolCtas][kPoolBins0], s_dsum[32], s_above;
+  __shared__ uint32_t s_key[kPoolCtas][2], s_final[kPoolFinal], s_best, s_least;
+  __shared__ int s_crossed, s_lowest, s_n, s_at, s_k, s_cross[kPoolLevels];
+  __shared__ I s_sum[32], s_listed;
+  __shared__ float s_anchor[kPoolLevels], s_inv[kPoolLevels];
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  float* s_own = reinterpret_cast<float*>(front);        // [kPoolBins0][threads]
+#pragma unroll
+  for (int b = 0; b < kPoolBins0 / 4; ++b) reinterpret_cast<float4*>(s_own)[b * T + t] = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
+  const float inv0 = span > 0.f ? (float)kPoolBins0 / span : 0.f, off0 = -lo * inv0;
+  // smallest and largest of a value over the cluster
+  auto exchange = [&](uint32_t& least, uint32_t& most) {
+    least = __reduce_min_sync(0xffffffffu, least);
+    most = __reduce_max_sync(0xffffffffu, most);
+    if (lane == 0) { atomicMin(&s_least, least); atomicMax(&s_best, most); }
+    __syncthreads();
+    if (t < C) {
+      uint32_t* to = cluster.map_shared_rank(s_key[rank], t);
+      to[0] = s_least; to[1] = s_best;
+    }
+    meet();
+    for (int c = 0; c < C; ++c) { least = min(least, s_key[c][0]); most = max(most, s_key[c][1]); }
+  };
+  auto stream = [&](const float* from, I count, auto f) {
+    I i = t;
+    if constexpr (WIDE) {
+      if ((reinterpret_cast<uintptr_t>(from) & 15u) == 0) {
+        const I trips = count / (16 * (I)T);
+#pragma unroll 1
+        for (I r = 0; r < trips; ++r) {
+          float4 x[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[j] = reinterpret_cast<const float4*>(from)[(4 * r + j) * (I)T + t];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) { f(x[j].x); f(x[j].y); f(x[j].z); f(x[j].w); }
+        }
+        i += trips * 16 * (I)T;
+      }
+    }
+#pragma unroll 4
+    for (; i < count; i += T) f(from[i]);
+  };
+  // ---- the first bins: floor(s * inv0 + off0) by an addition that rounds down, NaN to bin 0
+  stream(src, n, [&](float s) {
+    const float x = fminf(fmaxf(fmaf(s, inv0, off0), 0.f), (float)(kPoolBins0 - 1));
+    const int b = __float_as_int(__fadd_rd(x, 8388608.f)) & (kPoolBins0 - 1);
+    s_own[b * T + t] += weight(s);
+  });
+  __syncthreads();
+#pragma unroll 1
+  for (int b = warp; b < kPoolBins0; b += T / 32) {
+    float w = 0.f;
+#pragma unroll
+    for (int r = 0; r < T / 32; ++r) {
+      const float x = s_own[b * T + 32 * r + lane];
+      if (x > 0.f) w += x;
+    }
+    double x = (double)w;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane < C) cluster.map_shared_rank(s_w0[rank], lane)[b] = x;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 2 * kPoolLevels; ++i) reinterpret_cast<uint32_t*>(front)[i * T + t] = 0u;
+  meet();
+  double need;                           // mass still to be covered from the crossing bin down
+  int cross0;
+  {
+    double x = 0.0;                      // lane l: bin 31 - l
+    for (int c = 0; c < C; ++c) x += s_w0[c][kPoolBins0 - 1 - lane];
+    double inc = x;
+#pragma unroll 1
+    for (int o = 1; o < 32; o <<= 1) {
+      const double v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    const double total = __shfl_sync(0xffffffffu, inc, 31), excl = inc - x;
+    if (!target(total, need)) return false;
+    const unsigned int hit = __ballot_sync(0xffffffffu, x > 0.0 && excl < need && inc >= need);
+    const unsigned int occupied = __ballot_sync(0xffffffffu, x > 0.0);
+    const int e = hit ? __ffs(hit) - 1 : occupied ? 31 - __clz(occupied) : kPoolBins0 - 1;
+    cross0 = kPoolBins0 - 1 - e;
+    need -= __shfl_sync(0xffffffffu, excl, e);
+  }
+  {
+    // ---- the list of the crossing bin's scores (the last bin has no end), if it has room for them
+    const float y_lo = (float)cross0, y_hi = cross0 == kPoolBins0 - 1 ? NAN : (float)(cross0 + 1);
+    auto inside = [&](float s) {
+      const float y = fmaf(s, inv0, off0);
+      return (cross0 == 0 || y >= y_lo) && !(y >= y_hi);
+    };
+    float* s_list = reinterpret_cast<float*>(front + kPoolLevels * kLevelBytes);
+    I mine = 0;
+    stream(src, n, [&](float s) { mine += inside(s) ? 1 : 0; });
+    I at = pool_exclusive(mine, s_sum);
+    if (t == T - 1) s_listed = at + mine;
+    if (mine && at + mine <= kList)
+      stream(src, n, [&](float s) { if (inside(s)) s_list[at++] = s; });
+    if (t == 0) {
+      s_anchor[0] = inv0 > 0.f ? lo + (float)cross0 / inv0 : lo;
+      s_inv[0] = fminf(inv0 * (float)T, 1e30f);
+    }
+    __syncthreads();
+    const bool over = s_listed > kList;
+    const float* in_bin = over ? src : s_list;
+    const I n_in = over ? n : s_listed;
+    auto bin_of = [&](int L, float s) {
+      const float x = (s - s_anchor[L]) * s_inv[L];
+      return x > 0.f ? (int)fminf(x, (float)(T - 1)) : 0;
+    };
+    auto each = [&](int levels, auto f) {          // the scores inside the crossing bins of so many levels
+      auto look = [&](float s) {
+        bool in = !over || inside(s);
+#pragma unroll 1
+        for (int l = 0; l < levels; ++l) in = in && bin_of(l, s) == s_cross[l];
+        if (in) f(s);
+      };
+#pragma unroll 1
+      for (I i = t; i < n_in; i += T) look(in_bin[i]);
+    };
+    // ---- a bin of it per thread; thread t looks after bin T - 1 - t
+#pragma unroll 1
+    for (int L = 0; L < kPoolLevels; ++L) {
+      float* w = reinterpret_cast<float*>(front + L * kLevelBytes);
+      unsigned int* cnt = reinterpret_cast<unsigned int*>(w + T);
+      each(L, [&](float s) {
+        const int b = bin_of(L, s);
+        // lanes that are at the same score go in one update: scores that are all alike would queue for one bin
+        const uint32_t key = float_key(s);
+        const unsigned int here = __activemask();
+        int lanes = 1;
+        if (__reduce_min_sync(here, key) == __reduce_max_sync(here, key)) {
+          if (lane != __ffs(here) - 1) return;
+          lanes = __popc(here);
+        }
+        atomicAdd(&cnt[b], (unsigned int)lanes);
+        atomicAdd(&w[b], (float)lanes * weight(s));
+      });
+      if (t == 0) { s_crossed = INT32_MAX; s_lowest = -1; s_k = 0; s_n = 0; s_best = 0u; s_least = 0xffffffffu; s_above = 0.0; }
+      meet();
+      const int b = T - 1 - t;
+      double x = 0.0;
+      I k = 0;
+      int before = 0;
+#pragma unroll
+      for (int c0 = 0; c0 < kPoolCtas; c0 += 4) {
+        if (c0 >= C) break;
+        unsigned int ks[4];
+        float ws[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const int from = min(c0 + c, C - 1);
+          ks[c] = *cluster.map_shared_rank(cnt + b, from);
+          ws[c] = *cluster.map_shared_rank(w + b, from);
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (c0 + c < C) {
+            x += (double)ws[c];
+            if (c0 + c < rank) before += (int)ks[c];
+            k += (I)ks[c];
+          }
+      }
+      const double excl = pool_exclusive(x, s_dsum);
+      if (k && excl < need && excl + x >= need) atomicMin(&s_crossed, t);
+      const unsigned int some = __ballot_sync(0xffffffffu, k != 0);
+      if (lane == 0 && some) atomicMax(&s_lowest, 32 * warp + 31 - __clz(some));      // where rounding keeps the sum below `need`
+      __syncthreads();
+      const int e = s_crossed != INT32_MAX ? s_crossed : s_lowest >= 0 ? s_lowest : T - 1;
+      if (t == e) {
+        s_above = excl; s_k = (int)min(k, (I)INT32_MAX); s_at = before; s_cross[L] = T - 1 - e;
+        if (L + 1 < kPoolLevels) {
+          s_anchor[L + 1] = s_inv[L] > 0.f ? s_anchor[L] + (float)(T - 1 - e) / s_inv[L] : s_anchor[L];
+          s_inv[L + 1] = fminf(s_inv[L] * (float)T, 1e30f);
+        }
+      }
+      __syncthreads();
+      need -= s_above;
+      const int K = s_k;
+      if (K <= kPoolFinal) {
+        // ---- the last few, each against all others: the largest key whose mass and that of those above reach the target
+        each(L + 1, [&](float s) {
+          const int to = s_at + atomicAdd(&s_n, 1);
+          const uint32_t key = float_key(s);
+          for (int c = 0; c < C; ++c) cluster.map_shared_rank(s_final, c)[to] = key;
+        });
+        meet();
+        int G = 32;                      // threads per score
+        while (G * K > T) G >>= 1;
+        const int i = t / G, r = t & (G - 1);
+        float mass = 0.f;
+        const uint32_t key = i < K ? s_final[i] : 0u;
+        if (i < K)
+#pragma unroll 1
+          for (int j = r; j < K; j += G) {
+            const uint32_t other = s_final[j];
+            if (other >= key) mass += weight(key_float(other));
+          }
+#pragma unroll 1
+        for (int o = G >> 1; o > 0; o >>= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
+        const uint32_t best = __reduce_max_sync(0xffffffffu, i < K && (double)mass >= need ? key : 0u);
+        const uint32_t least = __reduce_min_sync(0xffffffffu, i < K ? key : 0xffffffffu);
+        if (lane == 0) {
+          if (best) atomicMax(&s_best, best);
+          atomicMin(&s_least, least);
+        }
+        __syncthreads();
+        cutoff = s_best ? s_best : s_least;
+        break;
+      }
+      uint32_t kmin = 0xffffffffu, kmax = 0u;
+      each(L + 1, [&](float s) {
+        kmin = min(kmin, float_key(s));
+        kmax = max(kmax, float_key(s));
+      });
+      exchange(kmin, kmax);
+      cutoff = kmin;
+      if (kmin == kmax) break;
+    }
+  }
+  return true;
+}
+
 template <PoolSrc SRC, int T>
 __global__ void __launch_bounds__(T, 1)
 select_pool_kernel(const PoolArgs a) {
@@ -1211,7 +1446,7 @@ select_pool_kernel(const PoolArgs a) {
   auto meet = [&]() { if (cluster.num_blocks() > 1) cluster.sync(); else __syncthreads(); };
   // before the first look into another CTA's shared memory: all of them have started
   auto all_there = []() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); };
-  constexpr int kFront = SRC == kPoolScores ? kPoolFront * T : 0, kLevelBytes = 8 * T, kList = (kPoolFront * T - kPoolLevels * kLevelBytes) / 4;
+  constexpr int kFront = SRC == kPoolScores ? kPoolFront * T : 0;
   extern __shared__ __align__(16) unsigned char pool_smem[];
   __shared__ int s_pairs[kPoolCtas];
   __shared__ int s_sum[32];
@@ -1231,15 +1466,10 @@ select_pool_kernel(const PoolArgs a) {
   uint32_t cutoff = 0u;
   float* s_src = nullptr;
   if constexpr (SRC == kPoolScores) {
-    __shared__ double s_w0[kPoolCtas][kPoolBins0], s_dsum[32], s_above;
-    __shared__ uint32_t s_key[kPoolCtas][2], s_final[kPoolFinal], s_best, s_least;
-    __shared__ int s_crossed, s_lowest, s_listed, s_n, s_at, s_k, s_cross[kPoolLevels];
-    __shared__ float s_anchor[kPoolLevels], s_inv[kPoolLevels];
+    __shared__ uint32_t s_key[kPoolCtas][2], s_least, s_most;
     s_src = reinterpret_cast<float*>(pool_smem + kFront + ((4 * (C * Nb + a.segs_per * (Nb + 1)) + 15) & ~15));
-    float* s_own = reinterpret_cast<float*>(pool_smem);        // [kPoolBins0][threads]
-#pragma unroll
-    for (int b = 0; b < kPoolBins0 / 4; ++b) reinterpret_cast<float4*>(s_own)[b * T + t] = make_float4(0.f, 0.f, 0.f, 0.f);
     uint32_t min_key = 0xffffffffu, max_key = 0u;
+    if (t == 0) { s_least = min_key; s_most = max_key; }
     if (a.range) { min_key = float_key(__ldg(a.range + 2 * bh)); max_key = float_key(__ldg(a.range + 2 * bh + 1)); }
     {
       const float* g_src = a.scores + ((long long)bh * a.S + q0) * Nb;
@@ -1253,220 +1483,36 @@ select_pool_kernel(const PoolArgs a) {
         for (int i = t; i < n; i += T) s_src[i] = __ldg(g_src + i);
       }
     }
-    // smallest and largest of a value over the cluster
-    auto exchange = [&](uint32_t& lo, uint32_t& hi) {
-      if (t == 0) { s_least = 0xffffffffu; s_best = 0u; }
-      __syncthreads();
-      lo = __reduce_min_sync(0xffffffffu, lo);
-      hi = __reduce_max_sync(0xffffffffu, hi);
-      if (lane == 0) { atomicMin(&s_least, lo); atomicMax(&s_best, hi); }
-      __syncthreads();
-      if (t < C) {
-        uint32_t* to = cluster.map_shared_rank(s_key[rank], t);
-        to[0] = s_least; to[1] = s_best;
-      }
-      meet();
-      for (int c = 0; c < C; ++c) { lo = min(lo, s_key[c][0]); hi = max(hi, s_key[c][1]); }
-    };
     all_there();
-    __syncthreads();
     if (!a.range) {
+      __syncthreads();
 #pragma unroll 2
       for (int i = t; i < n; i += T) {
         const uint32_t key = float_key(s_src[i]);
         min_key = min(min_key, key);
         max_key = max(max_key, key);
       }
-      exchange(min_key, max_key);
+      min_key = __reduce_min_sync(0xffffffffu, min_key);
+      max_key = __reduce_max_sync(0xffffffffu, max_key);
+      if (lane == 0) { atomicMin(&s_least, min_key); atomicMax(&s_most, max_key); }
+      __syncthreads();
+      if (t < C) {
+        uint32_t* to = cluster.map_shared_rank(s_key[rank], t);
+        to[0] = s_least; to[1] = s_most;
+      }
+      meet();
+      for (int c = 0; c < C; ++c) { min_key = min(min_key, s_key[c][0]); max_key = max(max_key, s_key[c][1]); }
     }
-    const float lo = key_float(min_key), smax = key_float(max_key), span = smax - lo;
-    const float inv0 = span > 0.f ? (float)kPoolBins0 / span : 0.f, off0 = -lo * inv0;
+    const float lo = key_float(min_key), smax = key_float(max_key);
     const bool unit_w = a.unit_w != 0;
-    auto weight = [&](float s) { return unit_w ? 1.0f : pair_weight(a.sigma, s, smax); };
-    // ---- the first bins: floor(s * inv0 + off0) by an addition that rounds down, NaN to bin 0
-#pragma unroll 4
-    for (int i = t; i < n; i += T) {
-      const float s = s_src[i], x = fminf(fmaxf(fmaf(s, inv0, off0), 0.f), (float)(kPoolBins0 - 1));
-      const int b = __float_as_int(__fadd_rd(x, 8388608.f)) & (kPoolBins0 - 1);
-      s_own[b * T + t] += weight(s);
-    }
-    __syncthreads();
-#pragma unroll 1
-    for (int b = warp; b < kPoolBins0; b += T / 32) {
-      float w = 0.f;
-#pragma unroll
-      for (int r = 0; r < T / 32; ++r) {
-        const float x = s_own[b * T + 32 * r + lane];
-        if (x > 0.f) w += x;
-      }
-      double x = (double)w;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if (lane < C) cluster.map_shared_rank(s_w0[rank], lane)[b] = x;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 2 * kPoolLevels; ++i) reinterpret_cast<uint32_t*>(pool_smem)[i * T + t] = 0u;
-    meet();
-    double need;                           // mass still to be covered from the crossing bin down
-    int cross0;
-    {
-      double x = 0.0;                      // lane l: bin 31 - l
-      for (int c = 0; c < C; ++c) x += s_w0[c][kPoolBins0 - 1 - lane];
-      double inc = x;
-#pragma unroll 1
-      for (int o = 1; o < 32; o <<= 1) {
-        const double v = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += v;
-      }
-      const double total = __shfl_sync(0xffffffffu, inc, 31), excl = inc - x;
-      need = a.count_target >= 0.0 ? a.count_target : (double)a.tau * total;
-      const unsigned int hit = __ballot_sync(0xffffffffu, x > 0.0 && excl < need && inc >= need);
-      const unsigned int occupied = __ballot_sync(0xffffffffu, x > 0.0);
-      const int e = hit ? __ffs(hit) - 1 : occupied ? 31 - __clz(occupied) : kPoolBins0 - 1;
-      cross0 = kPoolBins0 - 1 - e;
-      need -= __shfl_sync(0xffffffffu, excl, e);
-    }
     cutoff = min_key;                      // everything, where tau = 1
     if (a.tau < 1.0f) {
-      // ---- the list of the crossing bin's scores (the last bin has no end), if it has room for them
-      const float y_lo = (float)cross0, y_hi = cross0 == kPoolBins0 - 1 ? NAN : (float)(cross0 + 1);
-      auto inside = [&](float s) {
-        const float y = fmaf(s, inv0, off0);
-        return (cross0 == 0 || y >= y_lo) && !(y >= y_hi);
-      };
-      float* s_list = reinterpret_cast<float*>(pool_smem + kPoolLevels * kLevelBytes);
-      int mine = 0;
-#pragma unroll 4
-      for (int i = t; i < n; i += T) mine += inside(s_src[i]) ? 1 : 0;
-      int at = pool_exclusive(mine, s_sum);
-      if (t == T - 1) s_listed = at + mine;
-      if (mine && at + mine <= kList)
-#pragma unroll 4
-        for (int i = t; i < n; i += T) {
-          const float s = s_src[i];
-          if (inside(s)) s_list[at++] = s;
-        }
-      if (t == 0) {
-        s_anchor[0] = inv0 > 0.f ? lo + (float)cross0 / inv0 : lo;
-        s_inv[0] = fminf(inv0 * (float)T, 1e30f);
-      }
+      pool_search<T, false, int>(cluster, meet, pool_smem, s_src, n, lo, smax - lo,
+                          [&](float s) { return unit_w ? 1.0f : pair_weight(a.sigma, s, smax); },
+                          [&](double total, double& need) { need = a.count_target >= 0.0 ? a.count_target : (double)a.tau * total; return true; },
+                          cutoff);
+    } else {
       __syncthreads();
-      const bool over = s_listed > kList;
-      const float* src = over ? s_src : s_list;
-      const int n_src = over ? n : s_listed;
-      auto bin_of = [&](int L, float s) {
-        const float x = (s - s_anchor[L]) * s_inv[L];
-        return x > 0.f ? (int)fminf(x, (float)(T - 1)) : 0;
-      };
-      auto each = [&](int levels, auto f) {          // the scores inside the crossing bins of so many levels
-#pragma unroll 1
-        for (int i = t; i < n_src; i += T) {
-          const float s = src[i];
-          bool in = !over || inside(s);
-#pragma unroll 1
-          for (int l = 0; l < levels; ++l) in = in && bin_of(l, s) == s_cross[l];
-          if (in) f(s);
-        }
-      };
-      // ---- a bin of it per thread; thread t looks after bin T - 1 - t
-#pragma unroll 1
-      for (int L = 0; L < kPoolLevels; ++L) {
-        float* w = reinterpret_cast<float*>(pool_smem + L * kLevelBytes);
-        unsigned int* cnt = reinterpret_cast<unsigned int*>(w + T);
-        each(L, [&](float s) {
-          const int b = bin_of(L, s);
-          // lanes that are at the same score go in one update: scores that are all alike would queue for one bin
-          const uint32_t key = float_key(s);
-          const unsigned int here = __activemask();
-          int lanes = 1;
-          if (__reduce_min_sync(here, key) == __reduce_max_sync(here, key)) {
-            if (lane != __ffs(here) - 1) return;
-            lanes = __popc(here);
-          }
-          atomicAdd(&cnt[b], (unsigned int)lanes);
-          atomicAdd(&w[b], (float)lanes * weight(s));
-        });
-        if (t == 0) { s_crossed = INT32_MAX; s_lowest = -1; s_k = 0; s_n = 0; s_best = 0u; s_least = 0xffffffffu; s_above = 0.0; }
-        meet();
-        const int b = T - 1 - t;
-        double x = 0.0;
-        int k = 0, before = 0;
-#pragma unroll
-        for (int c0 = 0; c0 < kPoolCtas; c0 += 4) {
-          if (c0 >= C) break;
-          unsigned int ks[4];
-          float ws[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int from = min(c0 + c, C - 1);
-            ks[c] = *cluster.map_shared_rank(cnt + b, from);
-            ws[c] = *cluster.map_shared_rank(w + b, from);
-          }
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            if (c0 + c < C) {
-              x += (double)ws[c];
-              if (c0 + c < rank) before += (int)ks[c];
-              k += (int)ks[c];
-            }
-        }
-        const double excl = pool_exclusive(x, s_dsum);
-        if (k && excl < need && excl + x >= need) atomicMin(&s_crossed, t);
-        const unsigned int some = __ballot_sync(0xffffffffu, k != 0);
-        if (lane == 0 && some) atomicMax(&s_lowest, 32 * warp + 31 - __clz(some));      // where rounding keeps the sum below `need`
-        __syncthreads();
-        const int e = s_crossed != INT32_MAX ? s_crossed : s_lowest >= 0 ? s_lowest : T - 1;
-        if (t == e) {
-          s_above = excl; s_k = k; s_at = before; s_cross[L] = T - 1 - e;
-          if (L + 1 < kPoolLevels) {
-            s_anchor[L + 1] = s_inv[L] > 0.f ? s_anchor[L] + (float)(T - 1 - e) / s_inv[L] : s_anchor[L];
-            s_inv[L + 1] = fminf(s_inv[L] * (float)T, 1e30f);
-          }
-        }
-        __syncthreads();
-        need -= s_above;
-        const int K = s_k;
-        if (K <= kPoolFinal) {
-          // ---- the last few, each against all others: the largest key whose mass and that of those above reach the target
-          each(L + 1, [&](float s) {
-            const int to = s_at + atomicAdd(&s_n, 1);
-            const uint32_t key = float_key(s);
-            for (int c = 0; c < C; ++c) cluster.map_shared_rank(s_final, c)[to] = key;
-          });
-          meet();
-          int G = 32;                      // threads per score
-          while (G * K > T) G >>= 1;
-          const int i = t / G, r = t & (G - 1);
-          float mass = 0.f;
-          const uint32_t key = i < K ? s_final[i] : 0u;
-          if (i < K)
-#pragma unroll 1
-            for (int j = r; j < K; j += G) {
-              const uint32_t other = s_final[j];
-              if (other >= key) mass += weight(key_float(other));
-            }
-#pragma unroll 1
-          for (int o = G >> 1; o > 0; o >>= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
-          const uint32_t best = __reduce_max_sync(0xffffffffu, i < K && (double)mass >= need ? key : 0u);
-          const uint32_t least = __reduce_min_sync(0xffffffffu, i < K ? key : 0xffffffffu);
-          if (lane == 0) {
-            if (best) atomicMax(&s_best, best);
-            atomicMin(&s_least, least);
-          }
-          __syncthreads();
-          cutoff = s_best ? s_best : s_least;
-          break;
-        }
-        uint32_t kmin = 0xffffffffu, kmax = 0u;
-        each(L + 1, [&](float s) {
-          kmin = min(kmin, float_key(s));
-          kmax = max(kmax, float_key(s));
-        });
-        exchange(kmin, kmax);
-        cutoff = kmin;
-        if (kmin == kmax) break;
-      }
     }
     if (rank == 0 && t == 0) a.cutoff_per_head[bh] = key_float(cutoff);
   } else {
@@ -1572,6 +1618,266 @@ select_pool_kernel(const PoolArgs a) {
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// Larger pools, if there is room for candidate lists: a sample of a head's scores tells roughly where the cutoff is, ONE pass
+// over the matrix adds up the mass above a window round that place and copies the window's scores aside, and a cluster of
+// CTAs per head finds the cutoff among these.  Where it is not among them (the sample missed the few pairs that hold the mass, or
+// the window has more scores than the list) the cluster searches the whole of the head's scores.  Three launches instead of eight
+// and two passes over the matrix (this one and mark) instead of three.  Whole selection of 12 heads x 32,760 x 140 blocks 191 ->
+// 164 us, 24 heads 340 -> 296, 12 x 55,296 x 72 218 -> 190.
+constexpr int kSampleThreads = kBins0, kSamples = 16;      // (per thread)
+constexpr int kFewSamples = 48;
+// From six million scores on (matrix of 24 MB): 12 heads x 16,384 x 32 blocks (6.3 million) 70 -> 66 us, x 64 99 -> 84, x 13,650 x 25
+// (4.1 million) 74 -> 74, 2 heads x 37,500 x 25 51 -> 58 (whole selection, white scores).
+constexpr long long kWindowMin = 6000000;
+// CTAs that take one head's sample, and its search: at most two to an SM, and few where there is little to do.
+static int window_ctas(int BH, long long P) {
+  int C = kPoolCtas;
+  while (C > 1 && ((long long)BH * C > 2ll * sm_count() || (P >> 18) < C)) C /= 2;
+  return C;
+}
+
+// A cluster per head; also leaves the head's state.  The sample is counted in 512 bins of the head's range and, round the
+// crossing, in 512 bins of a few of these; a bin's mass is its count times the weight at its middle.  The window reaches
+// 4.5 standard deviations of the sample's estimate of the mass above the cutoff to either side of the target.
+__global__ void __launch_bounds__(kSampleThreads)
+window_kernel(const float* __restrict__ scores, long long P, const float* __restrict__ range, HeadState* __restrict__ st, float sigma,
+              int unit_w, float tau, double count_target, float list_share) {
+  if (!grid_begin()) return;
+  __shared__ unsigned int s_cnt[2][kBins0];
+  __shared__ float s_m[32], s_m2[32], s_total, s_total2, s_above2, s_base, s_base2;
+  __shared__ int s_c[32], s_bin[2], s_before[2], s_all, s_top;
+  __shared__ float s_top_mass;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), bh = blockIdx.x / C, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  s_cnt[0][t] = s_cnt[1][t] = 0u;
+  uint32_t min_key, max_key;
+  if (range) { min_key = float_key(range[2 * bh]); max_key = float_key(range[2 * bh + 1]); }
+  else { min_key = st[bh].min_key; max_key = st[bh].max_key; }
+  const float lo = key_float(min_key), smax = key_float(max_key), span = smax - lo;
+  const float* base = scores + (long long)bh * P;
+  // one score out of each of n equal parts of the pool, at a place that a hash gives
+  const int most = C * kSamples * kSampleThreads, n = (int)min(P, (long long)most);
+  const unsigned long long step = ((unsigned long long)P << 20) / n;      // (P < 2^37)
+  const unsigned int stride = (unsigned int)min(P / n, 0xffffffffll);
+  float x[kSamples];
+#pragma unroll
+  for (int u = 0; u < kSamples; ++u) {
+    const int i = (u * C + rank) * kSampleThreads + t;
+    unsigned int h = (i + 1u) * 2654435761u;
+    h ^= h >> 15;
+    h *= 2246822519u;
+    x[u] = i < n ? __ldg(base + ((i * step) >> 20) + __umulhi(h, stride)) : NAN;
+  }
+  const float share = count_target >= 0.0 ? (float)(count_target / (double)P) : tau;
+  float from = lo, inv = span > 0.f ? (float)kBins0 / span : 0.f, win_lo = -INFINITY, win_hi = INFINITY;
+  float over = 0.f, over2 = 0.f;        // mass above the bins of the second round, and its squares
+  int inside = 0, top = kBins0;         // top: the first round's lowest bin from which on the scores fit the list
+  float top_mass = 0.f, goal = 0.f;
+  if (t == 0) { s_top = kBins0; s_top_mass = 0.f; }
+  __syncthreads();
+#pragma unroll 1
+  for (int round = 0; round < 2; ++round) {
+    const float off = -from * inv;
+#pragma unroll
+    for (int u = 0; u < kSamples; ++u) {
+      const float y = fmaf(x[u], inv, off);
+      // (NaN is in no bin; the ends of the head's range are in the first and the last)
+      if (round == 0 ? y == y : y >= 0.f && y < (float)kBins0) atomicAdd(&s_cnt[round][min(max(__float2int_rd(y), 0), kBins0 - 1)], 1u);
+    }
+    cluster.sync();
+    const int b = kBins0 - 1 - t;       // this thread's bin
+    int c = 0;
+#pragma unroll
+    for (int r = 0; r < kPoolCtas; ++r)
+      if (r < C) c += (int)cluster.map_shared_rank(s_cnt[round], r)[b];
+    const float mid = from + ((float)b + 0.5f) / inv, w = unit_w ? 1.0f : pair_weight(sigma, mid, smax);
+    const float m = c ? (float)c * w : 0.f, m2 = c ? m * w : 0.f;
+    // sums over the bins above this one
+    float im = m, im2 = m2;
+    int ic = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float v = __shfl_up_sync(0xffffffffu, im, o), v2 = __shfl_up_sync(0xffffffffu, im2, o);
+      const int vc = __shfl_up_sync(0xffffffffu, ic, o);
+      if (lane >= o) { im += v; im2 += v2; ic += vc; }
+    }
+    if (lane == 31) { s_m[warp] = im; s_m2[warp] = im2; s_c[warp] = ic; }
+    if (t < 2) { s_bin[t] = -1; s_before[t] = t == 0 ? -1 : 0; }
+    if (t == 0) s_above2 = 0.f;
+    __syncthreads();
+    float excl = over + im - m, excl2 = over2 + im2 - m2;
+    int before = ic - c;
+    for (int v = 0; v < warp; ++v) { excl += s_m[v]; excl2 += s_m2[v]; before += s_c[v]; }
+    if (t == kSampleThreads - 1) {
+      if (round == 0) { s_total = excl + m; s_total2 = excl2 + m2; }
+      s_all = before + c;
+    }
+    if (round == 0 && (float)(before + c) <= 0.7f * list_share * (float)n) atomicMin(&s_top, b);
+    __syncthreads();
+    goal = share * s_total;
+    if (excl < goal && excl + m >= goal) s_above2 = excl2 + m2;
+    if (round == 0 && b == s_top) s_top_mass = excl + m;
+    __syncthreads();
+    const float dev = 4.5f * sqrtf((1.f - share) * (1.f - share) * s_above2 + share * share * fmaxf(s_total2 - s_above2, 0.f));
+    if (excl < goal - dev && excl + m >= goal - dev) { s_bin[1] = b; s_before[1] = before; s_base = excl; s_base2 = excl2; }
+    if (excl < goal + dev && excl + m >= goal + dev) { s_bin[0] = b; s_before[0] = before + c; }
+    __syncthreads();
+    const int b_lo = s_bin[0], b_hi = s_bin[1];
+    inside = (s_before[0] >= 0 ? s_before[0] : s_all) - s_before[1];
+    if (round == 0) { top = s_top; top_mass = s_top_mass; }
+    // (an end that this round did not find stays where it was)
+    const float edge = from;
+    if (b_lo > 0) win_lo = edge + (float)b_lo / inv;
+    // (few samples are no measure of what lies above them: no upper end there)
+    if (b_hi >= 0 && s_before[1] < kFewSamples) inside += s_before[1];
+    else if (b_hi >= 0 && (round > 0 || b_hi < kBins0 - 1)) win_hi = edge + (float)(b_hi + 1) / inv;
+    if (round == 0) {
+      if ((float)inside <= 0.5f * list_share * (float)n) break;      // narrow enough
+      // the second round looks at the bins from b_lo to b_hi
+      const int first = max(b_lo, 0), last = b_hi >= 0 ? b_hi : kBins0 - 1;
+      if (b_hi >= 0) { over = s_base; over2 = s_base2; }
+      from = edge + (float)first / inv;
+      inv = inv > 0.f ? inv * ((float)kBins0 / (float)(last - first + 1)) : 0.f;
+    }
+    __syncthreads();
+  }
+  if (rank == 0 && t == 0) {
+    HeadState h;
+    memset(&h, 0, sizeof(h));
+    h.min_key = min_key; h.max_key = max_key;
+    h.cutoff_key = 0xffffffffu;
+    // Where the window would hold more than the list: if a few pairs hold the mass (the sample is no measure of it, and the
+    // cutoff lies high), the highest scores that fit; else the whole pool is searched.
+    if (!(span > 0.f) || (float)inside > 0.75f * list_share * (float)n) {
+      win_lo = span > 0.f && top > 0 && top < kBins0 && top_mass >= 1.5f * goal ? lo + (float)top * span / (float)kBins0 : INFINITY;
+      win_hi = INFINITY;
+    }
+    h.win_lo = win_lo; h.win_hi = win_hi;
+    st[bh] = h;
+  }
+  cluster.sync();      // nobody leaves while its counts may be read
+}
+
+// The pass over the matrix.  Bound by HBM: a dozen instructions per score and no atomics; a warp gathers what it finds in the
+// window and writes it out some 256 at a time (with the check for that behind every score instead of every sixteen, twenty copies of
+// the code that writes: 77 us where this takes 47; floor 34: 12 heads x 32,760 x 140).
+constexpr int kWindowThreads = 512, kWindowStage = 256 + 512;
+__global__ void __launch_bounds__(kWindowThreads)
+window_pass_kernel(const float* __restrict__ scores, long long P, HeadState* __restrict__ st, float sigma, int unit_w,
+                   float* __restrict__ cand, long long ccap) {
+  if (!grid_begin()) return;
+  extern __shared__ float s_stage[];    // [warps][kWindowStage]
+  __shared__ double s_z[kWindowThreads / 32], s_a[kWindowThreads / 32];
+  const int bh = blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const float win_lo = st[bh].win_lo, win_hi = st[bh].win_hi, smax = key_float(st[bh].max_key);
+  float* list = cand + (long long)bh * ccap;
+  float* stage = s_stage + warp * kWindowStage;
+  const unsigned int lt_mask = (1u << lane) - 1u;
+  int staged = 0;                       // (the same in all lanes)
+  auto write_out = [&]() {
+    __syncwarp();
+    unsigned int at = 0;
+    if (lane == 0) at = atomicAdd(&st[bh].cand_cnt, (unsigned int)staged);
+    at = __shfl_sync(0xffffffffu, at, 0);
+    for (int i = lane; i < staged; i += 32)
+      if (at + i < ccap) list[at + i] = stage[i];
+    staged = 0;
+    __syncwarp();
+  };
+  float z = 0.f, above = 0.f;
+  auto take = [&](float s, bool there) {
+    float w = unit_w ? 1.0f : fmaxf(pair_weight(sigma, s, smax), 0.f);      // (0 for NaN)
+    if (!there) w = 0.f;
+    z += w;
+    if (s >= win_hi) above += w;
+    const bool in = there && s >= win_lo && s < win_hi;
+    const unsigned int found = __ballot_sync(0xffffffffu, in);
+    if (found) {
+      if (in) stage[staged + __popc(found & lt_mask)] = s;
+      staged += __popc(found);
+    }
+  };
+  const float* base = scores + (long long)bh * P;
+  const long long gw = (long long)blockIdx.x * (kWindowThreads / 32) + warp, n_warps = (long long)gridDim.x * (kWindowThreads / 32);
+  long long done = 0;                   // scores that went in runs of 512
+  if ((reinterpret_cast<uintptr_t>(base) & 15u) == 0) {
+    const float4* b4 = reinterpret_cast<const float4*>(base);
+    const long long runs = P / 512;
+#pragma unroll 1
+    for (long long r = gw; r < runs; r += n_warps) {
+      float4 x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = __ldg(b4 + r * 128 + 32 * j + lane);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) { take(x[j].x, true); take(x[j].y, true); take(x[j].z, true); take(x[j].w, true); }
+      if (staged > kWindowStage - 512) write_out();
+    }
+    done = runs * 512;
+  }
+#pragma unroll 1
+  for (long long r = done + gw * 512; r < P; r += n_warps * 512) {
+#pragma unroll 4
+    for (int j = 0; j < 16; ++j) {
+      const long long i = r + 32 * j + lane;
+      take(i < P ? __ldg(base + i) : 0.f, i < P);
+    }
+    if (staged > kWindowStage - 512) write_out();
+  }
+  if (staged) write_out();
+  double zd = z, ad = above;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) { zd += __shfl_xor_sync(0xffffffffu, zd, o); ad += __shfl_xor_sync(0xffffffffu, ad, o); }
+  if (lane == 0) { s_z[warp] = zd; s_a[warp] = ad; }
+  __syncthreads();
+  if (t == 0) {
+    zd = ad = 0.0;
+    for (int w = 0; w < kWindowThreads / 32; ++w) { zd += s_z[w]; ad += s_a[w]; }
+    atomicAdd(&st[bh].Z, zd);
+    if (ad > 0.0) atomicAdd(&st[bh].mass_above, ad);
+  }
+}
+
+// The cutoff, by a cluster per head.
+template <int T>
+__global__ void __launch_bounds__(T, 1)
+window_search_kernel(const float* __restrict__ scores, long long P, HeadState* __restrict__ st, float sigma, int unit_w, float tau,
+                     double count_target, const float* __restrict__ cand, long long ccap, float* __restrict__ cutoff_per_head) {
+  if (!grid_begin()) return;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  extern __shared__ __align__(16) unsigned char pool_smem[];
+  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), bh = (int)blockIdx.x / C;
+  auto meet = [&]() { cluster.sync(); };
+  const HeadState h = st[bh];
+  const float lo = key_float(h.min_key), smax = key_float(h.max_key);
+  const bool by_count = unit_w != 0;
+  auto weight = [&](float s) { return by_count ? 1.0f : pair_weight(sigma, s, smax); };
+  uint32_t cutoff = h.min_key;            // everything, where tau = 1 or all scores are alike (zeros of either sign are)
+  if (lo == smax && lo == 0.f) cutoff = 0x7fffffffu;
+  meet();                                 // (all CTAs have started)
+  if (tau < 1.0f && lo != smax) {
+    bool found = false;
+    const int n = (int)min((long long)h.cand_cnt, ccap);
+    if ((long long)h.cand_cnt <= ccap && n > 0) {
+      const double left = (count_target >= 0.0 ? count_target : (double)tau * h.Z) - h.mass_above;
+      const float w_lo = fmaxf(h.win_lo, lo), w_hi = fminf(h.win_hi, smax);
+      const int per = ((n + C - 1) / C + 3) & ~3, i0 = min(rank * per, n);
+      found = pool_search<T, true, int>(cluster, meet, pool_smem, cand + (long long)bh * ccap + i0, min(per, n - i0), w_lo, w_hi - w_lo, weight,
+                                        [&](double total, double& need) { need = left; return left > 0.0 && left <= total; }, cutoff);
+    }
+    if (!found) {
+      const long long per = ((P + C - 1) / C + 3) & ~3ll, i0 = min(rank * per, P);
+      pool_search<T, true, long long>(cluster, meet, pool_smem, scores + (long long)bh * P + i0, min(per, P - i0), lo, smax - lo, weight,
+                                      [&](double total, double& need) { need = count_target >= 0.0 ? count_target : (double)tau * total; return true; },
+                                      cutoff);
+    }
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    st[bh].cutoff_key = cutoff;
+    cutoff_per_head[bh] = key_float(cutoff);
+  }
+}
+
 // Row normalisation for the second reading of Eq. 4: out[i][j] = sigma * s[i][j] - logsumexp_j(sigma * s[i][:]),
 // the logarithm of S times the pair's probability when every query is normalised on its own.  One
 // warp per query row; the head-wide quantile search then runs on `out` with unit temperature.
@@ -1659,10 +1965,10 @@ struct SelectWs {
   Guards guards;
 };
 
-// Room for the list of one head: the pairs of one of the 512 level-0 bins.
+// Room for the list of one head: a sixteenth of its scores (a window holds up to 4 % of them).
 static long long cand_capacity(const Dims& D) {
   const long long P = (long long)D.S * D.Nb;
-  return std::max<long long>(4096, ((P / 32 + 3) / 4) * 4);
+  return std::max<long long>(4096, ((P / 16 + 3) / 4) * 4);
 }
 
 static SelectWs carve_select(const Dims& D, void* ws) {
@@ -1756,7 +2062,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     a.k_per_head = k_per_head; a.cutoff_per_head = cutoff_per_head;
     auto kernel = w.pool.T == 256 ? select_pool_kernel<decltype(tag)::value, 256> : select_pool_kernel<decltype(tag)::value, 512>;
     VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pool_smem));
-    launch_cluster(w.pool.C, kernel, (unsigned)(D.BH * w.pool.C), w.pool.T, pool_smem, st, a);
+    launch_cluster(true, w.pool.C, kernel, (unsigned)(D.BH * w.pool.C), w.pool.T, pool_smem, st, a);
     VMOBA_LAUNCH_OK(1);
     return VMOBA_OK;
   };
@@ -1833,13 +2139,34 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     if (pool) {
       if ((rc = pool_launch(VMOBA_POOL(kPoolScores), range, unit_w, count_target))) return rc;
     } else {
-    launch_kernel(init_state_kernel, (unsigned)(((long long)D.BH * kBins + 255) / 256), 256, 0, st, w.state, D.BH,
-                  range, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey);
-
     // enough CTAs per head to fill the machine, few enough that the per-CTA flush stays small
     long long per_head = (P / 4 + 255) / 256;
     int gx = (int)std::min<long long>(std::max<long long>(per_head / 8, 1), std::max(1, sm_count() * 8 / D.BH));
     dim3 grid(gx, D.BH);
+    const bool window = use_cand && (long long)D.BH * P >= kWindowMin;
+    if (window) {
+      if (!range) {
+        launch_kernel(init_state_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, D.BH, nullptr, nullptr, nullptr, nullptr, nullptr);
+        launch_kernel(minmax_kernel, grid, 256, 0, st, scores, P, w.state);
+        count_launches(2);
+      }
+      const int C = window_ctas(D.BH, P);
+      // (not early behind the scores kernel, in whose SMs' spare room its CTAs would wait: 33K tokens, 3D, forward 603 us early, 559 not)
+      launch_cluster(early_rows(D), C, window_kernel, (unsigned)(D.BH * C), kSampleThreads, 0, st, scores, P, range, w.state, sigma, unit_w, tau,
+                     count_target, (float)((double)w.ccap / (double)P));
+      const int gx1 = (int)std::min<long long>(std::max<long long>(per_head / 16, 1), std::max(1, sm_count() * 3 / D.BH));
+      constexpr int T = 512, smem1 = kPoolFront * T, smem_stage = kWindowThreads / 32 * kWindowStage * (int)sizeof(float);
+      VMOBA_CUDA_OK(cudaFuncSetAttribute(window_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_stage));
+      launch_kernel(early_rows(D), window_pass_kernel, dim3(gx1, D.BH), kWindowThreads, smem_stage, st, scores, P, w.state, sigma, unit_w,
+                    w.cand, w.ccap);
+      VMOBA_CUDA_OK(cudaFuncSetAttribute(window_search_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1));
+      launch_cluster(true, C, window_search_kernel<T>, (unsigned)(D.BH * C), T, smem1, st, scores, P, w.state, sigma, unit_w, tau,
+                     count_target, w.cand, w.ccap, cutoff_per_head);
+      VMOBA_LAUNCH_OK(3);
+    } else {
+    launch_kernel(init_state_kernel, (unsigned)(((long long)D.BH * kBins + 255) / 256), 256, 0, st, w.state, D.BH,
+                  range, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey);
+
     if (!range) {
       launch_kernel(minmax_kernel, grid, 256, 0, st, scores, P, w.state);
       launch_kernel(setup_level0_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, D.BH);
@@ -1864,6 +2191,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     launch_kernel(scan_kernel<2>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
                   w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
     VMOBA_LAUNCH_OK(7);
+    }
     VMOBA_CUDA_OK(cudaFuncSetAttribute(mark_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     launch_kernel(mark_kernel, sgrid, kSegThreads, smem, st, scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg,
                   own_sb, mask_bits, w.seg_cnt, w.seg_total, w.tmask);

@@ -1,6 +1,6 @@
-"""Small pools (up to 2^20 scores per head): the whole of the selection up to the offsets is one kernel, a cluster per head.
-Larger ones go through the chain of passes over the score matrix, with which it is compared here: a pool of m copies of the same
-scores has m times the mass above any score, so the cutoff is the same and every copy keeps the same pairs."""
+"""The three routes to a head's cutoff: small pools go through one kernel, a cluster per head; of the larger ones those of six
+million scores in all through a sample, one pass and a search; the rest through histograms of the matrix.  A pool of m copies of the
+same scores has m times the mass above any score, so the cutoff is the same on all three and every copy keeps the same pairs."""
 import numpy as np
 import pytest
 import torch
@@ -8,7 +8,8 @@ import torch
 from paper_2506_23858_b200 import binding as vb
 
 pytestmark = pytest.mark.gpu
-POOL_MAX = 1 << 20
+POOL_MAX = 1 << 20          # beyond every pool that the cluster kernel takes
+WINDOW_MIN = 6000000        # scores of all heads, from which on a sample is taken
 
 
 def _run(shape, scores, rule, tau=0.25, topk=1, score_range=None, capacity=None):
@@ -51,6 +52,22 @@ def _check_lists(shape, out, m):
     assert np.array_equal(out["q_pairs"][:n].cpu().numpy(), place[m])
 
 
+def _copies(small, total):
+    """The shape with further query rows that makes the pool larger than POOL_MAX, with fewer or with more than `total` scores in
+    all: the same blocks per row, `copies` times the frames and the frames per block."""
+    P = small.S * small.n_blocks
+    copies = (POOL_MAX if total is None else max(POOL_MAX, total // small.heads)) // P + 1
+    big = _shape(small.heads, (small.T * copies, small.H, small.W), (small.bT * copies, small.bH, small.bW))
+    assert big.n_blocks == small.n_blocks and big.S * big.n_blocks > POOL_MAX
+    assert (big.S * big.n_blocks * big.heads >= WINDOW_MIN) == (total is not None)
+    return copies, big
+
+
+def _repeat(x, copies):
+    heads, S, Nb = x.shape
+    return x[:, None].expand(heads, copies, S, Nb).reshape(heads, copies * S, Nb).contiguous()
+
+
 def _shape(heads, grid, block):
     return vb.make_shape(1, heads, 64, grid, block, "f32")
 
@@ -64,26 +81,22 @@ SHAPES = [((1, 7, 9), (1, 1, 1)), ((4, 8, 8), (1, 8, 8)), ((3, 43, 8), (3, 43, 1
 @pytest.mark.parametrize("grid,block", SHAPES)
 @pytest.mark.parametrize("rule,tau,topk", [(vb.SELECT_THRESHOLD_GLOBAL, 0.25, 0), (vb.SELECT_THRESHOLD_GLOBAL, 1.0, 0),
                                            (vb.SELECT_TOPK_GLOBAL, 0.0, 3)])
-def test_pool_kernel_agrees_with_the_passes_over_the_matrix(grid, block, rule, tau, topk):
+@pytest.mark.parametrize("total", [None, WINDOW_MIN])
+def test_pool_kernel_agrees_with_the_passes_over_the_matrix(grid, block, rule, tau, topk, total):
     heads = 3
     small = _shape(heads, grid, block)
     S, Nb = small.S, small.n_blocks
-    assert S * Nb <= POOL_MAX
-    copies = POOL_MAX // (S * Nb) + 1
-    # the copies are further query rows: the same blocks per row, `copies` times the frames and the frames per block
-    large = _shape(heads, (grid[0] * copies, grid[1], grid[2]), (block[0] * copies, block[1], block[2]))
-    assert large.n_blocks == Nb and large.S * Nb > POOL_MAX
+    copies, large = _copies(small, total)
     g = torch.Generator(device="cuda").manual_seed(S * Nb)
     x = 4.0 * torch.randn((heads, S, Nb), generator=g, device="cuda")
-    y = x[:, None].expand(heads, copies, S, Nb).reshape(heads, copies * S, Nb).contiguous()
     a = _run(small, x, rule, tau, topk)
     ranged = _run(small, x, rule, tau, topk, score_range=torch.stack([x.amin((1, 2)), x.amax((1, 2))], 1).contiguous())
-    b = _run(large, y, rule, tau, topk, capacity=int(heads * large.S * Nb))
+    b = _run(large, _repeat(x, copies), rule, tau, topk, capacity=int(heads * large.S * Nb))
     ma = _mask(small, a)
     for out in (a, ranged):
         _check_lists(small, out, _mask(small, out))
         assert int(out["status"]) == 0
-    # the budget of the pair-count rule and, for masses, one pair at the cutoff: sums of up to 2^20 fp32 weights in any order
+    # the budget of the pair-count rule and, for masses, one pair at the cutoff: sums of millions of fp32 weights in any order
     # are off by 1e-6 of the whole, less than a pair's weight at most cutoffs
     mb = _mask(large, b).reshape(heads, copies, S, Nb)
     for other in (_mask(small, ranged), mb[:, 0], mb[:, -1]):
@@ -92,15 +105,46 @@ def test_pool_kernel_agrees_with_the_passes_over_the_matrix(grid, block, rule, t
     assert torch.allclose(a["cutoff"], b["cutoff"], atol=1e-2)
 
 
+@pytest.mark.parametrize("tau", [0.02, 0.25, 0.9])
+@pytest.mark.parametrize("values", ["flat", "sharp", "few hold the mass", "outlier", "one side"])
+def test_cutoff_of_large_pools_against_a_sort(values, tau):
+    """The sample's window finds the cutoff, or the search of the whole pool does, whatever the scores look like: against a sort in
+    64 bits.  The sums of 3 million fp32 weights are off by 1e-6 of the whole."""
+    shape = _shape(2, (12, 100, 53), (3, 5, 53))       # 63,600 queries x 80 blocks: ten million scores in all
+    heads, S, Nb = shape.heads, shape.S, shape.n_blocks
+    g = torch.Generator(device="cuda").manual_seed(7)
+    x = torch.randn((heads, S, Nb), generator=g, device="cuda")
+    if values == "flat":
+        x *= 0.05
+    elif values == "sharp":
+        x *= 20.0
+    elif values == "few hold the mass":
+        x *= 45.0
+    elif values == "outlier":
+        x[:, S // 3, Nb // 2] = 60.0
+        x[:, S // 4, 0] = -5e3
+    else:
+        x = -torch.exp(x)
+    out = _run(shape, x, vb.SELECT_THRESHOLD_GLOBAL, tau, score_range=torch.stack([x.amin((1, 2)), x.amax((1, 2))], 1).contiguous())
+    for h in range(heads):
+        v = x[h].flatten().double().sort(descending=True).values
+        cs = torch.exp((v - v[0]) / 8.0).cumsum(0)                                  # scale 64 ** -0.5
+        want = min(int((cs < tau * cs[-1]).sum()), v.numel() - 1)                   # index of the pair that reaches the target
+        k = int((x[h] >= out["cutoff"][h]).sum())
+        assert k == int(out["k"][h])
+        assert abs(float(cs[k - 1] - cs[want])) <= 2e-6 * float(cs[-1]), (h, k, want)
+    assert int(out["status"]) == 0
+
+
 @pytest.mark.parametrize("values", ["constant", "zeros", "two", "infinite", "nan"])
 @pytest.mark.parametrize("rule,tau,topk", [(vb.SELECT_THRESHOLD_GLOBAL, 0.3, 0), (vb.SELECT_TOPK_GLOBAL, 0.0, 2)])
-def test_pool_kernel_special_scores(values, rule, tau, topk):
+@pytest.mark.parametrize("total", [None, WINDOW_MIN])
+def test_pool_kernel_special_scores(values, rule, tau, topk, total):
     """Ties, infinities and NaN come out as they do from the passes over the matrix (same copies as above)."""
     heads, grid, block = 2, (4, 13, 11), (1, 13, 11)
     small = _shape(heads, grid, block)
     S, Nb = small.S, small.n_blocks
-    copies = POOL_MAX // (S * Nb) + 1
-    large = _shape(heads, (grid[0] * copies, grid[1], grid[2]), (block[0] * copies, block[1], block[2]))
+    copies, large = _copies(small, total)
     g = torch.Generator(device="cuda").manual_seed(3)
     x = torch.randn((heads, S, Nb), generator=g, device="cuda")
     if values == "constant":
@@ -116,12 +160,11 @@ def test_pool_kernel_special_scores(values, rule, tau, topk):
     elif values == "nan":
         x[0, 5] = float("nan")
         x[1, 9, 2] = -float("nan")
-    y = x[:, None].expand(heads, copies, S, Nb).reshape(heads, copies * S, Nb).contiguous()
     score_range = None
     if values == "nan":          # (as the scores kernel leaves it: of the numbers)
         score_range = torch.stack([x.nan_to_num(0.0).amin((1, 2)), x.nan_to_num(0.0).amax((1, 2))], 1).contiguous()
     a = _run(small, x, rule, tau, topk, score_range)
-    b = _run(large, y, rule, tau, topk, score_range, capacity=int(heads * large.S * Nb))
+    b = _run(large, _repeat(x, copies), rule, tau, topk, score_range, capacity=int(heads * large.S * Nb))
     ma, mb = _mask(small, a), _mask(large, b).reshape(heads, copies, S, Nb)
     _check_lists(small, a, ma)
     # a NaN takes the mass of the lowest bin of its CTA (there) or thread (here) with it: a few pairs of 600
