@@ -164,15 +164,15 @@ inline void count_launches(int n) { g_kernel_launches.fetch_add((unsigned long l
 // range-checked build, where nothing is early, and the diagnostics' own kernel do neither).  An early launch does
 // not wait for the end of the kernel before it in the stream: its CTAs are set up while the other still runs, stop in
 // grid_begin() until that one has completed and its writes are visible, and then allow the same for the next.  A call is a
-// chain of some twenty kernels (23 in bf16 with the backward, 27 in fp32), many of a few microseconds, and each early launch
+// chain of a dozen kernels or more (12 to 17 in bf16 with the backward, 17 in fp32), many of a few microseconds, and each early launch
 // is worth 1.5 .. 3 us (forward of 33K tokens,
 // 12 heads: 659 -> 624 us; forward and backward of 1.9K tokens: 204 -> 171 us).
 //
 // Not early: a long kernel that lives by many loads in flight, after one with another shape.  CTAs that move in beside the
 // running kernel find the SM's shared memory / L1 split as that one has it, and keep it; and the SMs that run dry first take
 // more than their share of them.  Measured, early against not (33K tokens, 3D blocks): merge pass 1391 / 838 us, row-dot pass
-// 94 / 80 us, backward 494 / 433 us, first histogram 111 / 101 us, inverse permutation 81 / 72 us.  Such kernels are early
-// only where they are short themselves: early_rows().
+// 94 / 80 us, backward 494 / 433 us, first histogram 111 / 101 us.  Such kernels are early only where they are short themselves:
+// early_rows().
 template <typename... P, typename... A>
 inline void launch_kernel(bool early, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -393,6 +393,13 @@ __device__ __forceinline__ void block_exclusive_scan(In in, int* __restrict__ ou
   if (n <= 2 * (long long)blockDim.x) block_exclusive_scan_by<1>(in, out, n, total_out);
   else block_exclusive_scan_by<8>(in, out, n, total_out);
 }
+
+// Centroids as three bf16 numbers each, whose sum they are (scores_tc.cu): parts[part][head][Nb_pad][head_dim], pad rows zero.
+struct CentroidParts {
+  __nv_bfloat16* parts = nullptr;
+  int Nb_pad = 0;
+  long long n = 0;        // elements of one part
+};
 
 // Device counters set through vmoba_debug_wait_profile (null when diagnostics are off).
 unsigned long long* debug_wait_profile();

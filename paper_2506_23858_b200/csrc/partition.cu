@@ -90,7 +90,7 @@ static int launch_partition(const Dims& D, const PermGeom& g, int inverse, int n
                             int32_t* inv_perm, cudaStream_t st) {
   const long long n_rows = (long long)D.BH * D.S;
   auto go = [&](auto kernel, int rows) {
-    launch_kernel(early_rows(D), kernel, dim3((unsigned)((n_rows + 8 * rows - 1) / (8 * rows)), n), 256, 0, st, g, D.S, D.heads,
+    launch_kernel(kernel, dim3((unsigned)((n_rows + 8 * rows - 1) / (8 * rows)), n), 256, 0, st, g, D.S, D.heads,
                   (int)n_rows, inverse, t, perm, inv_perm);
   };
   // 32 rows per warp once that gives every SM its 64 warps; below, 8 rows, for more warps to hide a pass's latency

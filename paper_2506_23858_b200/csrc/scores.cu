@@ -13,8 +13,8 @@ namespace vmoba {
 
 // scores_tc.cu: tensor-core scores for bf16 / head_dim 128
 size_t scores_tc_ws_bytes(const Dims& D);
-int scores_tc(const Dims& D, const void* q_bm, const float* cent, float* scores, float* range, void* ws,
-              int32_t* status, cudaStream_t st);
+CentroidParts scores_tc_parts(const Dims& D, void* ws);
+int scores_tc(const Dims& D, const void* q_bm, const CentroidParts& cent, float* scores, float* range, int32_t* status, cudaStream_t st);
 
 size_t scores_ws_bytes(const Dims& D) {
   return (D.dtype == VMOBA_BF16 && D.d == 128) ? scores_tc_ws_bytes(D) : 256;
@@ -25,10 +25,14 @@ size_t scores_ws_bytes(const Dims& D) {
 // few blocks by the latency of a thread's chain of loads, hence the many in flight.
 // The blocks are taken from the last position of every head to the first: the partition of k, in token order over all heads,
 // ends there, and what it wrote last is still in L2.
+// For the tensor-core scores kernel it also leaves the centroids' parts (a launch of its own before), and in any case
+// the score range's starting values for the kernel that follows.
 template <typename T, int DH, int SPLIT>
 __global__ void __launch_bounds__((1024 / DH) * (DH * (int)sizeof(T) / 16 / SPLIT))
-centroid_kernel(const T* __restrict__ k_bm, float* __restrict__ cent, int sb, int BH, int Nb) {
+centroid_kernel(const T* __restrict__ k_bm, float* __restrict__ cent, int sb, int BH, int Nb, CentroidParts out, float* __restrict__ range) {
   if (!grid_begin()) return;
+  if (range && blockIdx.x == 0)
+    for (int h = threadIdx.x; h < BH; h += blockDim.x) { range[2 * h] = INFINITY; range[2 * h + 1] = -INFINITY; }
   constexpr int W = 16 / sizeof(T);          // columns per thread
   constexpr int V = DH / W / SPLIT;          // threads per row
   constexpr int RL = 1024 / DH;              // row lanes
@@ -65,20 +69,34 @@ centroid_kernel(const T* __restrict__ k_bm, float* __restrict__ cent, int sb, in
   for (int c = threadIdx.x; c < V * W; c += RL * V) {
     float s = red[0][c];
     for (int r = 1; r < RL; ++r) s += red[r][c];
-    cent[blk * DH + part * V * W + c] = s * inv;
+    const float x = s * inv;
+    cent[blk * DH + part * V * W + c] = x;
+    if constexpr (sizeof(T) == 2 && DH == 128) {
+      const __nv_bfloat16 b1 = __float2bfloat16_rn(x);
+      const float r1 = x - __bfloat162float(b1);
+      const __nv_bfloat16 b2 = __float2bfloat16_rn(r1);
+      const float r2 = r1 - __bfloat162float(b2);
+      const long long at = ((long long)bh * out.Nb_pad + j) * DH + part * V * W + c;
+      out.parts[at] = b1;
+      out.parts[out.n + at] = b2;
+      out.parts[2 * out.n + at] = __float2bfloat16_rn(r2);
+      if (j == Nb - 1)
+        for (int p = 0; p < 3; ++p)
+          for (int r = 1; r < out.Nb_pad - j; ++r) out.parts[p * out.n + at + r * DH] = __float2bfloat16_rn(0.f);
+    }
   }
 }
 
 template <typename T, int DH>
-static void run_centroids(const Dims& D, const T* k, float* cent, cudaStream_t st) {
+static void run_centroids(const Dims& D, const T* k, float* cent, const CentroidParts& parts, float* range, cudaStream_t st) {
   constexpr int THREADS = (1024 / DH) * (DH * (int)sizeof(T) / 16);
   const long long n = (long long)D.BH * D.Nb;
   // Four CTAs per block where one would not give every SM four.  12 heads: 24 blocks of 1,400 keys 41 us with one, 24 with
   // four; 16 blocks of 840 keys 20 and 8; 140 blocks of 234 keys 15 with one.
   if (n < sm_count() * 4ll)
-    launch_kernel(centroid_kernel<T, DH, 4>, (unsigned)(4 * n), THREADS / 4, 0, st, k, cent, D.sb, D.BH, D.Nb);
+    launch_kernel(centroid_kernel<T, DH, 4>, (unsigned)(4 * n), THREADS / 4, 0, st, k, cent, D.sb, D.BH, D.Nb, parts, range);
   else
-    launch_kernel(centroid_kernel<T, DH, 1>, (unsigned)n, THREADS, 0, st, k, cent, D.sb, D.BH, D.Nb);
+    launch_kernel(centroid_kernel<T, DH, 1>, (unsigned)n, THREADS, 0, st, k, cent, D.sb, D.BH, D.Nb, parts, range);
 }
 
 // fp32 tile GEMM: a CTA computes 64 queries x 64 blocks with the whole head_dim in shared
@@ -86,7 +104,7 @@ static void run_centroids(const Dims& D, const T* k, float* cent, cudaStream_t s
 template <typename T, int DH>
 __global__ void __launch_bounds__(256)
 scores_kernel(const T* __restrict__ q_bm, const float* __restrict__ cent, float* __restrict__ scores,
-              int S, int Nb) {
+              int S, int Nb, float* __restrict__ range) {
   if (!grid_begin()) return;
   extern __shared__ float smem[];
   constexpr int LD = 64 + 4;
@@ -110,6 +128,7 @@ scores_kernel(const T* __restrict__ q_bm, const float* __restrict__ cent, float*
   const int ty = tid / 16, tx = tid % 16;
   const float* ch = cent + (long long)bh * Nb * DH;
   float* out = scores + ((long long)bh * S + q0) * Nb;
+  float lo = INFINITY, hi = -INFINITY;      // of this thread's scores
   for (int j0 = 0; j0 < Nb; j0 += 64) {
     __syncthreads();
     for (int i = tid; i < 64 * V; i += 256) {
@@ -144,54 +163,37 @@ scores_kernel(const T* __restrict__ q_bm, const float* __restrict__ cent, float*
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         int col = j0 + tx * 4 + j;
-        if (col < Nb) out[(long long)r * Nb + col] = acc[i][j];
+        if (col < Nb) {
+          out[(long long)r * Nb + col] = acc[i][j];
+          lo = fminf(lo, acc[i][j]);
+          hi = fmaxf(hi, acc[i][j]);
+        }
       }
     }
   }
-}
-
-// Smallest and largest score of each head (the paths whose scores kernel does not take them on the way).
-__global__ void range_init_kernel(float* __restrict__ range, int BH) {
-  if (!grid_begin()) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < BH) { range[2 * i] = INFINITY; range[2 * i + 1] = -INFINITY; }
-}
-__global__ void __launch_bounds__(256)
-range_kernel(const float* __restrict__ scores, long long P, float* __restrict__ range) {
-  if (!grid_begin()) return;
-  const int bh = blockIdx.y;
-  const float* base = scores + (long long)bh * P;
-  float lo = INFINITY, hi = -INFINITY;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < P; i += (long long)gridDim.x * blockDim.x) {
-    const float s = base[i];
-    lo = fminf(lo, s); hi = fmaxf(hi, s);
-  }
+  if (range) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-    hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if ((tid & 31) == 0 && lo <= hi) { atomic_min_f32(range + 2 * bh, lo); atomic_max_f32(range + 2 * bh + 1, hi); }
   }
-  if ((threadIdx.x & 31) == 0 && lo <= hi) { atomic_min_f32(range + 2 * bh, lo); atomic_max_f32(range + 2 * bh + 1, hi); }
 }
 
 template <typename T, int DH>
 static int run_scores(const Dims& D, const void* q, const void* k, float* cent, float* scores, float* range, void* ws,
                       int32_t* status, cudaStream_t st) {
-  run_centroids<T, DH>(D, static_cast<const T*>(k), cent, st);
+  const bool tc = D.dtype == VMOBA_BF16 && DH == 128;
+  const CentroidParts parts = tc ? scores_tc_parts(D, ws) : CentroidParts();
+  run_centroids<T, DH>(D, static_cast<const T*>(k), cent, parts, range, st);
   VMOBA_LAUNCH_OK(1);
-  if (D.dtype == VMOBA_BF16 && DH == 128) return scores_tc(D, q, cent, scores, range, ws, status, st);
+  if (tc) return scores_tc(D, q, parts, scores, range, status, st);
   size_t smem = 2 * DH * (64 + 4) * sizeof(float);
   VMOBA_CUDA_OK(cudaFuncSetAttribute(scores_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   dim3 grid((D.S + 63) / 64, 1, D.BH);
-  launch_kernel(scores_kernel<T, DH>, grid, 256, smem, st, static_cast<const T*>(q), cent, scores, D.S, D.Nb);
+  launch_kernel(scores_kernel<T, DH>, grid, 256, smem, st, static_cast<const T*>(q), cent, scores, D.S, D.Nb, range);
   VMOBA_LAUNCH_OK(1);
-  if (range) {
-    const long long P = (long long)D.S * D.Nb;
-    launch_kernel(range_init_kernel, (D.BH + 127) / 128, 128, 0, st, range, D.BH);
-    const int gx = (int)std::min<long long>(std::max<long long>(P / 2048, 1), std::max(1, sm_count() * 8 / D.BH));
-    launch_kernel(range_kernel, dim3(gx, D.BH), 256, 0, st, scores, P, range);
-    VMOBA_LAUNCH_OK(2);
-  }
   return VMOBA_OK;
 }
 

@@ -62,34 +62,6 @@ struct Params {
   int32_t* status;
 };
 
-// Splits fp32 centroids into three bf16 parts: parts[part][bh][Nb_pad][128]; pad rows are zero.
-__global__ void __launch_bounds__(256)
-split_centroids_kernel(const float* __restrict__ cent, __nv_bfloat16* __restrict__ parts, int Nb, int Nb_pad, int BH,
-                       float* __restrict__ range) {
-  if (!grid_begin()) return;
-  const long long n = (long long)BH * Nb_pad * DH;
-  if (range) {     // the scores kernel that follows takes minima / maxima into these words
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < BH) { range[2 * t] = INFINITY; range[2 * t + 1] = -INFINITY; }
-  }
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i % DH);
-    const long long row = i / DH;
-    const int j = (int)(row % Nb_pad);
-    const long long bh = row / Nb_pad;
-    float x = 0.f;
-    if (j < Nb) x = cent[(bh * Nb + j) * DH + c];
-    const __nv_bfloat16 b1 = __float2bfloat16_rn(x);
-    const float r1 = x - __bfloat162float(b1);
-    const __nv_bfloat16 b2 = __float2bfloat16_rn(r1);
-    const float r2 = r1 - __bfloat162float(b2);
-    const __nv_bfloat16 b3 = __float2bfloat16_rn(r2);
-    parts[i] = b1;
-    parts[n + i] = b2;
-    parts[2 * n + i] = b3;
-  }
-}
-
 __global__ void __launch_bounds__(THREADS, 1)
 scores_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ CUtensorMap tmS, const Params p) {
@@ -317,18 +289,21 @@ size_t scores_tc_ws_bytes(const Dims& D) {
   return 3 * (size_t)D.BH * Nb_pad * sct::DH * sizeof(__nv_bfloat16) + 1024;
 }
 
-// scores [BH, S, Nb] fp32 from block-major bf16 q and fp32 centroids (already computed).
-int scores_tc(const Dims& D, const void* q_bm, const float* cent, float* scores, float* range, void* ws,
-              int32_t* status, cudaStream_t st) {
+// Where the centroid kernel leaves the parts: [3][BH][Nb_pad][128], rows of whole 32-column slabs (the epilogue's store unit).
+CentroidParts scores_tc_parts(const Dims& D, void* ws) {
+  CentroidParts c;
+  c.Nb_pad = (D.Nb + 31) / 32 * 32;
+  c.parts = reinterpret_cast<__nv_bfloat16*>((reinterpret_cast<uintptr_t>(ws) + 1023) & ~uintptr_t(1023));
+  c.n = (long long)D.BH * c.Nb_pad * sct::DH;
+  return c;
+}
+
+// scores [BH, S, Nb] fp32 from block-major bf16 q and the centroids' parts (already there; range, if given, starts at +inf, -inf).
+int scores_tc(const Dims& D, const void* q_bm, const CentroidParts& cent, float* scores, float* range, int32_t* status, cudaStream_t st) {
   using namespace sct;
-  // ranges of whole 32-column slabs (the epilogue's store unit)
-  const int Nb_pad = (D.Nb + 31) / 32 * 32;
+  const int Nb_pad = cent.Nb_pad;
   const int n_pass = (Nb_pad + NT_MAX - 1) / NT_MAX;
   const int rows_pass = ((Nb_pad + n_pass - 1) / n_pass + 31) / 32 * 32;
-  __nv_bfloat16* parts = reinterpret_cast<__nv_bfloat16*>((reinterpret_cast<uintptr_t>(ws) + 1023) & ~uintptr_t(1023));
-  const long long n = (long long)D.BH * Nb_pad * DH;
-  launch_kernel(split_centroids_kernel, (int)std::min<long long>((n + 255) / 256, sm_count() * 8), 256, 0, st, cent,
-                parts, D.Nb, Nb_pad, D.BH, range);
   CUtensorMap tmQ, tmB, tmS;
   const int tma_store = (D.Nb % 4 == 0) && (reinterpret_cast<uintptr_t>(scores) % 16 == 0);
   if (tma_store) {
@@ -337,7 +312,7 @@ int scores_tc(const Dims& D, const void* q_bm, const float* cent, float* scores,
     tmS = CUtensorMap{};
   }
   if (!sm100::make_tmap_bf16_rows(&tmQ, q_bm, (uint64_t)D.BH * D.S, DH, BM) ||
-      !sm100::make_tmap_bf16_rows(&tmB, parts, (uint64_t)3 * D.BH * Nb_pad, DH, rows_pass))
+      !sm100::make_tmap_bf16_rows(&tmB, cent.parts, (uint64_t)3 * D.BH * Nb_pad, DH, rows_pass))
     return VMOBA_ERR_CUDA;
   Params p;
   p.scores = scores; p.S = D.S; p.Nb = D.Nb; p.Nb_pad = Nb_pad; p.BH = D.BH; p.n_pass = n_pass; p.rows_pass = rows_pass;
@@ -350,7 +325,7 @@ int scores_tc(const Dims& D, const void* q_bm, const float* cent, float* scores,
   const long long items = (long long)D.BH * n_pass * ((D.S + BM - 1) / BM);
   launch_kernel(scores_tc_kernel, (int)std::max<long long>(1, std::min<long long>(items, sm_count())), THREADS,
                 smem_bytes(p.nq, rows_pass), st, tmQ, tmB, tmS, p);
-  VMOBA_LAUNCH_OK(2);
+  VMOBA_LAUNCH_OK(1);
   return VMOBA_OK;
 }
 
