@@ -81,7 +81,8 @@ static int simt_sparse_fwd(const Dims& D, const void* q, const void* k, const vo
   const long long n_kb = (long long)D.BH * D.Nb;
   launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
   long long max_items = cap / simt::kRows + n_kb;
-  launch_kernel(early_simt(D, (double)cap * D.sb), simt::attn_fwd_kernel<T, DH, false>, grid_for(max_items, 8), simt::kThreads, 0, st, (const T*)q,
+  VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_fwd_kernel<T, DH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kFwdSmem<DH>));
+  launch_kernel(early_simt(D, (double)cap * D.sb), simt::attn_fwd_kernel<T, DH, false>, grid_for(max_items, 8), simt::kThreads, simt::kFwdSmem<DH>, st, (const T*)q,
                 (const T*)k, (const T*)v, kb_ptr, q_idx, q_ptr, w.item_ptr, (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale,
                 (T*)o, (T*)o_resid, lse, w.part_o, w.part_lse, cap);
   long long nq = (long long)D.BH * D.S;
@@ -118,22 +119,24 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
     VMOBA_GUARDS_CHECK(w.guards, status, st);
     return VMOBA_OK;
   }
+  // fp32 gradients are added up in place (unless dq takes the place of something that is still read), others in an accumulator; the
+  // row-dot pass clears it
+  const bool in_place = D.dtype == VMOBA_F32 && dq != q && dq != k && dq != v && dq != o && dq != d_o;
+  float* acc = in_place ? reinterpret_cast<float*>(dq) : w.dq_acc;
   launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
-                (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), nullptr, nullptr, (T*)nullptr, nullptr, 0);
-  count_launches(1);
-  VMOBA_CUDA_OK(cudaMemsetAsync(w.dq_acc, 0, (size_t)nq * DH * sizeof(float), st));
-  launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
+                (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), acc, nullptr, (T*)nullptr, nullptr, 0);
   long long tiles = (D.sb + simt::kRows - 1) / simt::kRows;
-  const bool early = early_simt(D, (double)cap * D.sb);
-  launch_kernel(early, simt::attn_bwd_dkdv_kernel<T, DH, false>, grid_for(n_kb * tiles, 4), simt::kThreads, 0, st,
-                (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb, D.BH,
-                D.scale, cap, (T*)dk, (T*)dv);
-  launch_kernel(early, simt::attn_bwd_dq_kernel<T, DH, false>, grid_for(nq / simt::kRows * D.Nb + n_kb, 4), simt::kThreads,
-                0, st, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, w.item_ptr,
-                (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale, cap, w.dq_acc, (T*)dq);
-  launch_kernel(early_rows(D), simt::cast_kernel<T>, grid_for((nq * DH / 4 + 255) / 256, 16), 256, 0, st, w.dq_acc,
-                (T*)dq, nq * DH / 4);
-  VMOBA_LAUNCH_OK(4);
+  VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_bwd_dkdv_kernel<T, DH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kBwdSmem<DH>));
+  launch_kernel(early_simt(D, (double)cap * D.sb), simt::attn_bwd_dkdv_kernel<T, DH, false>, grid_for(n_kb * tiles, 4), simt::kThreads,
+                simt::kBwdSmem<DH>, st, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb,
+                D.BH, D.scale, cap, (T*)dk, (T*)dv, acc);
+  count_launches(2);
+  if (!in_place) {
+    launch_kernel(early_rows(D), simt::cast_kernel<T>, grid_for((nq * DH / 4 + 255) / 256, 16), 256, 0, st, w.dq_acc,
+                  (T*)dq, nq * DH / 4);
+    count_launches(1);
+  }
+  VMOBA_LAUNCH_OK(0);
   VMOBA_GUARDS_CHECK(w.guards, status, st);
   return VMOBA_OK;
 }
@@ -149,7 +152,8 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
     int rc = tc_dense_fwd(D, q, k, v, o, d_o ? w.o_resid : nullptr, lse, status, st);
     if (rc) return rc;
   } else {
-    launch_kernel(early, simt::attn_fwd_kernel<T, DH, true>, grid_for(D.BH * tiles, 8), simt::kThreads, 0, st, (const T*)q,
+    VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_fwd_kernel<T, DH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kFwdSmem<DH>));
+    launch_kernel(early, simt::attn_fwd_kernel<T, DH, true>, grid_for(D.BH * tiles, 8), simt::kThreads, simt::kFwdSmem<DH>, st, (const T*)q,
                   (const T*)k, (const T*)v, nullptr, nullptr, nullptr, nullptr, 0, D.S, 1, D.S, D.BH, D.scale, (T*)o,
                   d_o ? (T*)w.o_resid : nullptr, lse, nullptr, nullptr, 0);
     count_launches(1);
@@ -168,12 +172,13 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
       VMOBA_LAUNCH_OK(1);
       return VMOBA_OK;
     }
-    launch_kernel(early, simt::attn_bwd_dkdv_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, 0, st,
+    VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_bwd_dkdv_kernel<T, DH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kBwdSmem<DH>));
+    VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_bwd_dq_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kBwdSmem<DH>));
+    launch_kernel(early, simt::attn_bwd_dkdv_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, simt::kBwdSmem<DH>, st,
                   (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, D.S, 1, D.S,
-                  D.BH, D.scale, 0, (T*)dk, (T*)dv);
-    launch_kernel(early, simt::attn_bwd_dq_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, 0, st,
-                  (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, nullptr, 0, D.S,
-                  1, D.S, D.BH, D.scale, 0, nullptr, (T*)dq);
+                  D.BH, D.scale, 0, (T*)dk, (T*)dv, nullptr);
+    launch_kernel(early, simt::attn_bwd_dq_kernel<T, DH>, grid_for(D.BH * tiles, 4), simt::kThreads, simt::kBwdSmem<DH>, st, (const T*)q,
+                  (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, D.S, D.BH, D.scale, (T*)dq);
   }
   VMOBA_LAUNCH_OK(d_o ? 3 : 0);
   return VMOBA_OK;

@@ -18,9 +18,8 @@
 namespace vmoba {
 namespace simt {
 
-constexpr int kRows = 64;      // rows (queries, or keys in the dK/dV kernel) per CTA
-constexpr int kTile = 32;      // rows of the streamed operand per shared-memory tile
-constexpr int kThreads = 256;  // 4 threads per row, each owning head_dim/4 channels
+constexpr int kRows = 64;      // rows (queries, or keys in the dK/dV kernel) per CTA, and of a tile of the streamed operand
+constexpr int kThreads = 256;  // 16 x 16: a thread owns a 4 x 4 piece of a 64 x 64 product, 4 rows x DH / 16 columns of a result
 
 // item_desc[item] = {index of the (batch, head, key block) list, first list position, rows (<= rows_per_item), 0}; a warp
 // per list (a thread per list took 13 us for 240 lists of 77 items, bound by the latency of its loop).
@@ -103,130 +102,247 @@ __device__ __forceinline__ Item decode_sparse(int item, const int* __restrict__ 
   return it;
 }
 
-// Cooperative load of `kTile` rows x DH channels (converted to fp32) into shared memory;
-// rows beyond `n_valid` are zero-filled.  row_of(i) gives the in-head position of tile row i.
-template <typename T, int DH, typename RowOf>
-__device__ __forceinline__ void load_tile(float* __restrict__ dst, const T* __restrict__ head_base, int n_valid,
-                                          RowOf row_of) {
-  constexpr int V = DH / 4;
-  for (int i = threadIdx.x; i < kTile * V; i += kThreads) {
-    int r = i / V, c4 = i % V;
-    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r < n_valid) x = load4(head_base + (long long)row_of(r) * DH + c4 * 4);
-    *reinterpret_cast<float4*>(dst + r * DH + c4 * 4) = x;
+// Tiles in shared memory: 64 rows of DH (or 64) floats, four more to a row, so that sixteen consecutive rows' float4 lie in
+// different banks.
+//
+// The products below are bound by the FMA pipe: 64 FMAs per eight 16-byte loads from shared memory.  With four threads to a row,
+// each holding a quarter of its channels, a key cost a thread as many loads as four of its FMAs and two shuffles.
+// Forward and backward of 13 heads x 4,096 tokens, head_dim 128, 2450 -> 1095 us; of 2 x 256, head_dim 64, 98.6 -> 72.0.
+template <int DH> constexpr int kLd = DH + 4;
+template <int DH> constexpr int kTileFloats = kRows * kLd<DH>;
+constexpr int kLdP = kRows + 4;
+
+// A tile's rows, in registers on their way from global to shared memory (rows beyond n_valid: zeros).
+template <typename T, int DH>
+struct TileRegs {
+  static constexpr int V = DH / 4, N = kRows * V / kThreads;
+  float4 x[N];
+  template <typename RowOf>
+  __device__ __forceinline__ void fetch(const T* __restrict__ head_base, int n_valid, RowOf row_of) {
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      const int i = threadIdx.x + n * kThreads, r = i / V, c4 = i % V;
+      x[n] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r < n_valid) x[n] = load4(head_base + (long long)row_of(r) * DH + c4 * 4);
+    }
+  }
+  __device__ __forceinline__ void store(float* dst) const {
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      const int i = threadIdx.x + n * kThreads, r = i / V, c4 = i % V;
+      *reinterpret_cast<float4*>(dst + r * kLd<DH> + c4 * 4) = x[n];
+    }
+  }
+};
+
+// acc[i][j] = A[4 ty + i] . B[tx + 16 j] for the first NJ * 16 rows of B.  Sixteen channels at a time: sums of sums keep
+// the rounding error of one long sum, and more, away (o of 4 x 2,048 tokens, head_dim 128: 4.0e-7 off with a quarter of
+// the channels in a row, 5.1e-7 with all of them, 3.6e-7 so).
+template <int DH, int NJ>
+__device__ __forceinline__ void dot_tiles_n(const float* A, const float* B, int ty, int tx, float (&acc)[4][4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+#pragma unroll 1
+  for (int c0 = 0; c0 < DH; c0 += 16) {
+    float part[4][NJ];
+#pragma unroll
+    for (int c = 0; c < 16; c += 4) {
+      float4 a[4], b[NJ];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(A + (4 * ty + i) * kLd<DH> + c0 + c);
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) b[j] = *reinterpret_cast<const float4*>(B + (tx + 16 * j) * kLd<DH> + c0 + c);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+          part[i][j] = c == 0 ? a[i].x * b[j].x : fmaf(a[i].x, b[j].x, part[i][j]);
+          part[i][j] = fmaf(a[i].y, b[j].y, part[i][j]);
+          part[i][j] = fmaf(a[i].z, b[j].z, part[i][j]);
+          part[i][j] = fmaf(a[i].w, b[j].w, part[i][j]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) acc[i][j] += part[i][j];
   }
 }
+template <int DH>
+__device__ __forceinline__ void dot_tiles(const float* A, const float* B, int ty, int tx, int n_b, float (&acc)[4][4]) {
+  if (n_b > 32) dot_tiles_n<DH, 4>(A, B, ty, tx, acc);
+  else dot_tiles_n<DH, 2>(A, B, ty, tx, acc);
+}
 
-__device__ __forceinline__ float quad_sum(float x) {
-  x += __shfl_xor_sync(0xffffffffu, x, 1);
-  x += __shfl_xor_sync(0xffffffffu, x, 2);
+__device__ __forceinline__ void fma4(float* acc, float w, const float4& x) {
+  acc[0] = fmaf(w, x.x, acc[0]); acc[1] = fmaf(w, x.y, acc[1]); acc[2] = fmaf(w, x.z, acc[2]); acc[3] = fmaf(w, x.w, acc[3]);
+}
+// acc[i][4 g + c] += sum over the first n rows k of B: P[4 ty + i][k] * B[k][64 g + 4 tx + c]
+template <int DH>
+__device__ __forceinline__ void add_weighted(const float* P, const float* B, int ty, int tx, int n, float (&acc)[4][DH / 16]) {
+#pragma unroll 1
+  for (int k = 0; k < n; k += 4) {
+    float4 w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = *reinterpret_cast<const float4*>(P + (4 * ty + i) * kLdP + k);
+#pragma unroll
+    for (int g = 0; g < DH / 64; ++g) {
+      float4 x[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[e] = *reinterpret_cast<const float4*>(B + (k + e) * kLd<DH> + 64 * g + 4 * tx);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        fma4(&acc[i][4 * g], w[i].x, x[0]); fma4(&acc[i][4 * g], w[i].y, x[1]);
+        fma4(&acc[i][4 * g], w[i].z, x[2]); fma4(&acc[i][4 * g], w[i].w, x[3]);
+      }
+    }
+  }
+}
+// The same with P transposed: acc[i][..] += sum over k of P[k][4 ty + i] * B[k][..]
+template <int DH>
+__device__ __forceinline__ void add_weighted_t(const float* P, const float* B, int ty, int tx, int n, float (&acc)[4][DH / 16]) {
+#pragma unroll 4
+  for (int k = 0; k < n; ++k) {
+    const float4 w = *reinterpret_cast<const float4*>(P + k * kLdP + 4 * ty);
+#pragma unroll
+    for (int g = 0; g < DH / 64; ++g) {
+      const float4 x = *reinterpret_cast<const float4*>(B + k * kLd<DH> + 64 * g + 4 * tx);
+      fma4(&acc[0][4 * g], w.x, x); fma4(&acc[1][4 * g], w.y, x); fma4(&acc[2][4 * g], w.z, x); fma4(&acc[3][4 * g], w.w, x);
+    }
+  }
+}
+// over the sixteen threads of a row
+__device__ __forceinline__ float row_max(float x) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
   return x;
 }
+__device__ __forceinline__ float row_sum(float x) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+template <int DH> constexpr int kFwdSmem = (2 * kTileFloats<DH> + kRows * kLdP) * 4;      // Q, K or V, weights
 
 // ------------------------------------------------------------------------------ forward
 template <typename T, int DH, bool DENSE>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 2)
 attn_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                 const int* __restrict__ kb_ptr, const int* __restrict__ q_idx, const int* __restrict__ q_ptr,
                 const int* __restrict__ item_ptr, int n_kb, int S, int Nb, int sb, int BH, float scale,
                 T* __restrict__ o, T* __restrict__ o_resid, float* __restrict__ lse, float* __restrict__ part_o,
                 float* __restrict__ part_lse, long long capacity) {
   if (!grid_begin()) return;
-  constexpr int DP = DH / 4;   // channels per thread
-  constexpr int G = DP / 4;    // float4 groups per thread
-  __shared__ __align__(16) float Ks[kTile * DH];
-  __shared__ __align__(16) float Vs[kTile * DH];
-  const int r = threadIdx.x >> 2, part = threadIdx.x & 3;
+  extern __shared__ __align__(16) float simt_smem[];
+  float* Qs = simt_smem;
+  float* KVs = Qs + kTileFloats<DH>;
+  float* Ps = KVs + kTileFloats<DH>;
+  __shared__ int s_row[kRows];                 // in-head position of the query, -1 for none; bit 30: it has a single block
+  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
   const int tiles_per_head = (S + kRows - 1) / kRows;
   const int n_items = DENSE ? BH * tiles_per_head : item_ptr[n_kb];
   for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
     Item it;
-    int qpos = -1;
-    long long pos = -1;
+    int rows;
     if (DENSE) {
       it.bh = item / tiles_per_head;
-      int row = (item - it.bh * tiles_per_head) * kRows + r;
+      it.list_lo = (item - it.bh * tiles_per_head) * kRows;
       it.key_begin = 0; it.key_end = S;
-      if (row < S) qpos = row;
+      rows = min(kRows, S - it.list_lo);
     } else {
       it = decode_sparse(item, item_ptr, n_kb, kb_ptr, Nb, sb, kRows, capacity);
-      if (it.list_lo + r < it.list_hi) { pos = it.list_lo + r; qpos = q_idx[pos]; }
+      rows = it.list_hi - it.list_lo;
     }
     const long long head_off = (long long)it.bh * S;
     const T* kh = k + head_off * DH;
     const T* vh = v + head_off * DH;
-    float qr[DP], acc[DP];
-#pragma unroll
-    for (int g = 0; g < G; ++g) {
-      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (qpos >= 0) x = load4(q + (head_off + qpos) * DH + (part + 4 * g) * 4);
-      qr[4 * g] = x.x; qr[4 * g + 1] = x.y; qr[4 * g + 2] = x.z; qr[4 * g + 3] = x.w;
-      acc[4 * g] = acc[4 * g + 1] = acc[4 * g + 2] = acc[4 * g + 3] = 0.f;
+    constexpr int kSingle = 1 << 30;
+    __syncthreads();                           // (the item before is through with the shared memory)
+    if (t < kRows) {
+      int x = -1;
+      if (t < rows) {
+        x = DENSE ? it.list_lo + t : q_idx[it.list_lo + t];
+        if (DENSE || q_ptr[head_off + x + 1] - q_ptr[head_off + x] == 1) x |= kSingle;
+      }
+      s_row[t] = x;
     }
-    float m = -INFINITY, l = 0.f;
-    for (int t0 = it.key_begin; t0 < it.key_end; t0 += kTile) {
-      const int nv = min(kTile, it.key_end - t0);
-      __syncthreads();
-      load_tile<T, DH>(Ks, kh, nv, [&](int i) { return t0 + i; });
-      load_tile<T, DH>(Vs, vh, nv, [&](int i) { return t0 + i; });
-      __syncthreads();
-#pragma unroll 1
-      for (int kk = 0; kk < kTile; kk += 16) {
-        if (kk >= nv) break;
-        float s[16];
+    TileRegs<T, DH> next;
+    next.fetch(kh, min(kRows, it.key_end - it.key_begin), [&](int i) { return it.key_begin + i; });
+    __syncthreads();
+    {
+      TileRegs<T, DH> qt;
+      qt.fetch(q + head_off * DH, rows, [&](int i) { return s_row[i] & (kSingle - 1); });
+      qt.store(Qs);
+    }
+    next.store(KVs);
+    float m[4], l[4], acc[4][DH / 16];         // l: of this thread's keys only
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float a = 0.f;
+    for (int i = 0; i < 4; ++i) {
+      m[i] = -INFINITY; l[i] = 0.f;
 #pragma unroll
-          for (int g = 0; g < G; ++g) {
-            float4 kv = *reinterpret_cast<const float4*>(Ks + (kk + i) * DH + (part + 4 * g) * 4);
-            a = fmaf(qr[4 * g], kv.x, a); a = fmaf(qr[4 * g + 1], kv.y, a);
-            a = fmaf(qr[4 * g + 2], kv.z, a); a = fmaf(qr[4 * g + 3], kv.w, a);
+      for (int c = 0; c < DH / 16; ++c) acc[i][c] = 0.f;
+    }
+    const bool live = (ty & ~1) * 4 < rows;    // (a warp has eight rows)
+    __syncthreads();
+    for (int t0 = it.key_begin; t0 < it.key_end; t0 += kRows) {
+      const int nv = min(kRows, it.key_end - t0);
+      next.fetch(vh, nv, [&](int i) { return t0 + i; });
+      if (live) {
+        float s[4][4];
+        dot_tiles<DH>(Qs, KVs, ty, tx, nv, s);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float mx = -INFINITY;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            s[i][j] = tx + 16 * j < nv ? s[i][j] * scale : -INFINITY;
+            mx = fmaxf(mx, s[i][j]);
           }
-          a = quad_sum(a);
-          s[i] = (kk + i < nv) ? a * scale : -INFINITY;
-        }
-        float mx = s[0];
+          const float m_new = fmaxf(m[i], row_max(mx));
+          const float corr = m[i] == -INFINITY ? 0.f : expf(m[i] - m_new);
+          l[i] *= corr;
 #pragma unroll
-        for (int i = 1; i < 16; ++i) mx = fmaxf(mx, s[i]);
-        const float m_new = fmaxf(m, mx);
-        const float corr = (m == -INFINITY) ? 0.f : expf(m - m_new);
-        l *= corr;
+          for (int c = 0; c < DH / 16; ++c) acc[i][c] *= corr;
 #pragma unroll
-        for (int c = 0; c < DP; ++c) acc[c] *= corr;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          const float p = (s[i] == -INFINITY) ? 0.f : expf(s[i] - m_new);
-          l += p;
-#pragma unroll
-          for (int g = 0; g < G; ++g) {
-            float4 vv = *reinterpret_cast<const float4*>(Vs + (kk + i) * DH + (part + 4 * g) * 4);
-            acc[4 * g] = fmaf(p, vv.x, acc[4 * g]); acc[4 * g + 1] = fmaf(p, vv.y, acc[4 * g + 1]);
-            acc[4 * g + 2] = fmaf(p, vv.z, acc[4 * g + 2]); acc[4 * g + 3] = fmaf(p, vv.w, acc[4 * g + 3]);
+          for (int j = 0; j < 4; ++j) {
+            const float p = s[i][j] == -INFINITY ? 0.f : expf(s[i][j] - m_new);
+            l[i] += p;
+            Ps[(4 * ty + i) * kLdP + tx + 16 * j] = p;
           }
+          m[i] = m_new;
         }
-        m = m_new;
+      }
+      __syncthreads();
+      next.store(KVs);
+      __syncthreads();
+      const int t1 = t0 + kRows;
+      if (t1 < it.key_end) next.fetch(kh, min(kRows, it.key_end - t1), [&](int i) { return t1 + i; });
+      if (live) add_weighted<DH>(Ps, KVs, ty, tx, nv, acc);
+      if (t1 < it.key_end) {
+        __syncthreads();
+        next.store(KVs);
+        __syncthreads();
       }
     }
-    if (qpos >= 0) {
-      const float inv = 1.0f / l;
-      const float row_lse = m + logf(l);
-      const long long G_ = head_off + qpos;
-      bool direct = DENSE;
-      if (!DENSE) direct = (q_ptr[G_ + 1] - q_ptr[G_]) == 1;
-      if (direct) {
+    if (!live) continue;
 #pragma unroll
-        for (int g = 0; g < G; ++g)
-          store4_resid(o + G_ * DH + (part + 4 * g) * 4, o_resid ? o_resid + G_ * DH + (part + 4 * g) * 4 : nullptr,
-                       make_float4(acc[4 * g] * inv, acc[4 * g + 1] * inv, acc[4 * g + 2] * inv, acc[4 * g + 3] * inv));
-        if (part == 0) lse[G_] = row_lse;
-      } else {
+    for (int i = 0; i < 4; ++i) {
+      const float total = row_sum(l[i]);
+      const int x = s_row[4 * ty + i];
+      if (x < 0) continue;
+      const float inv = 1.0f / total, row_lse = m[i] + logf(total);
+      const long long G_ = head_off + (x & (kSingle - 1)), pos = (long long)it.list_lo + 4 * ty + i;
+      const bool direct = (x & kSingle) != 0;
 #pragma unroll
-        for (int g = 0; g < G; ++g)
-          store4(part_o + pos * DH + (part + 4 * g) * 4,
-                 make_float4(acc[4 * g] * inv, acc[4 * g + 1] * inv, acc[4 * g + 2] * inv, acc[4 * g + 3] * inv));
-        if (part == 0) part_lse[pos] = row_lse;
+      for (int g = 0; g < DH / 64; ++g) {
+        const int col = 64 * g + 4 * tx;
+        const float4 r = make_float4(acc[i][4 * g] * inv, acc[i][4 * g + 1] * inv, acc[i][4 * g + 2] * inv, acc[i][4 * g + 3] * inv);
+        if (direct) store4_resid(o + G_ * DH + col, o_resid ? o_resid + G_ * DH + col : nullptr, r);
+        else store4(part_o + pos * DH + col, r);
       }
+      if (tx == 0) { if (direct) lse[G_] = row_lse; else part_lse[pos] = row_lse; }
     }
   }
 }
@@ -585,20 +701,26 @@ rowdot_kernel(const T* __restrict__ o, const T* __restrict__ o_resid, const T* _
   }
 }
 
-// dK, dV: key-stationary.  A CTA owns 64 keys of one key block (or of the whole sequence when
-// DENSE) and streams the queries that selected the block; no atomics, deterministic.
+// dK, dV: key-stationary.  A CTA owns 64 keys of one key block (or of the whole sequence when DENSE) and streams the queries that
+// selected the block; dK and dV are written once.  Sparse: dQ of every tile of queries is added into dq_acc (fp32, cleared
+// before), in whatever order the items come to it; dense: dQ has a kernel of its own, so that it repeats.
+template <int DH> constexpr int kBwdSmem = (4 * kTileFloats<DH> + kRows * kLdP) * 4;      // K, V, Q, dO, weights
 template <typename T, int DH, bool DENSE>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, DH == 64 ? 2 : 1)
 attn_bwd_dkdv_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
                      const T* __restrict__ d_o, const float* __restrict__ lse, const float* __restrict__ Dv,
                      const int* __restrict__ kb_ptr, const int* __restrict__ q_idx, int S, int Nb, int sb, int BH,
-                     float scale, long long capacity, T* __restrict__ dk, T* __restrict__ dv) {
+                     float scale, long long capacity, T* __restrict__ dk, T* __restrict__ dv, float* __restrict__ dq_acc) {
   if (!grid_begin()) return;
-  constexpr int DP = DH / 4, G = DP / 4;
-  __shared__ __align__(16) float Qs[kTile * DH];
-  __shared__ __align__(16) float dOs[kTile * DH];
-  __shared__ float s_lse[kTile], s_D[kTile];
-  const int r = threadIdx.x >> 2, part = threadIdx.x & 3;
+  extern __shared__ __align__(16) float simt_smem[];
+  float* Ks = simt_smem;
+  float* Vs = Ks + kTileFloats<DH>;
+  float* Qs = Vs + kTileFloats<DH>;
+  float* dOs = Qs + kTileFloats<DH>;
+  float* Ps = dOs + kTileFloats<DH>;           // [key][query]: weights, then dS
+  __shared__ float s_lse[kRows], s_D[kRows];
+  __shared__ int s_row[kRows];
+  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
   const int span = DENSE ? S : sb;
   const int tiles = (span + kRows - 1) / kRows;
   const long long n_items = (long long)BH * (DENSE ? 1 : Nb) * tiles;
@@ -606,167 +728,178 @@ attn_bwd_dkdv_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* 
     const int tile = (int)(item % tiles);
     const long long kbi = item / tiles;          // DENSE: bh ; sparse: bh * Nb + j
     const int bh = DENSE ? (int)kbi : (int)(kbi / Nb);
-    const int j = DENSE ? 0 : (int)(kbi - (long long)bh * Nb);
-    const int key_in_span = tile * kRows + r;
-    const bool key_ok = key_in_span < span;
-    const int kpos = j * sb + key_in_span;
+    const int j0 = DENSE ? 0 : (int)(kbi - (long long)bh * Nb);
+    const int key0 = j0 * sb + tile * kRows, keys = min(kRows, span - tile * kRows);
     const long long head_off = (long long)bh * S;
     long long list_lo = 0, list_hi = S;
     if (!DENSE) { list_lo = min((long long)kb_ptr[kbi], capacity); list_hi = min((long long)kb_ptr[kbi + 1], capacity); }
-    float kr[DP], vr[DP], dkr[DP], dvr[DP];
+    float dk_[4][DH / 16], dv_[4][DH / 16];
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-      if (key_ok) {
-        x = load4(k + (head_off + kpos) * DH + (part + 4 * g) * 4);
-        y = load4(v + (head_off + kpos) * DH + (part + 4 * g) * 4);
-      }
-      kr[4 * g] = x.x; kr[4 * g + 1] = x.y; kr[4 * g + 2] = x.z; kr[4 * g + 3] = x.w;
-      vr[4 * g] = y.x; vr[4 * g + 1] = y.y; vr[4 * g + 2] = y.z; vr[4 * g + 3] = y.w;
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) dkr[4 * g + c] = dvr[4 * g + c] = 0.f;
+      for (int c = 0; c < DH / 16; ++c) dk_[i][c] = dv_[i][c] = 0.f;
+    const bool live = (ty & ~1) * 4 < keys;    // (a warp has eight rows)
+    __syncthreads();                           // (the item before is through with the shared memory)
+    {
+      TileRegs<T, DH> x, y;
+      x.fetch(k + head_off * DH, keys, [&](int i) { return key0 + i; });
+      y.fetch(v + head_off * DH, keys, [&](int i) { return key0 + i; });
+      x.store(Ks);
+      y.store(Vs);
     }
-    for (long long t0 = list_lo; t0 < list_hi; t0 += kTile) {
-      const int nv = (int)min((long long)kTile, list_hi - t0);
+    for (long long t0 = list_lo; t0 < list_hi; t0 += kRows) {
+      const int nq = (int)min((long long)kRows, list_hi - t0);
       __syncthreads();
-      auto row_of = [&](int i) { return DENSE ? (int)(t0 + i) : q_idx[t0 + i]; };
-      load_tile<T, DH>(Qs, q + head_off * DH, nv, row_of);
-      load_tile<T, DH>(dOs, d_o + head_off * DH, nv, row_of);
-      if (threadIdx.x < kTile) {
-        float a = INFINITY, b = 0.f;
-        if (threadIdx.x < nv) {
-          long long g_ = head_off + row_of(threadIdx.x);
-          a = lse[g_]; b = Dv[g_];
+      if (t < kRows) {
+        float a = INFINITY, b = 0.f;             // (lse = +inf for rows that are none: their weights are 0)
+        int x = 0;
+        if (t < nq) {
+          x = DENSE ? (int)t0 + t : q_idx[t0 + t];
+          a = lse[head_off + x]; b = Dv[head_off + x];
         }
-        s_lse[threadIdx.x] = a; s_D[threadIdx.x] = b;
+        s_lse[t] = a; s_D[t] = b; s_row[t] = x;
       }
       __syncthreads();
-#pragma unroll 2
-      for (int i = 0; i < kTile; ++i) {
-        if (i >= nv) break;
-        float s = 0.f, dp = 0.f;
+      {
+        TileRegs<T, DH> x, y;
+        x.fetch(q + head_off * DH, nq, [&](int i) { return s_row[i]; });
+        y.fetch(d_o + head_off * DH, nq, [&](int i) { return s_row[i]; });
+        x.store(Qs);
+        y.store(dOs);
+      }
+      __syncthreads();
+      const int nq4 = (nq + 3) & ~3;
+      float p[4][4];
+      if (live) {
+        dot_tiles<DH>(Ks, Qs, ty, tx, nq, p);
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-          float4 qv = *reinterpret_cast<const float4*>(Qs + i * DH + (part + 4 * g) * 4);
-          float4 gv = *reinterpret_cast<const float4*>(dOs + i * DH + (part + 4 * g) * 4);
-          s = fmaf(qv.x, kr[4 * g], s); s = fmaf(qv.y, kr[4 * g + 1], s);
-          s = fmaf(qv.z, kr[4 * g + 2], s); s = fmaf(qv.w, kr[4 * g + 3], s);
-          dp = fmaf(gv.x, vr[4 * g], dp); dp = fmaf(gv.y, vr[4 * g + 1], dp);
-          dp = fmaf(gv.z, vr[4 * g + 2], dp); dp = fmaf(gv.w, vr[4 * g + 3], dp);
-        }
-        s = quad_sum(s); dp = quad_sum(dp);
-        const float p = expf(s * scale - s_lse[i]);      // lse = +inf for padded rows -> p = 0
-        const float ds = p * (dp - s_D[i]);
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-          float4 qv = *reinterpret_cast<const float4*>(Qs + i * DH + (part + 4 * g) * 4);
-          float4 gv = *reinterpret_cast<const float4*>(dOs + i * DH + (part + 4 * g) * 4);
-          dkr[4 * g] = fmaf(ds, qv.x, dkr[4 * g]); dkr[4 * g + 1] = fmaf(ds, qv.y, dkr[4 * g + 1]);
-          dkr[4 * g + 2] = fmaf(ds, qv.z, dkr[4 * g + 2]); dkr[4 * g + 3] = fmaf(ds, qv.w, dkr[4 * g + 3]);
-          dvr[4 * g] = fmaf(p, gv.x, dvr[4 * g]); dvr[4 * g + 1] = fmaf(p, gv.y, dvr[4 * g + 1]);
-          dvr[4 * g + 2] = fmaf(p, gv.z, dvr[4 * g + 2]); dvr[4 * g + 3] = fmaf(p, gv.w, dvr[4 * g + 3]);
+          for (int j = 0; j < 4; ++j) {
+            const int qq = tx + 16 * j;
+            p[i][j] = 4 * ty + i < keys && qq < nq ? expf(p[i][j] * scale - s_lse[qq]) : 0.f;
+            Ps[(4 * ty + i) * kLdP + qq] = p[i][j];
+          }
+        __syncwarp();                          // (a warp reads its own eight rows)
+        add_weighted<DH>(Ps, dOs, ty, tx, nq4, dv_);
+        float s[4][4];
+        dot_tiles<DH>(Vs, dOs, ty, tx, nq, s);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int qq = tx + 16 * j;
+            Ps[(4 * ty + i) * kLdP + qq] = qq < nq ? p[i][j] * (s[i][j] - s_D[qq]) : 0.f;
+          }
+        __syncwarp();
+        add_weighted<DH>(Ps, Qs, ty, tx, nq4, dk_);
+      }
+      if constexpr (!DENSE) {
+        __syncthreads();
+        if ((ty & ~1) * 4 < nq) {              // thread: queries 4 ty + i
+          float dq_[4][DH / 16];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < DH / 16; ++c) dq_[i][c] = 0.f;
+          add_weighted_t<DH>(Ps, Ks, ty, tx, keys, dq_);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            if (4 * ty + i >= nq) break;
+            float* row = dq_acc + (head_off + s_row[4 * ty + i]) * DH + 4 * tx;
+#pragma unroll
+            for (int g = 0; g < DH / 64; ++g)
+              asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(row + 64 * g), "f"(dq_[i][4 * g] * scale),
+                           "f"(dq_[i][4 * g + 1] * scale), "f"(dq_[i][4 * g + 2] * scale), "f"(dq_[i][4 * g + 3] * scale)
+                           : "memory");
+          }
         }
       }
     }
-    if (key_ok) {
 #pragma unroll
-      for (int g = 0; g < G; ++g) {
-        store4(dk + (head_off + kpos) * DH + (part + 4 * g) * 4,
-               make_float4(dkr[4 * g] * scale, dkr[4 * g + 1] * scale, dkr[4 * g + 2] * scale, dkr[4 * g + 3] * scale));
-        store4(dv + (head_off + kpos) * DH + (part + 4 * g) * 4,
-               make_float4(dvr[4 * g], dvr[4 * g + 1], dvr[4 * g + 2], dvr[4 * g + 3]));
+    for (int i = 0; i < 4; ++i) {
+      if (4 * ty + i >= keys) break;
+#pragma unroll
+      for (int g = 0; g < DH / 64; ++g) {
+        const long long at = (head_off + key0 + 4 * ty + i) * DH + 64 * g + 4 * tx;
+        store4(dk + at, make_float4(dk_[i][4 * g] * scale, dk_[i][4 * g + 1] * scale, dk_[i][4 * g + 2] * scale, dk_[i][4 * g + 3] * scale));
+        store4(dv + at, make_float4(dv_[i][4 * g], dv_[i][4 * g + 1], dv_[i][4 * g + 2], dv_[i][4 * g + 3]));
       }
     }
   }
 }
 
-// dQ: query-stationary over the same work items as the forward.  Sparse: the per-block
-// contributions of a query are added into an fp32 accumulator (atomics); dense: written directly.
-template <typename T, int DH, bool DENSE>
-__global__ void __launch_bounds__(kThreads)
+// dQ of the dense path: query-stationary, written directly.
+template <typename T, int DH>
+__global__ void __launch_bounds__(kThreads, DH == 64 ? 2 : 1)
 attn_bwd_dq_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __restrict__ v,
-                   const T* __restrict__ d_o, const float* __restrict__ lse, const float* __restrict__ Dv,
-                   const int* __restrict__ kb_ptr, const int* __restrict__ q_idx, const int* __restrict__ item_ptr,
-                   int n_kb, int S, int Nb, int sb, int BH, float scale, long long capacity,
-                   float* __restrict__ dq_acc, T* __restrict__ dq) {
+                   const T* __restrict__ d_o, const float* __restrict__ lse, const float* __restrict__ Dv, int S, int BH,
+                   float scale, T* __restrict__ dq) {
   if (!grid_begin()) return;
-  constexpr int DP = DH / 4, G = DP / 4;
-  __shared__ __align__(16) float Ks[kTile * DH];
-  __shared__ __align__(16) float Vs[kTile * DH];
-  const int r = threadIdx.x >> 2, part = threadIdx.x & 3;
-  const int tiles_per_head = (S + kRows - 1) / kRows;
-  const int n_items = DENSE ? BH * tiles_per_head : item_ptr[n_kb];
+  extern __shared__ __align__(16) float simt_smem[];
+  float* Qs = simt_smem;
+  float* dOs = Qs + kTileFloats<DH>;
+  float* Ks = dOs + kTileFloats<DH>;
+  float* Vs = Ks + kTileFloats<DH>;
+  float* Ps = Vs + kTileFloats<DH>;            // [query][key]: dS
+  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+  const int tiles_per_head = (S + kRows - 1) / kRows, n_items = BH * tiles_per_head;
   for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-    Item it;
-    int qpos = -1;
-    if (DENSE) {
-      it.bh = item / tiles_per_head;
-      int row = (item - it.bh * tiles_per_head) * kRows + r;
-      it.key_begin = 0; it.key_end = S;
-      if (row < S) qpos = row;
-    } else {
-      it = decode_sparse(item, item_ptr, n_kb, kb_ptr, Nb, sb, kRows, capacity);
-      if (it.list_lo + r < it.list_hi) qpos = q_idx[it.list_lo + r];
-    }
-    const long long head_off = (long long)it.bh * S;
-    const T* kh = k + head_off * DH;
-    const T* vh = v + head_off * DH;
-    float qr[DP], gr[DP], acc[DP];
-    float row_lse = INFINITY, row_D = 0.f;
-    if (qpos >= 0) { row_lse = lse[head_off + qpos]; row_D = Dv[head_off + qpos]; }
+    const int bh = item / tiles_per_head, row0 = (item - bh * tiles_per_head) * kRows, rows = min(kRows, S - row0);
+    const long long head_off = (long long)bh * S;
+    float row_lse[4], row_D[4], acc[4][DH / 16];
 #pragma unroll
-    for (int g = 0; g < G; ++g) {
-      float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-      if (qpos >= 0) {
-        x = load4(q + (head_off + qpos) * DH + (part + 4 * g) * 4);
-        y = load4(d_o + (head_off + qpos) * DH + (part + 4 * g) * 4);
-      }
-      qr[4 * g] = x.x; qr[4 * g + 1] = x.y; qr[4 * g + 2] = x.z; qr[4 * g + 3] = x.w;
-      gr[4 * g] = y.x; gr[4 * g + 1] = y.y; gr[4 * g + 2] = y.z; gr[4 * g + 3] = y.w;
-      acc[4 * g] = acc[4 * g + 1] = acc[4 * g + 2] = acc[4 * g + 3] = 0.f;
+    for (int i = 0; i < 4; ++i) {
+      const bool ok = 4 * ty + i < rows;
+      row_lse[i] = ok ? lse[head_off + row0 + 4 * ty + i] : INFINITY;
+      row_D[i] = ok ? Dv[head_off + row0 + 4 * ty + i] : 0.f;
+#pragma unroll
+      for (int c = 0; c < DH / 16; ++c) acc[i][c] = 0.f;
     }
-    for (int t0 = it.key_begin; t0 < it.key_end; t0 += kTile) {
-      const int nv = min(kTile, it.key_end - t0);
+    __syncthreads();                           // (the item before is through with the shared memory)
+    {
+      TileRegs<T, DH> x, y;
+      x.fetch(q + head_off * DH, rows, [&](int i) { return row0 + i; });
+      y.fetch(d_o + head_off * DH, rows, [&](int i) { return row0 + i; });
+      x.store(Qs);
+      y.store(dOs);
+    }
+    const bool live = (ty & ~1) * 4 < rows;    // (a warp has eight rows)
+    for (int t0 = 0; t0 < S; t0 += kRows) {
+      const int nv = min(kRows, S - t0);
+      {
+        TileRegs<T, DH> x, y;
+        x.fetch(k + head_off * DH, nv, [&](int i) { return t0 + i; });
+        y.fetch(v + head_off * DH, nv, [&](int i) { return t0 + i; });
+        __syncthreads();
+        x.store(Ks);
+        y.store(Vs);
+      }
       __syncthreads();
-      load_tile<T, DH>(Ks, kh, nv, [&](int i) { return t0 + i; });
-      load_tile<T, DH>(Vs, vh, nv, [&](int i) { return t0 + i; });
-      __syncthreads();
-#pragma unroll 2
-      for (int i = 0; i < kTile; ++i) {
-        if (i >= nv) break;
-        float s = 0.f, dp = 0.f;
+      if (live) {
+        float p[4][4], s[4][4];
+        dot_tiles<DH>(Qs, Ks, ty, tx, nv, p);
+        dot_tiles<DH>(dOs, Vs, ty, tx, nv, s);
+        __syncwarp();
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-          float4 kv = *reinterpret_cast<const float4*>(Ks + i * DH + (part + 4 * g) * 4);
-          float4 vv = *reinterpret_cast<const float4*>(Vs + i * DH + (part + 4 * g) * 4);
-          s = fmaf(qr[4 * g], kv.x, s); s = fmaf(qr[4 * g + 1], kv.y, s);
-          s = fmaf(qr[4 * g + 2], kv.z, s); s = fmaf(qr[4 * g + 3], kv.w, s);
-          dp = fmaf(gr[4 * g], vv.x, dp); dp = fmaf(gr[4 * g + 1], vv.y, dp);
-          dp = fmaf(gr[4 * g + 2], vv.z, dp); dp = fmaf(gr[4 * g + 3], vv.w, dp);
-        }
-        s = quad_sum(s); dp = quad_sum(dp);
-        const float p = expf(s * scale - row_lse);
-        const float ds = p * (dp - row_D);
+        for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int g = 0; g < G; ++g) {
-          float4 kv = *reinterpret_cast<const float4*>(Ks + i * DH + (part + 4 * g) * 4);
-          acc[4 * g] = fmaf(ds, kv.x, acc[4 * g]); acc[4 * g + 1] = fmaf(ds, kv.y, acc[4 * g + 1]);
-          acc[4 * g + 2] = fmaf(ds, kv.z, acc[4 * g + 2]); acc[4 * g + 3] = fmaf(ds, kv.w, acc[4 * g + 3]);
-        }
+          for (int j = 0; j < 4; ++j) {
+            const int key = tx + 16 * j;
+            Ps[(4 * ty + i) * kLdP + key] = key < nv ? expf(p[i][j] * scale - row_lse[i]) * (s[i][j] - row_D[i]) : 0.f;
+          }
+        __syncwarp();                          // (a warp reads its own eight rows)
+        add_weighted<DH>(Ps, Ks, ty, tx, (nv + 3) & ~3, acc);
       }
     }
-    if (qpos >= 0) {
-      const long long G_ = head_off + qpos;
 #pragma unroll
-      for (int g = 0; g < G; ++g) {
-        if (DENSE) {
-          store4(dq + G_ * DH + (part + 4 * g) * 4,
-                 make_float4(acc[4 * g] * scale, acc[4 * g + 1] * scale, acc[4 * g + 2] * scale, acc[4 * g + 3] * scale));
-        } else {
+    for (int i = 0; i < 4; ++i) {
+      if (4 * ty + i >= rows) break;
 #pragma unroll
-          for (int c = 0; c < 4; ++c) atomicAdd(dq_acc + G_ * DH + (part + 4 * g) * 4 + c, acc[4 * g + c] * scale);
-        }
-      }
+      for (int g = 0; g < DH / 64; ++g)
+        store4(dq + (head_off + row0 + 4 * ty + i) * DH + 64 * g + 4 * tx,
+               make_float4(acc[i][4 * g] * scale, acc[i][4 * g + 1] * scale, acc[i][4 * g + 2] * scale, acc[i][4 * g + 3] * scale));
     }
   }
 }
