@@ -1189,17 +1189,17 @@ template <typename T>
 __device__ __noinline__ T pool_exclusive(T x, T* s_warp) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   T inc = x;
-#pragma unroll 1
+#pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const T v = __shfl_up_sync(0xffffffffu, inc, o);
     if (lane >= o) inc += v;
   }
   if (lane == 31) s_warp[warp] = inc;
   __syncthreads();
-  T before = lane < warp ? s_warp[lane] : T(0);
-#pragma unroll 1
-  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
-  return before + (inc - x);
+  T before = lane < warp ? s_warp[lane] : T(0);      // (at most sixteen warps)
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o, 16);
+  return __shfl_sync(0xffffffffu, before, 0) + (inc - x);
 }
 
 // The search for a head's cutoff among the scores src[0 .. n) of every CTA of a cluster, which lie in [lo, lo + span] (shared or
@@ -1261,18 +1261,25 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
     s_own[b * T + t] += weight(s);
   });
   __syncthreads();
-#pragma unroll 1
-  for (int b = warp; b < kPoolBins0; b += T / 32) {
-    float w = 0.f;
+  {
+    constexpr int kMine = kPoolBins0 / (T / 32);       // bins of a warp, worked out side by side
+    double x[kMine];
 #pragma unroll
-    for (int r = 0; r < T / 32; ++r) {
-      const float x = s_own[b * T + 32 * r + lane];
-      if (x > 0.f) w += x;
+    for (int m = 0; m < kMine; ++m) {
+      const float* own = s_own + (warp + m * (T / 32)) * T + lane;
+      float w = 0.f;
+#pragma unroll
+      for (int r = 0; r < T / 32; ++r)
+        if (own[32 * r] > 0.f) w += own[32 * r];
+      x[m] = (double)w;
     }
-    double x = (double)w;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane < C) cluster.map_shared_rank(s_w0[rank], lane)[b] = x;
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int m = 0; m < kMine; ++m) x[m] += __shfl_xor_sync(0xffffffffu, x[m], o);
+    if (lane < C)
+#pragma unroll
+      for (int m = 0; m < kMine; ++m) cluster.map_shared_rank(s_w0[rank], lane)[warp + m * (T / 32)] = x[m];
   }
   __syncthreads();
 #pragma unroll
@@ -1448,8 +1455,9 @@ select_pool_kernel(const PoolArgs a) {
   auto all_there = []() { asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); };
   constexpr int kFront = SRC == kPoolScores ? kPoolFront * T : 0;
   extern __shared__ __align__(16) unsigned char pool_smem[];
-  __shared__ int s_pairs[kPoolCtas];
+  __shared__ int s_pairs[kPoolCtas], s_mine;      // pairs of the cluster's CTAs
   __shared__ int s_sum[32];
+  if (threadIdx.x == 0) s_mine = 0;
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), bh = (int)blockIdx.x / C;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int Nb = a.Nb, mw = a.mw, TW = a.QSEG >> 5;
@@ -1581,9 +1589,9 @@ select_pool_kernel(const PoolArgs a) {
     for (int c = 0; c < C; ++c) cluster.map_shared_rank(s_tot + rank * Nb, c)[j] = sum;
     pairs += sum;
   }
-  const int before = pool_exclusive(pairs, s_sum);
-  if (t == T - 1)
-    for (int c = 0; c < C; ++c) cluster.map_shared_rank(s_pairs, c)[rank] = before + pairs;
+  if (pairs) atomicAdd(&s_mine, pairs);
+  __syncthreads();
+  if (t < C) cluster.map_shared_rank(s_pairs, t)[rank] = s_mine;
   meet();      // (what is read from here on is the CTA's own: it may leave when it is done)
   const int per = (Nb + T - 1) / T, j0 = min(t * per, Nb), j1 = min(j0 + per, Nb);
   int run_all = 0;
