@@ -173,8 +173,12 @@ def _ws_args(ws):
     return _ptr(ws), ws.numel() * ws.element_size()
 
 
+_I64x3 = ctypes.c_int64 * 3
+_MANY = {n: (ctypes.c_int64 * (3 * n), ctypes.c_void_p * n) for n in range(1, 5)}     # argument arrays of partition_many
+
+
 def vmoba_partition(shape, inverse, src, dst, raster_strides_bsh, perm=None, inv_perm=None, stream=None):
-    strides = (ctypes.c_int64 * 3)(*[int(x) for x in raster_strides_bsh])
+    strides = _I64x3(*map(int, raster_strides_bsh))
     _check(lib().vmoba_partition(ctypes.byref(shape), int(inverse), _ptr(src), _ptr(dst), strides, _ptr(perm),
                                  _ptr(inv_perm), _stream(stream)), "vmoba_partition")
 
@@ -182,9 +186,10 @@ def vmoba_partition(shape, inverse, src, dst, raster_strides_bsh, perm=None, inv
 def vmoba_partition_many(shape, inverse, srcs, dsts, raster_strides_bsh, perm=None, inv_perm=None, stream=None):
     """vmoba_partition of up to four tensors in one launch; raster_strides_bsh: one (batch, token, head) triple each."""
     n = len(srcs)
-    strides = (ctypes.c_int64 * (3 * n))(*[x for t in raster_strides_bsh for x in t])
-    src = (ctypes.c_void_p * n)(*[t.data_ptr() for t in srcs])
-    dst = (ctypes.c_void_p * n)(*[t.data_ptr() for t in dsts])
+    i64s, ptrs = _MANY.get(n) or (ctypes.c_int64 * (3 * n), ctypes.c_void_p * n)
+    strides = i64s(*[x for t in raster_strides_bsh for x in t])
+    src = ptrs(*[t.data_ptr() for t in srcs])
+    dst = ptrs(*[t.data_ptr() for t in dsts])
     _check(lib().vmoba_partition_many(ctypes.byref(shape), inverse, n, src, dst, strides, _ptr(perm), _ptr(inv_perm),
                                       _stream(stream)), "vmoba_partition_many")
 
@@ -267,7 +272,7 @@ def vmoba_attn_bwd(shape, q_bm, k_bm, v_bm, o_bm, o_resid, lse, do_bm, kb_ptr, q
 def vmoba_attn_fwd_raster(shape, q_bm, k_bm, v_bm, kb_ptr, q_idx, q_ptr, q_pairs, capacity, o, o_strides_bsh, perm,
                           o_resid_bm, lse, dev_status, ws, stream=None):
     p, n = _ws_args(ws)
-    os_ = (ctypes.c_int64 * 3)(*[int(x) for x in o_strides_bsh])
+    os_ = _I64x3(*map(int, o_strides_bsh))
     _check(lib().vmoba_attn_fwd_raster(ctypes.byref(shape), _ptr(q_bm), _ptr(k_bm), _ptr(v_bm), _ptr(kb_ptr), _ptr(q_idx),
                                        _ptr(q_ptr), _ptr(q_pairs), int(capacity), _ptr(o), os_, _ptr(perm),
                                        _ptr(o_resid_bm), _ptr(lse), _ptr(dev_status), p, n, _stream(stream)),
@@ -278,9 +283,9 @@ def vmoba_attn_bwd_raster(shape, q_bm, k_bm, v_bm, o, o_strides_bsh, o_resid, ls
                           q_ptr, capacity, dq, dk, dv, grad_strides_bsh, perm, dev_status, ws, stream=None, do_bm=None):
     """do_bm: with a raster-order d_o, a block-major tensor that takes a copy of it on the way."""
     p, n = _ws_args(ws)
-    dos = None if do_strides_bsh is None else (ctypes.c_int64 * 3)(*[int(x) for x in do_strides_bsh])
-    os_ = None if o_strides_bsh is None else (ctypes.c_int64 * 3)(*[int(x) for x in o_strides_bsh])
-    gs = (ctypes.c_int64 * 3)(*[int(x) for x in grad_strides_bsh])
+    dos = None if do_strides_bsh is None else _I64x3(*map(int, do_strides_bsh))
+    os_ = None if o_strides_bsh is None else _I64x3(*map(int, o_strides_bsh))
+    gs = _I64x3(*map(int, grad_strides_bsh))
     if do_bm is not None:
         _check(lib().vmoba_attn_bwd_raster_do(ctypes.byref(shape), _ptr(q_bm), _ptr(k_bm), _ptr(v_bm), _ptr(o), os_,
                                               _ptr(o_resid), _ptr(lse), _ptr(d_o), dos, _ptr(do_bm), _ptr(kb_ptr),

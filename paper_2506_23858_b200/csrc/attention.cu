@@ -81,7 +81,7 @@ static int simt_sparse_fwd(const Dims& D, const void* q, const void* k, const vo
   const long long n_kb = (long long)D.BH * D.Nb;
   launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
   long long max_items = cap / simt::kRows + n_kb;
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_fwd_kernel<T, DH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kFwdSmem<DH>));
+  VMOBA_CUDA_OK(allow_smem(simt::attn_fwd_kernel<T, DH, false>, simt::kFwdSmem<DH>));
   launch_kernel(early_simt(D, (double)cap * D.sb), simt::attn_fwd_kernel<T, DH, false>, grid_for(max_items, 8), simt::kThreads, simt::kFwdSmem<DH>, st, (const T*)q,
                 (const T*)k, (const T*)v, kb_ptr, q_idx, q_ptr, w.item_ptr, (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale,
                 (T*)o, (T*)o_resid, lse, w.part_o, w.part_lse, cap);
@@ -126,7 +126,7 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
   launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
                 (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), acc, nullptr, (T*)nullptr, nullptr, 0);
   long long tiles = (D.sb + simt::kRows - 1) / simt::kRows;
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_bwd_dkdv_kernel<T, DH, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kBwdSmem<DH>));
+  VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dkdv_kernel<T, DH, false>, simt::kBwdSmem<DH>));
   launch_kernel(early_simt(D, (double)cap * D.sb), simt::attn_bwd_dkdv_kernel<T, DH, false>, grid_for(n_kb * tiles, 4), simt::kThreads,
                 simt::kBwdSmem<DH>, st, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb,
                 D.BH, D.scale, cap, (T*)dk, (T*)dv, acc);
@@ -152,7 +152,7 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
     int rc = tc_dense_fwd(D, q, k, v, o, d_o ? w.o_resid : nullptr, lse, status, st);
     if (rc) return rc;
   } else {
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_fwd_kernel<T, DH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kFwdSmem<DH>));
+    VMOBA_CUDA_OK(allow_smem(simt::attn_fwd_kernel<T, DH, true>, simt::kFwdSmem<DH>));
     launch_kernel(early, simt::attn_fwd_kernel<T, DH, true>, grid_for(D.BH * tiles, 8), simt::kThreads, simt::kFwdSmem<DH>, st, (const T*)q,
                   (const T*)k, (const T*)v, nullptr, nullptr, nullptr, nullptr, 0, D.S, 1, D.S, D.BH, D.scale, (T*)o,
                   d_o ? (T*)w.o_resid : nullptr, lse, nullptr, nullptr, 0);
@@ -172,8 +172,8 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
       VMOBA_LAUNCH_OK(1);
       return VMOBA_OK;
     }
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_bwd_dkdv_kernel<T, DH, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kBwdSmem<DH>));
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(simt::attn_bwd_dq_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, simt::kBwdSmem<DH>));
+    VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dkdv_kernel<T, DH, true>, simt::kBwdSmem<DH>));
+    VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dq_kernel<T, DH>, simt::kBwdSmem<DH>));
     launch_kernel(early, simt::attn_bwd_dkdv_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, simt::kBwdSmem<DH>, st,
                   (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, D.S, 1, D.S,
                   D.BH, D.scale, 0, (T*)dk, (T*)dv, nullptr);

@@ -791,7 +791,7 @@ static int launch(const Dims& D, const void* k, const void* v, KvParams& kp, cud
   if (items > (long long)INT32_MAX - 4096) return VMOBA_ERR_SHAPE;
   const int grid = DENSE ? (int)items : (int)std::max<long long>(1, std::min<long long>(items, sm_count()));
   auto kernel = kp.prof ? attn_bwd_fused_kernel<DENSE, MULTI, true> : attn_bwd_fused_kernel<DENSE, MULTI, false>;
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+  VMOBA_CUDA_OK(allow_smem(kernel, (int)SMEM_BYTES));
   launch_kernel(early_rows(D), kernel, grid, THREADS, SMEM_BYTES, st, tmK, tmV, tmQ, tmO, kp);
   VMOBA_LAUNCH_OK(1);
   return VMOBA_OK;

@@ -589,7 +589,7 @@ static int launch_wide(const Dims& D, const void* q, const void* k, const void* 
       !sm100::make_tmap_bf16_heads(&tmQ, q, D.BH, D.S, DH, BM))      // dense: consecutive rows; sparse: not used
     return VMOBA_ERR_CUDA;
   auto kernel = p.prof ? attn_fwd_wide_kernel<DENSE, RASTER, true> : attn_fwd_wide_kernel<DENSE, RASTER, false>;
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+  VMOBA_CUDA_OK(allow_smem(kernel, (int)SMEM_BYTES));
   launch_kernel(kernel, grid, THREADS, SMEM_BYTES, st, tmK, tmV, tmQ, p);
   VMOBA_LAUNCH_OK(1);
   return VMOBA_OK;

@@ -579,7 +579,7 @@ int tc_sparse_fwd_narrow(const Dims& D, const void* q, const void* k, const void
   p.o_map = o_map;
   const long long items = std::max<long long>(1, std::min<long long>(cap / BM + n_kb, 2LL * sm_count()));
   auto kernel = o_map.perm ? attn_fwd_narrow_kernel<true> : attn_fwd_narrow_kernel<false>;
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES));
+  VMOBA_CUDA_OK(allow_smem(kernel, (int)SMEM_BYTES));
   launch_kernel(kernel, (int)items, THREADS, SMEM_BYTES, st, tmK, tmV, p);
   simt::merge_batched(D, q_ptr, q_pairs, p.part_o, part_lse, part_scale, cap, o, o_resid, lse, o_map, st);
   VMOBA_LAUNCH_OK(2);

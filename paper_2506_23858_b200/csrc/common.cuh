@@ -100,6 +100,21 @@ inline int sm_count() {
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Lets a kernel have so much dynamic shared memory.  The runtime is asked once per kernel, device and thread: a layer call of
+// ten launches asked six times.
+template <typename... P>
+inline cudaError_t allow_smem(void (*kernel)(P...), int bytes) {
+  struct Seen { void (*kernel)(P...); int dev, bytes; };
+  thread_local Seen seen[16] = {};
+  int dev = 0;
+  if (cudaError_t e = cudaGetDevice(&dev)) return e;
+  Seen& s = seen[(reinterpret_cast<uintptr_t>(kernel) >> 4) % 16];
+  if (s.kernel == kernel && s.dev == dev && s.bytes >= bytes) return cudaSuccess;
+  if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) return e;
+  s = {kernel, dev, bytes};
+  return cudaSuccess;
+}
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // The debug build (-DVMOBA_DEBUG, lib/libvmoba_debug.so) stands in for a memory checker: every index read from a

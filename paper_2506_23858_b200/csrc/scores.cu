@@ -190,7 +190,7 @@ static int run_scores(const Dims& D, const void* q, const void* k, float* cent, 
   VMOBA_LAUNCH_OK(1);
   if (tc) return scores_tc(D, q, parts, scores, range, status, st);
   size_t smem = 2 * DH * (64 + 4) * sizeof(float);
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(scores_kernel<T, DH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  VMOBA_CUDA_OK(allow_smem(scores_kernel<T, DH>, (int)smem));
   dim3 grid((D.S + 63) / 64, 1, D.BH);
   launch_kernel(scores_kernel<T, DH>, grid, 256, smem, st, static_cast<const T*>(q), cent, scores, D.S, D.Nb, range);
   VMOBA_LAUNCH_OK(1);

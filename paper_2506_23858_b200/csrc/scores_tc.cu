@@ -321,7 +321,7 @@ int scores_tc(const Dims& D, const void* q_bm, const CentroidParts& cent, float*
   while (smem_bytes(p.nq, rows_pass) > SMEM_MAX) --p.nq;      // (two tiles fit beside 160 rows)
   p.range = range;
   p.status = status;
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(scores_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX));
+  VMOBA_CUDA_OK(allow_smem(scores_tc_kernel, SMEM_MAX));
   const long long items = (long long)D.BH * n_pass * ((D.S + BM - 1) / BM);
   launch_kernel(scores_tc_kernel, (int)std::max<long long>(1, std::min<long long>(items, sm_count())), THREADS,
                 smem_bytes(p.nq, rows_pass), st, tmQ, tmB, tmS, p);

@@ -2069,7 +2069,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     a.mask_bits = mask_bits; a.tmask = w.tmask; a.seg_cnt = w.seg_cnt; a.seg_qoff = w.seg_qoff; a.kb_excl = w.kb_total;
     a.k_per_head = k_per_head; a.cutoff_per_head = cutoff_per_head;
     auto kernel = w.pool.T == 256 ? select_pool_kernel<decltype(tag)::value, 256> : select_pool_kernel<decltype(tag)::value, 512>;
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pool_smem));
+    VMOBA_CUDA_OK(allow_smem(kernel, (int)pool_smem));
     launch_cluster(true, w.pool.C, kernel, (unsigned)(D.BH * w.pool.C), w.pool.T, pool_smem, st, a);
     VMOBA_LAUNCH_OK(1);
     return VMOBA_OK;
@@ -2131,7 +2131,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
       if ((rc = pool_launch(VMOBA_POOL(kPoolMask), nullptr, 0, -1.0))) return rc;
     } else {
     launch_kernel(local_cutoff_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, cutoff_per_head, D.BH);
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(mark_from_mask_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VMOBA_CUDA_OK(allow_smem(mark_from_mask_kernel, (int)smem));
     launch_kernel(mark_from_mask_kernel, sgrid, kSegThreads, smem, st, mask_bits, D.S, D.Nb, D.mask_words, QSEG, nseg,
                   w.seg_cnt, w.seg_total, w.tmask);
     VMOBA_LAUNCH_OK(2);
@@ -2164,10 +2164,10 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
                      count_target, (float)((double)w.ccap / (double)P));
       const int gx1 = (int)std::min<long long>(std::max<long long>(per_head / 16, 1), std::max(1, sm_count() * 3 / D.BH));
       constexpr int T = 512, smem1 = kPoolFront * T, smem_stage = kWindowThreads / 32 * kWindowStage * (int)sizeof(float);
-      VMOBA_CUDA_OK(cudaFuncSetAttribute(window_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_stage));
+      VMOBA_CUDA_OK(allow_smem(window_pass_kernel, smem_stage));
       launch_kernel(early_rows(D), window_pass_kernel, dim3(gx1, D.BH), kWindowThreads, smem_stage, st, scores, P, w.state, sigma, unit_w,
                     w.cand, w.ccap);
-      VMOBA_CUDA_OK(cudaFuncSetAttribute(window_search_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1));
+      VMOBA_CUDA_OK(allow_smem(window_search_kernel<T>, smem1));
       launch_cluster(true, C, window_search_kernel<T>, (unsigned)(D.BH * C), T, smem1, st, scores, P, w.state, sigma, unit_w, tau,
                      count_target, w.cand, w.ccap, cutoff_per_head);
       VMOBA_LAUNCH_OK(3);
@@ -2182,7 +2182,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     }
     {
       constexpr int smem0 = kBins0 * kRep * (int)sizeof(float);
-      VMOBA_CUDA_OK(cudaFuncSetAttribute(hist0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem0));
+      VMOBA_CUDA_OK(allow_smem(hist0_kernel, smem0));
       // three 512-thread CTAs per SM hold their replicated bins side by side
       int gx0 = (int)std::min<long long>(std::max<long long>(per_head / 16, 1), std::max(1, sm_count() * 3 / D.BH));
       launch_kernel(early_rows(D), hist0_kernel, dim3(gx0, D.BH), 512, smem0, st, scores, P, w.state, sigma, unit_w,
@@ -2200,7 +2200,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
                   w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
     VMOBA_LAUNCH_OK(7);
     }
-    VMOBA_CUDA_OK(cudaFuncSetAttribute(mark_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    VMOBA_CUDA_OK(allow_smem(mark_kernel, (int)smem));
     launch_kernel(mark_kernel, sgrid, kSegThreads, smem, st, scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg,
                   own_sb, mask_bits, w.seg_cnt, w.seg_total, w.tmask);
     VMOBA_LAUNCH_OK(1);
@@ -2209,7 +2209,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
 #undef VMOBA_POOL
 
   const size_t smem_fill = ((size_t)QSEG * D.mask_words + 2 * (size_t)D.Nb * (QSEG >> 5) + 2 * (size_t)D.Nb + 1 + 2 * kStage) * 4;
-  VMOBA_CUDA_OK(cudaFuncSetAttribute(fill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_fill));
+  VMOBA_CUDA_OK(allow_smem(fill_kernel, (int)smem_fill));
   long long nkb = (long long)D.BH * D.Nb;
   if (!pool) {
     launch_kernel(seg_prefix_kernel, (unsigned)(D.BH * ((D.Nb + 31) / 32)), 32 * std::min(32, (nseg + 7) / 8), 0, st,

@@ -66,8 +66,9 @@ class VmobaLayer:
     @staticmethod
     def raster_strides(x):
         """Element strides (batch, token, head) of a [B, S, heads, d] tensor."""
-        assert x.stride(3) == 1
-        return (x.stride(0), x.stride(1), x.stride(2))
+        s = x.stride()
+        assert s[3] == 1
+        return s[:3]
 
     def partition(self, raster, bm, inverse=False, perm=None, inv_perm=None):
         src, dst = (bm, raster) if inverse else (raster, bm)
