@@ -526,24 +526,26 @@ offsets_kernel(const int* __restrict__ kb_total, int* __restrict__ kb_ptr, long 
 // set bits.  The position of a pair in q_idx is that of its block's first selecting query in the segment plus the
 // selecting queries below in the block's column of the segment (column words of the mark kernel, prefixed per word).  Both
 // lists of a segment are put together in shared memory, by block and by query, and written out in runs; a segment with
-// more than kStage pairs writes its entries one by one.  8.2 million pairs, nine per query: 119 us (273 with a warp per key
-// block that wrote q_pairs entry by entry); 12.6 million, 32 per query, beyond the stage: 154 (173).
+// more pairs than the stage holds writes its entries one by one.  Bound by the latency of a CTA's steps, so that the shared
+// memory is kept small: with what counts a segment's queries in 16 bits, and a stage of the rule's size where that is known, three
+// CTAs share an SM.  8.2 million pairs, nine per query: 106 us (137 with 32 bits and two CTAs, 273 with a warp per key block that
+// wrote q_pairs entry by entry); 0.33 million 23 (31); 12.6 million, 32 per query, beyond the stage: 155.
 constexpr int kStage = 6144;
 __global__ void __launch_bounds__(kSegThreads)
 fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__ tmask, int S, int Nb, int mw, int QSEG,
             int nseg, int* __restrict__ kb_ptr, const int* __restrict__ seg_cnt, const int* __restrict__ seg_qoff,
             int* __restrict__ q_idx, int* __restrict__ q_ptr, int* __restrict__ q_pairs, long long capacity,
-            const int* __restrict__ kb_excl, const int64_t* __restrict__ k_per_head, int32_t* __restrict__ dev_status) {
+            const int* __restrict__ kb_excl, const int64_t* __restrict__ k_per_head, int32_t* __restrict__ dev_status, int stage) {
   if (!grid_begin()) return;
   extern __shared__ uint32_t sm[];
   const int TW = QSEG >> 5;
   uint32_t* s_mask = sm;                                    // [QSEG][mw]
   uint32_t* s_tm = s_mask + QSEG * mw;                      // [TW][Nb] column words
-  int* s_pre = reinterpret_cast<int*>(s_tm + Nb * TW);      // [TW][Nb] entries of the segment in front of that word, by block
-  int* s_off = s_pre + Nb * TW;                             // [Nb + 1] entries in front of the block
+  int* s_off = reinterpret_cast<int*>(s_tm + Nb * TW);      // [Nb + 1] entries in front of the block
   int* s_pos = s_off + Nb + 1;                              // [Nb] position of the segment's first entry of the block in q_idx
-  int* s_idx = s_pos + Nb;                                  // [kStage] q_idx entries by block
-  int* s_pair = s_idx + kStage;                             // [kStage] q_pairs entries by query
+  int* s_pair = s_pos + Nb;                                 // [stage] q_pairs entries by query
+  uint16_t* s_idx = reinterpret_cast<uint16_t*>(s_pair + stage);      // [stage] queries of the segment, by block
+  uint16_t* s_pre = s_idx + stage;                          // [TW][Nb] the block's entries in front of that word
   __shared__ int s_warp[kSegThreads / 32];
   const int seg = blockIdx.x, bh = blockIdx.y;
   const int q0 = seg * QSEG;
@@ -605,7 +607,7 @@ fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__
     int run = scan(c);
     for (int j = j0; j < j1; ++j) {
       s_off[j] = run;
-      for (int w = 0; w < TW; ++w) { s_pre[w * Nb + j] = run; run += __popc(s_tm[w * Nb + j]); }
+      for (int w = 0; w < TW; ++w) { s_pre[w * Nb + j] = (uint16_t)(run - s_off[j]); run += __popc(s_tm[w * Nb + j]); }
     }
     if (j1 == Nb && j0 < j1) s_off[Nb] = run;
   }
@@ -615,7 +617,7 @@ fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__
   int mine = scan(cnt);                              // this query's next entry of q_pairs, counted from the segment's first
   const int total = s_off[Nb];
   if (t < nq) q_ptr[(long long)bh * S + q0 + t] = (int)min(qbase + mine, (long long)INT32_MAX);
-  const bool staged = total <= kStage;
+  const bool staged = total <= stage;
   if (t < nq) {
     const uint32_t lt_mask = (1u << lane) - 1u;
     for (int w = 0; w < mw; ++w) {
@@ -623,11 +625,11 @@ fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__
       while (word) {
         const int j = 32 * w + __ffs(word) - 1;
         word &= word - 1;
-        const int e = s_pre[warp * Nb + j] + __popc(s_tm[warp * Nb + j] & lt_mask);
-        const long long pos = (long long)s_pos[j] + (e - s_off[j]);
+        const int in_block = s_pre[warp * Nb + j] + __popc(s_tm[warp * Nb + j] & lt_mask);
+        const long long pos = (long long)s_pos[j] + in_block;
         const int entry = (int)min(pos, (long long)INT32_MAX);
         if (staged) {
-          s_idx[e] = q0 + t;
+          s_idx[s_off[j] + in_block] = (uint16_t)t;
           s_pair[mine] = entry;
         } else if (pos < capacity) {
           q_idx[pos] = q0 + t;
@@ -646,7 +648,7 @@ fill_kernel(const uint32_t* __restrict__ mask_bits, const uint32_t* __restrict__
     const int o0 = s_off[j], n = s_off[j + 1] - o0;
     const long long pos = s_pos[j];
     for (int i = t & 7; i < n; i += 8)
-      if (pos + i < capacity) q_idx[pos + i] = s_idx[o0 + i];
+      if (pos + i < capacity) q_idx[pos + i] = q0 + s_idx[o0 + i];
   }
 }
 
@@ -713,7 +715,8 @@ __device__ __forceinline__ float warp_min(float x) {
 // score itself, whose ties are then taken in block order.  The first probe is the threshold of the row before (rows
 // of a run are neighbours of one head), the next ones step away from it by doubling amounts, and once two probes
 // enclose the threshold the interval is halved.  A step is a compare and an add per word and one warp reduction: the
-// kernel is bound by instruction issue.  280 blocks, k = 9, 907,200 rows (1.0 GB of scores): 0.43 ms; plain halving
+// kernel is bound by instruction issue.  280 blocks, k = 9, 907,200 rows (1.0 GB of scores): 0.38 ms (0.44 with the row's smallest
+// score looked for as well and ten words instead of nine); plain halving
 // from the row's minimum and maximum 0.80 ms, a search over the 32 key bits in an instantiation of 16 words 3.08 ms.
 template <int MW>
 __global__ void __launch_bounds__(256)
@@ -751,17 +754,24 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
   float t_prev = NAN;                   // threshold of the row before
   for (long long row = row_begin; row < row_end; ++row) {
     float x[MW];
-    float mx = -INFINITY, mn = INFINITY;
+    float mx = -INFINITY;
 #pragma unroll
     for (int i = 0; i < MW; ++i) {
       x[i] = next[i];
       mx = max_nan(mx, x[i]);
-      if (lane + 32 * i < Nb) mn = fminf(mn, x[i]);
     }
     src += Nb;
     if (row + 1 < row_end) load_row(src);
+    // the row's smallest score, which only a search that does not start from the row before needs
+    auto smallest = [&]() {
+      float mn = INFINITY;
+#pragma unroll
+      for (int i = 0; i < MW; ++i)
+        if (lane + 32 * i < Nb) mn = fminf(mn, x[i]);
+      return warp_min(mn);
+    };
     // invariant: at least k scores reach lo, fewer than k reach hi (or lo == hi)
-    float lo = warp_min(mn), hi = warp_max_nan(mx);
+    float hi = warp_max_nan(mx), lo = -INFINITY;
     const bool has_nan = hi != hi;
     bool exact = false;                 // exactly k scores reach lo
     if (k < Nb && !has_nan) {
@@ -772,12 +782,15 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
         for (int i = 0; i < MW; ++i) n += x[i] >= c ? 1 : 0;
         return __reduce_add_sync(0xffffffffu, n);
       };
-      float mid = t_prev, step = 0.015625f * (hi - lo);
-      bool below = false, above = false;
-      if (!(mid > lo && mid < hi) && !split_interval(lo, hi, mid)) {
-        lo = hi;                        // two neighbouring values at most: is the larger one the k-th?
-        if (count_ge(hi) < k) lo = warp_min(mn);
-      } else {
+      float mid = t_prev, step = (k > 4 ? 0.0625f : 0.125f) * (hi - mid);
+      bool below = false, above = false, go = mid < hi;
+      if (!go) {
+        lo = smallest();
+        step = 0.015625f * (hi - lo);
+        go = split_interval(lo, hi, mid);
+        if (!go && count_ge(hi) >= k) lo = hi;      // two neighbouring values at most: is the larger one the k-th?
+      }
+      if (go) {
         for (;;) {
           const int n = count_ge(mid);
           if (n >= k) { lo = mid; below = true; } else { hi = mid; above = true; }
@@ -2111,9 +2124,12 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
       else if (mw <= 4) topk_words(VMOBA_INT(4));
       else if (mw <= 5) topk_words(VMOBA_INT(5));
       else if (mw <= 6) topk_words(VMOBA_INT(6));
+      else if (mw <= 7) topk_words(VMOBA_INT(7));
       else if (mw <= 8) topk_words(VMOBA_INT(8));
+      else if (mw <= 9) topk_words(VMOBA_INT(9));
       else if (mw <= 10) topk_words(VMOBA_INT(10));
       else if (mw <= 12) topk_words(VMOBA_INT(12));
+      else if (mw <= 14) topk_words(VMOBA_INT(14));
       else if (mw <= 16) topk_words(VMOBA_INT(16));
       else if (mw <= 24) topk_words(VMOBA_INT(24));
       else topk_words(VMOBA_INT(kLocalMaxWords));
@@ -2208,7 +2224,12 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
   }
 #undef VMOBA_POOL
 
-  const size_t smem_fill = ((size_t)QSEG * D.mask_words + 2 * (size_t)D.Nb * (QSEG >> 5) + 2 * (size_t)D.Nb + 1 + 2 * kStage) * 4;
+  // (the top-k rule's segments have so many pairs and no more)
+  const int stage = rule == VMOBA_SELECT_TOPK_LOCAL
+                        ? (int)std::min<long long>(kStage, (long long)QSEG * (std::min(topk, D.Nb) + (own_sb > 0 ? 1 : 0)) + 1 & ~1ll)
+                        : kStage;
+  const size_t cols = (size_t)D.Nb * (QSEG >> 5);
+  const size_t smem_fill = ((size_t)QSEG * D.mask_words + cols + 2 * (size_t)D.Nb + 1 + stage) * 4 + (stage + cols) * 2;
   VMOBA_CUDA_OK(allow_smem(fill_kernel, (int)smem_fill));
   long long nkb = (long long)D.BH * D.Nb;
   if (!pool) {
@@ -2224,7 +2245,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
   const int fill_threads = QSEG >= 128 ? QSEG : kSegThreads;
   launch_kernel(fill_kernel, sgrid, fill_threads, smem_fill, st, mask_bits, w.tmask, D.S, D.Nb, D.mask_words, QSEG, nseg,
                 kb_ptr, w.seg_cnt, w.seg_qoff, q_idx, q_ptr, q_pairs, capacity, pool ? w.kb_total : nullptr, k_per_head,
-                dev_status);
+                dev_status, stage);
   VMOBA_LAUNCH_OK(1);
   VMOBA_GUARDS_CHECK(w.guards, dev_status, st);
   return VMOBA_OK;
