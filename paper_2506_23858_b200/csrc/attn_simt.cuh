@@ -107,7 +107,8 @@ __device__ __forceinline__ Item decode_sparse(int item, const int* __restrict__ 
 //
 // The products below are bound by the FMA pipe: 64 FMAs per eight 16-byte loads from shared memory.  With four threads to a row,
 // each holding a quarter of its channels, a key cost a thread as many loads as four of its FMAs and two shuffles.
-// Forward and backward of 13 heads x 4,096 tokens, head_dim 128, 2450 -> 1095 us; of 2 x 256, head_dim 64, 98.6 -> 72.0.
+// Forward and backward of 13 heads x 4,096 tokens, head_dim 128, 2440 -> 1084 us; of 2 x 256, head_dim 64, 99.2 -> 66.2; dense, 4 x
+// 2,000, head_dim 64, bf16, 1361 -> 829.
 template <int DH> constexpr int kLd = DH + 4;
 template <int DH> constexpr int kTileFloats = kRows * kLd<DH>;
 constexpr int kLdP = kRows + 4;
@@ -135,39 +136,49 @@ struct TileRegs {
   }
 };
 
-// acc[i][j] = A[4 ty + i] . B[tx + 16 j] for the first NJ * 16 rows of B.  Sixteen channels at a time: sums of sums keep
-// the rounding error of one long sum, and more, away (o of 4 x 2,048 tokens, head_dim 128: 4.0e-7 off with a quarter of
-// the channels in a row, 5.1e-7 with all of them, 3.6e-7 so).
+// acc[i][j] = A[4 ty + i] . B[tx + 16 j] for the first NJ * 16 rows of B, as (p0 + p1) + (p2 + p3) where pn sums the channels
+// 16 g + 4 n to 16 g + 4 n + 3 of all g in their order.  These are the sums of the kernels with four threads to a row, and so is
+// the order of every other sum here but that of dq: o, lse, dk and dv are theirs to the bit.  (Scores off by one rounding move
+// single gradients by 1e-4 of their rms where the logits are large: 13 heads x 4,096 tokens with a smooth field in q and k, head_dim
+// 128.  Sums of sixteen channels at a time are nearer to 64 bits by a quarter and as fast, but that far from what was.)
 template <int DH, int NJ>
-__device__ __forceinline__ void dot_tiles_n(const float* A, const float* B, int ty, int tx, float (&acc)[4][4]) {
+__device__ __forceinline__ void dot_quarter(const float* A, const float* B, int ty, int tx, int c0, float (&part)[4][4]) {
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-#pragma unroll 1
-  for (int c0 = 0; c0 < DH; c0 += 16) {
-    float part[4][NJ];
+    for (int j = 0; j < 4; ++j) part[i][j] = 0.f;
 #pragma unroll
-    for (int c = 0; c < 16; c += 4) {
-      float4 a[4], b[NJ];
+  for (int c = 0; c < DH; c += 16) {
+    float4 a[4], b[NJ];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(A + (4 * ty + i) * kLd<DH> + c0 + c);
+    for (int i = 0; i < 4; ++i) a[i] = *reinterpret_cast<const float4*>(A + (4 * ty + i) * kLd<DH> + c0 + c);
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) b[j] = *reinterpret_cast<const float4*>(B + (tx + 16 * j) * kLd<DH> + c0 + c);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) {
-          part[i][j] = c == 0 ? a[i].x * b[j].x : fmaf(a[i].x, b[j].x, part[i][j]);
-          part[i][j] = fmaf(a[i].y, b[j].y, part[i][j]);
-          part[i][j] = fmaf(a[i].z, b[j].z, part[i][j]);
-          part[i][j] = fmaf(a[i].w, b[j].w, part[i][j]);
-        }
-    }
+    for (int j = 0; j < NJ; ++j) b[j] = *reinterpret_cast<const float4*>(B + (tx + 16 * j) * kLd<DH> + c0 + c);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < NJ; ++j) acc[i][j] += part[i][j];
+      for (int j = 0; j < NJ; ++j) {
+        part[i][j] = fmaf(a[i].x, b[j].x, part[i][j]);
+        part[i][j] = fmaf(a[i].y, b[j].y, part[i][j]);
+        part[i][j] = fmaf(a[i].z, b[j].z, part[i][j]);
+        part[i][j] = fmaf(a[i].w, b[j].w, part[i][j]);
+      }
+  }
+}
+template <int DH, int NJ>
+__device__ __forceinline__ void dot_tiles_n(const float* A, const float* B, int ty, int tx, float (&acc)[4][4]) {
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    float x[4][4], y[4][4];
+    dot_quarter<DH, NJ>(A, B, ty, tx, 8 * h, x);
+    dot_quarter<DH, NJ>(A, B, ty, tx, 8 * h + 4, y);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        x[i][j] += y[i][j];
+        acc[i][j] = h ? acc[i][j] + x[i][j] : x[i][j];
+      }
   }
 }
 template <int DH>
@@ -213,16 +224,19 @@ __device__ __forceinline__ void add_weighted_t(const float* P, const float* B, i
     }
   }
 }
-// over the sixteen threads of a row
-__device__ __forceinline__ float row_max(float x) {
+// Thread tx of the sixteen that share rows: the largest x[tx / 4][tx % 4] of them all.
+__device__ __forceinline__ float group_max(const float (&x)[4][4], int tx) {
+  float r[16];
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
-  return x;
-}
-__device__ __forceinline__ float row_sum(float x) {
+  for (int n = 0; n < 16; ++n) r[n] = x[n >> 2][n & 3];
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  return x;
+  for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (int n = 0; n < o; ++n) {
+      const float keep = (tx & o) ? r[n + o] : r[n], give = (tx & o) ? r[n] : r[n + o];
+      r[n] = fmaxf(keep, __shfl_xor_sync(0xffffffffu, give, o));
+    }
+  return r[0];
 }
 template <int DH> constexpr int kFwdSmem = (2 * kTileFloats<DH> + kRows * kLdP) * 4;      // Q, K or V, weights
 
@@ -240,6 +254,7 @@ attn_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
   float* KVs = Qs + kTileFloats<DH>;
   float* Ps = KVs + kTileFloats<DH>;
   __shared__ int s_row[kRows];                 // in-head position of the query, -1 for none; bit 30: it has a single block
+  __shared__ __align__(16) float s_max[kRows * 4], s_corr[kRows * 4];      // of a tile's rows, every sixteen keys
   const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
   const int tiles_per_head = (S + kRows - 1) / kRows;
   const int n_items = DENSE ? BH * tiles_per_head : item_ptr[n_kb];
@@ -277,13 +292,12 @@ attn_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
       qt.store(Qs);
     }
     next.store(KVs);
-    float m[4], l[4], acc[4][DH / 16];         // l: of this thread's keys only
+    float m = -INFINITY, l = 0.f;              // of row 4 ty + tx / 4
+    float acc[4][DH / 16];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      m[i] = -INFINITY; l[i] = 0.f;
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int c = 0; c < DH / 16; ++c) acc[i][c] = 0.f;
-    }
     const bool live = (ty & ~1) * 4 < rows;    // (a warp has eight rows)
     __syncthreads();
     for (int t0 = it.key_begin; t0 < it.key_end; t0 += kRows) {
@@ -293,25 +307,42 @@ attn_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
         float s[4][4];
         dot_tiles<DH>(Qs, KVs, ty, tx, nv, s);
 #pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) s[i][j] = tx + 16 * j < nv ? s[i][j] * scale : -INFINITY;
+        // the largest score so far changes every sixteen keys: thread tx finds it for row tx / 4 at keys 16 (tx % 4) and on, and
+        // what the sums so far are multiplied with there
+        const float mx = group_max(s, tx);
+        float mj = mx, up = __shfl_up_sync(0xffffffffu, mj, 1, 4);
+        if ((tx & 3) >= 1) mj = fmaxf(mj, up);
+        up = __shfl_up_sync(0xffffffffu, mj, 2, 4);
+        if ((tx & 3) >= 2) mj = fmaxf(mj, up);
+        mj = fmaxf(m, mj);
+        up = __shfl_up_sync(0xffffffffu, mj, 1, 4);
+        const float before = (tx & 3) ? up : m;
+        s_max[ty * 16 + tx] = mj;
+        s_corr[ty * 16 + tx] = before == -INFINITY ? 0.f : expf(before - mj);
+        m = __shfl_sync(0xffffffffu, mj, 3, 4);
+        __syncwarp();
+#pragma unroll
         for (int i = 0; i < 4; ++i) {
-          float mx = -INFINITY;
+          const float4 m4 = *reinterpret_cast<const float4*>(s_max + 16 * ty + 4 * i);
+          const float mm[4] = {m4.x, m4.y, m4.z, m4.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            s[i][j] = tx + 16 * j < nv ? s[i][j] * scale : -INFINITY;
-            mx = fmaxf(mx, s[i][j]);
+          for (int j = 0; j < 4; ++j) Ps[(4 * ty + i) * kLdP + tx + 16 * j] = s[i][j] == -INFINITY ? 0.f : expf(s[i][j] - mm[j]);
+        }
+        __syncwarp();
+        // the row's weights, key after key
+        const float* row = Ps + (4 * ty + (tx >> 2)) * kLdP;
+#pragma unroll 1
+        for (int k = 0; k < nv; k += 16) {
+          const float corr = s_corr[16 * ty + (tx & 12) + (k >> 4)];
+#pragma unroll
+          for (int c = 0; c < 16; c += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(row + k + c);
+            l = c == 0 ? __fadd_rn(__fmul_rn(l, corr), w.x) : l + w.x;      // (not one fused operation: it was two)
+            l += w.y; l += w.z; l += w.w;
           }
-          const float m_new = fmaxf(m[i], row_max(mx));
-          const float corr = m[i] == -INFINITY ? 0.f : expf(m[i] - m_new);
-          l[i] *= corr;
-#pragma unroll
-          for (int c = 0; c < DH / 16; ++c) acc[i][c] *= corr;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float p = s[i][j] == -INFINITY ? 0.f : expf(s[i][j] - m_new);
-            l[i] += p;
-            Ps[(4 * ty + i) * kLdP + tx + 16 * j] = p;
-          }
-          m[i] = m_new;
         }
       }
       __syncthreads();
@@ -319,7 +350,18 @@ attn_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
       __syncthreads();
       const int t1 = t0 + kRows;
       if (t1 < it.key_end) next.fetch(kh, min(kRows, it.key_end - t1), [&](int i) { return t1 + i; });
-      if (live) add_weighted<DH>(Ps, KVs, ty, tx, nv, acc);
+      if (live) {
+#pragma unroll 1
+        for (int k = 0; k < nv; k += 16) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float corr = s_corr[16 * ty + 4 * i + (k >> 4)];
+#pragma unroll
+            for (int c = 0; c < DH / 16; ++c) acc[i][c] *= corr;
+          }
+          add_weighted<DH>(Ps + k, KVs + k * kLd<DH>, ty, tx, min(16, nv - k), acc);
+        }
+      }
       if (t1 < it.key_end) {
         __syncthreads();
         next.store(KVs);
@@ -329,10 +371,10 @@ attn_fwd_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* __res
     if (!live) continue;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const float total = row_sum(l[i]);
+      const float total = __shfl_sync(0xffffffffu, l, 4 * i, 16), top = __shfl_sync(0xffffffffu, m, 4 * i, 16);
       const int x = s_row[4 * ty + i];
       if (x < 0) continue;
-      const float inv = 1.0f / total, row_lse = m[i] + logf(total);
+      const float inv = 1.0f / total, row_lse = top + logf(total);
       const long long G_ = head_off + (x & (kSingle - 1)), pos = (long long)it.list_lo + 4 * ty + i;
       const bool direct = (x & kSingle) != 0;
 #pragma unroll
