@@ -68,9 +68,10 @@ static int grid_for(long long items, int per_sm) {
 
 // Whether the CUDA-core kernels are launched ahead of the end of the kernel before them.  Several of their CTAs share an SM, and
 // early ones go where that kernel has left room: two to an SM while others stay empty, which costs a long kernel more than the
-// launch it saves.  Dense forward and backward, early against not: 4 heads x 2,000 tokens (bf16, head_dim 64) 1842 / 1366 us,
-// 12 x 512 483 / 370; a sparse forward of 4 x 256 (three early launches) 31 / 39.  pairs: (query, key) pairs at most.
-static bool early_simt(const Dims& D, double pairs) { return pairs * D.d <= (double)(1 << 26); }
+// launch it saves.  Dense forward and backward in bf16, head_dim 64, early against not: 8 heads x 256 tokens 113.6 / 118.8 us,
+// 12 x 256 144.6 / 118.8, 12 x 512 310 / 223, 4 x 2,000 1273 / 772; a sparse layer, fp32, of 2 x 256 66.0 / 70.5.  pairs: (query,
+// key) pairs at most.
+static bool early_simt(const Dims& D, double pairs) { return pairs * D.d <= (double)(1 << 25); }
 
 template <typename T, int DH>
 static int simt_sparse_fwd(const Dims& D, const void* q, const void* k, const void* v, const int* kb_ptr,
