@@ -4,19 +4,22 @@
 //
 // Sorting the head's pool and accumulating normalised similarity until tau is reached is
 // equivalent to finding the weighted quantile of the scores under the softmax weights:
-// the cutoff is the largest score c with mass{score >= c} >= tau * Z.  That is found without
-// a sort by three histogram refinements (2048 bins each, linear in the score, fp64 bin
-// masses), after which the mask is one comparison per pair.  Every kernel streams the score
-// matrix with 16-byte loads; the stage is bound by HBM bandwidth.
+// the cutoff is the largest score c with mass{score >= c} >= tau * Z.  That is found without a sort, by one of three
+// routes that the size of the pool decides:
 //
-//   init (+ minmax, unless the caller hands over each head's score range)
-//           -> hist level 0 -> scan -> hist level 1 -> scan -> hist level 2 -> scan (cutoff)
-//   (level 1 copies the pairs of the level-0 crossing bin aside, and level 2 reads that short list instead of the
-//    score matrix: three traversals of the matrix, levels 0 and 1 and mark)
-//   mark    : mask bits + per (segment, block) counts + per-segment pair totals
+//   small   : select_pool_kernel, a cluster per head with the scores on chip, does everything before fill (pool_plan)
+//   large   : window (sample) -> window pass (mass above the window, its scores aside) -> window search (cutoff), if there is
+//             room for the lists (kWindowMin); then mark .. fill
+//   between : init (+ minmax, unless the caller hands over each head's score range)
+//             -> hist level 0 -> scan -> hist level 1 -> scan -> hist level 2 -> scan (cutoff): histogram refinements, linear in
+//             the score, fp64 bin masses; level 1 copies the pairs of the level-0 crossing bin aside, and level 2 reads that
+//             short list instead of the score matrix; then mark .. fill
+//
+//   mark    : mask bits (one comparison per pair) + per (segment, block) counts + per-segment pair totals
 //   offsets : CSR offsets by key block (kb_ptr) and by query (q_ptr)
 //   fill    : q_idx (queries of each key block, ascending) and q_pairs (pairs of each query)
-// Small pools take select_pool_kernel instead of everything before fill (pool_plan).
+//
+// Every pass streams the score matrix with 16-byte loads and is bound by HBM bandwidth, the small route by latency.
 #include <algorithm>
 #include <type_traits>
 
