@@ -1654,6 +1654,10 @@ constexpr int kFewSamples = 48;
 // From six million scores on (matrix of 24 MB): 12 heads x 16,384 x 32 blocks (6.3 million) 70 -> 66 us, x 64 99 -> 84, x 13,650 x 25
 // (4.1 million) 74 -> 74, 2 heads x 37,500 x 25 51 -> 58 (whole selection, white scores).
 constexpr long long kWindowMin = 6000000;
+// And where the sample is one score in eighty or more.  Thinner, it can miss the few pairs that hold a smooth layer's mass, the window
+// comes out too wide, and the search of the whole pool takes many times what the histogram passes do: 40 heads x 75,600, three
+// layers of 21, 40 and 280 blocks (one score in 48, 92 and 646), selection 4.2 ms by the passes, 32.6 where all three took the window.
+constexpr long long kSampleShare = 80;
 // CTAs that take one head's sample, and its search: at most two to an SM, and few where there is little to do.
 static int window_ctas(int BH, long long P) {
   int C = kPoolCtas;
@@ -2170,7 +2174,8 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     long long per_head = (P / 4 + 255) / 256;
     int gx = (int)std::min<long long>(std::max<long long>(per_head / 8, 1), std::max(1, sm_count() * 8 / D.BH));
     dim3 grid(gx, D.BH);
-    const bool window = use_cand && (long long)D.BH * P >= kWindowMin;
+    const bool window = use_cand && (long long)D.BH * P >= kWindowMin &&
+                        P <= kSampleShare * window_ctas(D.BH, P) * kSamples * kSampleThreads;
     if (window) {
       if (!range) {
         launch_kernel(init_state_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, D.BH, nullptr, nullptr, nullptr, nullptr, nullptr);
