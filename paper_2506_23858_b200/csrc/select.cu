@@ -1655,8 +1655,8 @@ constexpr int kFewSamples = 48;
 // (4.1 million) 74 -> 74, 2 heads x 37,500 x 25 51 -> 58 (whole selection, white scores).
 constexpr long long kWindowMin = 6000000;
 // And where the sample is one score in eighty or more.  Thinner, it can miss the few pairs that hold a smooth layer's mass, the window
-// comes out too wide, and the search of the whole pool takes many times what the histogram passes do: 40 heads x 75,600, three
-// layers of 21, 40 and 280 blocks (one score in 48, 92 and 646), selection 4.2 ms by the passes, 32.6 where all three took the window.
+// comes out too wide, and the search of the whole pool takes many times what the histogram passes do.  40 heads x 75,600: 21 blocks (one
+// score in 48) search 26 us, 40 blocks (one in 92) 31, 280 blocks (one in 646) 24,000.
 constexpr long long kSampleShare = 80;
 // CTAs that take one head's sample, and its search: at most two to an SM, and few where there is little to do.
 static int window_ctas(int BH, long long P) {
