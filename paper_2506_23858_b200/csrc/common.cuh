@@ -179,7 +179,7 @@ inline void count_launches(int n) { g_kernel_launches.fetch_add((unsigned long l
 // range-checked build, where nothing is early, and the diagnostics' own kernel do neither).  An early launch does
 // not wait for the end of the kernel before it in the stream: its CTAs are set up while the other still runs, stop in
 // grid_begin() until that one has completed and its writes are visible, and then allow the same for the next.  A call is a
-// chain of a dozen kernels or more (12 to 17 in bf16 with the backward, 17 in fp32), many of a few microseconds, and each early launch
+// chain of a dozen kernels or more (12 to 21 in bf16 with the backward), many of a few microseconds, and each early launch
 // is worth 1.5 .. 3 us (forward of 33K tokens,
 // 12 heads: 659 -> 624 us; forward and backward of 1.9K tokens: 204 -> 171 us).
 //

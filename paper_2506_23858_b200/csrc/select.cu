@@ -4,13 +4,11 @@
 //
 // Sorting the head's pool and accumulating normalised similarity until tau is reached is
 // equivalent to finding the weighted quantile of the scores under the softmax weights:
-// the cutoff is the largest score c with mass{score >= c} >= tau * Z.  That is found without a sort, by one of three
+// the cutoff is the largest score c with mass{score >= c} >= tau * Z.  That is found without a sort, by one of two
 // routes that the size of the pool decides:
 //
 //   small   : select_pool_kernel, a cluster per head with the scores on chip, does everything before fill (pool_plan)
-//   large   : window (sample) -> window pass (mass above the window, its scores aside) -> window search (cutoff), if there is
-//             room for the lists (kWindowMin); then mark .. fill
-//   between : init (+ minmax, unless the caller hands over each head's score range)
+//   larger  : init (+ minmax, unless the caller hands over each head's score range)
 //             -> hist level 0 -> scan -> hist level 1 -> scan -> hist level 2 -> scan (cutoff): histogram refinements, linear in
 //             the score, fp64 bin masses; level 1 copies the pairs of the level-0 crossing bin aside, and level 2 reads that
 //             short list instead of the score matrix; then mark .. fill
@@ -48,7 +46,6 @@ struct HeadState {
   unsigned int cand_cnt;       // pairs of the level-0 crossing bin, copied aside by the level-1 pass
   int cand_ok;                 // every one of them found room in the list: level 2 reads the list
   float bin0_off;              // -anchor[0] * inv[0]: the level-0 bin of s is floor(s * inv[0] + bin0_off)
-  float win_lo, win_hi;        // the window that a sample gives the cutoff
   uint32_t pad;
 };
 
@@ -1220,9 +1217,8 @@ __device__ __noinline__ T pool_exclusive(T x, T* s_warp) {
 
 // The search for a head's cutoff among the scores src[0 .. n) of every CTA of a cluster, which lie in [lo, lo + span] (shared or
 // global memory; I: a type that holds n).  target(total, need): the mass to be covered, given that of all these scores; false: they
-// cannot hold the cutoff, and the search ends.  front: kPoolFront * T bytes of shared memory.  WIDE: from global memory, sixteen bytes
-// per load.
-template <int T, bool WIDE, typename I, typename Meet, typename Weight, typename Target>
+// cannot hold the cutoff, and the search ends.  front: kPoolFront * T bytes of shared memory.
+template <int T, typename I, typename Meet, typename Weight, typename Target>
 __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& cluster, Meet meet, unsigned char* front, const float* src,
                                             I n, float lo, float span, Weight weight, Target target, uint32_t& cutoff) {
   constexpr int kLevelBytes = 8 * T, kList = (kPoolFront * T - kPoolLevels * kLevelBytes) / 4;
@@ -1253,20 +1249,6 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
   };
   auto stream = [&](const float* from, I count, auto f) {
     I i = t;
-    if constexpr (WIDE) {
-      if ((reinterpret_cast<uintptr_t>(from) & 15u) == 0) {
-        const I trips = count / (16 * (I)T);
-#pragma unroll 1
-        for (I r = 0; r < trips; ++r) {
-          float4 x[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) x[j] = reinterpret_cast<const float4*>(from)[(4 * r + j) * (I)T + t];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) { f(x[j].x); f(x[j].y); f(x[j].z); f(x[j].w); }
-        }
-        i += trips * 16 * (I)T;
-      }
-    }
 #pragma unroll 4
     for (; i < count; i += T) f(from[i]);
   };
@@ -1531,7 +1513,7 @@ select_pool_kernel(const PoolArgs a) {
     const bool unit_w = a.unit_w != 0;
     cutoff = min_key;                      // everything, where tau = 1
     if (a.tau < 1.0f) {
-      pool_search<T, false, int>(cluster, meet, pool_smem, s_src, n, lo, smax - lo,
+      pool_search<T, int>(cluster, meet, pool_smem, s_src, n, lo, smax - lo,
                           [&](float s) { return unit_w ? 1.0f : pair_weight(a.sigma, s, smax); },
                           [&](double total, double& need) { need = a.count_target >= 0.0 ? a.count_target : (double)a.tau * total; return true; },
                           cutoff);
@@ -1642,270 +1624,6 @@ select_pool_kernel(const PoolArgs a) {
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// Larger pools, if there is room for candidate lists: a sample of a head's scores tells roughly where the cutoff is, ONE pass
-// over the matrix adds up the mass above a window round that place and copies the window's scores aside, and a cluster of
-// CTAs per head finds the cutoff among these.  Where it is not among them (the sample missed the few pairs that hold the mass, or
-// the window has more scores than the list) the cluster searches the whole of the head's scores.  Three launches instead of eight
-// and two passes over the matrix (this one and mark) instead of three.  Whole selection of 12 heads x 32,760 x 140 blocks 191 ->
-// 164 us, 24 heads 340 -> 296, 12 x 55,296 x 72 218 -> 190.
-constexpr int kSampleThreads = kBins0, kSamples = 16;      // (per thread)
-constexpr int kFewSamples = 48;
-// From six million scores on (matrix of 24 MB): 12 heads x 16,384 x 32 blocks (6.3 million) 70 -> 66 us, x 64 99 -> 84, x 13,650 x 25
-// (4.1 million) 74 -> 74, 2 heads x 37,500 x 25 51 -> 58 (whole selection, white scores).
-constexpr long long kWindowMin = 6000000;
-// And where the sample is one score in eighty or more.  Thinner, it can miss the few pairs that hold a smooth layer's mass, the window
-// comes out too wide, and the search of the whole pool takes many times what the histogram passes do.  40 heads x 75,600: 21 blocks (one
-// score in 48) search 26 us, 40 blocks (one in 92) 31, 280 blocks (one in 646) 24,000.
-constexpr long long kSampleShare = 80;
-// CTAs that take one head's sample, and its search: at most two to an SM, and few where there is little to do.
-static int window_ctas(int BH, long long P) {
-  int C = kPoolCtas;
-  while (C > 1 && ((long long)BH * C > 2ll * sm_count() || (P >> 18) < C)) C /= 2;
-  return C;
-}
-
-// A cluster per head; also leaves the head's state.  The sample is counted in 512 bins of the head's range and, round the
-// crossing, in 512 bins of a few of these; a bin's mass is its count times the weight at its middle.  The window reaches
-// 4.5 standard deviations of the sample's estimate of the mass above the cutoff to either side of the target.
-__global__ void __launch_bounds__(kSampleThreads)
-window_kernel(const float* __restrict__ scores, long long P, const float* __restrict__ range, HeadState* __restrict__ st, float sigma,
-              int unit_w, float tau, double count_target, float list_share) {
-  if (!grid_begin()) return;
-  __shared__ unsigned int s_cnt[2][kBins0];
-  __shared__ float s_m[32], s_m2[32], s_total, s_total2, s_above2, s_base, s_base2;
-  __shared__ int s_c[32], s_bin[2], s_before[2], s_all, s_top;
-  __shared__ float s_top_mass;
-  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
-  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), bh = blockIdx.x / C, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  s_cnt[0][t] = s_cnt[1][t] = 0u;
-  uint32_t min_key, max_key;
-  if (range) { min_key = float_key(range[2 * bh]); max_key = float_key(range[2 * bh + 1]); }
-  else { min_key = st[bh].min_key; max_key = st[bh].max_key; }
-  const float lo = key_float(min_key), smax = key_float(max_key), span = smax - lo;
-  const float* base = scores + (long long)bh * P;
-  // one score out of each of n equal parts of the pool, at a place that a hash gives
-  const int most = C * kSamples * kSampleThreads, n = (int)min(P, (long long)most);
-  const unsigned long long step = ((unsigned long long)P << 20) / n;      // (P < 2^37)
-  const unsigned int stride = (unsigned int)min(P / n, 0xffffffffll);
-  float x[kSamples];
-#pragma unroll
-  for (int u = 0; u < kSamples; ++u) {
-    const int i = (u * C + rank) * kSampleThreads + t;
-    unsigned int h = (i + 1u) * 2654435761u;
-    h ^= h >> 15;
-    h *= 2246822519u;
-    x[u] = i < n ? __ldg(base + ((i * step) >> 20) + __umulhi(h, stride)) : NAN;
-  }
-  const float share = count_target >= 0.0 ? (float)(count_target / (double)P) : tau;
-  float from = lo, inv = span > 0.f ? (float)kBins0 / span : 0.f, win_lo = -INFINITY, win_hi = INFINITY;
-  float over = 0.f, over2 = 0.f;        // mass above the bins of the second round, and its squares
-  int inside = 0, top = kBins0;         // top: the first round's lowest bin from which on the scores fit the list
-  float top_mass = 0.f, goal = 0.f;
-  if (t == 0) { s_top = kBins0; s_top_mass = 0.f; }
-  __syncthreads();
-#pragma unroll 1
-  for (int round = 0; round < 2; ++round) {
-    const float off = -from * inv;
-#pragma unroll
-    for (int u = 0; u < kSamples; ++u) {
-      const float y = fmaf(x[u], inv, off);
-      // (NaN is in no bin; the ends of the head's range are in the first and the last)
-      if (round == 0 ? y == y : y >= 0.f && y < (float)kBins0) atomicAdd(&s_cnt[round][min(max(__float2int_rd(y), 0), kBins0 - 1)], 1u);
-    }
-    cluster.sync();
-    const int b = kBins0 - 1 - t;       // this thread's bin
-    int c = 0;
-#pragma unroll
-    for (int r = 0; r < kPoolCtas; ++r)
-      if (r < C) c += (int)cluster.map_shared_rank(s_cnt[round], r)[b];
-    const float mid = from + ((float)b + 0.5f) / inv, w = unit_w ? 1.0f : pair_weight(sigma, mid, smax);
-    const float m = c ? (float)c * w : 0.f, m2 = c ? m * w : 0.f;
-    // sums over the bins above this one
-    float im = m, im2 = m2;
-    int ic = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const float v = __shfl_up_sync(0xffffffffu, im, o), v2 = __shfl_up_sync(0xffffffffu, im2, o);
-      const int vc = __shfl_up_sync(0xffffffffu, ic, o);
-      if (lane >= o) { im += v; im2 += v2; ic += vc; }
-    }
-    if (lane == 31) { s_m[warp] = im; s_m2[warp] = im2; s_c[warp] = ic; }
-    if (t < 2) { s_bin[t] = -1; s_before[t] = t == 0 ? -1 : 0; }
-    if (t == 0) s_above2 = 0.f;
-    __syncthreads();
-    float excl = over + im - m, excl2 = over2 + im2 - m2;
-    int before = ic - c;
-    for (int v = 0; v < warp; ++v) { excl += s_m[v]; excl2 += s_m2[v]; before += s_c[v]; }
-    if (t == kSampleThreads - 1) {
-      if (round == 0) { s_total = excl + m; s_total2 = excl2 + m2; }
-      s_all = before + c;
-    }
-    if (round == 0 && (float)(before + c) <= 0.7f * list_share * (float)n) atomicMin(&s_top, b);
-    __syncthreads();
-    goal = share * s_total;
-    if (excl < goal && excl + m >= goal) s_above2 = excl2 + m2;
-    if (round == 0 && b == s_top) s_top_mass = excl + m;
-    __syncthreads();
-    const float dev = 4.5f * sqrtf((1.f - share) * (1.f - share) * s_above2 + share * share * fmaxf(s_total2 - s_above2, 0.f));
-    if (excl < goal - dev && excl + m >= goal - dev) { s_bin[1] = b; s_before[1] = before; s_base = excl; s_base2 = excl2; }
-    if (excl < goal + dev && excl + m >= goal + dev) { s_bin[0] = b; s_before[0] = before + c; }
-    __syncthreads();
-    const int b_lo = s_bin[0], b_hi = s_bin[1];
-    inside = (s_before[0] >= 0 ? s_before[0] : s_all) - s_before[1];
-    if (round == 0) { top = s_top; top_mass = s_top_mass; }
-    // (an end that this round did not find stays where it was)
-    const float edge = from;
-    if (b_lo > 0) win_lo = edge + (float)b_lo / inv;
-    // (few samples are no measure of what lies above them: no upper end there)
-    if (b_hi >= 0 && s_before[1] < kFewSamples) inside += s_before[1];
-    else if (b_hi >= 0 && (round > 0 || b_hi < kBins0 - 1)) win_hi = edge + (float)(b_hi + 1) / inv;
-    if (round == 0) {
-      if ((float)inside <= 0.5f * list_share * (float)n) break;      // narrow enough
-      // the second round looks at the bins from b_lo to b_hi
-      const int first = max(b_lo, 0), last = b_hi >= 0 ? b_hi : kBins0 - 1;
-      if (b_hi >= 0) { over = s_base; over2 = s_base2; }
-      from = edge + (float)first / inv;
-      inv = inv > 0.f ? inv * ((float)kBins0 / (float)(last - first + 1)) : 0.f;
-    }
-    __syncthreads();
-  }
-  if (rank == 0 && t == 0) {
-    HeadState h;
-    memset(&h, 0, sizeof(h));
-    h.min_key = min_key; h.max_key = max_key;
-    h.cutoff_key = 0xffffffffu;
-    // Where the window would hold more than the list: if a few pairs hold the mass (the sample is no measure of it, and the
-    // cutoff lies high), the highest scores that fit; else the whole pool is searched.
-    if (!(span > 0.f) || (float)inside > 0.75f * list_share * (float)n) {
-      win_lo = span > 0.f && top > 0 && top < kBins0 && top_mass >= 1.5f * goal ? lo + (float)top * span / (float)kBins0 : INFINITY;
-      win_hi = INFINITY;
-    }
-    h.win_lo = win_lo; h.win_hi = win_hi;
-    st[bh] = h;
-  }
-  cluster.sync();      // nobody leaves while its counts may be read
-}
-
-// The pass over the matrix.  Bound by HBM: a dozen instructions per score and no atomics; a warp gathers what it finds in the
-// window and writes it out some 256 at a time (with the check for that behind every score instead of every sixteen, twenty copies of
-// the code that writes: 77 us where this takes 47; floor 34: 12 heads x 32,760 x 140).
-constexpr int kWindowThreads = 512, kWindowStage = 256 + 512;
-__global__ void __launch_bounds__(kWindowThreads)
-window_pass_kernel(const float* __restrict__ scores, long long P, HeadState* __restrict__ st, float sigma, int unit_w,
-                   float* __restrict__ cand, long long ccap) {
-  if (!grid_begin()) return;
-  extern __shared__ float s_stage[];    // [warps][kWindowStage]
-  __shared__ double s_z[kWindowThreads / 32], s_a[kWindowThreads / 32];
-  const int bh = blockIdx.y, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const float win_lo = st[bh].win_lo, win_hi = st[bh].win_hi, smax = key_float(st[bh].max_key);
-  float* list = cand + (long long)bh * ccap;
-  float* stage = s_stage + warp * kWindowStage;
-  const unsigned int lt_mask = (1u << lane) - 1u;
-  int staged = 0;                       // (the same in all lanes)
-  auto write_out = [&]() {
-    __syncwarp();
-    unsigned int at = 0;
-    if (lane == 0) at = atomicAdd(&st[bh].cand_cnt, (unsigned int)staged);
-    at = __shfl_sync(0xffffffffu, at, 0);
-    for (int i = lane; i < staged; i += 32)
-      if (at + i < ccap) list[at + i] = stage[i];
-    staged = 0;
-    __syncwarp();
-  };
-  float z = 0.f, above = 0.f;
-  auto take = [&](float s, bool there) {
-    float w = unit_w ? 1.0f : fmaxf(pair_weight(sigma, s, smax), 0.f);      // (0 for NaN)
-    if (!there) w = 0.f;
-    z += w;
-    if (s >= win_hi) above += w;
-    const bool in = there && s >= win_lo && s < win_hi;
-    const unsigned int found = __ballot_sync(0xffffffffu, in);
-    if (found) {
-      if (in) stage[staged + __popc(found & lt_mask)] = s;
-      staged += __popc(found);
-    }
-  };
-  const float* base = scores + (long long)bh * P;
-  const long long gw = (long long)blockIdx.x * (kWindowThreads / 32) + warp, n_warps = (long long)gridDim.x * (kWindowThreads / 32);
-  long long done = 0;                   // scores that went in runs of 512
-  if ((reinterpret_cast<uintptr_t>(base) & 15u) == 0) {
-    const float4* b4 = reinterpret_cast<const float4*>(base);
-    const long long runs = P / 512;
-#pragma unroll 1
-    for (long long r = gw; r < runs; r += n_warps) {
-      float4 x[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] = __ldg(b4 + r * 128 + 32 * j + lane);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { take(x[j].x, true); take(x[j].y, true); take(x[j].z, true); take(x[j].w, true); }
-      if (staged > kWindowStage - 512) write_out();
-    }
-    done = runs * 512;
-  }
-#pragma unroll 1
-  for (long long r = done + gw * 512; r < P; r += n_warps * 512) {
-#pragma unroll 4
-    for (int j = 0; j < 16; ++j) {
-      const long long i = r + 32 * j + lane;
-      take(i < P ? __ldg(base + i) : 0.f, i < P);
-    }
-    if (staged > kWindowStage - 512) write_out();
-  }
-  if (staged) write_out();
-  double zd = z, ad = above;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) { zd += __shfl_xor_sync(0xffffffffu, zd, o); ad += __shfl_xor_sync(0xffffffffu, ad, o); }
-  if (lane == 0) { s_z[warp] = zd; s_a[warp] = ad; }
-  __syncthreads();
-  if (t == 0) {
-    zd = ad = 0.0;
-    for (int w = 0; w < kWindowThreads / 32; ++w) { zd += s_z[w]; ad += s_a[w]; }
-    atomicAdd(&st[bh].Z, zd);
-    if (ad > 0.0) atomicAdd(&st[bh].mass_above, ad);
-  }
-}
-
-// The cutoff, by a cluster per head.
-template <int T>
-__global__ void __launch_bounds__(T, 1)
-window_search_kernel(const float* __restrict__ scores, long long P, HeadState* __restrict__ st, float sigma, int unit_w, float tau,
-                     double count_target, const float* __restrict__ cand, long long ccap, float* __restrict__ cutoff_per_head) {
-  if (!grid_begin()) return;
-  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
-  extern __shared__ __align__(16) unsigned char pool_smem[];
-  const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank(), bh = (int)blockIdx.x / C;
-  auto meet = [&]() { cluster.sync(); };
-  const HeadState h = st[bh];
-  const float lo = key_float(h.min_key), smax = key_float(h.max_key);
-  const bool by_count = unit_w != 0;
-  auto weight = [&](float s) { return by_count ? 1.0f : pair_weight(sigma, s, smax); };
-  uint32_t cutoff = h.min_key;            // everything, where tau = 1 or all scores are alike (zeros of either sign are)
-  if (lo == smax && lo == 0.f) cutoff = 0x7fffffffu;
-  meet();                                 // (all CTAs have started)
-  if (tau < 1.0f && lo != smax) {
-    bool found = false;
-    const int n = (int)min((long long)h.cand_cnt, ccap);
-    if ((long long)h.cand_cnt <= ccap && n > 0) {
-      const double left = (count_target >= 0.0 ? count_target : (double)tau * h.Z) - h.mass_above;
-      const float w_lo = fmaxf(h.win_lo, lo), w_hi = fminf(h.win_hi, smax);
-      const int per = ((n + C - 1) / C + 3) & ~3, i0 = min(rank * per, n);
-      found = pool_search<T, true, int>(cluster, meet, pool_smem, cand + (long long)bh * ccap + i0, min(per, n - i0), w_lo, w_hi - w_lo, weight,
-                                        [&](double total, double& need) { need = left; return left > 0.0 && left <= total; }, cutoff);
-    }
-    if (!found) {
-      const long long per = ((P + C - 1) / C + 3) & ~3ll, i0 = min(rank * per, P);
-      pool_search<T, true, long long>(cluster, meet, pool_smem, scores + (long long)bh * P + i0, min(per, P - i0), lo, smax - lo, weight,
-                                      [&](double total, double& need) { need = count_target >= 0.0 ? count_target : (double)tau * total; return true; },
-                                      cutoff);
-    }
-  }
-  if (rank == 0 && threadIdx.x == 0) {
-    st[bh].cutoff_key = cutoff;
-    cutoff_per_head[bh] = key_float(cutoff);
-  }
-}
-
 // Row normalisation for the second reading of Eq. 4: out[i][j] = sigma * s[i][j] - logsumexp_j(sigma * s[i][:]),
 // the logarithm of S times the pair's probability when every query is normalised on its own.  One
 // warp per query row; the head-wide quantile search then runs on `out` with unit temperature.
@@ -1993,10 +1711,10 @@ struct SelectWs {
   Guards guards;
 };
 
-// Room for the list of one head: a sixteenth of its scores (a window holds up to 4 % of them).
+// Room for the list of one head: the pairs of one of the 512 level-0 bins.
 static long long cand_capacity(const Dims& D) {
   const long long P = (long long)D.S * D.Nb;
-  return std::max<long long>(4096, ((P / 16 + 3) / 4) * 4);
+  return std::max<long long>(4096, ((P / 32 + 3) / 4) * 4);
 }
 
 static SelectWs carve_select(const Dims& D, void* ws) {
@@ -2174,28 +1892,6 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     long long per_head = (P / 4 + 255) / 256;
     int gx = (int)std::min<long long>(std::max<long long>(per_head / 8, 1), std::max(1, sm_count() * 8 / D.BH));
     dim3 grid(gx, D.BH);
-    const bool window = use_cand && (long long)D.BH * P >= kWindowMin &&
-                        P <= kSampleShare * window_ctas(D.BH, P) * kSamples * kSampleThreads;
-    if (window) {
-      if (!range) {
-        launch_kernel(init_state_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, D.BH, nullptr, nullptr, nullptr, nullptr, nullptr);
-        launch_kernel(minmax_kernel, grid, 256, 0, st, scores, P, w.state);
-        count_launches(2);
-      }
-      const int C = window_ctas(D.BH, P);
-      // (not early behind the scores kernel, in whose SMs' spare room its CTAs would wait: 33K tokens, 3D, forward 603 us early, 559 not)
-      launch_cluster(early_rows(D), C, window_kernel, (unsigned)(D.BH * C), kSampleThreads, 0, st, scores, P, range, w.state, sigma, unit_w, tau,
-                     count_target, (float)((double)w.ccap / (double)P));
-      const int gx1 = (int)std::min<long long>(std::max<long long>(per_head / 16, 1), std::max(1, sm_count() * 3 / D.BH));
-      constexpr int T = 512, smem1 = kPoolFront * T, smem_stage = kWindowThreads / 32 * kWindowStage * (int)sizeof(float);
-      VMOBA_CUDA_OK(allow_smem(window_pass_kernel, smem_stage));
-      launch_kernel(early_rows(D), window_pass_kernel, dim3(gx1, D.BH), kWindowThreads, smem_stage, st, scores, P, w.state, sigma, unit_w,
-                    w.cand, w.ccap);
-      VMOBA_CUDA_OK(allow_smem(window_search_kernel<T>, smem1));
-      launch_cluster(true, C, window_search_kernel<T>, (unsigned)(D.BH * C), T, smem1, st, scores, P, w.state, sigma, unit_w, tau,
-                     count_target, w.cand, w.ccap, cutoff_per_head);
-      VMOBA_LAUNCH_OK(3);
-    } else {
     launch_kernel(init_state_kernel, (unsigned)(((long long)D.BH * kBins + 255) / 256), 256, 0, st, w.state, D.BH,
                   range, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey);
 
@@ -2223,7 +1919,6 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     launch_kernel(scan_kernel<2>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
                   w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
     VMOBA_LAUNCH_OK(7);
-    }
     VMOBA_CUDA_OK(allow_smem(mark_kernel, (int)smem));
     launch_kernel(mark_kernel, sgrid, kSegThreads, smem, st, scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg,
                   own_sb, mask_bits, w.seg_cnt, w.seg_total, w.tmask);

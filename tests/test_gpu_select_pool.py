@@ -9,7 +9,7 @@ from paper_2506_23858_b200 import binding as vb
 
 pytestmark = pytest.mark.gpu
 POOL_MAX = 1 << 20          # beyond every pool that the cluster kernel takes
-WINDOW_MIN = 6000000        # scores of all heads, from which on a sample is taken
+WINDOW_MIN = 6000000        # scores of all heads of a large pool
 
 
 def _run(shape, scores, rule, tau=0.25, topk=1, score_range=None, capacity=None):
@@ -108,7 +108,7 @@ def test_pool_kernel_agrees_with_the_passes_over_the_matrix(grid, block, rule, t
 @pytest.mark.parametrize("tau", [0.02, 0.25, 0.9])
 @pytest.mark.parametrize("values", ["flat", "sharp", "few hold the mass", "outlier", "one side"])
 def test_cutoff_of_large_pools_against_a_sort(values, tau):
-    """The sample's window finds the cutoff, or the search of the whole pool does, whatever the scores look like: against a sort in
+    """The passes over the matrix find the cutoff whatever the scores look like: against a sort in
     64 bits.  The sums of 3 million fp32 weights are off by 1e-6 of the whole."""
     shape = _shape(2, (12, 100, 53), (3, 5, 53))       # 63,600 queries x 80 blocks: ten million scores in all
     heads, S, Nb = shape.heads, shape.S, shape.n_blocks
