@@ -100,20 +100,16 @@ inline int sm_count() {
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Lets a kernel have so much dynamic shared memory.  The runtime is asked once per kernel, device and thread: a layer call of
-// ten launches asked six times.
+// Lets a kernel have up to `bytes` of dynamic shared memory, ahead of every launch that needs more than 48 KB.  The limit is one
+// setting per kernel and context for all threads, and a smaller one replaces a larger: every launch of a kernel gives the same number,
+// whatever its shape, or one thread's small call would make another's large one fail.  It is not remembered either (57 ns of
+// host time per call): a context that is new, after a reset or beside another, starts without it.
 template <typename... P>
 inline cudaError_t allow_smem(void (*kernel)(P...), int bytes) {
-  struct Seen { void (*kernel)(P...); int dev, bytes; };
-  thread_local Seen seen[16] = {};
-  int dev = 0;
-  if (cudaError_t e = cudaGetDevice(&dev)) return e;
-  Seen& s = seen[(reinterpret_cast<uintptr_t>(kernel) >> 4) % 16];
-  if (s.kernel == kernel && s.dev == dev && s.bytes >= bytes) return cudaSuccess;
-  if (cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) return e;
-  s = {kernel, dev, bytes};
-  return cudaSuccess;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
+// The number for kernels whose need depends on the shape: what a CTA may have (227 KB) less room for static shared memory.
+constexpr int kSmemMost = 222 * 1024;
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 

@@ -1807,7 +1807,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     a.mask_bits = mask_bits; a.tmask = w.tmask; a.seg_cnt = w.seg_cnt; a.seg_qoff = w.seg_qoff; a.kb_excl = w.kb_total;
     a.k_per_head = k_per_head; a.cutoff_per_head = cutoff_per_head;
     auto kernel = w.pool.T == 256 ? select_pool_kernel<decltype(tag)::value, 256> : select_pool_kernel<decltype(tag)::value, 512>;
-    VMOBA_CUDA_OK(allow_smem(kernel, (int)pool_smem));
+    VMOBA_CUDA_OK(allow_smem(kernel, kSmemMost));
     launch_cluster(true, w.pool.C, kernel, (unsigned)(D.BH * w.pool.C), w.pool.T, pool_smem, st, a);
     VMOBA_LAUNCH_OK(1);
     return VMOBA_OK;
@@ -1872,7 +1872,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
       if ((rc = pool_launch(VMOBA_POOL(kPoolMask), nullptr, 0, -1.0))) return rc;
     } else {
     launch_kernel(local_cutoff_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, cutoff_per_head, D.BH);
-    VMOBA_CUDA_OK(allow_smem(mark_from_mask_kernel, (int)smem));
+    VMOBA_CUDA_OK(allow_smem(mark_from_mask_kernel, kSmemMost));
     launch_kernel(mark_from_mask_kernel, sgrid, kSegThreads, smem, st, mask_bits, D.S, D.Nb, D.mask_words, QSEG, nseg,
                   w.seg_cnt, w.seg_total, w.tmask);
     VMOBA_LAUNCH_OK(2);
@@ -1919,7 +1919,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     launch_kernel(scan_kernel<2>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
                   w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
     VMOBA_LAUNCH_OK(7);
-    VMOBA_CUDA_OK(allow_smem(mark_kernel, (int)smem));
+    VMOBA_CUDA_OK(allow_smem(mark_kernel, kSmemMost));
     launch_kernel(mark_kernel, sgrid, kSegThreads, smem, st, scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg,
                   own_sb, mask_bits, w.seg_cnt, w.seg_total, w.tmask);
     VMOBA_LAUNCH_OK(1);
@@ -1933,7 +1933,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
                         : kStage;
   const size_t cols = (size_t)D.Nb * (QSEG >> 5);
   const size_t smem_fill = ((size_t)QSEG * D.mask_words + cols + 2 * (size_t)D.Nb + 1 + stage) * 4 + (stage + cols) * 2;
-  VMOBA_CUDA_OK(allow_smem(fill_kernel, (int)smem_fill));
+  VMOBA_CUDA_OK(allow_smem(fill_kernel, kSmemMost));
   long long nkb = (long long)D.BH * D.Nb;
   if (!pool) {
     launch_kernel(seg_prefix_kernel, (unsigned)(D.BH * ((D.Nb + 31) / 32)), 32 * std::min(32, (nseg + 7) / 8), 0, st,
