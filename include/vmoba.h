@@ -271,8 +271,9 @@ int vmoba_attn_fwd_raster(const vmoba_shape* shape, const void* q_bm, const void
  * dq, dk, dv [B, heads, S, head_dim] (dtype) from do_bm, the forward's o_bm (+ o_resid) and lse.
  * Queries without a selected block get dq = 0.  The paper states no gradient formula; this is
  * the softmax-attention gradient restricted to the selected pairs.  `capacity` is the one given
- * to vmoba_select (list positions at or beyond it are never read).  dk and dv repeat bit for bit; the blocks' parts of
- * a row of dq are added in fp32 in any order.
+ * to vmoba_select (list positions at or beyond it are never read).  dk and dv repeat bit for bit.  A row of dq is
+ * a sum in fp32 of parts that are added in any order: one per selected block (so that it repeats for a query with one or two
+ * blocks), but with bf16 and head_dim 128 one per 128 keys of a block.
  */
 int vmoba_attn_bwd(const vmoba_shape* shape, const void* q_bm, const void* k_bm, const void* v_bm,
                    const void* o_bm, const void* o_resid_or_null, const float* lse, const void* do_bm,

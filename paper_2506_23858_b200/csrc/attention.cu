@@ -126,12 +126,25 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
   float* acc = in_place ? reinterpret_cast<float*>(dq) : w.dq_acc;
   launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
                 (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), acc, nullptr, (T*)nullptr, nullptr, 0);
-  long long tiles = (D.sb + simt::kRows - 1) / simt::kRows;
-  VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dkdv_kernel<T, DH, false>, simt::kBwdSmem<DH>));
-  launch_kernel(early_simt(D, (double)cap * D.sb), simt::attn_bwd_dkdv_kernel<T, DH, false>, grid_for(n_kb * tiles, 4), simt::kThreads,
-                simt::kBwdSmem<DH>, st, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb,
-                D.BH, D.scale, cap, (T*)dk, (T*)dv, acc);
+  const long long tiles = (D.sb + simt::kRows - 1) / simt::kRows;
+  const bool early = early_simt(D, (double)cap * D.sb);
+  auto dkdv = tiles == 1                      ? simt::attn_bwd_dkdv_kernel<T, DH, false, simt::kDqTile>
+              : tiles <= simt::kDqClusterMax ? simt::attn_bwd_dkdv_kernel<T, DH, false, simt::kDqCluster>
+                                             : simt::attn_bwd_dkdv_kernel<T, DH, false, simt::kDqNone>;
+  const int C = tiles <= simt::kDqClusterMax ? (int)tiles : 1;
+  VMOBA_CUDA_OK(allow_smem(dkdv, simt::kBwdSmem<DH>));
+  launch_cluster(early, C, dkdv, C * grid_for(n_kb * tiles / C, std::max(1, 4 / C)), simt::kThreads, simt::kBwdSmem<DH>, st,
+                 (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb, D.BH, D.scale, cap,
+                 (T*)dk, (T*)dv, acc);
   count_launches(2);
+  if (tiles > simt::kDqClusterMax) {
+    launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);
+    VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dq_kernel<T, DH, false>, simt::kBwdSmem<DH>));
+    launch_kernel(early, simt::attn_bwd_dq_kernel<T, DH, false>, grid_for(cap / simt::kRows + n_kb, 4), simt::kThreads,
+                  simt::kBwdSmem<DH>, st, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, w.item_ptr,
+                  (int)n_kb, D.S, D.Nb, D.sb, D.BH, D.scale, cap, (T*)nullptr, acc);
+    count_launches(2);
+  }
   if (!in_place) {
     launch_kernel(early_rows(D), simt::cast_kernel<T>, grid_for((nq * DH / 4 + 255) / 256, 16), 256, 0, st, w.dq_acc,
                   (T*)dq, nq * DH / 4);
@@ -173,13 +186,14 @@ static int simt_dense(const Dims& D, const void* q, const void* k, const void* v
       VMOBA_LAUNCH_OK(1);
       return VMOBA_OK;
     }
-    VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dkdv_kernel<T, DH, true>, simt::kBwdSmem<DH>));
-    VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dq_kernel<T, DH>, simt::kBwdSmem<DH>));
-    launch_kernel(early, simt::attn_bwd_dkdv_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, simt::kBwdSmem<DH>, st,
+    VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dkdv_kernel<T, DH, true, simt::kDqNone>, simt::kBwdSmem<DH>));
+    VMOBA_CUDA_OK(allow_smem(simt::attn_bwd_dq_kernel<T, DH, true>, simt::kBwdSmem<DH>));
+    launch_kernel(early, simt::attn_bwd_dkdv_kernel<T, DH, true, simt::kDqNone>, grid_for(D.BH * tiles, 4), simt::kThreads, simt::kBwdSmem<DH>, st,
                   (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, D.S, 1, D.S,
                   D.BH, D.scale, 0, (T*)dk, (T*)dv, nullptr);
-    launch_kernel(early, simt::attn_bwd_dq_kernel<T, DH>, grid_for(D.BH * tiles, 4), simt::kThreads, simt::kBwdSmem<DH>, st, (const T*)q,
-                  (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, D.S, D.BH, D.scale, (T*)dq);
+    launch_kernel(early, simt::attn_bwd_dq_kernel<T, DH, true>, grid_for(D.BH * tiles, 4), simt::kThreads, simt::kBwdSmem<DH>, st,
+                  (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, nullptr, nullptr, nullptr, 0, D.S, 1, D.S, D.BH,
+                  D.scale, 0, (T*)dq, nullptr);
   }
   VMOBA_LAUNCH_OK(d_o ? 3 : 0);
   return VMOBA_OK;
