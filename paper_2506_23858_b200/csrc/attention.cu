@@ -120,9 +120,16 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
     VMOBA_GUARDS_CHECK(w.guards, status, st);
     return VMOBA_OK;
   }
-  // fp32 gradients are added up in place (unless dq takes the place of something that is still read), others in an accumulator; the
-  // row-dot pass clears it
-  const bool in_place = D.dtype == VMOBA_F32 && dq != q && dq != k && dq != v && dq != o && dq != d_o;
+  // fp32 gradients are added up in place (unless dq lies over something that is still read), others in an accumulator; the row-dot
+  // pass clears it
+  const size_t tensor = (size_t)nq * DH * sizeof(T);
+  auto apart = [&](const void* x, size_t bytes) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(dq), b = reinterpret_cast<uintptr_t>(x);
+    return a + tensor <= b || b + bytes <= a;
+  };
+  const bool in_place = D.dtype == VMOBA_F32 && apart(q, tensor) && apart(k, tensor) && apart(v, tensor) && apart(o, tensor) &&
+                        apart(d_o, tensor) && apart(lse, (size_t)nq * sizeof(float)) &&
+                        apart(kb_ptr, ((size_t)n_kb + 1) * sizeof(int)) && apart(q_idx, (size_t)cap * sizeof(int));
   float* acc = in_place ? reinterpret_cast<float*>(dq) : w.dq_acc;
   launch_kernel(early_rows(D), simt::rowdot_kernel<T, DH>, grid_for((nq + 7) / 8, 16), 256, 0, st, (const T*)o,
                 (const T*)o_resid, (const T*)d_o, nq, w.Dv, do_map, RowMap(), acc, nullptr, (T*)nullptr, nullptr, 0);

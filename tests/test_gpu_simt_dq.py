@@ -1,6 +1,6 @@
 """dq of the sparse CUDA-core backward (fp32, and bf16 with head_dim 64).  A query's row of it is the sum of one part per selected
 block, each part worked out in a fixed order: a query with one or two blocks has the same dq in every call, whatever the order in
-which the parts come."""
+which the parts come.  And dq may lie over an input: it is written when everything that is read has been."""
 import numpy as np
 import pytest
 import torch
@@ -49,6 +49,29 @@ def test_queries_of_one_or_two_blocks_repeat(sb, nb, d, dtype):
         assert torch.allclose(L.dq_bm.float(), first[0].float(), rtol=2.0 ** -7, atol=1e-4)
     assert (first[0][0][blocks == 0] == 0).all()
     L.check_status()
+
+
+@pytest.mark.parametrize("sb,nb", [(64, 4), (130, 3)])
+@pytest.mark.parametrize("shift", [0, 4, 64 * 5, -64 * 5])
+@pytest.mark.parametrize("over", ["q_bm", "k_bm", "v_bm", "o_bm", "do_bm", "lse", "kb_ptr", "q_idx"])
+def test_dq_may_lie_over_an_input(over, shift, sb, nb):
+    d = 64
+    L, blocks = _layer(sb, nb, d, "f32", heads=2, seed=5)
+    L.attn_bwd()
+    want, dk, dv = L.dq_bm.clone(), L.dk_bm.clone(), L.dv_bm.clone()
+    src = getattr(L, over)
+    n, pad = want.numel(), 1024
+    room = torch.zeros(max(n, src.numel()) + 2 * pad, device="cuda")
+    at = room[pad:pad + src.numel()].view(src.dtype).view(src.shape)
+    at.copy_(src)
+    setattr(L, over, at)
+    L.dq_bm = room[pad + shift:pad + shift + n].view(want.shape)
+    L.attn_bwd()
+    L.check_status()
+    few = blocks <= 2
+    assert torch.equal(L.dk_bm, dk) and torch.equal(L.dv_bm, dv)
+    assert torch.equal(L.dq_bm[0][few], want[0][few])
+    assert torch.allclose(L.dq_bm, want, rtol=1e-5, atol=1e-5)
 
 
 @pytest.mark.parametrize("d,dtype", [(64, "f32"), (128, "f32"), (64, "bf16")])
