@@ -100,13 +100,21 @@ __device__ __forceinline__ void for_each_score(const float* __restrict__ base, l
   }
 }
 
+// Key of a score under the head-wide rules: that of float_key, but a NaN without a sign has the place of -0 (one with a sign lies
+// below -inf), so that a diverged score neither sets the head's range nor is taken for its largest.  Said here, because what
+// float_key makes of a NaN is the compiler's choice: where the value is also a float, it may take `bits | sign` for a float negation,
+// which returns any NaN.
+__device__ __forceinline__ uint32_t pool_key(float f) {
+  return __float_as_int(f) > 0x7f800000 ? 0x7fffffffu : float_key(f);
+}
+
 __global__ void __launch_bounds__(256)
 minmax_kernel(const float* __restrict__ scores, long long P, HeadState* __restrict__ st) {
   if (!grid_begin()) return;
   const int bh = blockIdx.y;
   uint32_t kmin = 0xffffffffu, kmax = 0u;
   for_each_score<false>(scores + (long long)bh * P, P, [&](float s) {
-    uint32_t k = float_key(s);
+    const uint32_t k = pool_key(s);
     kmin = min(kmin, k);
     kmax = max(kmax, k);
   });
@@ -195,8 +203,9 @@ hist_kernel(const float* __restrict__ scores, long long P, const HeadState* __re
     int b = bin_at(hs, L, s);
     atomicAdd(&s_cnt[b], 1u);
     atomicAdd(&s_w[b], unit_w ? 1.0f : pair_weight(sigma, s, smax));
-    atomicMin(&s_min[b], float_key(s));
-    if (L == 1) atomicMax(&s_max[b], float_key(s));
+    const uint32_t key = pool_key(s);
+    atomicMin(&s_min[b], key);
+    if (L == 1) atomicMax(&s_max[b], key);
   });
   __syncthreads();
   if (L == 1 && list) {
@@ -410,7 +419,7 @@ mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, 
   // least 0.5 / Nb away from an integer, the rounding error far less (a fix-up step covers the rest)
   const float inv_nb = 1.0f / (float)Nb;
   auto mark = [&](long long i, float s) {
-    const bool sel = float_key(s) >= cutoff;
+    const bool sel = pool_key(s) >= cutoff;
     if (!sel && own_sb <= 0) return;          // the common case: no index arithmetic at all
     const int ii = (int)i;
     int ql = (int)(((float)ii + 0.5f) * inv_nb), j = ii - ql * Nb;
@@ -1346,7 +1355,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
       each(L, [&](float s) {
         const int b = bin_of(L, s);
         // lanes that are at the same score go in one update: scores that are all alike would queue for one bin
-        const uint32_t key = float_key(s);
+        const uint32_t key = pool_key(s);
         const unsigned int here = __activemask();
         int lanes = 1;
         if (__reduce_min_sync(here, key) == __reduce_max_sync(here, key)) {
@@ -1401,7 +1410,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
         // ---- the last few, each against all others: the largest key whose mass and that of those above reach the target
         each(L + 1, [&](float s) {
           const int to = s_at + atomicAdd(&s_n, 1);
-          const uint32_t key = float_key(s);
+          const uint32_t key = pool_key(s);
           for (int c = 0; c < C; ++c) cluster.map_shared_rank(s_final, c)[to] = key;
         });
         meet();
@@ -1430,8 +1439,8 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
       }
       uint32_t kmin = 0xffffffffu, kmax = 0u;
       each(L + 1, [&](float s) {
-        kmin = min(kmin, float_key(s));
-        kmax = max(kmax, float_key(s));
+        kmin = min(kmin, pool_key(s));
+        kmax = max(kmax, pool_key(s));
       });
       exchange(kmin, kmax);
       cutoff = kmin;
@@ -1494,7 +1503,7 @@ select_pool_kernel(const PoolArgs a) {
       __syncthreads();
 #pragma unroll 2
       for (int i = t; i < n; i += T) {
-        const uint32_t key = float_key(s_src[i]);
+        const uint32_t key = pool_key(s_src[i]);
         min_key = min(min_key, key);
         max_key = max(max_key, key);
       }
@@ -1548,11 +1557,7 @@ select_pool_kernel(const PoolArgs a) {
             int j = lane & ((1 << (31 - __clz(width))) - 1);
 #pragma unroll 4
             for (int r = 0; r < width; ++r) {
-              // (a NaN without a sign goes as -0, as it does in mark_kernel, whose key the compiler takes for a float operation)
-              const float x = s[j];
-              uint32_t key = float_key(x);
-              if (x != x && key > 0x80000000u) key = 0x7fffffffu;
-              if (key >= cutoff) word |= 1u << j;
+              if (pool_key(s[j]) >= cutoff) word |= 1u << j;
               if (++j == width) j = 0;
             }
             if (a.own_sb > 0) {             // the query's own block, if it is to be kept
