@@ -1417,17 +1417,17 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
         int G = 32;                      // threads per score
         while (G * K > T) G >>= 1;
         const int i = t / G, r = t & (G - 1);
-        float mass = 0.f;
+        double mass = 0.0;
         const uint32_t key = i < K ? s_final[i] : 0u;
         if (i < K)
 #pragma unroll 1
           for (int j = r; j < K; j += G) {
             const uint32_t other = s_final[j];
-            if (other >= key) mass += weight(key_float(other));
+            if (other >= key) mass += (double)weight(key_float(other));
           }
 #pragma unroll 1
         for (int o = G >> 1; o > 0; o >>= 1) mass += __shfl_xor_sync(0xffffffffu, mass, o);
-        const uint32_t best = __reduce_max_sync(0xffffffffu, i < K && (double)mass >= need ? key : 0u);
+        const uint32_t best = __reduce_max_sync(0xffffffffu, i < K && mass >= need ? key : 0u);
         const uint32_t least = __reduce_min_sync(0xffffffffu, i < K ? key : 0xffffffffu);
         if (lane == 0) {
           if (best) atomicMax(&s_best, best);

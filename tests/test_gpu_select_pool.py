@@ -1,6 +1,8 @@
 """The three routes to a head's cutoff: small pools go through one kernel, a cluster per head; of the larger ones those of six
 million scores in all through a sample, one pass and a search; the rest through histograms of the matrix.  A pool of m copies of the
 same scores has m times the mass above any score, so the cutoff is the same on all three and every copy keeps the same pairs."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -134,6 +136,27 @@ def test_cutoff_of_large_pools_against_a_sort(values, tau):
         assert k == int(out["k"][h])
         assert abs(float(cs[k - 1] - cs[want])) <= 2e-6 * float(cs[-1]), (h, k, want)
     assert int(out["status"]) == 0
+
+
+def test_last_candidates_of_a_small_pool_are_added_up_in_64_bits():
+    """One pair of weight 1, 30 of 2^-25 and one of 2^-26, all among the last candidates: which of the small ones reaches the target
+    does not show in fp32, where 1 + 2^-25 is 1.  (A candidate per warp lane, so that the mass of the pool is exact.)"""
+    heads = 8
+    shape = _shape(heads, (4, 64, 1), (1, 64, 1))
+    S, Nb = shape.S, shape.n_blocks
+    per_unit = 0.125 * math.log2(math.e)                       # octaves of weight per unit of score: scale 64 ** -0.5
+    x = torch.linspace(-2e6, -1.9e6, S * Nb, dtype=torch.float64)
+    x[0] = 0.0
+    for j in range(30):
+        x[1 + j] = -25.0 / per_unit * (1 + j * 2.0 ** -20)
+    x[31] = -26.0 / per_unit
+    x = x.float().reshape(1, S, Nb).expand(heads, S, Nb).contiguous().cuda()
+    v = x[0].flatten().double().sort(descending=True).values
+    cs = torch.exp(v / 8.0).cumsum(0)
+    for m in range(1, 15):
+        tau = 1.0 - m * 2.0 ** -24
+        out = _run(shape, x, vb.SELECT_THRESHOLD_GLOBAL, tau)
+        assert out["k"].tolist() == [int((cs < tau * cs[-1]).sum()) + 1] * heads, m
 
 
 @pytest.mark.parametrize("values", ["constant", "zeros", "two", "infinite", "nan"])
