@@ -1722,10 +1722,10 @@ static long long cand_capacity(const Dims& D) {
   return std::max<long long>(4096, ((P / 32 + 3) / 4) * 4);
 }
 
-static SelectWs carve_select(const Dims& D, void* ws) {
+static SelectWs lay_out_select(const Dims& D, const PoolPlan& pool, void* ws) {
   SelectWs w;
   Carver c(ws);
-  w.pool = pool_plan(D);
+  w.pool = pool;
   const int QSEG = w.QSEG = w.pool.C ? w.pool.QSEG : seg_queries(D.mask_words);
   const long long nseg = w.nseg = (D.S + QSEG - 1) / QSEG;
   w.state = c.take<HeadState>(D.BH);
@@ -1738,7 +1738,7 @@ static SelectWs carve_select(const Dims& D, void* ws) {
   w.seg_cnt = c.take<int>((size_t)D.BH * nseg * D.Nb);
   w.seg_total = c.take<int>((size_t)D.BH * nseg);
   w.seg_qoff = c.take<int>((size_t)D.BH * nseg + 1);
-  w.kb_total = c.take<int>((size_t)D.BH * (D.Nb + 1));
+  w.kb_total = c.take<int>((size_t)D.BH * (D.Nb + (w.pool.C ? 1 : 0)));
   w.base_bytes = c.total();
   w.ccap = w.pool.C ? 0 : cand_capacity(D);
   w.cand = c.take<float>((size_t)D.BH * w.ccap);
@@ -1747,12 +1747,26 @@ static SelectWs carve_select(const Dims& D, void* ws) {
   return w;
 }
 
-size_t select_ws_bytes(const Dims& D) { return carve_select(D, nullptr).bytes; }
+// The scratch that a call needs is that of the passes over the matrix, whichever route it takes: how many heads go to
+// select_pool_kernel depends on the GPU, and a size that was asked for on one (or without one) holds on another.  The small route
+// lives in the same bytes, without the bins, which leaves it room to spare.
+static SelectWs carve_select(const Dims& D, void* ws) {
+  const SelectWs passes = lay_out_select(D, PoolPlan(), ws);
+  const PoolPlan plan = pool_plan(D);
+  if (!plan.C) return passes;
+  SelectWs w = lay_out_select(D, plan, ws);
+  if (w.bytes > passes.base_bytes) return passes;
+  w.base_bytes = passes.base_bytes;
+  w.bytes = passes.bytes;
+  return w;
+}
+
+size_t select_ws_bytes(const Dims& D) { return lay_out_select(D, PoolPlan(), nullptr).bytes; }
 // the least the selection can work with (no candidate lists: levels 1 and 2 read the score matrix)
-size_t select_base_ws_bytes(const Dims& D) { return carve_select(D, nullptr).base_bytes; }
+size_t select_base_ws_bytes(const Dims& D) { return lay_out_select(D, PoolPlan(), nullptr).base_bytes; }
 // the row-normalised rule also keeps a transformed copy of the score matrix behind the common scratch
 size_t select_rownorm_ws_bytes(const Dims& D) {
-  return ((carve_select(D, nullptr).bytes + 255) / 256) * 256 + (size_t)D.BH * D.S * D.Nb * sizeof(float);
+  return ((select_ws_bytes(D) + 255) / 256) * 256 + (size_t)D.BH * D.S * D.Nb * sizeof(float);
 }
 
 }  // namespace vmoba
@@ -1785,7 +1799,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
   if (ws_bytes < (rownorm ? select_rownorm_ws_bytes(D) : (allow_base_ws ? w.base_bytes : w.bytes))) return VMOBA_ERR_WORKSPACE;
   // the candidate lists are the last slice: a caller with a fixed scratch area may have no room for them
   const bool use_cand = ws_bytes >= w.bytes;
-  if (!use_cand) { w.cand = nullptr; w.ccap = -1; if (w.guards.n > 0) w.guards.n -= 1; }
+  if (!use_cand && !w.pool.C) { w.cand = nullptr; w.ccap = -1; if (w.guards.n > 0) w.guards.n -= 1; }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const long long P = (long long)D.S * D.Nb;
   float sigma = D.scale;
