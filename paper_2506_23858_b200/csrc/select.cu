@@ -1181,9 +1181,10 @@ enum PoolSrc { kPoolScores, kPoolMask };
 constexpr int kPoolCtas = 8;                  // what every device schedules as one cluster
 constexpr int kPoolBins0 = 32, kPoolLevels = 3, kPoolFinal = 256;
 constexpr int kPoolSmemMax = 224 * 1024;
-// A second (fourth, eighth) CTA shares a head from more than 4,096 scores per CTA on, as long as all heads run at once: 12 heads x
+// A second (fourth, eighth) CTA shares a head from more than 4,096 scores per CTA on, as long as there is an SM for each: 12 heads x
 // 15,000 scores 19.0 us (one CTA 25), x 33,000 21.2 (16,384 per CTA 26; whole selection, 37.7 by the passes over the matrix).
 constexpr long long kPoolSlice = 4096;
+constexpr long long kPoolSecond[2] = {28672, 22528};      // scores per CTA of a cluster of four, of eight: see pool_plan()
 // Up to 2,048 scores a CTA has 256 threads, else 512: a step that every thread takes costs their number (x 1,024 scores 14.8
 // us with 256, 15.2 with 512, 16.7 with 1,024; x 15,000 in two CTAs 24.1, 21.6, 23.0).
 constexpr long long kPoolShort = 2048;
@@ -1662,10 +1663,18 @@ static int seg_queries(int mw) {
   return q;
 }
 
-// How select_pool_kernel divides a head (C = 0: it does not take it, the passes over the matrix do).  It takes what runs in one
-// wave: 12 heads x 215,000 scores 56.6 -> 38.7 us, but 40 heads of them, in two and a half, 89.6 -> 103.7.
+// How select_pool_kernel divides a head (C = 0: it does not take it, the passes over the matrix do).
+//
+// One CTA of 512 threads or two of 256 fit an SM by their registers, and 148 SMs hold 148 clusters of one, 74 of two, 33 of four and 15
+// of eight (a cluster lies within one GPC).  What runs in one wave is taken (us, small route / passes: 15 heads x 131,072 scores
+// 34 / 58, x 299,776 52 / 71; 148 x 19,968 38 / 75), and of what takes more
+//   * as many CTAs as shared memory and 2,048 threads per SM would let run: 296 heads x 1,024 scores 21 / 60, 740, in three waves,
+//     38 / 95, 296 x 7,488 48 / 83;
+//   * a second wave of clusters of four or eight while their slices are short (kPoolSecond): 18 heads x 162,816 60 / 65, but 16 x
+//     215,040 71 / 67 and x 299,776 83 / 73; 37 x 107,520 69 / 73, but x 149,760 83 / 79.
+// The per-query rules' masks (`scores` false) have no slice to search: 18 heads x 299,776 49 / 50, 37 x 149,760 49 / 52.
 struct PoolPlan { int C, T, QSEG, nseg, segs_per; size_t smem, smem_mask; };
-static PoolPlan pool_plan(const Dims& D) {
+static PoolPlan pool_plan(const Dims& D, bool scores) {
   PoolPlan p = {};
   const long long P = (long long)D.S * D.Nb;
   if (P > kPoolCtas * (long long)kPoolSmemMax / 4 || D.Nb > 1024) return p;
@@ -1682,9 +1691,11 @@ static PoolPlan pool_plan(const Dims& D) {
     p.smem = kPoolFront * p.T + p.smem_mask + 4 * (size_t)p.segs_per * p.QSEG * D.Nb;
     return p.smem <= (size_t)kPoolSmemMax;
   };
-  auto at_once = [&](int C) {
-    const long long per_sm = std::min<long long>((227 * 1024) / (long long)(p.smem + 5 * 1024), 2048 / p.T);
-    return (long long)D.BH * C <= sm_count() * per_sm;
+  auto takes = [&](int C) {
+    const long long per_sm = std::min<long long>((227 * 1024) / (long long)(p.smem + 5 * 1024), 2048 / p.T), sms = sm_count();
+    const long long whole = C == 8 ? sms * 5 / 6 : C == 4 ? sms * 9 / 10 : sms;      // SMs that clusters of C come to fill
+    if (scores && C >= 4 && (long long)D.BH * C > whole && P / C > kPoolSecond[C == 8]) return false;
+    return (long long)D.BH * C <= sms * per_sm;
   };
   int C = 1;
   while (C < kPoolCtas && P / C > kPoolSlice && (long long)D.BH * 2 * C <= sm_count()) C *= 2;
@@ -1692,7 +1703,7 @@ static PoolPlan pool_plan(const Dims& D) {
     if (C == kPoolCtas) { p.C = 0; return p; }
     C *= 2;
   }
-  if (!at_once(C)) p.C = 0;
+  if (!takes(C)) p.C = 0;
   return p;
 }
 
@@ -1750,9 +1761,9 @@ static SelectWs lay_out_select(const Dims& D, const PoolPlan& pool, void* ws) {
 // The scratch that a call needs is that of the passes over the matrix, whichever route it takes: how many heads go to
 // select_pool_kernel depends on the GPU, and a size that was asked for on one (or without one) holds on another.  The small route
 // lives in the same bytes, without the bins, which leaves it room to spare.
-static SelectWs carve_select(const Dims& D, void* ws) {
+static SelectWs carve_select(const Dims& D, bool scores, void* ws) {
   const SelectWs passes = lay_out_select(D, PoolPlan(), ws);
-  const PoolPlan plan = pool_plan(D);
+  const PoolPlan plan = pool_plan(D, scores);
   if (!plan.C) return passes;
   SelectWs w = lay_out_select(D, plan, ws);
   if (w.bytes > passes.base_bytes) return passes;
@@ -1795,7 +1806,7 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
   if (!aligned16(scores) || !aligned16(ws)) return VMOBA_ERR_ARG;
   if (capacity <= 0 || capacity > (int64_t)INT32_MAX) return VMOBA_ERR_ARG;
   if (D.Nb > 8192 || (local && D.Nb > 32 * kLocalMaxWords)) return VMOBA_ERR_SHAPE;
-  SelectWs w = carve_select(D, ws);
+  SelectWs w = carve_select(D, !local, ws);
   if (ws_bytes < (rownorm ? select_rownorm_ws_bytes(D) : (allow_base_ws ? w.base_bytes : w.bytes))) return VMOBA_ERR_WORKSPACE;
   // the candidate lists are the last slice: a caller with a fixed scratch area may have no room for them
   const bool use_cand = ws_bytes >= w.bytes;

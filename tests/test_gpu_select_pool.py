@@ -196,6 +196,37 @@ def test_pool_kernel_special_scores(values, rule, tau, topk, total):
         assert np.array_equal(ma[0, 5], mb[0, 0, 5]) and ma[1, 9, 2] == mb[1, 0, 9, 2]
 
 
+# heads, grid, block, whether the heads go to one cluster each (with fill: two launches): heads of a wave and of several, more than the
+# 32 heads before it that a warp adds up at a time; two waves of clusters of eight and of four, of short slices and of long ones
+ROUTES = [(33, (4, 8, 8), (1, 8, 8), True), (34, (4, 8, 8), (1, 8, 8), True), (70, (3, 43, 8), (3, 43, 1), True), (149, (4, 8, 8), (1, 8, 8), True),
+          (740, (4, 8, 8), (1, 8, 8), True), (741, (4, 8, 8), (1, 8, 8), False),
+          (15, (16, 28, 30), (1, 28, 30), True), (16, (16, 28, 30), (1, 28, 30), False), (18, (16, 16, 32), (1, 16, 32), True),
+          (33, (16, 19, 30), (1, 19, 30), True), (34, (16, 19, 30), (1, 19, 30), False), (37, (16, 14, 30), (1, 14, 30), True)]
+
+
+@pytest.mark.parametrize("heads,grid,block,small", ROUTES)
+@pytest.mark.parametrize("rule,topk", [(vb.SELECT_THRESHOLD_GLOBAL, 0), (vb.SELECT_TOPK_GLOBAL, 2), (vb.SELECT_TOPK_LOCAL, 2)])
+def test_many_heads(heads, grid, block, small, rule, topk):
+    """The lists of many heads, on both sides of the rule that gives them to a cluster each; each head's pairs are those that it has
+    by itself."""
+    shape, one = _shape(heads, grid, block), _shape(1, grid, block)
+    S, Nb = shape.S, shape.n_blocks
+    g = torch.Generator(device="cuda").manual_seed(heads)
+    x = 3.0 * torch.randn((heads, S, Nb), generator=g, device="cuda")
+    score_range = torch.stack([x.amin((1, 2)), x.amax((1, 2))], 1).contiguous()
+    before = vb.kernel_launches()
+    out = _run(shape, x, rule, 0.25, topk, score_range)
+    if rule != vb.SELECT_TOPK_LOCAL:
+        assert (vb.kernel_launches() - before == 2) == small
+    m = _mask(shape, out)
+    _check_lists(shape, out, m)
+    assert int(out["status"]) == 0
+    for h in {0, heads // 3, heads - 2, heads - 1}:
+        alone = _run(one, x[h:h + 1].contiguous(), rule, 0.25, topk, score_range[h:h + 1].contiguous())
+        # (the cutoff of a mass may fall a pair further: sums of fp32 weights in another order)
+        assert (_mask(one, alone)[0] != m[h]).sum() <= (1 if rule == vb.SELECT_THRESHOLD_GLOBAL else 0)
+
+
 @pytest.mark.parametrize("rule,topk", [(vb.SELECT_TOPK_LOCAL, 3), (vb.SELECT_THRESHOLD_LOCAL, 0),
                                        (vb.SELECT_THRESHOLD_GLOBAL | vb.SELECT_KEEP_OWN_BLOCK, 0)])
 @pytest.mark.parametrize("grid,block", SHAPES[1:])
