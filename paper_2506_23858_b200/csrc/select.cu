@@ -791,17 +791,28 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
         for (int i = 0; i < MW; ++i) n += x[i] >= c ? 1 : 0;
         return __reduce_add_sync(0xffffffffu, n);
       };
+      // First step: a share of the way from the threshold before to the row's maximum, which holds more of the row the larger k is.
+      // 280 blocks x 201,600 rows, whole selection, 1/8 against 1/16: rows alike, k = 9, 134 / 131 us, k = 2 112 / 113; at random, k = 9,
+      // 150 / 152, k = 2 135 / 139.
+      // Where the threshold before lies at or above the row's largest score, or every score reaches it, the row is unlike the one
+      // before, and the search starts from the middle of its own range: rows a thousand apart 181 us (198 without; 140 blocks 136 and
+      // 154, 48 blocks 113 and 134).
       float mid = t_prev, step = (k > 4 ? 0.0625f : 0.125f) * (hi - mid);
       bool below = false, above = false, go = mid < hi;
+      int n = 0;
+      if (go) {
+        n = count_ge(mid);
+        go = n < Nb;
+      }
       if (!go) {
         lo = smallest();
         step = 0.015625f * (hi - lo);
         go = split_interval(lo, hi, mid);
-        if (!go && count_ge(hi) >= k) lo = hi;      // two neighbouring values at most: is the larger one the k-th?
+        if (go) n = count_ge(mid);
+        else if (count_ge(hi) >= k) lo = hi;        // two neighbouring values at most: is the larger one the k-th?
       }
       if (go) {
         for (;;) {
-          const int n = count_ge(mid);
           if (n >= k) { lo = mid; below = true; } else { hi = mid; above = true; }
           if (n == k) { exact = true; break; }
           const float far = below ? lo + step : hi - step;
@@ -813,6 +824,7 @@ select_topk_kernel(const float* __restrict__ scores, int S, int Nb, int mw, int 
             if (!above && count_ge(hi) >= k) lo = hi;
             break;
           }
+          n = count_ge(mid);
         }
         t_prev = lo;
       }

@@ -57,3 +57,30 @@ def test_exactly_k_blocks_in_key_order(nb):
         assert L.k_per_head.tolist() == [S * kk] * heads
         cutoff = np.where(want, keys, np.uint32(0xffffffff)).reshape(heads, -1).min(axis=1)
         assert np.array_equal(_keys(L.cutoff.cpu().numpy()), cutoff), k
+
+
+@pytest.mark.parametrize("nb", [40, 140, 280])
+def test_rows_unlike_the_one_before(nb):
+    """The search starts from the threshold of the row before: rows of other scales, beyond and below it, and up to 1e38 away."""
+    heads, S = 2, 24 * nb
+    shape = vb.make_shape(1, heads, 64, (nb, S // nb, 1), (1, S // nb, 1), "f32")
+    L = VmobaLayer(shape, heads * S * nb)
+    rng = np.random.default_rng(nb)
+    x = rng.standard_normal((heads, S, nb)).astype(np.float32)
+    kind = rng.integers(0, 8, (heads, S, 1))
+    size = np.float32(10.0) ** rng.integers(-30, 30, (heads, S, 1)).astype(np.float32)
+    x = np.where(kind == 0, x * size, x)
+    x = np.where(kind == 1, x + 1000 * rng.standard_normal((heads, S, 1)).astype(np.float32), x)
+    x = np.where(kind == 2, np.where(np.arange(nb) == 3, np.float32(2.0), np.float32(1e-4) * x), x)
+    x = np.where(kind == 3, np.float32(1e38) * np.sign(x), x)      # (ties)
+    x = np.where(kind == 4, np.minimum(x, 0) - np.float32(1e38), x)
+    x = np.where(kind == 5, np.where(np.arange(nb) % 3 == 0, np.float32(-np.inf), x), x).astype(np.float32)
+    L.scores.copy_(torch.from_numpy(x).view(L.scores.shape))
+    keys = _keys(x)
+    order = np.argsort(-keys.astype(np.int64), axis=2, kind="stable")
+    for k in (1, 2, 5, 9, nb // 2):
+        L.select_rule(vb.SELECT_TOPK_LOCAL, topk=k)
+        L.check_status()
+        want = np.zeros(x.shape, dtype=bool)
+        np.put_along_axis(want, order[..., :k], True, axis=2)
+        assert np.array_equal(U.unpack_mask(L.mask_bits, heads, S, nb), want), k
