@@ -1237,18 +1237,18 @@ __device__ __noinline__ T pool_exclusive(T x, T* s_warp) {
   return __shfl_sync(0xffffffffu, before, 0) + (inc - x);
 }
 
-// The search for a head's cutoff among the scores src[0 .. n) of every CTA of a cluster, which lie in [lo, lo + span] (shared or
-// global memory; I: a type that holds n).  target(total, need): the mass to be covered, given that of all these scores; false: they
-// cannot hold the cutoff, and the search ends.  front: kPoolFront * T bytes of shared memory.
-template <int T, typename I, typename Meet, typename Weight, typename Target>
-__device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& cluster, Meet meet, unsigned char* front, const float* src,
-                                            I n, float lo, float span, Weight weight, Target target, uint32_t& cutoff) {
+// The search for a head's cutoff among the scores src[0 .. n) of every CTA of a cluster, in shared memory, which lie in [lo, lo +
+// span].  target(total): the mass to be covered, given that of all these scores.  front: kPoolFront * T bytes of shared memory.
+template <int T, typename Meet, typename Weight, typename Target>
+__device__ __forceinline__ uint32_t pool_search(cooperative_groups::cluster_group& cluster, Meet meet, unsigned char* front, const float* src,
+                                                int n, float lo, float span, Weight weight, Target target) {
   constexpr int kLevelBytes = 8 * T, kList = (kPoolFront * T - kPoolLevels * kLevelBytes) / 4;
   __shared__ double s_w0[kPoolCtas][kPoolBins0], s_dsum[32], s_above;
   __shared__ uint32_t s_key[kPoolCtas][2], s_final[kPoolFinal], s_best, s_least;
   __shared__ int s_crossed, s_lowest, s_n, s_at, s_k, s_cross[kPoolLevels];
-  __shared__ I s_sum[32], s_listed;
+  __shared__ int s_sum[32], s_listed;
   __shared__ float s_anchor[kPoolLevels], s_inv[kPoolLevels];
+  uint32_t cutoff = 0u;
   const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   float* s_own = reinterpret_cast<float*>(front);        // [kPoolBins0][threads]
@@ -1269,8 +1269,8 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
     meet();
     for (int c = 0; c < C; ++c) { least = min(least, s_key[c][0]); most = max(most, s_key[c][1]); }
   };
-  auto stream = [&](const float* from, I count, auto f) {
-    I i = t;
+  auto stream = [&](const float* from, int count, auto f) {
+    int i = t;
 #pragma unroll 4
     for (; i < count; i += T) f(from[i]);
   };
@@ -1317,7 +1317,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
       if (lane >= o) inc += v;
     }
     const double total = __shfl_sync(0xffffffffu, inc, 31), excl = inc - x;
-    if (!target(total, need)) return false;
+    need = target(total);
     const unsigned int hit = __ballot_sync(0xffffffffu, x > 0.0 && excl < need && inc >= need);
     const unsigned int occupied = __ballot_sync(0xffffffffu, x > 0.0);
     const int e = hit ? __ffs(hit) - 1 : occupied ? 31 - __clz(occupied) : kPoolBins0 - 1;
@@ -1332,9 +1332,9 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
       return (cross0 == 0 || y >= y_lo) && !(y >= y_hi);
     };
     float* s_list = reinterpret_cast<float*>(front + kPoolLevels * kLevelBytes);
-    I mine = 0;
+    int mine = 0;
     stream(src, n, [&](float s) { mine += inside(s) ? 1 : 0; });
-    I at = pool_exclusive(mine, s_sum);
+    int at = pool_exclusive(mine, s_sum);
     if (t == T - 1) s_listed = at + mine;
     if (mine && at + mine <= kList)
       stream(src, n, [&](float s) { if (inside(s)) s_list[at++] = s; });
@@ -1345,7 +1345,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
     __syncthreads();
     const bool over = s_listed > kList;
     const float* in_bin = over ? src : s_list;
-    const I n_in = over ? n : s_listed;
+    const int n_in = over ? n : s_listed;
     auto bin_of = [&](int L, float s) {
       const float x = (s - s_anchor[L]) * s_inv[L];
       return x > 0.f ? (int)fminf(x, (float)(T - 1)) : 0;
@@ -1358,7 +1358,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
         if (in) f(s);
       };
 #pragma unroll 1
-      for (I i = t; i < n_in; i += T) look(in_bin[i]);
+      for (int i = t; i < n_in; i += T) look(in_bin[i]);
     };
     // ---- a bin of it per thread; thread t looks after bin T - 1 - t
 #pragma unroll 1
@@ -1382,8 +1382,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
       meet();
       const int b = T - 1 - t;
       double x = 0.0;
-      I k = 0;
-      int before = 0;
+      int k = 0, before = 0;
 #pragma unroll
       for (int c0 = 0; c0 < kPoolCtas; c0 += 4) {
         if (c0 >= C) break;
@@ -1400,7 +1399,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
           if (c0 + c < C) {
             x += (double)ws[c];
             if (c0 + c < rank) before += (int)ks[c];
-            k += (I)ks[c];
+            k += (int)ks[c];
           }
       }
       const double excl = pool_exclusive(x, s_dsum);
@@ -1410,7 +1409,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
       __syncthreads();
       const int e = s_crossed != INT32_MAX ? s_crossed : s_lowest >= 0 ? s_lowest : T - 1;
       if (t == e) {
-        s_above = excl; s_k = (int)min(k, (I)INT32_MAX); s_at = before; s_cross[L] = T - 1 - e;
+        s_above = excl; s_k = k; s_at = before; s_cross[L] = T - 1 - e;
         if (L + 1 < kPoolLevels) {
           s_anchor[L + 1] = s_inv[L] > 0.f ? s_anchor[L] + (float)(T - 1 - e) / s_inv[L] : s_anchor[L];
           s_inv[L + 1] = fminf(s_inv[L] * (float)T, 1e30f);
@@ -1460,7 +1459,7 @@ __device__ __forceinline__ bool pool_search(cooperative_groups::cluster_group& c
       if (kmin == kmax) break;
     }
   }
-  return true;
+  return cutoff;
 }
 
 template <PoolSrc SRC, int T>
@@ -1535,10 +1534,9 @@ select_pool_kernel(const PoolArgs a) {
     const bool unit_w = a.unit_w != 0;
     cutoff = min_key;                      // everything, where tau = 1
     if (a.tau < 1.0f) {
-      pool_search<T, int>(cluster, meet, pool_smem, s_src, n, lo, smax - lo,
-                          [&](float s) { return unit_w ? 1.0f : pair_weight(a.sigma, s, smax); },
-                          [&](double total, double& need) { need = a.count_target >= 0.0 ? a.count_target : (double)a.tau * total; return true; },
-                          cutoff);
+      cutoff = pool_search<T>(cluster, meet, pool_smem, s_src, n, lo, smax - lo,
+                              [&](float s) { return unit_w ? 1.0f : pair_weight(a.sigma, s, smax); },
+                              [&](double total) { return a.count_target >= 0.0 ? a.count_target : (double)a.tau * total; });
     } else {
       __syncthreads();
     }
@@ -1913,11 +1911,11 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     if (pool) {
       if ((rc = pool_launch(VMOBA_POOL(kPoolMask), nullptr, 0, -1.0))) return rc;
     } else {
-    launch_kernel(local_cutoff_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, cutoff_per_head, D.BH);
-    VMOBA_CUDA_OK(allow_smem(mark_from_mask_kernel, kSmemMost));
-    launch_kernel(mark_from_mask_kernel, sgrid, kSegThreads, smem, st, mask_bits, D.S, D.Nb, D.mask_words, QSEG, nseg,
-                  w.seg_cnt, w.seg_total, w.tmask);
-    VMOBA_LAUNCH_OK(2);
+      launch_kernel(local_cutoff_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, cutoff_per_head, D.BH);
+      VMOBA_CUDA_OK(allow_smem(mark_from_mask_kernel, kSmemMost));
+      launch_kernel(mark_from_mask_kernel, sgrid, kSegThreads, smem, st, mask_bits, D.S, D.Nb, D.mask_words, QSEG, nseg,
+                    w.seg_cnt, w.seg_total, w.tmask);
+      VMOBA_LAUNCH_OK(2);
     }
   } else {
     // head-wide rules: weighted quantile of the pool (unit weights and a pair budget for top-k)
@@ -1930,41 +1928,41 @@ static int select_impl(const vmoba_shape* shape, const float* scores, const floa
     if (pool) {
       if ((rc = pool_launch(VMOBA_POOL(kPoolScores), range, unit_w, count_target))) return rc;
     } else {
-    // enough CTAs per head to fill the machine, few enough that the per-CTA flush stays small
-    long long per_head = (P / 4 + 255) / 256;
-    int gx = (int)std::min<long long>(std::max<long long>(per_head / 8, 1), std::max(1, sm_count() * 8 / D.BH));
-    dim3 grid(gx, D.BH);
-    launch_kernel(init_state_kernel, (unsigned)(((long long)D.BH * kBins + 255) / 256), 256, 0, st, w.state, D.BH,
-                  range, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey);
+      // enough CTAs per head to fill the machine, few enough that the per-CTA flush stays small
+      long long per_head = (P / 4 + 255) / 256;
+      int gx = (int)std::min<long long>(std::max<long long>(per_head / 8, 1), std::max(1, sm_count() * 8 / D.BH));
+      dim3 grid(gx, D.BH);
+      launch_kernel(init_state_kernel, (unsigned)(((long long)D.BH * kBins + 255) / 256), 256, 0, st, w.state, D.BH,
+                    range, w.g_cnt, w.g_w, w.g_minkey, w.g_maxkey);
 
-    if (!range) {
-      launch_kernel(minmax_kernel, grid, 256, 0, st, scores, P, w.state);
-      launch_kernel(setup_level0_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, D.BH);
-      count_launches(2);
-    }
-    {
-      constexpr int smem0 = kBins0 * kRep * (int)sizeof(float);
-      VMOBA_CUDA_OK(allow_smem(hist0_kernel, smem0));
-      // three 512-thread CTAs per SM hold their replicated bins side by side
-      int gx0 = (int)std::min<long long>(std::max<long long>(per_head / 16, 1), std::max(1, sm_count() * 3 / D.BH));
-      launch_kernel(early_rows(D), hist0_kernel, dim3(gx0, D.BH), 512, smem0, st, scores, P, w.state, sigma, unit_w,
-                    w.g_w);
-    }
-    launch_kernel(scan_kernel<0>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
-                  w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
-    launch_kernel(hist_kernel<1>, grid, 256, 0, st, scores, P, w.state, sigma, unit_w, w.g_cnt, w.g_w, w.g_minkey,
-                  w.g_maxkey, w.cand, w.ccap, &w.state->cand_cnt);
-    launch_kernel(scan_kernel<1>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
-                  w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
-    launch_kernel(hist_kernel<2>, grid, 256, 0, st, scores, P, w.state, sigma, unit_w, w.g_cnt, w.g_w, w.g_minkey,
-                  w.g_maxkey, w.cand, w.ccap, &w.state->cand_cnt);
-    launch_kernel(scan_kernel<2>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
-                  w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
-    VMOBA_LAUNCH_OK(7);
-    VMOBA_CUDA_OK(allow_smem(mark_kernel, kSmemMost));
-    launch_kernel(mark_kernel, sgrid, kSegThreads, smem, st, scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg,
-                  own_sb, mask_bits, w.seg_cnt, w.seg_total, w.tmask);
-    VMOBA_LAUNCH_OK(1);
+      if (!range) {
+        launch_kernel(minmax_kernel, grid, 256, 0, st, scores, P, w.state);
+        launch_kernel(setup_level0_kernel, (D.BH + 127) / 128, 128, 0, st, w.state, D.BH);
+        count_launches(2);
+      }
+      {
+        constexpr int smem0 = kBins0 * kRep * (int)sizeof(float);
+        VMOBA_CUDA_OK(allow_smem(hist0_kernel, smem0));
+        // three 512-thread CTAs per SM hold their replicated bins side by side
+        int gx0 = (int)std::min<long long>(std::max<long long>(per_head / 16, 1), std::max(1, sm_count() * 3 / D.BH));
+        launch_kernel(early_rows(D), hist0_kernel, dim3(gx0, D.BH), 512, smem0, st, scores, P, w.state, sigma, unit_w,
+                      w.g_w);
+      }
+      launch_kernel(scan_kernel<0>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
+                    w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
+      launch_kernel(hist_kernel<1>, grid, 256, 0, st, scores, P, w.state, sigma, unit_w, w.g_cnt, w.g_w, w.g_minkey,
+                    w.g_maxkey, w.cand, w.ccap, &w.state->cand_cnt);
+      launch_kernel(scan_kernel<1>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
+                    w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
+      launch_kernel(hist_kernel<2>, grid, 256, 0, st, scores, P, w.state, sigma, unit_w, w.g_cnt, w.g_w, w.g_minkey,
+                    w.g_maxkey, w.cand, w.ccap, &w.state->cand_cnt);
+      launch_kernel(scan_kernel<2>, D.BH, 1024, 0, st, w.state, tau, count_target, w.g_cnt, w.g_w, w.g_minkey,
+                    w.g_maxkey, k_per_head, cutoff_per_head, w.ccap);
+      VMOBA_LAUNCH_OK(7);
+      VMOBA_CUDA_OK(allow_smem(mark_kernel, kSmemMost));
+      launch_kernel(mark_kernel, sgrid, kSegThreads, smem, st, scores, w.state, D.S, D.Nb, D.mask_words, QSEG, nseg,
+                    own_sb, mask_bits, w.seg_cnt, w.seg_total, w.tmask);
+      VMOBA_LAUNCH_OK(1);
     }
   }
 #undef VMOBA_POOL
