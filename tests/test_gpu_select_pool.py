@@ -1,6 +1,6 @@
-"""The three routes to a head's cutoff: small pools go through one kernel, a cluster per head; of the larger ones those of six
-million scores in all through a sample, one pass and a search; the rest through histograms of the matrix.  A pool of m copies of the
-same scores has m times the mass above any score, so the cutoff is the same on all three and every copy keeps the same pairs."""
+"""The two routes to a head's cutoff: small pools go through one kernel, a cluster per head, larger ones through histograms of the
+matrix.  A pool of m copies of the same scores has m times the mass above any score, so the cutoff is the same on both and every copy
+keeps the same pairs."""
 import math
 
 import numpy as np
@@ -11,7 +11,6 @@ from paper_2506_23858_b200 import binding as vb
 
 pytestmark = pytest.mark.gpu
 POOL_MAX = 1 << 20          # beyond every pool that the cluster kernel takes
-WINDOW_MIN = 6000000        # scores of all heads of a large pool
 
 
 def _run(shape, scores, rule, tau=0.25, topk=1, score_range=None, capacity=None):
@@ -54,14 +53,12 @@ def _check_lists(shape, out, m):
     assert np.array_equal(out["q_pairs"][:n].cpu().numpy(), place[m])
 
 
-def _copies(small, total):
-    """The shape with further query rows that makes the pool larger than POOL_MAX, with fewer or with more than `total` scores in
-    all: the same blocks per row, `copies` times the frames and the frames per block."""
-    P = small.S * small.n_blocks
-    copies = (POOL_MAX if total is None else max(POOL_MAX, total // small.heads)) // P + 1
+def _copies(small):
+    """The shape with further query rows that makes the pool larger than POOL_MAX: the same blocks per row, `copies` times the frames
+    and the frames per block."""
+    copies = POOL_MAX // (small.S * small.n_blocks) + 1
     big = _shape(small.heads, (small.T * copies, small.H, small.W), (small.bT * copies, small.bH, small.bW))
     assert big.n_blocks == small.n_blocks and big.S * big.n_blocks > POOL_MAX
-    assert (big.S * big.n_blocks * big.heads >= WINDOW_MIN) == (total is not None)
     return copies, big
 
 
@@ -75,24 +72,25 @@ def _shape(heads, grid, block):
 
 
 # grid, block: one CTA; several, some of them without a segment; rows of an odd number of blocks (slices off 16-byte boundaries); short
-# rows; rows of several mask words; slices that stay in shared memory and, from 320K scores on, that do not
+# rows; rows of several mask words; up to the largest slices that shared memory holds (319,488 scores in eight CTAs)
 SHAPES = [((1, 7, 9), (1, 1, 1)), ((4, 8, 8), (1, 8, 8)), ((3, 43, 8), (3, 43, 1)), ((5, 13, 11), (1, 13, 11)), ((2, 33, 37), (1, 3, 37)),
-          ((8, 24, 35), (2, 3, 35)), ((7, 40, 35), (7, 10, 5)), ((6, 40, 35), (3, 10, 5)), ((5, 25, 34), (5, 5, 2))]
+          ((8, 24, 35), (2, 3, 35)), ((7, 40, 35), (7, 10, 5)), ((20, 17, 6), (1, 17, 1)), ((8, 24, 52), (2, 6, 26))]
 
 
 @pytest.mark.parametrize("grid,block", SHAPES)
 @pytest.mark.parametrize("rule,tau,topk", [(vb.SELECT_THRESHOLD_GLOBAL, 0.25, 0), (vb.SELECT_THRESHOLD_GLOBAL, 1.0, 0),
                                            (vb.SELECT_TOPK_GLOBAL, 0.0, 3)])
-@pytest.mark.parametrize("total", [None, WINDOW_MIN])
-def test_pool_kernel_agrees_with_the_passes_over_the_matrix(grid, block, rule, tau, topk, total):
+def test_pool_kernel_agrees_with_the_passes_over_the_matrix(grid, block, rule, tau, topk):
     heads = 3
     small = _shape(heads, grid, block)
     S, Nb = small.S, small.n_blocks
-    copies, large = _copies(small, total)
+    copies, large = _copies(small)
     g = torch.Generator(device="cuda").manual_seed(S * Nb)
     x = 4.0 * torch.randn((heads, S, Nb), generator=g, device="cuda")
+    before = vb.kernel_launches()
     a = _run(small, x, rule, tau, topk)
     ranged = _run(small, x, rule, tau, topk, score_range=torch.stack([x.amin((1, 2)), x.amax((1, 2))], 1).contiguous())
+    assert vb.kernel_launches() - before == 4                  # the two kernels of the small route, twice
     b = _run(large, _repeat(x, copies), rule, tau, topk, capacity=int(heads * large.S * Nb))
     ma = _mask(small, a)
     for out in (a, ranged):
@@ -109,10 +107,12 @@ def test_pool_kernel_agrees_with_the_passes_over_the_matrix(grid, block, rule, t
 
 @pytest.mark.parametrize("tau", [0.02, 0.25, 0.9])
 @pytest.mark.parametrize("values", ["flat", "sharp", "few hold the mass", "outlier", "one side"])
-def test_cutoff_of_large_pools_against_a_sort(values, tau):
-    """The passes over the matrix find the cutoff whatever the scores look like: against a sort in
-    64 bits.  The sums of 3 million fp32 weights are off by 1e-6 of the whole."""
-    shape = _shape(2, (12, 100, 53), (3, 5, 53))       # 63,600 queries x 80 blocks: ten million scores in all
+# 63,600 queries x 80 blocks (ten million scores in all: the passes), and small pools of one, four and eight CTAs
+@pytest.mark.parametrize("grid,block", [((12, 100, 53), (3, 5, 53)), ((4, 13, 11), (1, 13, 11)), ((6, 12, 26), (3, 6, 13)), ((8, 24, 35), (2, 3, 35))])
+def test_cutoff_against_a_sort(grid, block, values, tau):
+    """Both routes find the cutoff whatever the scores look like: against a sort in 64 bits.  The sums of 3 million fp32 weights are
+    off by 1e-6 of the whole, those of the small route (up to 112 per thread) by no more."""
+    shape = _shape(2, grid, block)
     heads, S, Nb = shape.heads, shape.S, shape.n_blocks
     g = torch.Generator(device="cuda").manual_seed(7)
     x = torch.randn((heads, S, Nb), generator=g, device="cuda")
@@ -161,13 +161,12 @@ def test_last_candidates_of_a_small_pool_are_added_up_in_64_bits():
 
 @pytest.mark.parametrize("values", ["constant", "zeros", "two", "infinite", "nan"])
 @pytest.mark.parametrize("rule,tau,topk", [(vb.SELECT_THRESHOLD_GLOBAL, 0.3, 0), (vb.SELECT_TOPK_GLOBAL, 0.0, 2)])
-@pytest.mark.parametrize("total", [None, WINDOW_MIN])
-def test_pool_kernel_special_scores(values, rule, tau, topk, total):
+def test_pool_kernel_special_scores(values, rule, tau, topk):
     """Ties, infinities and NaN come out as they do from the passes over the matrix (same copies as above)."""
     heads, grid, block = 2, (4, 13, 11), (1, 13, 11)
     small = _shape(heads, grid, block)
     S, Nb = small.S, small.n_blocks
-    copies, large = _copies(small, total)
+    copies, large = _copies(small)
     g = torch.Generator(device="cuda").manual_seed(3)
     x = torch.randn((heads, S, Nb), generator=g, device="cuda")
     if values == "constant":
