@@ -408,6 +408,7 @@ mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, 
   const int q0 = seg * QSEG;
   const int nq = min(QSEG, S - q0);
   const uint32_t cutoff = st[bh].cutoff_key;
+  const float cut = key_float(cutoff);
   for (int i = threadIdx.x; i < QSEG * mw; i += blockDim.x) s_mask[i] = 0u;
   for (int i = threadIdx.x; i < Nb; i += blockDim.x) s_cnt[i] = 0;
   for (int i = threadIdx.x; i < Nb * TW; i += blockDim.x) s_tm[i] = 0u;
@@ -419,8 +420,9 @@ mark_kernel(const float* __restrict__ scores, const HeadState* __restrict__ st, 
   // least 0.5 / Nb away from an integer, the rounding error far less (a fix-up step covers the rest)
   const float inv_nb = 1.0f / (float)Nb;
   auto mark = [&](long long i, float s) {
+    if (s < cut && own_sb <= 0) return;       // the common case: one comparison, no index arithmetic (what is left: NaN, zeros, the selected)
     const bool sel = pool_key(s) >= cutoff;
-    if (!sel && own_sb <= 0) return;          // the common case: no index arithmetic at all
+    if (!sel && own_sb <= 0) return;
     const int ii = (int)i;
     int ql = (int)(((float)ii + 0.5f) * inv_nb), j = ii - ql * Nb;
     if (j < 0) { --ql; j += Nb; } else if (j >= Nb) { ++ql; j -= Nb; }     // belt and braces for huge Nb
