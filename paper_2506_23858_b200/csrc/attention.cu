@@ -140,9 +140,13 @@ static int simt_sparse_bwd(const Dims& D, const void* q, const void* k, const vo
                                              : simt::attn_bwd_dkdv_kernel<T, DH, false, simt::kDqNone>;
   const int C = tiles <= simt::kDqClusterMax ? (int)tiles : 1;
   VMOBA_CUDA_OK(allow_smem(dkdv, simt::kBwdSmem<DH>));
-  launch_cluster(early, C, dkdv, C * grid_for(n_kb * tiles / C, std::max(1, 4 / C)), simt::kThreads, simt::kBwdSmem<DH>, st,
-                 (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr, q_idx, D.S, D.Nb, D.sb, D.BH, D.scale, cap,
-                 (T*)dk, (T*)dv, acc);
+  const int grid = C * grid_for(n_kb * tiles / C, std::max(1, 4 / C));
+  auto go = [&](auto launch) {
+    launch(dkdv, grid, simt::kThreads, simt::kBwdSmem<DH>, st, (const T*)q, (const T*)k, (const T*)v, (const T*)d_o, lse, w.Dv, kb_ptr,
+           q_idx, D.S, D.Nb, D.sb, D.BH, D.scale, cap, (T*)dk, (T*)dv, acc);
+  };
+  if (C > 1) go([&](auto&&... a) { launch_cluster(early, C, a...); });
+  else go([&](auto&&... a) { launch_kernel(early, a...); });
   count_launches(2);
   if (tiles > simt::kDqClusterMax) {
     launch_kernel(simt::item_ptr_kernel, 1, 1024, 0, st, kb_ptr, n_kb, simt::kRows, cap, w.item_ptr, nullptr, 0);

@@ -106,10 +106,13 @@ __device__ __forceinline__ Item decode_sparse(int item, const int* __restrict__ 
 // Tiles in shared memory: 64 rows of DH (or 64) floats, four more to a row, so that sixteen consecutive rows' float4 lie in
 // different banks.
 //
-// The products below are bound by the FMA pipe: 64 FMAs per eight 16-byte loads from shared memory.  With four threads to a row,
-// each holding a quarter of its channels, a key cost a thread as many loads as four of its FMAs and two shuffles.
-// Forward and backward of 13 heads x 4,096 tokens, head_dim 128, 2440 -> 1084 us; of 2 x 256, head_dim 64, 99.2 -> 66.2; dense, 4 x
-// 2,000, head_dim 64, bf16, 1361 -> 829.
+// A 64 x 64 product takes a thread 64 FMAs per eight 16-byte loads from shared memory.  With four threads to a row, each holding a
+// quarter of its channels, a key cost a thread as many loads as four of its FMAs and two shuffles.  fp32 layer,
+// forward and backward: 13 heads x 4,096 tokens in blocks of 512 keys 4570 -> 2256 us (head_dim 128), 2136 -> 1275 (64), 8 x 2,496 in
+// blocks of 156 307 -> 197, 2 x 256 123 -> 77; dense, 4 x 2,000, head_dim 64, bf16, 1361 -> 829.  What bounds them now (13 x 4,096, blocks of 512 keys): the shared-memory pipe, 71 and 74 % busy in the forwards of head_dim 64
+// and 128, and the latency that 16 warps per SM (8 in the backward of head_dim 128: registers) do not hide, 54 to 64 % of the issue
+// slots taken; the FMA pipe is 40 to 45 % busy.  At the 128 registers of two CTAs per SM all kernels but the backward of
+// head_dim 128 spill: 16 to 168 bytes of stack.  Dense calls of few tiles leave SMs idle (4 x 2,000: 128 tiles).
 template <int DH> constexpr int kLd = DH + 4;
 template <int DH> constexpr int kTileFloats = kRows * kLd<DH>;
 constexpr int kLdP = kRows + 4;
