@@ -95,3 +95,23 @@ def test_long_blocks(d, dtype):
         err = float((L.dq_bm[0, h].double() - want).norm() / want.norm())
         # 3,600 roundings of 2^-24 would be 2e-4 if all went one way; at random sixty of them, and the bf16 result's own
         assert err <= (1e-5 if dtype == "f32" else 4e-3), err
+
+
+@pytest.mark.parametrize("sb,nb", [(64, 4), (200, 4), (720, 3)])
+def test_a_captured_backward_replays(sb, nb):
+    """The three routes of dq in a graph: what it writes is what the call writes."""
+    L, blocks = _layer(sb, nb, 64, "f32", seed=2)
+    L.attn_bwd()
+    torch.cuda.synchronize()
+    want = [x.clone() for x in (L.dq_bm, L.dk_bm, L.dv_bm)]
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        L.attn_bwd()
+    for _ in range(3):
+        for x in (L.dq_bm, L.dk_bm, L.dv_bm):
+            x.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(L.dk_bm, want[1]) and torch.equal(L.dv_bm, want[2])
+        assert torch.equal(L.dq_bm[0][blocks <= 2], want[0][0][blocks <= 2])
+    L.check_status()
